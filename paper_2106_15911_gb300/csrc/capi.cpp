@@ -14,6 +14,7 @@
 #include "handle.h"
 #include "host_math.h"
 #include "kernels.h"
+#include "m2l.h"
 #include "nf_tc.h"
 #include "nf_crt.h"
 #include "pfmm_internal.h"
@@ -357,6 +358,7 @@ int pfmm::apply_same_step(pfmm_handle *H, const double *x, double *f, int ns, vo
     g.perm = H->d_perm;
     g.nsm = H->nsm;
     g.m2l_force = H->m2l_force;
+    g.fold = H->fold;
     launch_permute_in(x, xint, H->mixed, 1, g, st);
     if (H->otf) {
         cudaMemsetAsync(fint, 0, sizeof(double) * ns * (size_t)H->nt, st);
@@ -682,6 +684,32 @@ static int build_impl(const pfmm_mesh *mesh, const pfmm_params *prm, cudaStream_
             if ((rc = H->alloc(&E1, ne)) || (rc = H->alloc(&pref, 2 * (size_t)na * na))) return rc;
             launch_e1_table(na, prm->m_t, mx, L.G, L.hx, L.hxp, L.ht, H->alpha, E1, pref, st);
             CK(cudaGetLastError());
+            if (L.G == 4 && H->fprec != 0) {  // before E1 is converted in place
+                if ((rc = H->alloc(&D.EF, m2l_fold_table_floats(na, mx, H->fprec)))) return rc;
+                launch_m2l_fold_table(E1, na, mx, D.ntr, H->fprec, D.EF, st);
+                for (int s = 0; s < 2; ++s) {
+                    const int eng = s ? kM2LFusedSliced : kM2LFused;
+                    if (H->fold[s].units || m2l_engine_for(H->fprec, 4, H->nk, H->ne, mx, s ? 4 : 2) != eng) continue;
+                    const M2LFoldPlan P = m2l_fold_plan(H->fprec, mx, kinv, s == 1);
+                    M2LFoldDev &F = H->fold[s];
+                    int *units = nullptr, *urow = nullptr;
+                    if ((rc = upload(H, &units, P.units, st)) || (rc = upload(H, &urow, P.urow, st))) return rc;
+                    CK(cudaStreamSynchronize(st));  // P's arrays go out of scope
+                    F.urows = P.urows;
+                    F.nslice = P.nslice;
+                    F.nunits = (int)P.units.size() / 2;
+                    F.first3 = P.first3;
+                    F.q3 = P.q3;
+                    for (int i = 0; i < 2; ++i) F.ntask[i] = P.ntask[i];
+                    for (int i = 0; i < kM2LMaxSlices; ++i) {
+                        F.first2[i] = P.first2[i];
+                        F.ntask2[i] = P.ntask2[i];
+                    }
+                    F.smem = P.smem;
+                    F.units = units;
+                    F.urow = urow;
+                }
+            }
             if ((rc = device_to_R(H, &D.E1, E1, ne, st)) || (rc = device_to_R(H, &D.pref, pref, 2 * (size_t)na * na, st)))
                 return rc;
         }
@@ -912,6 +940,7 @@ static int apply_impl(pfmm_handle *H, int op, const double *x, double *f, int nr
     g.eoff = H->d_eoff;
     g.nsm = H->nsm;
     g.m2l_force = H->m2l_force;
+    g.fold = H->fold;
     if ((int)t.panels.size() == g.nbox_leaf) {  // one row panel per leaf box: its 64-row tiles
         g.tiles = H->d_tiles;
         g.ntiles = H->ntiles;

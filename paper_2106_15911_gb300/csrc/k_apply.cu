@@ -19,6 +19,7 @@
 #include "df64.cuh"
 #include "device_math.cuh"
 #include "kernels.h"
+#include "m2l.h"
 
 namespace pfmm {
 
@@ -810,7 +811,7 @@ __global__ void k_m2l_s3(M2LArgs A, const R *__restrict__ E1, const R *__restric
 // Split mode (levels with too few intervals to fill the GPU): one CTA per (k, b, source term)
 // with source term = (J, a) of the interaction list; each term's locals go to its own slice of a
 // workspace and k_m2l_sum_terms adds the slices in a fixed order (deterministic).
-constexpr int FGMax = 4;  // padded grid extent per direction: 4, or 2 for the coarse levels (G <= 2)
+constexpr int FGMax = 4;  // largest grid extent of the fused kernels
 
 // C(n, 4), 0 for n < 4: the budget rows of all triples with |t| <= n - 4 (slice offsets of T2)
 __host__ __device__ inline int binom4(int n) { return n < 4 ? 0 : n * (n - 1) * (n - 2) * (n - 3) / 24; }
@@ -1219,7 +1220,13 @@ int m2l_fused_fg(int G) { return G <= 2 ? 2 : FGMax; }
 
 size_t m2l_fused_smem(int G, int nk, int ne, int mx, size_t es, bool sliced)
 {
-    const int FG = m2l_fused_fg(G), CS = FG * FG * FG + 1, m1 = mx + 1;
+    const int FG = m2l_fused_fg(G), m1 = mx + 1;
+    if (FG == FGMax) {  // the folded kernel: rows of 64 cells, eight coefficients, unit tables (padded tasks)
+        const size_t urows = sliced ? (size_t)nk : (size_t)std::max(ne, nk);
+        return es * (((size_t)ne + urows) * 64 + (size_t)m1 * m1 * 8) +
+               8 * ((size_t)2 * nk + ne + 4 * m1 * (2 + kM2LMaxSlices / 2)) + 4 * (64 + (size_t)nk);
+    }
+    const int CS = FG * FG * FG + 1;
     const size_t urows = sliced ? (size_t)nk : (size_t)std::max(ne, nk);
     return es * (((size_t)ne + urows) * CS + (size_t)7 * m1 * m1) +
            4 * ((size_t)3 * nk + (size_t)m1 * m1 * m1 + FG * FG * FG + ne);
@@ -1282,6 +1289,10 @@ int launch_m2l(int prec, const DevLevel &L, int l, const void *mu, void *lam, in
         using R = decltype(tag);
         if (engine == kM2LFused || engine == kM2LFusedSliced) {
             const bool sl = engine == kM2LFusedSliced;
+            if (m2l_fused_fg(L.G) == FGMax) {
+                rc = launch_m2l_folded(prec, L, g.fold[sl ? 1 : 0], mb, lb, nrhs, g, T1, ws_elems, st);
+                return;
+            }
             const size_t fsm = m2l_fused_smem(L.G, g.nk, g.ne, g.mx, es, sl);
             M2LArgs A{L.G, L.ntr, na, g.nk, g.mx, g.ne, L.nint, L.nbox, L.cellbox, L.boxcell, L.pk, L.pJ, 0,
                       g.kidx, g.kinv, g.eoff};
@@ -1292,8 +1303,7 @@ int launch_m2l(int prec, const DevLevel &L, int l, const void *mu, void *lam, in
             const int64_t split_ctas = (int64_t)kM2LSplitCtasPerSm * (g.nsm > 0 ? g.nsm : 152);
             const int split = ((int64_t)L.nint * na * nrhs < split_ctas && (size_t)nterm * nlev <= ws_elems) ? 1 : 0;
             const dim3 grd(L.nint * na * (split ? nterm : 1), nrhs);
-            auto kf = m2l_fused_fg(L.G) == 2 ? (sl ? k_m2l_fused<R, 2, true> : k_m2l_fused<R, 2, false>)
-                                             : (sl ? k_m2l_fused<R, FGMax, true> : k_m2l_fused<R, FGMax, false>);
+            auto kf = sl ? k_m2l_fused<R, 2, true> : k_m2l_fused<R, 2, false>;
             cudaFuncSetAttribute(kf, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fsm);
             kf<<<grd, kM2LThreads, fsm, st>>>(A, (const R *)mb, (const R *)L.E1, (const R *)L.pref, (R *)lb, nrhs,
                                               split, (R *)T1);

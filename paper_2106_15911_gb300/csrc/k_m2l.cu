@@ -1,0 +1,670 @@
+// k_m2l.cu -- M2L of the levels with 4^3 cells (Eq. m2l with Eq. exp_coeffs_3d, one direction at a
+// time; the passes and their budget rows are described at launch_m2l), with every direction folded
+// into its even and odd part.
+//
+// The one-directional coefficients satisfy E_{k,nu}(-o) = (-1)^{k+nu} E_{k,nu}(o), so on the four
+// cells of a direction they are a 4 x 4 Toeplitz matrix that the reflection of the cells maps to
+// itself (k + nu even) or to its negative (odd).  In the folded coordinates
+//   (y0 + y3, y1 + y2 | y0 - y3, y1 - y2)   (index = 2 sector + j, sector 0: even, 1: odd)
+// it is two 2 x 2 blocks, input sector s to output sector s ^ ((k + nu) & 1), with
+//   M^s_ij = (t_{i-j} + (-1)^s t_{i-(3-j)}) / 2,  t_o = E_{k,nu}(o),
+// so a step costs 8 multiply-adds per fibre of four cells instead of 16, and 8 coefficients
+// instead of 7.  The moments are folded once when a CTA loads them, the locals unfolded once when
+// it writes them; the factor 1/2 of the inverse sits in M.
+//
+// One CTA per (target interval k, time node b, chunk of source terms (J, a), rhs).  T1 and T2 live
+// in shared memory, one row of 64 cells per (triple, budget) entry; a row is 16 chunks of four
+// consecutive values, and the four values of a chunk are a fibre of the direction that the next
+// pass sums over, so a fibre is one vector load:
+//   U  row (k2, k3; k1):        [Y3][Y2][Y1]       pass 1 sums over k1, Y1
+//   T1 row (nu1, k3; k2, C):    [X1][Y3][Y2]       pass 2 sums over k2, Y2   (C: budget of T1)
+//   T2 row (nu1, nu2, B'; k3):  [X2][X1][Y3]       pass 3 sums over k3, Y3
+// The rows of one sum are consecutive (passes 1 and 3) or at steps that shrink by one row (pass 2),
+// so all passes are the same short chain: a unit (its rows and its nu) is given to 16 / NF lanes,
+// each with NF fibres in registers, and a warp takes a task of 2 NF units of one length, whose
+// chain is unrolled for that length.  Where the lengths allow it the units of a task share nu
+// (their coefficient loads are one broadcast) and differ in the row key (k3 of T1, nu1 of T2, modulo
+// 4): the chunks of a row are stored at chunk ^ 2 key, so the units' stores go to different banks.
+// Tasks are dealt to the warps longest first, back and forth.  The parity of k + nu alternates with
+// k, so the accumulators are kept relative to the parity of nu and swapped by addressing when they
+// are written.  Double-FP32 rows hold 64 high then 64 low parts.
+#include <cuda_runtime.h>
+
+#include <algorithm>
+#include <cstdint>
+#include <vector>
+
+#include "df64.cuh"
+#include "kernels.h"
+#include "m2l.h"
+
+namespace pfmm {
+
+namespace {
+
+template <typename R>
+struct Form;  // planes: FP32 words per value; NF: fibres per lane; threads and CTAs per SM
+template <>
+struct Form<float> {
+    static constexpr int planes = 1, NF = 2, threads = 256, ctas = 2;
+};
+template <>
+struct Form<df64> {
+    static constexpr int planes = 2, NF = 1, threads = 384, ctas = 1;
+};
+
+__device__ __forceinline__ void load4(const float *p, float (&v)[4])
+{
+    const float4 a = *reinterpret_cast<const float4 *>(p);
+    v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
+}
+__device__ __forceinline__ void load4(const float *p, df64 (&v)[4])
+{
+    const float4 a = *reinterpret_cast<const float4 *>(p), b = *reinterpret_cast<const float4 *>(p + 64);
+    v[0] = df_make(a.x, b.x); v[1] = df_make(a.y, b.y); v[2] = df_make(a.z, b.z); v[3] = df_make(a.w, b.w);
+}
+__device__ __forceinline__ void store1(float *p, float v) { *p = v; }
+__device__ __forceinline__ void store1(float *p, df64 v)
+{
+    v = df_fast_two_sum(v.hi, v.lo);
+    p[0] = v.hi;
+    p[64] = v.lo;
+}
+__device__ __forceinline__ void store4(float *p, const float (&v)[4])
+{
+    *reinterpret_cast<float4 *>(p) = make_float4(v[0], v[1], v[2], v[3]);
+}
+__device__ __forceinline__ void store4(float *p, const df64 (&v)[4])
+{
+    *reinterpret_cast<float4 *>(p) = make_float4(v[0].hi, v[1].hi, v[2].hi, v[3].hi);
+    *reinterpret_cast<float4 *>(p + 64) = make_float4(v[0].lo, v[1].lo, v[2].lo, v[3].lo);
+}
+// the eight coefficients of (nu, k)
+__device__ __forceinline__ void load8(const float *p, float (&e)[8])
+{
+    const float4 a = *reinterpret_cast<const float4 *>(p), b = *reinterpret_cast<const float4 *>(p + 4);
+    e[0] = a.x; e[1] = a.y; e[2] = a.z; e[3] = a.w;
+    e[4] = b.x; e[5] = b.y; e[6] = b.z; e[7] = b.w;
+}
+__device__ __forceinline__ void load8(const float *p, df64 (&e)[8])
+{
+    float h[8], l[8];
+    load8(p, h);
+    load8(p + 8, l);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) e[i] = df_make(h[i], l[i]);
+}
+// acc += a b.  Double-FP32: the high parts by an error-free sum, everything else into the low part,
+// which is normalised only when the sum is stored (12 operations instead of 15)
+__device__ __forceinline__ void step(float &acc, float a, float b) { acc = fmaf(a, b, acc); }
+__device__ __forceinline__ void step(df64 &acc, df64 a, df64 b)
+{
+    const float p = __fmul_rn(a.hi, b.hi);
+    float e = __fmaf_rn(a.hi, b.hi, -p);
+    e = __fmaf_rn(a.hi, b.lo, e);
+    e = __fmaf_rn(a.lo, b.hi, e);
+    float s, t;
+    df_two_sum(acc.hi, p, s, t);
+    acc.hi = s;
+    acc.lo = __fadd_rn(acc.lo, __fadd_rn(t, e));
+}
+__device__ __forceinline__ float norm(float v) { return v; }
+__device__ __forceinline__ df64 norm(df64 v) { return df_fast_two_sum(v.hi, v.lo); }
+__device__ __forceinline__ float diff(float a, float b) { return a - b; }
+__device__ __forceinline__ df64 diff(df64 a, df64 b) { return a + (-b); }
+__device__ __forceinline__ float shfl_x(float v, int m) { return __shfl_xor_sync(0xffffffffu, v, m); }
+__device__ __forceinline__ df64 shfl_x(df64 v, int m)
+{
+    return df_make(__shfl_xor_sync(0xffffffffu, v.hi, m), __shfl_xor_sync(0xffffffffu, v.lo, m));
+}
+
+// one (k, nu) step of a fibre; `odd`: k is odd, the input sectors feed the other accumulators
+template <typename R>
+__device__ __forceinline__ void fibre_step(R (&acc)[4], const R (&in)[4], const R (&e)[8], bool odd)
+{
+    const int o = odd ? 2 : 0;
+    step(acc[o], e[0], in[0]);
+    step(acc[o + 1], e[2], in[0]);
+    step(acc[2 - o], e[4], in[2]);
+    step(acc[3 - o], e[6], in[2]);
+    step(acc[o], e[1], in[1]);
+    step(acc[o + 1], e[3], in[1]);
+    step(acc[2 - o], e[5], in[3]);
+    step(acc[3 - o], e[7], in[3]);
+}
+
+// the chain of a unit: LEN steps from row address p (rows `stride` words apart, then `stride - dec`
+// and so on; fibre f is f chunks of LPU further on) with the coefficients at e; after(j) sees the
+// partial sums of every step
+template <typename R, int LEN, typename After>
+__device__ __forceinline__ void chain(R (&acc)[Form<R>::NF][4], const float *p, int stride, int dec, int fstep,
+                                      const float *e, After after)
+{
+    constexpr int PL = Form<R>::planes, NF = Form<R>::NF;
+#pragma unroll
+    for (int f = 0; f < NF; ++f)
+#pragma unroll
+        for (int r = 0; r < 4; ++r) acc[f][r] = R(0);
+#pragma unroll
+    for (int j = 0; j < LEN; ++j) {
+        R ev[8], in[NF][4];
+        load8(e + j * 8 * PL, ev);
+        load4(p, in[0]);
+        if (NF == 2) load4(p + fstep, in[NF - 1]);
+#pragma unroll
+        for (int f = 0; f < NF; ++f) fibre_step(acc[f], in[f], ev, j & 1);
+        after(j);
+        p += stride;
+        stride -= dec;
+    }
+}
+
+// run the chain for the task's length (at most m_x + 1 = 9): in FP32 unrolled for that length; in
+// double-FP32 two steps at a time (a step is some 120 instructions: unrolled for every length the
+// three passes no longer fit the instruction cache, and the 12288 x 256 product's M2L took 1.79 ms
+// instead of 0.97)
+template <typename After>
+__device__ __forceinline__ void chain_of(int len, float (&acc)[Form<float>::NF][4], const float *p, int stride, int dec,
+                                         int fstep, const float *e, After after)
+{
+    switch (len) {
+    case 1: chain<float, 1>(acc, p, stride, dec, fstep, e, after); break;
+    case 2: chain<float, 2>(acc, p, stride, dec, fstep, e, after); break;
+    case 3: chain<float, 3>(acc, p, stride, dec, fstep, e, after); break;
+    case 4: chain<float, 4>(acc, p, stride, dec, fstep, e, after); break;
+    case 5: chain<float, 5>(acc, p, stride, dec, fstep, e, after); break;
+    case 6: chain<float, 6>(acc, p, stride, dec, fstep, e, after); break;
+    case 7: chain<float, 7>(acc, p, stride, dec, fstep, e, after); break;
+    case 8: chain<float, 8>(acc, p, stride, dec, fstep, e, after); break;
+    default: chain<float, 9>(acc, p, stride, dec, fstep, e, after); break;
+    }
+}
+template <typename After>
+__device__ __forceinline__ void chain_of(int len, df64 (&acc)[Form<df64>::NF][4], const float *p, int stride, int dec,
+                                         int fstep, const float *e, After after)
+{
+#pragma unroll
+    for (int r = 0; r < 4; ++r) acc[0][r] = df64(0);
+#pragma unroll 1
+    for (int j = 0; j < len; j += 2) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            if (h == 1 && j + 1 >= len) break;
+            df64 ev[8], in[4];
+            load8(e, ev);
+            load4(p, in);
+            fibre_step(acc[0], in, ev, h == 1);
+            after(j + h);
+            e += 16;
+            p += stride;
+            stride -= dec;
+        }
+    }
+}
+
+// offsets within a row of the four values of chunk c's output fibre: position pos of the chunk goes
+// to chunk (4 pos + c / 4) ^ 2 key, word c % 4; the relative position r is pos ^ 2 (nu mod 2)
+__device__ __forceinline__ void out_offsets(int (&q)[4], int c, int nu, int key)
+{
+    const int base = ((((c >> 2) ^ ((key & 1) << 1)) << 2) | (c & 3)), x = (((nu & 1) << 1) ^ (key >> 1)) << 4;
+#pragma unroll
+    for (int r = 0; r < 4; ++r) q[r] = base + ((r << 4) ^ x);
+}
+
+// a unit's words
+struct UnitBits {
+    int row, nu, key, okey, step, slice, len, out;
+    bool valid;
+    __device__ __forceinline__ explicit UnitBits(int2 d)
+    {
+        row = d.x & 1023;
+        nu = (d.x >> 10) & 15;
+        key = (d.x >> 14) & 3;
+        okey = (d.x >> 16) & 3;
+        step = (d.x >> 18) & 15;
+        len = (d.x >> 22) & 15;
+        slice = (d.x >> 26) & 7;
+        valid = d.x < 0;
+        out = d.y;
+    }
+};
+
+}  // namespace
+
+template <typename R, int Q3>
+__global__ void __launch_bounds__(Form<R>::threads, Form<R>::ctas)
+k_m2l_folded(M2LFoldArgs A, const R *__restrict__ mu, R *__restrict__ lam)
+{
+    using F = Form<R>;
+    constexpr int PL = F::planes, NF = F::NF, LPU = 16 / NF, UPW = 32 / LPU, W = F::threads / 32, RW = 64 * PL;
+    extern __shared__ __align__(16) float sm[];
+    const int nk = A.nk, na = A.na, m1 = A.mx + 1;
+    float *T1 = sm, *U = T1 + A.ne * RW, *Es = U + A.urows * RW;
+    int2 *un = reinterpret_cast<int2 *>(Es + m1 * m1 * 8 * PL);
+    int *cbo = reinterpret_cast<int *>(un + A.nunits);  // [z][x][y] element offset of the cell's box, -1: empty
+    int *urow = cbo + 64;                               // [nk] row of U of a moment
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, sub = lane / LPU, cl = lane % LPU;
+    // grid x: (interval, node, chunk); even intervals have half the terms of odd ones
+    const int chunk = blockIdx.x % A.nchunk, kb = blockIdx.x / A.nchunk;
+    const int b = kb % na, k = A.k_lo + kb / na, rhs = blockIdx.y;
+    const int nterm = k < 2 ? 0 : (k & 1 ? 2 * na : na);
+    const int t_lo = chunk * A.tpc, t_hi = min(nterm, t_lo + A.tpc);
+    if (A.part && t_lo >= t_hi) return;
+    for (int i = threadIdx.x; i < A.nunits; i += F::threads) un[i] = A.units[i];
+    for (int i = threadIdx.x; i < nk; i += F::threads) urow[i] = A.urow[i];
+    for (int i = threadIdx.x; i < 64; i += F::threads) {
+        const int box = A.cellbox[i];
+        cbo[(i & 3) * 16 + (i >> 2)] = box < 0 ? -1 : box * na * nk;
+    }
+
+    R lamr[Q3][NF][4];
+#pragma unroll
+    for (int q = 0; q < Q3; ++q)
+#pragma unroll
+        for (int f = 0; f < NF; ++f)
+#pragma unroll
+            for (int r = 0; r < 4; ++r) lamr[q][f][r] = R(0);
+
+    for (int t = t_lo; t < t_hi; ++t) {
+        // terms (J, a): odd intervals J = k - 3 then k - 2, even ones k - 2
+        const int a = t % na, D = (k & 1) ? 3 - t / na : 2, J = k - D;
+        __syncthreads();  // tables in place; the previous term's pass 3 is done with U and Es
+        const float4 *Eg = reinterpret_cast<const float4 *>(A.EF) + (size_t)(((D - 2) * na + a) * na + b) * m1 * m1 * 2 * PL;
+        for (int i = threadIdx.x; i < m1 * m1 * 2 * PL; i += F::threads) reinterpret_cast<float4 *>(Es)[i] = Eg[i];
+        const R coef = reinterpret_cast<const R *>(A.pref)[((D - 2) * na + a) * na + b];
+        // moments of (J, a): lane = (multi-index, Y3) takes the 16 cells (Y1, Y2), folds them in x and
+        // y and, with the lane of the mirrored Y3, in z
+        const R *mJ = mu + (((size_t)rhs * A.nint + J) * A.nbox * na + a) * nk;
+        for (int i = threadIdx.x; i < ((nk + 7) & ~7) * 4; i += F::threads) {
+            const int z = i & 3, ik = i >> 2;
+            const bool ok = ik < nk;
+            const R *mi = mJ + (ok ? ik : 0);
+            R v[4][4];
+#pragma unroll
+            for (int x = 0; x < 4; ++x) {
+                const int4 o = *reinterpret_cast<const int4 *>(cbo + z * 16 + x * 4);
+                v[x][0] = o.x >= 0 ? mi[o.x] : R(0);
+                v[x][1] = o.y >= 0 ? mi[o.y] : R(0);
+                v[x][2] = o.z >= 0 ? mi[o.z] : R(0);
+                v[x][3] = o.w >= 0 ? mi[o.w] : R(0);
+            }
+#pragma unroll
+            for (int y = 0; y < 4; ++y) {
+                const R a0 = v[0][y], a1 = v[1][y], a2 = v[2][y], a3 = v[3][y];
+                v[0][y] = a0 + a3; v[1][y] = a1 + a2; v[2][y] = diff(a0, a3); v[3][y] = diff(a1, a2);
+            }
+            float *p = U + (ok ? urow[ik] : 0) * RW + (z < 2 ? z : 5 - z) * 16;
+#pragma unroll
+            for (int x = 0; x < 4; ++x) {
+                const R a0 = v[x][0], a1 = v[x][1], a2 = v[x][2], a3 = v[x][3];
+                v[x][0] = a0 + a3; v[x][1] = a1 + a2; v[x][2] = diff(a0, a3); v[x][3] = diff(a1, a2);
+            }
+#pragma unroll
+            for (int y = 0; y < 4; ++y) {
+                R s[4];
+#pragma unroll
+                for (int x = 0; x < 4; ++x) {
+                    const R o = shfl_x(v[x][y], 3);
+                    s[x] = z < 2 ? v[x][y] + o : diff(o, v[x][y]);
+                }
+                if (ok) store4(p + y * 4, s);
+            }
+        }
+        __syncthreads();
+        // pass 1: unit (k2, k3, nu1); the sum over k1 is cumulative, every partial sum is a row of T1
+        for (int ts = warp; ts < A.ntask[0]; ts += W) {
+            const UnitBits u(un[ts * UPW + sub]);
+            int q[NF][4];
+#pragma unroll
+            for (int f = 0; f < NF; ++f) out_offsets(q[f], cl + f * LPU, u.nu, u.okey);
+            float *o = T1 + u.out * RW;
+            R acc[NF][4];
+            chain_of(u.len, acc, U + u.row * RW + cl * 4, RW, 0, LPU * 4, Es + u.nu * m1 * 8 * PL, [&](int j) {
+                if (u.valid) {
+#pragma unroll
+                    for (int f = 0; f < NF; ++f)
+#pragma unroll
+                        for (int r = 0; r < 4; ++r) store1(o + q[f][r] + j * RW, acc[f][r]);
+                }
+            });
+        }
+        __syncthreads();
+        for (int sl = 0; sl < A.nslice; ++sl) {
+            if (sl > 0) __syncthreads();  // pass 3 of the previous slice is done with U
+            // pass 2: unit = row of T2
+            for (int ts = warp; ts < A.ntask2[sl]; ts += W) {
+                const UnitBits u(un[A.first2[sl] + ts * UPW + sub]);
+                R acc[NF][4];
+                chain_of(u.len, acc, T1 + u.row * RW + ((cl ^ (u.key << 1)) << 2), u.step * RW, RW, LPU * 4,
+                            Es + u.nu * m1 * 8 * PL, [](int) {});
+                if (u.valid) {
+                    float *o = U + u.out * RW;
+#pragma unroll
+                    for (int f = 0; f < NF; ++f) {
+                        int q[4];
+                        out_offsets(q, cl + f * LPU, u.nu, u.okey);
+#pragma unroll
+                        for (int r = 0; r < 4; ++r) store1(o + q[r], acc[f][r]);
+                    }
+                }
+            }
+            __syncthreads();
+            // pass 3: unit = multi-index of the locals, fixed per lane over all terms
+#pragma unroll
+            for (int q = 0; q < Q3; ++q) {
+                const int ts = warp + q * W;
+                if (ts >= A.ntask[1]) break;
+                const UnitBits u(un[A.first3 + ts * UPW + sub]);
+                if (u.slice != sl) continue;
+                R acc[NF][4];
+                chain_of(u.len, acc, U + u.row * RW + ((cl ^ (u.key << 1)) << 2), RW, 0, LPU * 4,
+                            Es + u.nu * m1 * 8 * PL, [](int) {});
+#pragma unroll
+                for (int f = 0; f < NF; ++f)
+#pragma unroll
+                    for (int r = 0; r < 4; ++r) step(lamr[q][f][r], coef, norm(acc[f][r]));
+            }
+        }
+    }
+    // unfold: in z per lane (row = multi-index: [X3][X2][X1]), then in y and x per (multi-index, X3)
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < Q3; ++q) {
+        const int ts = warp + q * W;
+        if (ts >= A.ntask[1]) break;
+        const UnitBits u(un[A.first3 + ts * UPW + sub]);
+        if (!u.valid) continue;
+        const bool odd = u.nu & 1;
+#pragma unroll
+        for (int f = 0; f < NF; ++f) {
+            const R(&l)[4] = lamr[q][f];
+            const R p0 = norm(odd ? l[2] : l[0]), p1 = norm(odd ? l[3] : l[1]), n0 = norm(odd ? l[0] : l[2]),
+                    n1 = norm(odd ? l[1] : l[3]);
+            float *p = U + u.out * RW + cl + f * LPU;
+            store1(p, p0 + n0);
+            store1(p + 16, p1 + n1);
+            store1(p + 32, diff(p1, n1));
+            store1(p + 48, diff(p0, n0));
+        }
+    }
+    __syncthreads();
+    R *out = (A.part ? reinterpret_cast<R *>(A.part) + (size_t)chunk * A.nlev : lam) +
+             (((size_t)rhs * A.nint + k) * A.nbox * na + b) * nk;
+    for (int i = threadIdx.x; i < nk * 4; i += F::threads) {
+        const int z = i & 3, iv = i >> 2;
+        const float *p = U + iv * RW + z * 16;
+        R v[4][4];  // [y][x]
+#pragma unroll
+        for (int y = 0; y < 4; ++y) {
+            R q[4];
+            load4(p + y * 4, q);
+            v[y][0] = q[0] + q[2]; v[y][1] = q[1] + q[3]; v[y][2] = diff(q[1], q[3]); v[y][3] = diff(q[0], q[2]);
+        }
+        const int4 *co = reinterpret_cast<const int4 *>(cbo + z * 16);
+        R *ov = out + iv;
+#pragma unroll
+        for (int x = 0; x < 4; ++x) {
+            const R q0 = v[0][x], q1 = v[1][x], q2 = v[2][x], q3 = v[3][x];
+            const int4 o = co[x];
+            if (o.x >= 0) ov[o.x] = q0 + q2;
+            if (o.y >= 0) ov[o.y] = q1 + q3;
+            if (o.z >= 0) ov[o.z] = diff(q1, q3);
+            if (o.w >= 0) ov[o.w] = diff(q0, q2);
+        }
+    }
+}
+
+// lam = sum of the chunk slices in order; interval k has ceil(terms / tpc) slices (none for k < 2)
+template <typename R>
+__global__ void k_m2l_sum_chunks(const R *__restrict__ part, int na, int tpc, size_t n, size_t per_k, int nint,
+                                 R *__restrict__ lam)
+{
+    const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const int k = (int)((i / per_k) % nint);
+    const int nterm = k < 2 ? 0 : (k & 1 ? 2 * na : na), nc = (nterm + tpc - 1) / tpc;
+    R s = R(0);
+    for (int t = 0; t < nc; ++t) s += part[(size_t)t * n + i];
+    lam[i] = s;
+}
+
+// folded coefficients of a level from its FP64 table E1 [D][a][b][o][k][nu] (offsets beyond the
+// interaction radius are zero): EF [D][a][b][nu][k][8], in FP32 or as 8 high and 8 low parts
+__global__ void k_m2l_fold_table(const double *__restrict__ E1, int na, int m1, int ntr, int planes, float *__restrict__ EF)
+{
+    const int gid = blockIdx.x * blockDim.x + threadIdx.x, esz = m1 * m1;
+    if (gid >= 2 * na * na * esz) return;
+    const int k = gid % m1, nu = (gid / m1) % m1;
+    const double *E = E1 + (size_t)(gid / esz) * 7 * esz + k * m1 + nu;
+    float *o = EF + (size_t)gid * 8 * planes;
+    for (int s = 0; s < 2; ++s)
+        for (int i = 0; i < 2; ++i)
+            for (int j = 0; j < 2; ++j) {
+                const int o1 = i - j, o2 = i - 3 + j;
+                const double t1 = (o1 < 0 ? -o1 : o1) <= ntr ? E[(o1 + 3) * esz] : 0.0;
+                const double t2 = (o2 < 0 ? -o2 : o2) <= ntr ? E[(o2 + 3) * esz] : 0.0;
+                const double m = 0.5 * (s == 0 ? t1 + t2 : t1 - t2);
+                const int at = s * 4 + i * 2 + j;
+                o[at] = (float)m;
+                if (planes == 2) o[at + 8] = (float)(m - (double)(float)m);
+            }
+}
+
+void launch_m2l_fold_table(const double *E1, int na, int mx, int ntr, int prec, float *EF, cudaStream_t st)
+{
+    const int n = 2 * na * na * (mx + 1) * (mx + 1);
+    k_m2l_fold_table<<<(n + 127) / 128, 128, 0, st>>>(E1, na, mx + 1, ntr, prec == 1 ? 1 : 2, EF);
+}
+
+size_t m2l_fold_table_floats(int na, int mx, int prec)
+{
+    return (size_t)2 * na * na * (mx + 1) * (mx + 1) * 8 * (prec == 1 ? 1 : 2);
+}
+
+namespace {
+
+struct Unit {
+    int row, nu, key, okey, step, slice, len, out;
+    bool valid;
+    int word() const
+    {
+        return row | nu << 10 | key << 14 | okey << 16 | step << 18 | len << 22 | slice << 26 | (valid ? INT32_MIN : 0);
+    }
+};
+
+// units into tasks of `upw` of one length and slice, of one nu and different okey where that can be
+// had; incomplete tasks are filled with units that store nothing.  Longest tasks first, dealt to
+// `warps` warps back and forth.  Appends the units' words, returns the number of tasks
+int deal(const std::vector<Unit> &u, int upw, int warps, std::vector<int> &out)
+{
+    std::vector<std::vector<Unit>> tasks;
+    int maxlen = 0, maxslice = 0;
+    for (const Unit &q : u) {
+        maxlen = std::max(maxlen, q.len);
+        maxslice = std::max(maxslice, q.slice);
+    }
+    for (int sl = 0; sl <= maxslice; ++sl)
+        for (int len = maxlen; len >= 1; --len) {
+            std::vector<Unit> g;
+            for (const Unit &q : u)
+                if (q.slice == sl && q.len == len) g.push_back(q);
+            while (!g.empty()) {
+                std::vector<Unit> t;
+                while ((int)t.size() < upw && !g.empty()) {
+                    size_t best = 0;
+                    int score = -1;
+                    for (size_t i = 0; i < g.size(); ++i) {
+                        bool fresh = true;
+                        for (const Unit &q : t) fresh = fresh && q.okey != g[i].okey;
+                        const int sc = (fresh ? 2 : 0) + (t.empty() || t[0].nu == g[i].nu ? 1 : 0);
+                        if (sc > score) {
+                            score = sc;
+                            best = i;
+                        }
+                    }
+                    t.push_back(g[best]);
+                    g.erase(g.begin() + best);
+                }
+                while ((int)t.size() < upw) {
+                    Unit d = t[0];
+                    d.valid = false;
+                    t.push_back(d);
+                }
+                tasks.push_back(t);
+            }
+        }
+    std::stable_sort(tasks.begin(), tasks.end(), [](const std::vector<Unit> &a, const std::vector<Unit> &b) { return a[0].len > b[0].len; });
+    const int n = (int)tasks.size();
+    const size_t at = out.size();
+    out.resize(at + 2 * (size_t)n * upw);
+    for (int t = 0; t < n; ++t) {
+        const int r = t / warps, w = t % warps, last = std::min(warps, n - r * warps);
+        const int pos = r * warps + (r & 1 ? last - 1 - w : w);
+        for (int i = 0; i < upw; ++i) {
+            out[at + 2 * ((size_t)pos * upw + i)] = tasks[t][i].word();
+            out[at + 2 * ((size_t)pos * upw + i) + 1] = tasks[t][i].out;
+        }
+    }
+    return n;
+}
+
+}  // namespace
+
+M2LFoldPlan m2l_fold_plan(int prec, int mx, const std::vector<int> &kinv, bool sliced)
+{
+    const int m1 = mx + 1, nf = prec == 1 ? Form<float>::NF : Form<df64>::NF, upw = 2 * nf;
+    const int warps = (prec == 1 ? Form<float>::threads : Form<df64>::threads) / 32;
+    auto iv = [&](int a, int b, int c) { return kinv[((size_t)a * m1 + b) * m1 + c]; };
+    auto tri = [](int n) { return n * (n + 1) / 2; };
+    M2LFoldPlan P;
+    P.nk = (mx + 1) * (mx + 2) * (mx + 3) / 6;
+    P.ne = P.nk * (mx + 4) / 4;
+    // rows of U: (k2, k3), then k1; of T1: (nu1, k3), then k2, then C = nu1 + k3 + k2 .. m_x
+    P.urow.assign(P.nk, 0);
+    std::vector<int> ub((size_t)m1 * m1, 0), tb((size_t)m1 * m1, 0);
+    int r = 0, rt = 0;
+    for (int i = 0; i <= mx; ++i)
+        for (int j = 0; i + j <= mx; ++j) {
+            ub[i * m1 + j] = r;
+            for (int k1 = 0; k1 + i + j <= mx; ++k1) P.urow[iv(k1, i, j)] = r++;
+            tb[i * m1 + j] = rt;
+            rt += tri(mx - i - j + 1);
+        }
+    // slices of nu1: consecutive values whose rows of T2 fit the rows of the moments
+    std::vector<int> slice(m1, 0);
+    auto rows2 = [&](int nu1) {
+        int n = 0;
+        for (int nu2 = 0; nu1 + nu2 <= mx; ++nu2) n += tri(mx - nu1 - nu2 + 1);
+        return n;
+    };
+    P.nslice = 1;
+    P.urows = P.nk;
+    for (int v = 0, fill = 0; v <= mx; ++v) {
+        if (sliced && fill && fill + rows2(v) > P.nk) {
+            P.nslice++;
+            fill = 0;
+        }
+        fill += rows2(v);
+        slice[v] = P.nslice - 1;
+        P.urows = std::max(P.urows, fill);
+    }
+    std::vector<Unit> u1, u3;
+    std::vector<std::vector<Unit>> u2(P.nslice);
+    for (int k2 = 0; k2 <= mx; ++k2)
+        for (int k3 = 0; k2 + k3 <= mx; ++k3)
+            for (int nu1 = 0; nu1 + k2 + k3 <= mx; ++nu1) {
+                const int n = mx - nu1 - k3;  // T1 rows of k2 start after n + 1, n, ... rows of smaller k2
+                u1.push_back({ub[k2 * m1 + k3], nu1, 0, k3 & 3, 0, 0, n - k2 + 1,
+                              tb[nu1 * m1 + k3] + k2 * (n + 1) - tri(k2 - 1), true});
+            }
+    std::vector<int> t2b((size_t)m1 * m1, 0), fill(P.nslice, 0);
+    for (int nu1 = 0; nu1 <= mx; ++nu1)
+        for (int nu2 = 0; nu1 + nu2 <= mx; ++nu2) {
+            t2b[nu1 * m1 + nu2] = fill[slice[nu1]];
+            fill[slice[nu1]] += tri(mx - nu1 - nu2 + 1);
+        }
+    for (int nu1 = 0; nu1 <= mx; ++nu1)
+        for (int nu2 = 0; nu1 + nu2 <= mx; ++nu2) {
+            for (int k3 = 0; nu1 + nu2 + k3 <= mx; ++k3)
+                for (int B = nu1 + nu2 + k3; B <= mx; ++B) {
+                    const int C = B - nu2, s = nu1 + k3;  // k2 = 0 .. C - s; from k2 to k2 + 1: n - k2 rows
+                    u2[slice[nu1]].push_back({tb[nu1 * m1 + k3] + C - s, nu2, k3 & 3, nu1 & 3, mx - s, 0, C - s + 1,
+                                              t2b[nu1 * m1 + nu2] + tri(B - nu1 - nu2) + k3, true});
+                }
+            for (int nu3 = 0; nu1 + nu2 + nu3 <= mx; ++nu3)
+                u3.push_back({t2b[nu1 * m1 + nu2] + tri(mx - nu3 - nu1 - nu2), nu3, nu1 & 3, 0, 0, slice[nu1],
+                              mx - nu1 - nu2 - nu3 + 1, iv(nu1, nu2, nu3), true});
+        }
+    P.ntask[0] = deal(u1, upw, warps, P.units);
+    for (int s = 0; s < P.nslice; ++s) {
+        P.first2[s] = (int)P.units.size() / 2;
+        P.ntask2[s] = deal(u2[s], upw, warps, P.units);
+    }
+    P.first3 = (int)P.units.size() / 2;
+    P.ntask[1] = deal(u3, upw, warps, P.units);
+    P.q3 = (P.ntask[1] + warps - 1) / warps;
+    const int planes = prec == 1 ? 1 : 2;
+    P.smem = sizeof(float) * planes * ((size_t)(P.ne + P.urows) * 64 + (size_t)m1 * m1 * 8) + sizeof(int) * P.units.size() +
+             sizeof(int) * (64 + P.nk);
+    return P;
+}
+
+template <typename R>
+static int launch_T(const M2LFoldArgs &A, int q3, size_t smem, dim3 grd, const void *mu, void *lam, cudaStream_t st)
+{
+    auto kf = q3 <= 4 ? k_m2l_folded<R, 4> : k_m2l_folded<R, 7>;
+    if (q3 > 7) return -1;
+    if (cudaFuncSetAttribute(kf, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return -1;
+    kf<<<grd, Form<R>::threads, smem, st>>>(A, (const R *)mu, (R *)lam);
+    return 0;
+}
+
+int launch_m2l_folded(int prec, const DevLevel &L, const M2LFoldDev &P, const void *mu, void *lam, int nrhs,
+                      const ApplyGeo &g, void *ws, size_t ws_elems, cudaStream_t st)
+{
+    M2LFoldArgs A{};
+    A.na = g.na;
+    A.nk = g.nk;
+    A.mx = g.mx;
+    A.ne = g.ne;
+    A.nint = L.nint;
+    A.nbox = L.nbox;
+    A.urows = P.urows;
+    A.nslice = P.nslice;
+    A.nunits = P.nunits;
+    A.first3 = P.first3;
+    for (int i = 0; i < 2; ++i) A.ntask[i] = P.ntask[i];
+    for (int i = 0; i < kM2LMaxSlices; ++i) {
+        A.first2[i] = P.first2[i];
+        A.ntask2[i] = P.ntask2[i];
+    }
+    A.units = (const int2 *)P.units;
+    A.urow = P.urow;
+    A.cellbox = L.cellbox;
+    A.EF = L.EF;
+    A.pref = L.pref;
+    const size_t per_k = (size_t)L.nbox * g.na * g.nk, nlev = (size_t)nrhs * L.nint * per_k;
+    // terms per CTA: all 2 m_t + 2 of an interval, or, while that leaves fewer than eight CTAs per SM,
+    // three, with the chunks' locals added afterwards
+    const int all = 2 * g.na, tpc = 3, nchunk = (all + tpc - 1) / tpc;
+    const int64_t few = (int64_t)8 * (g.nsm > 0 ? g.nsm : 152);
+    const bool split = (int64_t)L.nint * g.na * nrhs < few && (size_t)nchunk * nlev <= ws_elems;
+    A.tpc = split ? tpc : all;
+    A.nchunk = split ? nchunk : 1;
+    A.k_lo = split ? 2 : 0;
+    A.part = split ? ws : nullptr;
+    A.nlev = nlev;
+    const dim3 grd((unsigned)((L.nint - A.k_lo) * g.na * A.nchunk), nrhs);
+    const int rc = prec == 1 ? launch_T<float>(A, P.q3, P.smem, grd, mu, lam, st) : launch_T<df64>(A, P.q3, P.smem, grd, mu, lam, st);
+    if (rc) return rc;
+    if (split) {
+        const unsigned blocks = (unsigned)((nlev + 255) / 256);
+        if (prec == 1)
+            k_m2l_sum_chunks<float><<<blocks, 256, 0, st>>>((const float *)ws, g.na, A.tpc, nlev, per_k, L.nint, (float *)lam);
+        else
+            k_m2l_sum_chunks<df64><<<blocks, 256, 0, st>>>((const df64 *)ws, g.na, A.tpc, nlev, per_k, L.nint, (df64 *)lam);
+    }
+    return 0;
+}
+
+}  // namespace pfmm

@@ -68,6 +68,15 @@ struct OtfArgs {
 void launch_nf_otf(bool mixed, bool kop, const OtfArgs &a, int nsm, cudaStream_t st);
 
 // ---- apply ------------------------------------------------------------------------------
+// unit tables of the folded M2L of 4^3 levels on the device (k_m2l.cu); units null: not built
+constexpr int kM2LMaxSlices = 8;
+struct M2LFoldDev {
+    int urows, nslice, nunits, first3, q3;
+    int ntask[2], first2[kM2LMaxSlices], ntask2[kM2LMaxSlices];
+    const int *units, *urow;
+    size_t smem;
+};
+
 struct ApplyGeo {
     int nt, nv, Et, ls, nd, na, nk, mx, p;
     const int *perm;       // [nt] internal -> caller triangle
@@ -83,6 +92,7 @@ struct ApplyGeo {
     const int *box_tiles;  // [nbox_p + 1] first tile of each leaf box (tiles are box-major)
     int nsm;               // streaming multiprocessors of the device (grid sizing)
     int m2l_force;         // M2L engine asked for by the batch autotuner (PFMM_M2L_* code, 0: none)
+    const M2LFoldDev *fold;// [2] unit tables of the folded M2L: T2 whole, T2 sliced
 };
 
 // prec of the FMM launchers: 0 FP64, 1 FP32 (mixed mode), 2 double-FP32 (FP64 mode); every

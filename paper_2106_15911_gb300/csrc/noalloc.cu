@@ -125,6 +125,7 @@ extern "C" int pfmm_apply_V_noalloc(pfmm_handle *H, const double *w, double *f, 
     g.eoff = H->d_eoff;
     g.nsm = H->nsm;
     g.m2l_force = H->m2l_force;
+    g.fold = H->fold;
     if ((int)H->tree.panels.size() == g.nbox_leaf) {  // one row panel per leaf box: its 64-row tiles
         g.tiles = H->d_tiles;
         g.ntiles = H->ntiles;
