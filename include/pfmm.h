@@ -105,8 +105,8 @@ typedef struct pfmm_params {
                            numbers, about 48 significant bits, on the FP32 pipe); 1: every phase on
                            the FP64 pipe (reference mode, about 50x slower on GB300) */
     int32_t nf_form;    /* FP64 tensor-core nearfield kernel form: 0 (default) the faster of the two,
-                           timed at build; 1 one 128-row tile and two moduli per work item; 2 two
-                           row tiles sharing each input stage, one modulus per item */
+                           timed at build; 1 work items of up to 128 leaf intervals; 2 of up to 64
+                           (twice the items, each reading the blocks again) */
 } pfmm_params;
 
 typedef struct pfmm_handle pfmm_handle;

@@ -289,26 +289,21 @@ int pfmm::run_nf_crt(pfmm_handle *H, int op, const double *x, int nrhs, double *
     uint64_t dims[5] = {(uint64_t)cols, 2, (uint64_t)nint, (uint64_t)nrhs, (uint64_t)kCrtModuli};
     uint64_t str[4] = {(uint64_t)cols * 2, (uint64_t)cols * 4, (uint64_t)cols * 4 * nint,
                        (uint64_t)cols * 4 * nint * nrhs};
-    uint32_t box[5] = {64, 1, 128, 1, 1};
+    uint32_t box[5] = {64, 1, (uint32_t)nf_crt_intervals(nint, H->crt_form), 1, 1};
     CUtensorMap mW;
     if ((rc = encode_map(&mW, H->d_Wres, 5, dims, str, box))) return rc;
     NfCrtParams P{};
-    P.panels = H->d_panels;
-    P.tiles = H->d_tiles128;
-    P.ntiles = H->ntiles128;
-    P.nib = (nint + 127) / 128;
+    P.A = op == 0 ? H->d_AVres : H->d_AKres;
+    P.ntiles = (H->nt + 127) / 128;
     P.nkb = cols / 64;
     P.nrhs = nrhs;
-    P.nitems = (kCrtModuli / 2) * nrhs * P.ntiles * P.nib;
-    P.cols_pad = cols;
-    P.kop = op;
     P.nint = nint;
     P.Et = H->Et;
     P.nt = H->nt;
     P.res = H->d_res8;
     P.err = H->d_err;
     if (H->cur_ev) cudaEventRecord(H->cur_ev->ev[9], st);
-    if (launch_nf_apply_crt(op == 0 ? H->mapAVres : H->mapAKres, mW, P, H->nsm, st, H->crt_form))
+    if (launch_nf_apply_crt(mW, P, H->nsm, st, H->crt_form))
         return fail(PFMM_ERR_CUDA, std::string("FP64 tensor-core nearfield launch: ") +
                                        cudaGetErrorString(cudaGetLastError()));
     if (H->cur_ev) {
@@ -399,8 +394,8 @@ int pfmm_default_params(pfmm_params *p)
     return PFMM_OK;
 }
 
-// The faster of the two forms of the FP64 tensor-core nearfield (one row tile and two moduli per
-// work item, or two row tiles sharing each input stage), timed with CUDA events on this handle's
+// The faster of the two forms of the FP64 tensor-core nearfield (work items of up to 128 or of up to
+// 64 leaf intervals), timed with CUDA events on this handle's
 // V product of a zero input (the work does not depend on the values).
 static int tune_crt_form(pfmm_handle *H, cudaStream_t st)
 {
@@ -446,14 +441,15 @@ static int tune_crt_form(pfmm_handle *H, cudaStream_t st)
 
 // FP64 mode on panels that span all columns: per-row exponents and the residues of the scaled,
 // rounded panels for the exact tensor-core nearfield.  Skipped (CUDA-core FP64 engine kept) when
-// the residues (32 bytes per stored element) would not leave room on the device.
+// the residues (16 bytes per stored element) would not leave room on the device.
 static int build_crt(pfmm_handle *H, const Tree &t, bool fullV, bool fullK, cudaStream_t st)
 {
     using namespace pfmm;
     if (crt_upload_constants(st)) return fail(PFMM_ERR_CUDA, "CRT constants upload failed");
     size_t free_b = 0, total_b = 0;
     CK(cudaMemGetInfo(&free_b, &total_b));
-    const size_t need = (fullV ? (size_t)t.sizeV : 0) * 2 * kCrtModuli + (fullK ? (size_t)t.sizeK : 0) * 2 * kCrtModuli;
+    const int colsV = t.panels[0].colsV_pad, colsK = t.panels[0].colsK_pad;
+    const size_t need = (fullV ? crt_panel_bytes(H->nt, colsV) : 0) + (fullK ? crt_panel_bytes(H->nt, colsK) : 0);
     if (need > free_b / 10 * 7) return PFMM_OK;
     const int nd = H->nd, npanel = (int)t.panels.size();
     unsigned long long *rowmax = nullptr;
@@ -461,36 +457,27 @@ static int build_crt(pfmm_handle *H, const Tree &t, bool fullV, bool fullK, cuda
     if ((rc = H->alloc(&rowmax, (size_t)H->nt))) return rc;
     for (int op = 0; op < 2; ++op) {
         if (!(op == 0 ? fullV : fullK)) continue;
-        const int cols = op == 0 ? t.panels[0].colsV_pad : t.panels[0].colsK_pad;
-        const size_t n = op == 0 ? (size_t)t.sizeV : (size_t)t.sizeK;
+        const int cols = op == 0 ? colsV : colsK;
         const int b = crt_bits(4ll * cols);
-        int *rexp = nullptr, *rexpR = nullptr;
-        uint16_t *res = nullptr;
-        if ((rc = H->alloc(&rexp, (size_t)H->nt)) || (rc = H->alloc(&rexpR, n / cols)) ||
-            (rc = H->alloc(&res, n * kCrtModuli)))
-            return rc;
+        int *rexp = nullptr;
+        unsigned char *res = nullptr;
+        if ((rc = H->alloc(&rexp, (size_t)H->nt)) || (rc = H->alloc(&res, crt_panel_bytes(H->nt, cols)))) return rc;
         const double *A = (const double *)(op == 0 ? H->d_AV : H->d_AK);
-        launch_crt_row_exps(A, H->d_panels, npanel, op, nd, cols, b, rowmax, H->nt, rexp, rexpR, st);
-        launch_crt_split_panel(A, rexpR, n, cols, res, st);
+        launch_crt_row_exps(A, H->d_panels, npanel, op, nd, b, rowmax, H->nt, rexp, st);
+        launch_crt_split_panel(A, H->d_panels, H->d_tri_leaf, rexp, op, H->nt, cols, res, st);
         CK(cudaStreamSynchronize(st));
         CK(cudaGetLastError());
-        H->release(rexpR);
-        // [modulus][block][64 rows][64 columns]
-        uint64_t dims[4] = {64, 64, (uint64_t)(n / 4096), (uint64_t)kCrtModuli}, str[3] = {128, 8192, (n / 4096) * 8192};
-        uint32_t box[4] = {64, 64, 1, 1};
         if (op == 0) {
             H->colsV_u = cols;
             H->crt_bV = b;
             H->d_AVres = res;
             H->d_rexpV = rexp;
-            if ((rc = encode_map(&H->mapAVres, res, 4, dims, str, box))) return rc;
             H->crtV = true;
         } else {
             H->colsK_u = cols;
             H->crt_bK = b;
             H->d_AKres = res;
             H->d_rexpK = rexp;
-            if ((rc = encode_map(&H->mapAKres, res, 4, dims, str, box))) return rc;
             H->crtK = true;
         }
     }
@@ -1153,7 +1140,8 @@ int pfmm_get_info(const pfmm_handle *h, pfmm_info *info)
     info->nf_form_ms[0] = h->crt_form_ms[0];
     info->nf_form_ms[1] = h->crt_form_ms[1];
     if (h->crtV || h->crtK)
-        info->nearfield_bytes += (h->crtV ? t.sizeV : 0) * 2 * pfmm::kCrtModuli + (h->crtK ? t.sizeK : 0) * 2 * pfmm::kCrtModuli;
+        info->nearfield_bytes += (h->crtV ? pfmm::crt_panel_bytes(h->nt, h->colsV_u) : 0) +
+                                 (h->crtK ? pfmm::crt_panel_bytes(h->nt, h->colsK_u) : 0);
     info->nearfield_v_elements = t.sizeV;
     info->nf_dense_columns = t.dense_cols ? 1 : 0;
     // separable M2L work per level: pass 1 over cells (X1, Y2, Y3) and the budget chains of every

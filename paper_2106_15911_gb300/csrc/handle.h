@@ -103,11 +103,10 @@ struct pfmm_handle {
     // FP64 mode, exact residue-arithmetic nearfield on the tensor cores (k_nf_crt.cu)
     bool crtV = false, crtK = false;
     int crt_bV = 0, crt_bK = 0;                       // fixed-point bits of the operands
-    int crt_form = 1, crt_best_form = 1;              // kernel form (1: two moduli, 2: two row tiles per item)
+    int crt_form = 1, crt_best_form = 1;              // kernel form (intervals per work item: up to 128, up to 64)
     double crt_form_ms[2] = {0, 0};                   // build-time timing of the two forms
-    uint16_t *d_AVres = nullptr, *d_AKres = nullptr;  // FP16 residues [16][panel elements]
+    unsigned char *d_AVres = nullptr, *d_AKres = nullptr;  // residue bytes [16][panel elements]
     int *d_rexpV = nullptr, *d_rexpK = nullptr;       // row scale exponents by triangle
-    CUtensorMap mapAVres{}, mapAKres{};
     uint16_t *d_Wres = nullptr;                       // input residues [16][nrhs][E_t][cols]
     unsigned char *d_res8 = nullptr;                  // output residues [16][nrhs][E_t][E_x]
     uint16_t *d_Whi = nullptr, *d_Wlo = nullptr;  // FP16 input parts

@@ -12,8 +12,8 @@
 //     b chosen so that the exact integer product X = sum A' W' satisfies 2 |X| < M;
 //   * X is computed modulo 16 primes p_i < 256 (M = prod p_i ~ 2^123): the residues of A' and W'
 //     in [-(p-1)/2, (p-1)/2] are exact FP16 numbers, their products are below 2^14, and a tcgen05
-//     kind::f16 MMA chain accumulates them in FP32 exactly (integers below 2^24) over chunks of
-//     1024 columns; after each chunk the epilogue reduces the accumulator modulo p in place
+//     kind::f16 MMA chain accumulates them in FP32 exactly (integers below 2^24) over a chunk of
+//     products; after each chunk the epilogue reduces the accumulator modulo p in place
 //     (tcgen05.ld / .st), so the next chunk adds onto a small residue;
 //   * the 16 residues of X are combined by Garner's mixed-radix algorithm (balanced digits, exact
 //     FP32 arithmetic), X is assembled exactly in 128-bit integers and X 2^-(e_r + s) is rounded
@@ -21,13 +21,28 @@
 // The only rounding before the final FP64 result is that of A and W to b-bit fixed point per row /
 // per rhs (b = 52..53): the product is as accurate as an FP64 dot product of the same terms.
 //
-// Tiles as in the FP16-split kernel: 128 rows x 256 columns (128 leaf intervals x 2 steps), W a
-// TMA tensor [modulus][rhs][interval][phase][column] so the time shift d is a coordinate offset
-// and causality the zero fill.  A work item is (moduli pair, row tile, interval block, rhs): the
-// two moduli alternate chunk by chunk between two TMEM accumulators (2 x 256 columns), so the MMA
-// of one overlaps the epilogue's reduction of the other.  Warp roles (192 threads): warp 0 TMA,
-// warp 1 TMEM allocation and MMA issue, warps 2-5 epilogue (one 32-lane TMEM quadrant each).
-// Four 48 KB smem stages.  Every mbarrier wait is bounded (error word, clean exit).
+// The residues of A' are stored as bytes (r + 128), half the bytes of FP16, because the stored
+// blocks are the bulk of the traffic: 16 bytes per element.  All panels index the same columns, so
+// the rows are tiled regardless of panels: tile t holds the target triangles 128 t .. 128 t + 127, and
+// the four step offsets of one 64-column block of a tile are 32 KB in one piece, [modulus][tile]
+// [column block][d][row][64], brought in by one bulk copy.  Converter warps turn the bytes into FP16
+// in registers (byte permute onto 1024 + u, one subtraction, exact) and write them to tensor memory,
+// from where tcgen05.mma takes them as the A operand.
+//
+// Tiles: 128 rows x (NI leaf intervals x 2 phases) columns; W is a TMA tensor [modulus][rhs]
+// [interval][phase][column], so the time shift d is a coordinate offset and causality the zero fill.
+// For one column block the four step offsets need only four W tiles, (phase 0 or 1) x (interval
+// shift 0 or 1); stored in the order (0, 1), (1, 1), (0, 0), (1, 0), phase ph of offset d is tile
+// 2 + ph - d, so both phases of an offset are one contiguous operand of 2 NI rows, and each W tile is
+// brought in once for its two uses.  A work item is (modulus, row tile, interval block, rhs).  The
+// accumulator of phase 0 is reduced modulo p before column blocks r, 2 r, ..., that of phase 1
+// before r / 2, 3 r / 2, ... (r = 4 .. 8 by the modulus: 256 r products of two residues stay below
+// 2^24): the other phase's MMAs of that block are issued first and hide the reduction.
+// The roles meet once per column block (16 MMAs): a wait, the issue and the commit of a step cost the
+// issuing thread some 400 cycles, which one step per offset (448 cycles of MMAs) did not hide.
+// Warps: 0 TMA of W, 1 TMEM allocation and MMA issue, 2-9 converters (two groups of four, two offsets
+// each, one 32-lane TMEM quadrant per warp), 10-17 epilogue (two warps per quadrant, half the columns
+// each), 18 bulk copies of A.  Every mbarrier wait is bounded (error word, clean exit).
 #include <cuda.h>
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
@@ -50,25 +65,24 @@ using namespace tc;
 __constant__ int c_p[kCrtModuli];              // the moduli
 __constant__ float c_invp[kCrtModuli];         // 1 / p (FP32)
 __constant__ float c_pf[kCrtModuli];           // the moduli (FP32)
+__constant__ int c_red[kCrtModuli];            // column blocks between two reductions of an accumulator (even)
 __constant__ float c_pow11[kCrtModuli][5];     // 2^(11 k) mod p_i (FP32), k = 0 .. 4
 __constant__ float c_pjmodpif[kCrtModuli][kCrtModuli];  // (p_0 ... p_{j-1}) mod p_i, j < i (FP32)
 __constant__ float c_invPif[kCrtModuli];       // (p_0 ... p_{i-1})^-1 mod p_i (FP32)
 
 constexpr int BM = 128, BK = 64;
-constexpr int A_TILE = BM * BK * 2;      // 16 KB
-constexpr int B_HALF = 128 * BK * 2;     // 16 KB per phase
-constexpr int STAGE_BYTES = A_TILE + 2 * B_HALF;  // 48 KB
-constexpr int NSTAGE = 4;
-constexpr int CHUNK = 16;                // stages per exact FP32 accumulation chunk (1024 columns)
+constexpr int A8_TILE = BM * BK;         // 8 KB of residue bytes
+constexpr int A8_STAGE = 4 * A8_TILE;    // the four offsets of a column block
+constexpr int NST = 2;                   // column blocks in flight (bytes, FP16 tiles in tensor memory, W)
+constexpr int kCrtThreads = 608;
+constexpr int kTmemA = 256;              // first tensor memory column of the A tiles (32 columns each, four a stage)
 constexpr uint64_t kTimeoutNs = 2000000000ull;
 
-__device__ __forceinline__ void tma_4d(void *dst, const CUtensorMap *map, int x, int y, int z, int w, uint64_t *bar)
+__device__ __forceinline__ void bulk_copy(void *dst, const void *src, uint32_t bytes, uint64_t *bar)
 {
-    asm volatile(
-        "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], "
-        "[%6];" ::"r"(su32(dst)),
-        "l"((uint64_t)map), "r"(x), "r"(y), "r"(z), "r"(w), "r"(su32(bar))
-        : "memory");
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(su32(dst)),
+                 "l"(src), "r"(bytes), "r"(su32(bar))
+                 : "memory");
 }
 
 __device__ __forceinline__ void tma_5d(void *dst, const CUtensorMap *map, int x, int y, int z, int w, int v,
@@ -87,16 +101,36 @@ __host__ __device__ constexpr uint32_t idesc_f16(int M, int N)
     return (1u << 4) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
-__device__ __forceinline__ void mma_f16(uint32_t dt, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc)
+// The issuing warp runs its loop as a whole, so that addresses and descriptors stay in uniform
+// registers, and one lane issues (16 MMAs from a single lane's branch took 94 cycles each).
+__device__ __forceinline__ uint32_t elect_lane()
+{
+    uint32_t e;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(e));
+    return e;
+}
+
+// A from tensor memory, B from shared memory at descriptor low word blo (K-major, 128-byte swizzle)
+__device__ __forceinline__ void mma_f16_ts(uint32_t issue, uint32_t dt, uint32_t a, uint32_t blo, uint32_t idesc,
+                                           uint32_t acc)
+{
+    constexpr uint32_t hi = (1024 >> 4) | 1u << 14 | 2u << 29;  // 8-row groups 1024 bytes apart, version, swizzle
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t.reg .b64 b;\n\tmov.b64 b, {%2, %6};\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 q, %5, "
+        "0;\n\t@q tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], b, %3, p;\n\t}\n" ::"r"(dt),
+        "r"(a), "r"(blo), "r"(idesc), "r"(acc), "r"(issue), "n"(hi)
+        : "memory");
+}
+__device__ __forceinline__ void mma_commit_if(uint32_t issue, uint64_t *b)
 {
     asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\ttcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::
-            "r"(dt),
-        "l"(a), "l"(b), "r"(idesc), "r"(acc)
+        "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %1, 0;\n\t@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 "
+        "[%0];\n\t}" ::"r"(su32(b)),
+        "r"(issue)
         : "memory");
 }
 
-__device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&r)[32])
+__device__ __forceinline__ void tmem_st32_async(uint32_t taddr, const uint32_t (&r)[32])
 {
     asm volatile(
         "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
@@ -106,60 +140,84 @@ __device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&r)[32
         "r"(r[19]), "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]), "r"(r[24]), "r"(r[25]), "r"(r[26]), "r"(r[27]),
         "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31])
         : "memory");
+}
+
+__device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&r)[32])
+{
+    tmem_st32_async(taddr, r);
     asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
 }
 
 struct CItem {
-    int panel, r0, ib, rhs, m0;  // row tile, interval block, rhs, first modulus of the pair
+    int m, rhs, ib, tile;
+    __device__ __forceinline__ CItem(const NfCrtParams &P, int nib, int it)
+    {
+        // modulus-major: consecutive CTAs share the modulus (its W residues stay in L2)
+        const int per_m = P.ntiles * nib * P.nrhs;
+        m = it / per_m;
+        int r_ = it % per_m;
+        rhs = r_ / (P.ntiles * nib);
+        r_ %= P.ntiles * nib;
+        ib = r_ % nib;
+        tile = r_ / nib;
+    }
 };
 
-__device__ __forceinline__ CItem decode_citem(const NfCrtParams &P, int it)
+// four residue bytes u = r + 128 to FP16: the bytes below 0x64 are 1024 + u, less 1152 is r (exact)
+__device__ __forceinline__ void bytes_to_half(uint32_t w, uint32_t &lo, uint32_t &hi)
 {
-    // pair-major: consecutive CTAs share the moduli (their W residues stay in L2)
-    const int ntile = P.ntiles * P.nib * P.nrhs;
-    CItem I;
-    I.m0 = 2 * (it / ntile);
-    int tile = it % ntile;
-    I.rhs = tile / (P.ntiles * P.nib);
-    int r_ = tile % (P.ntiles * P.nib);
-    I.ib = r_ % P.nib;
-    int rt = r_ / P.nib;
-    I.panel = P.tiles[2 * rt];
-    I.r0 = P.tiles[2 * rt + 1];
-    return I;
+    const __half2 off = __half2half2(__ushort_as_half(0x6480));  // 1152
+    const uint32_t a = __byte_perm(w, 0x64646464u, 0x4140), b = __byte_perm(w, 0x64646464u, 0x4342);
+    const __half2 x = __hsub2(*reinterpret_cast<const __half2 *>(&a), off);
+    const __half2 y = __hsub2(*reinterpret_cast<const __half2 *>(&b), off);
+    lo = *reinterpret_cast<const uint32_t *>(&x);
+    hi = *reinterpret_cast<const uint32_t *>(&y);
 }
 
+template <int NI>
+struct CrtSmem {
+    static constexpr int W_TILE = NI * BK * 2, W_STAGE = 4 * W_TILE;
+    static constexpr size_t bytes = (size_t)NST * (W_STAGE + A8_STAGE) + 1024 + 256;
+};
+
 // x mod p into [-(p-1)/2 - p, (p-1)/2 + p] for an integer-valued |x| < 2^24 (exact): the FP32
-// quotient may be one off near a half-integer, which leaves a congruent value within 1.5 p
+// quotient may be one off near a half-integer, which leaves a congruent value within 1.5 p.  The
+// quotient (below 2^22) is rounded by adding and subtracting 1.5 2^23: rintf runs at an eighth of the
+// FP32 rate, and 64 columns of an accumulator took 1650 cycles to reduce instead of 450
 __device__ __forceinline__ float mod_small(float x, float p, float invp)
 {
-    const float q = rintf(x * invp);
+    const float q = __fsub_rn(__fmaf_rn(x, invp, 12582912.f), 12582912.f);
     return fmaf(-q, p, x);
 }
 
 }  // namespace
 
-__global__ void __launch_bounds__(192, 1) k_nf_apply_crt(const __grid_constant__ CUtensorMap mapA,
-                                                          const __grid_constant__ CUtensorMap mapW, NfCrtParams P)
+template <int NI>
+__global__ void __launch_bounds__(kCrtThreads, 1) k_nf_apply_crt(const __grid_constant__ CUtensorMap mapW, NfCrtParams P)
 {
+    using S = CrtSmem<NI>;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char *smem = (unsigned char *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    uint64_t *full = (uint64_t *)(smem + NSTAGE * STAGE_BYTES);
-    uint64_t *empty = full + NSTAGE;
-    uint64_t *tfull = empty + NSTAGE;
-    uint64_t *tempty = tfull + 2;
+    unsigned char *sA = smem + NST * S::W_STAGE;
+    uint64_t *wfull = (uint64_t *)(sA + NST * A8_STAGE);  // W of a stage has arrived
+    uint64_t *a8full = wfull + NST, *a8empty = a8full + NST;  // residue bytes arrived / read
+    uint64_t *aready = a8empty + NST, *done = aready + NST;   // FP16 tiles in TMEM / the stage's MMAs have completed
+    uint64_t *tfull = done + NST, *tempty = tfull + 2;
     uint32_t *tmem_slot = (uint32_t *)(tempty + 2);
     __shared__ volatile int s_abort;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
-        for (int s = 0; s < NSTAGE; ++s) {
-            mbar_init(&full[s], 1);
-            mbar_init(&empty[s], 1);
+        for (int s = 0; s < NST; ++s) {
+            mbar_init(&wfull[s], 1);
+            mbar_init(&a8full[s], 1);
+            mbar_init(&a8empty[s], 8);  // one arrival per converter warp
+            mbar_init(&aready[s], 8);
+            mbar_init(&done[s], 1);
         }
         for (int a = 0; a < 2; ++a) {
             mbar_init(&tfull[a], 1);
-            mbar_init(&tempty[a], 128);
+            mbar_init(&tempty[a], 8);  // one arrival per epilogue warp
         }
         s_abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -173,361 +231,231 @@ __global__ void __launch_bounds__(192, 1) k_nf_apply_crt(const __grid_constant__
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = *tmem_slot;
-    uint64_t deadline = gtimer() + kTimeoutNs;  // renewed per chunk: each wait is bounded by 2 s
-    const int nst = 4 * P.nkb;                   // stages per modulus: d = 0..3 x column blocks
-    const int nch = (nst + CHUNK - 1) / CHUNK;   // exact accumulation chunks
+    const int nib = (P.nint + NI - 1) / NI;
+    // each wait is bounded by about 2 s; the abort flag ends the other roles' loops
+    auto wait = [&](uint64_t *bar, uint32_t parity, int code) {
+        if (mbar_wait_bounded<true>(bar, parity)) return true;
+        atomicExch(P.err, code);
+        s_abort = 1;
+        return false;
+    };
+    // the same for a whole warp, which goes on or stops together (its TMEM accesses are warp-wide):
+    // one lane polls
+    auto warp_wait = [&](uint64_t *bar, uint32_t parity, int code) {
+        bool go = true;
+        if (lane == 0) go = wait(bar, parity, code) && !s_abort;
+        return __all_sync(0xffffffffu, go) != 0;
+    };
 
     if (warp == 0) {
-        // ---------------- TMA producer: (chunk, slot, stage) in the MMA's order
+        // ---------------- TMA of W: the four (phase, shift) tiles of a column block
         if (lane == 0) {
             int g = 0;
             for (int it = blockIdx.x; it < P.nitems && !s_abort; it += gridDim.x) {
-                const CItem I = decode_citem(P, it);
-                const PanelGPU &Pn = P.panels[I.panel];
-                const bool two = I.r0 + 64 < Pn.nrows;
-                const long long rbase = (P.kop ? Pn.offK : Pn.offV) / P.cols_pad + I.r0;
-                for (int ch = 0; ch < nch && !s_abort; ++ch)
-                    for (int slot = 0; slot < 2 && !s_abort; ++slot) {
-                        deadline = gtimer() + kTimeoutNs;
-                        const int m = I.m0 + slot;
-                        const int st1 = min(nst, (ch + 1) * CHUNK);
-                        for (int st = ch * CHUNK; st < st1; ++st, ++g) {
-                            const int s = g % NSTAGE;
-                            if (!mbar_wait(&empty[s], ((g / NSTAGE) & 1) ^ 1, deadline)) {
-                                atomicExch(P.err, 11);
-                                s_abort = 1;
-                                break;
-                            }
-                            const int d = st / P.nkb, kb = st % P.nkb;
-                            unsigned char *sA = smem + s * STAGE_BYTES;
-                            const uint32_t abytes = two ? A_TILE : A_TILE / 2;
-                            mbar_expect_tx(&full[s], abytes + (d < 3 ? 2 : 1) * B_HALF);
-                            const int blk = (int)((rbase + (long long)d * Pn.rows_pad) >> 6) * P.nkb + kb;
-                            tma_4d(sA, &mapA, 0, 0, blk, m, &full[s]);
-                            if (two) tma_4d(sA + A_TILE / 2, &mapA, 0, 0, blk + P.nkb, m, &full[s]);
-                            unsigned char *sB = sA + A_TILE;
-                            for (int ph = (d < 3 ? 0 : 1); ph < 2; ++ph) {
-                                const int phs = ((ph - d) % 2 + 2) % 2, q = (phs - (ph - d)) / 2;
-                                tma_5d(sB + ph * B_HALF, &mapW, kb * BK, phs, I.ib * 128 - q, I.rhs, m, &full[s]);
-                            }
-                        }
-                    }
+                const CItem I(P, nib, it);
+                for (int kb = 0; kb < P.nkb; ++kb, ++g) {
+                    const int s = g % NST;
+                    if (!wait(&done[s], ((g / NST) & 1) ^ 1, 11) || s_abort) break;
+                    unsigned char *d = smem + s * S::W_STAGE;
+                    mbar_expect_tx(&wfull[s], S::W_STAGE);
+#pragma unroll
+                    for (int q = 0; q < 4; ++q)  // (0, 1), (1, 1), (0, 0), (1, 0)
+                        tma_5d(d + q * S::W_TILE, &mapW, kb * BK, q & 1, I.ib * NI - (q < 2 ? 1 : 0), I.rhs, I.m,
+                               &wfull[s]);
+                }
             }
             const uint64_t dl2 = gtimer() + kTimeoutNs / 20;
-            for (int j = (g > NSTAGE ? g - NSTAGE : 0); j < g; ++j) mbar_wait(&full[j % NSTAGE], (j / NSTAGE) & 1, dl2);
+            for (int j = (g > NST ? g - NST : 0); j < g; ++j) mbar_wait(&wfull[j % NST], (j / NST) & 1, dl2);
+        }
+    } else if (warp == 18) {
+        // ---------------- bulk copies of the A bytes
+        if (lane == 0) {
+            int g = 0;
+            for (int it = blockIdx.x; it < P.nitems && !s_abort; it += gridDim.x) {
+                const CItem I(P, nib, it);
+                const unsigned char *src = P.A + ((size_t)I.m * P.ntiles + I.tile) * P.nkb * A8_STAGE;
+                for (int kb = 0; kb < P.nkb; ++kb, ++g, src += A8_STAGE) {
+                    const int s = g % NST;
+                    if (!wait(&a8empty[s], ((g / NST) & 1) ^ 1, 12) || s_abort) break;
+                    mbar_expect_tx(&a8full[s], A8_STAGE);
+                    bulk_copy(sA + s * A8_STAGE, src, A8_STAGE, &a8full[s]);
+                }
+            }
+            const uint64_t dl2 = gtimer() + kTimeoutNs / 20;
+            for (int j = (g > NST ? g - NST : 0); j < g; ++j) mbar_wait(&a8full[j % NST], (j / NST) & 1, dl2);
         }
     } else if (warp == 1) {
         // ---------------- MMA issuer
-        if (lane == 0) {
-            int g = 0, u = 0;  // u: accumulator uses (both slots advance together)
-            const uint32_t id256 = idesc_f16(BM, 256), id128 = idesc_f16(BM, 128);
-            for (int it = blockIdx.x; it < P.nitems && !s_abort; it += gridDim.x) {
-                for (int ch = 0; ch < nch && !s_abort; ++ch, ++u)
-                    for (int slot = 0; slot < 2 && !s_abort; ++slot) {
-                        deadline = gtimer() + kTimeoutNs;
-                        if (!mbar_wait(&tempty[slot], (u & 1) ^ 1, deadline)) {
-                            atomicExch(P.err, 12);
-                            s_abort = 1;
-                            break;
-                        }
-                        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                        const uint32_t dcol = tmem + slot * 256;
-                        const int st1 = min(nst, (ch + 1) * CHUNK);
-                        for (int st = ch * CHUNK; st < st1; ++st, ++g) {
-                            const int s = g % NSTAGE;
-                            if (!mbar_wait(&full[s], (g / NSTAGE) & 1, deadline)) {
-                                atomicExch(P.err, 13);
-                                s_abort = 1;
-                                break;
-                            }
-                            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                            const int d = st / P.nkb;
-                            const uint32_t a0 = su32(smem + s * STAGE_BYTES), b0 = a0 + A_TILE;
-#pragma unroll
-                            for (int kk = 0; kk < BK / 16; ++kk) {
-                                const uint32_t ko = kk * 32;
-                                // the item's first MMA starts from zero (d = 0 covers both phases)
-                                const uint32_t accf = (ch == 0 && st == 0 && kk == 0) ? 0u : 1u;
-                                if (d < 3)
-                                    mma_f16(dcol, sw128_desc(a0 + ko), sw128_desc(b0 + ko), id256, accf);
-                                else
-                                    mma_f16(dcol + 128, sw128_desc(a0 + ko), sw128_desc(b0 + B_HALF + ko), id128, 1u);
-                            }
-                            mma_commit(&empty[s]);
-                        }
-                        mma_commit(&tfull[slot]);
-                    }
-            }
-        }
-    } else {
-        // ---------------- epilogue: warps 2..5, TMEM lane quadrant = warp % 4
-        const int quad = warp & 3;
-        const int row_l = quad * 32 + lane;
-        int u = 0;
+        const uint32_t issue = elect_lane(), tm = __shfl_sync(0xffffffffu, tmem, 0);
+        const uint32_t wlo = __shfl_sync(0xffffffffu, (su32(smem) >> 4) & 0x3FFFu, 0) | 1u << 16;
+        constexpr uint32_t id2 = idesc_f16(BM, 2 * NI), id1 = idesc_f16(BM, NI), WT = S::W_TILE >> 4;
+        int g = 0;
+        uint32_t ev0 = 0, ev1 = 0;  // accumulator hand-overs of the phases
         for (int it = blockIdx.x; it < P.nitems && !s_abort; it += gridDim.x) {
-            const CItem I = decode_citem(P, it);
-            const PanelGPU &Pn = P.panels[I.panel];
-            const int row = I.r0 + row_l;
-            const bool row_ok = row < Pn.nrows;
-            for (int ch = 0; ch < nch && !s_abort; ++ch, ++u)
-                for (int slot = 0; slot < 2 && !s_abort; ++slot) {
-                    deadline = gtimer() + kTimeoutNs;
-                    if (!mbar_wait(&tfull[slot], u & 1, deadline)) {
-                        atomicExch(P.err, 14);
-                        s_abort = 1;
-                        break;
+            const CItem I(P, nib, it);
+            const int rp = c_red[I.m];
+            // the previous item's outputs have been read
+            bool ok = (ev0 == 0 || wait(&tempty[0], (ev0 - 1) & 1, 13)) && (ev1 == 0 || wait(&tempty[1], (ev1 - 1) & 1, 13));
+            int next0 = rp, next1 = rp / 2;  // column blocks before which a phase is reduced
+            for (int kb = 0; kb < P.nkb && ok; ++kb, ++g) {
+                const int s = g % NST;
+                const uint32_t w0 = wlo + s * (S::W_STAGE >> 4), at = tm + kTmemA + s * 128;
+                const bool r0 = kb == next0, r1 = kb == next1;
+                if (r0) {
+                    mma_commit_if(issue, &tfull[0]);
+                    ++ev0;
+                    next0 += rp;
+                }
+                if (r1) {
+                    mma_commit_if(issue, &tfull[1]);
+                    ++ev1;
+                    next1 += rp;
+                }
+                ok = wait(&wfull[s], (g / NST) & 1, 14) && wait(&aready[s], (g / NST) & 1, 15);
+                if (!ok) break;
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                if (!r0 && !r1) {
+                    const uint32_t more = kb > 0 ? 1u : 0u;  // an item's first MMA starts both phases from zero
+#pragma unroll
+                    for (int d = 0; d < 3; ++d)
+#pragma unroll
+                        for (int kk = 0; kk < BK / 16; ++kk)
+                            mma_f16_ts(issue, tm, at + d * 32 + kk * 8, w0 + (2 - d) * WT + kk * 2, id2,
+                                       d == 0 && kk == 0 ? more : 1u);
+#pragma unroll
+                    for (int kk = 0; kk < BK / 16; ++kk) mma_f16_ts(issue, tm + NI, at + 96 + kk * 8, w0 + kk * 2, id1, 1u);
+                } else {
+                    // the other phase first, while the epilogue reduces this one
+                    auto phase = [&](int ph) {
+#pragma unroll
+                        for (int d = 0; d < 3; ++d)
+#pragma unroll
+                            for (int kk = 0; kk < BK / 16; ++kk)
+                                mma_f16_ts(issue, tm + ph * NI, at + d * 32 + kk * 8, w0 + (2 + ph - d) * WT + kk * 2, id1, 1u);
+                        if (ph == 1)
+#pragma unroll
+                            for (int kk = 0; kk < BK / 16; ++kk)
+                                mma_f16_ts(issue, tm + NI, at + 96 + kk * 8, w0 + kk * 2, id1, 1u);
+                    };
+                    if (r0) {
+                        phase(1);
+                        if (!(ok = wait(&tempty[0], (ev0 - 1) & 1, 16))) break;
+                        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                        phase(0);
+                    } else {
+                        phase(0);
+                        if (!(ok = wait(&tempty[1], (ev1 - 1) & 1, 17))) break;
+                        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                        phase(1);
                     }
+                }
+                mma_commit_if(issue, &done[s]);
+            }
+            mma_commit_if(issue, &tfull[0]);
+            mma_commit_if(issue, &tfull[1]);
+            ++ev0;
+            ++ev1;
+        }
+    } else if (warp < 10) {
+        // ---------------- converters: thread = row; the bytes of two offsets to FP16 pairs in TMEM
+        const int row = (warp & 3) * 32 + lane, d0 = (warp - 2) >> 2 << 1;
+        const uint32_t tq = tmem + ((uint32_t)((warp & 3) * 32) << 16) + kTmemA + d0 * 32;
+        int g = 0;
+        bool ok = true;
+        for (int it = blockIdx.x; it < P.nitems && ok; it += gridDim.x)
+            for (int kb = 0; kb < P.nkb; ++kb, ++g) {
+                const int s = g % NST;
+                if (!(ok = warp_wait(&a8full[s], (g / NST) & 1, 18))) break;
+                uint4 b[2][4];
+#pragma unroll
+                for (int d = 0; d < 2; ++d) {
+                    // 16-byte chunk c of row r is at c ^ ((r / 2) mod 4): a quarter warp reads all banks
+                    const unsigned char *src = sA + s * A8_STAGE + (d0 + d) * A8_TILE + row * 64;
+#pragma unroll
+                    for (int c = 0; c < 4; ++c)
+                        b[d][c] = *reinterpret_cast<const uint4 *>(src + ((c ^ ((row >> 1) & 3)) << 4));
+                }
+                uint32_t v[32];
+                auto convert = [&](const uint4(&q)[4]) {
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) {
+                        bytes_to_half(q[c].x, v[8 * c], v[8 * c + 1]);
+                        bytes_to_half(q[c].y, v[8 * c + 2], v[8 * c + 3]);
+                        bytes_to_half(q[c].z, v[8 * c + 4], v[8 * c + 5]);
+                        bytes_to_half(q[c].w, v[8 * c + 6], v[8 * c + 7]);
+                    }
+                };
+                convert(b[0]);
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&a8empty[s]);
+                if (!(ok = warp_wait(&done[s], ((g / NST) & 1) ^ 1, 19))) break;
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                tmem_st32_async(tq + s * 128, v);
+                convert(b[1]);
+                tmem_st32_async(tq + s * 128 + 32, v);
+                asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+                asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&aready[s]);
+            }
+    } else {
+        // ---------------- epilogue: warps 10..17, TMEM lane quadrant = warp % 4, half of a phase's columns
+        constexpr int NC = NI >= 64 ? NI / 2 : NI;  // columns of a phase per warp
+        const int quad = warp & 3, half = (warp - 10) >> 2, c00 = half * NC;
+        const bool active = NI >= 64 || half == 0;
+        uint32_t ev[2] = {0, 0};
+        bool ok = true;
+        for (int it = blockIdx.x; it < P.nitems && ok; it += gridDim.x) {
+            const CItem I(P, nib, it);
+            const float p = c_pf[I.m], invp = c_invp[I.m];
+            const int rp = c_red[I.m];
+            bool odd = true;  // phase 1 is reduced first, then in turn
+            for (int kb = rp / 2; ok; kb += rp / 2, odd = !odd) {
+                const bool last = kb >= P.nkb;
+#pragma unroll
+                for (int ph = 0; ph < 2; ++ph) {
+                    if (!ok || (!last && (ph == 1) != odd)) continue;
+                    if (!(ok = warp_wait(&tfull[ph], ev[ph]++ & 1, 20))) continue;
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                    const int m = I.m0 + slot;
-                    const float p = (float)c_p[m], invp = c_invp[m];
-                    const uint32_t tbase = tmem + ((uint32_t)(quad * 32) << 16) + slot * 256;
-                    const bool last = ch == nch - 1;
-                    unsigned char *out = P.res + ((size_t)m * P.nrhs + I.rhs) * P.Et * (size_t)P.nt + Pn.row0 + row;
+                    const uint32_t tb = tmem + ((uint32_t)(quad * 32) << 16) + ph * NI + c00;
+                    if (active && !last) {
+                        uint32_t v[NC / 32][32];
+#pragma unroll
+                        for (int c = 0; c < NC / 32; ++c) tmem_ld32_async(tb + c * 32, v[c]);
+                        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+                        for (int c = 0; c < NC / 32; ++c) {
+#pragma unroll
+                            for (int j = 0; j < 32; ++j)
+                                v[c][j] = __float_as_uint(mod_small(__uint_as_float(v[c][j]), p, invp));
+                            tmem_st32_async(tb + c * 32, v[c]);
+                        }
+                        asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+                    } else if (active) {
+                        const int row = I.tile * BM + quad * 32 + lane;
+                        unsigned char *out = P.res + ((size_t)I.m * P.nrhs + I.rhs) * P.Et * (size_t)P.nt + row;
 #pragma unroll 1
-                    for (int c0 = 0; c0 < 256; c0 += 32) {
-                        uint32_t v[32];
-                        tmem_ld32(tbase + c0, v);
-                        if (!last) {
+                        for (int c0 = 0; c0 < NC; c0 += 32) {
+                            uint32_t v[32];
+                            tmem_ld32(tb + c0, v);
+                            if (row < P.nt) {
 #pragma unroll
-                            for (int j = 0; j < 32; ++j) v[j] = __float_as_uint(mod_small(__uint_as_float(v[j]), p, invp));
-                            tmem_st32(tbase + c0, v);
-                        } else if (row_ok) {
-#pragma unroll
-                            for (int j = 0; j < 32; ++j) {
-                                const int c = c0 + j, ph = c >> 7, iv = I.ib * 128 + (c & 127);
-                                float r = mod_small(__uint_as_float(v[j]), p, invp);
-                                r = r < 0.f ? r + p : r;
-                                r = r < 0.f ? r + p : r;
-                                r = r >= p ? r - p : r;
-                                if (iv < P.nint) out[(size_t)(2 * iv + ph) * P.nt] = (unsigned char)(int)r;
+                                for (int j = 0; j < 32; ++j) {
+                                    const int iv = I.ib * NI + c00 + c0 + j;
+                                    float r = mod_small(__uint_as_float(v[j]), p, invp);
+                                    r = r < 0.f ? r + p : r;
+                                    r = r < 0.f ? r + p : r;
+                                    r = r >= p ? r - p : r;
+                                    if (iv < P.nint) out[(unsigned)(2 * iv + ph) * (unsigned)P.nt] = (unsigned char)(int)r;
+                                }
                             }
                         }
                     }
                     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-                    mbar_arrive(&tempty[slot]);
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&tempty[ph]);
                 }
-        }
-    }
-    __syncthreads();
-    if (warp == 1) {
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512));
-    }
-}
-
-// ------------------------------------------------------------------------------------------
-// Two row tiles per CTA: the W stage (32 KB) feeds the MMAs of two 128-row tiles, so every byte
-// brought from L2 / HBM serves twice the tensor work of the form above.  A work item is (modulus,
-// pair of row tiles, interval block, rhs); the two tiles' accumulators take all 512 TMEM columns,
-// so the epilogue's reduction after each 1024-column chunk pauses the MMAs (about 900 of 16000
-// cycles).  Warps: 0 TMA, 1 MMA, 2..9 epilogue (warp w serves tile (w - 2) / 4 and TMEM lane
-// quadrant w % 4).  Three 64 KB stages.
-constexpr int STAGE2 = 2 * A_TILE + 2 * B_HALF;  // 64 KB
-constexpr int NSTAGE2 = 3;
-constexpr int kCrt2Threads = 320;
-
-struct CItem2 {
-    int m, rhs, ib;
-    int panel[2], r0[2];
-    bool has1;
-};
-
-__device__ __forceinline__ CItem2 decode_citem2(const NfCrtParams &P, int it)
-{
-    const int ntp = (P.ntiles + 1) / 2, per_m = ntp * P.nib * P.nrhs;
-    CItem2 I;
-    I.m = it / per_m;  // modulus-major: consecutive CTAs share the modulus (its W residues stay in L2)
-    int r_ = it % per_m;
-    I.rhs = r_ / (ntp * P.nib);
-    r_ %= ntp * P.nib;
-    I.ib = r_ % P.nib;
-    const int tp = r_ / P.nib;
-    const int t0 = 2 * tp, t1 = 2 * tp + 1;
-    I.panel[0] = P.tiles[2 * t0];
-    I.r0[0] = P.tiles[2 * t0 + 1];
-    I.has1 = t1 < P.ntiles;
-    I.panel[1] = I.has1 ? P.tiles[2 * t1] : I.panel[0];
-    I.r0[1] = I.has1 ? P.tiles[2 * t1 + 1] : I.r0[0];
-    return I;
-}
-
-__global__ void __launch_bounds__(kCrt2Threads, 1) k_nf_apply_crt2(const __grid_constant__ CUtensorMap mapA,
-                                                                   const __grid_constant__ CUtensorMap mapW,
-                                                                   NfCrtParams P)
-{
-    extern __shared__ __align__(1024) unsigned char smem_raw[];
-    unsigned char *smem = (unsigned char *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    uint64_t *full = (uint64_t *)(smem + NSTAGE2 * STAGE2);
-    uint64_t *empty = full + NSTAGE2;
-    uint64_t *tfull = empty + NSTAGE2;
-    uint64_t *tempty = tfull + 1;
-    uint32_t *tmem_slot = (uint32_t *)(tempty + 1);
-    __shared__ volatile int s_abort;
-
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (threadIdx.x == 0) {
-        for (int s = 0; s < NSTAGE2; ++s) {
-            mbar_init(&full[s], 1);
-            mbar_init(&empty[s], 1);
-        }
-        mbar_init(tfull, 1);
-        mbar_init(tempty, 256);
-        s_abort = 0;
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
-    if (warp == 1) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(tmem_slot)),
-                     "r"(512));
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
-    }
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    const uint32_t tmem = *tmem_slot;
-    uint64_t deadline = gtimer() + kTimeoutNs;  // renewed per chunk: each wait is bounded by 2 s
-    const int nst = 4 * P.nkb;
-    const int nch = (nst + CHUNK - 1) / CHUNK;
-
-    if (warp == 0) {
-        // ---------------- TMA producer
-        if (lane == 0) {
-            int g = 0;
-            for (int it = blockIdx.x; it < P.nitems && !s_abort; it += gridDim.x) {
-                const CItem2 I = decode_citem2(P, it);
-                bool two[2];
-                long long rbase[2];
-                int rpad[2];
-                for (int q = 0; q < 2; ++q) {
-                    const PanelGPU &Pn = P.panels[I.panel[q]];
-                    two[q] = I.r0[q] + 64 < Pn.nrows;
-                    rbase[q] = (P.kop ? Pn.offK : Pn.offV) / P.cols_pad + I.r0[q];
-                    rpad[q] = Pn.rows_pad;
-                }
-                for (int ch = 0; ch < nch && !s_abort; ++ch) {
-                    deadline = gtimer() + kTimeoutNs;
-                    const int st1 = min(nst, (ch + 1) * CHUNK);
-                    for (int st = ch * CHUNK; st < st1; ++st, ++g) {
-                        const int s = g % NSTAGE2;
-                        if (!mbar_wait(&empty[s], ((g / NSTAGE2) & 1) ^ 1, deadline)) {
-                            atomicExch(P.err, 21);
-                            s_abort = 1;
-                            break;
-                        }
-                        const int d = st / P.nkb, kb = st % P.nkb;
-                        unsigned char *sA = smem + s * STAGE2;
-                        uint32_t bytes = (d < 3 ? 2 : 1) * B_HALF;
-                        for (int q = 0; q < (I.has1 ? 2 : 1); ++q) bytes += two[q] ? A_TILE : A_TILE / 2;
-                        mbar_expect_tx(&full[s], bytes);
-                        for (int q = 0; q < (I.has1 ? 2 : 1); ++q) {
-                            const int blk = (int)((rbase[q] + (long long)d * rpad[q]) >> 6) * P.nkb + kb;
-                            tma_4d(sA + q * A_TILE, &mapA, 0, 0, blk, I.m, &full[s]);
-                            if (two[q]) tma_4d(sA + q * A_TILE + A_TILE / 2, &mapA, 0, 0, blk + P.nkb, I.m, &full[s]);
-                        }
-                        unsigned char *sB = sA + 2 * A_TILE;
-                        for (int ph = (d < 3 ? 0 : 1); ph < 2; ++ph) {
-                            const int phs = ((ph - d) % 2 + 2) % 2, q = (phs - (ph - d)) / 2;
-                            tma_5d(sB + ph * B_HALF, &mapW, kb * BK, phs, I.ib * 128 - q, I.rhs, I.m, &full[s]);
-                        }
-                    }
-                }
-            }
-            const uint64_t dl2 = gtimer() + kTimeoutNs / 20;
-            for (int j = (g > NSTAGE2 ? g - NSTAGE2 : 0); j < g; ++j)
-                mbar_wait(&full[j % NSTAGE2], (j / NSTAGE2) & 1, dl2);
-        }
-    } else if (warp == 1) {
-        // ---------------- MMA issuer
-        if (lane == 0) {
-            int g = 0, u = 0;
-            const uint32_t id256 = idesc_f16(BM, 256), id128 = idesc_f16(BM, 128);
-            for (int it = blockIdx.x; it < P.nitems && !s_abort; it += gridDim.x) {
-                const CItem2 I = decode_citem2(P, it);
-                for (int ch = 0; ch < nch && !s_abort; ++ch, ++u) {
-                    deadline = gtimer() + kTimeoutNs;
-                    if (!mbar_wait(tempty, (u & 1) ^ 1, deadline)) {
-                        atomicExch(P.err, 22);
-                        s_abort = 1;
-                        break;
-                    }
-                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                    const int st1 = min(nst, (ch + 1) * CHUNK);
-                    for (int st = ch * CHUNK; st < st1; ++st, ++g) {
-                        const int s = g % NSTAGE2;
-                        if (!mbar_wait(&full[s], (g / NSTAGE2) & 1, deadline)) {
-                            atomicExch(P.err, 23);
-                            s_abort = 1;
-                            break;
-                        }
-                        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                        const int d = st / P.nkb;
-                        const uint32_t a0 = su32(smem + s * STAGE2), b0 = a0 + 2 * A_TILE;
-#pragma unroll
-                        for (int kk = 0; kk < BK / 16; ++kk) {
-                            const uint32_t ko = kk * 32;
-                            const uint32_t accf = (ch == 0 && st == 0 && kk == 0) ? 0u : 1u;
-#pragma unroll
-                            for (int q = 0; q < 2; ++q) {
-                                if (q == 1 && !I.has1) break;
-                                const uint32_t aq = a0 + q * A_TILE + ko, dq = tmem + q * 256;
-                                if (d < 3)
-                                    mma_f16(dq, sw128_desc(aq), sw128_desc(b0 + ko), id256, accf);
-                                else
-                                    mma_f16(dq + 128, sw128_desc(aq), sw128_desc(b0 + B_HALF + ko), id128, 1u);
-                            }
-                        }
-                        mma_commit(&empty[s]);
-                    }
-                    mma_commit(tfull);
-                }
-            }
-        }
-    } else {
-        // ---------------- epilogue: warps 2..9; tile (warp - 2) / 4, TMEM lane quadrant warp % 4
-        const int quad = warp & 3, tq = (warp - 2) >> 2;
-        const int row_l = quad * 32 + lane;
-        int u = 0;
-        for (int it = blockIdx.x; it < P.nitems && !s_abort; it += gridDim.x) {
-            const CItem2 I = decode_citem2(P, it);
-            const bool active = tq == 0 || I.has1;
-            const PanelGPU &Pn = P.panels[I.panel[tq]];
-            const int row = I.r0[tq] + row_l;
-            const bool row_ok = active && row < Pn.nrows;
-            const float p = (float)c_p[I.m], invp = c_invp[I.m];
-            const uint32_t tbase = tmem + ((uint32_t)(quad * 32) << 16) + tq * 256;
-            unsigned char *out = P.res + ((size_t)I.m * P.nrhs + I.rhs) * P.Et * (size_t)P.nt + Pn.row0 + row;
-            for (int ch = 0; ch < nch && !s_abort; ++ch, ++u) {
-                deadline = gtimer() + kTimeoutNs;
-                if (!mbar_wait(tfull, u & 1, deadline)) {
-                    atomicExch(P.err, 24);
-                    s_abort = 1;
-                    break;
-                }
-                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const bool last = ch == nch - 1;
-                if (active) {
-#pragma unroll 1
-                    for (int c0 = 0; c0 < 256; c0 += 32) {
-                        uint32_t v[32];
-                        tmem_ld32(tbase + c0, v);
-                        if (!last) {
-#pragma unroll
-                            for (int j = 0; j < 32; ++j) v[j] = __float_as_uint(mod_small(__uint_as_float(v[j]), p, invp));
-                            tmem_st32(tbase + c0, v);
-                        } else if (row_ok) {
-#pragma unroll
-                            for (int j = 0; j < 32; ++j) {
-                                const int c = c0 + j, ph = c >> 7, iv = I.ib * 128 + (c & 127);
-                                float r = mod_small(__uint_as_float(v[j]), p, invp);
-                                r = r < 0.f ? r + p : r;
-                                r = r < 0.f ? r + p : r;
-                                r = r >= p ? r - p : r;
-                                if (iv < P.nint) out[(size_t)(2 * iv + ph) * P.nt] = (unsigned char)(int)r;
-                            }
-                        }
-                    }
-                }
-                asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-                mbar_arrive(tempty);
+                if (last) break;
             }
         }
     }
@@ -614,35 +542,48 @@ __device__ __forceinline__ void residues16(long long a, float (&r)[kCrtModuli])
     }
 }
 
-// FP64 panels -> residues of A' = rint(2^e_R A) for every modulus, [modulus][n] in the 64 x 64
-// block layout of nf_tiled_index (row R of the concatenated panels has exponent rowexp_R[R])
-__global__ void k_crt_split_panel(const double *__restrict__ A, const int *__restrict__ rowexp_R, size_t n, int ncp,
-                                  __half *__restrict__ res)
+// FP64 panels -> residues of A' = rint(2^e_x A) for every modulus as bytes r + 128, [modulus][tile]
+// [column block][d][128 rows][64 columns] with the 16-byte chunks of row r at c ^ ((r / 2) mod 4); rows
+// past the last triangle are zero.  Thread per (row, d, four columns)
+__global__ void k_crt_split_panel(const double *__restrict__ A, const PanelGPU *__restrict__ panels,
+                                  const int *__restrict__ tri_leaf, const int *__restrict__ rowexp, int kop, int nt,
+                                  int ntiles, int ncp, unsigned char *__restrict__ res)
 {
     const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const size_t R = i / ncp;
-    const int c = (int)(i - R * ncp);
-    const size_t o = nf_tiled_index(R, c, ncp >> 6);
-    float r[kCrtModuli];
-    residues16(__double2ll_rn(A[i] * pow2(rowexp_R[R])), r);
+    const int nq = ncp / 4, c = (int)(i % nq) * 4;
+    const size_t rd = i / nq;
+    const int d = (int)(rd & 3), x = (int)(rd >> 2);
+    if (x >= ntiles * BM) return;
+    const int nkb = ncp / BK, row = x & (BM - 1), ch = ((c & 63) >> 4) ^ ((row >> 1) & 3);
+    double4 v = make_double4(0.0, 0.0, 0.0, 0.0);
+    if (x < nt) {
+        const PanelGPU &Pn = panels[tri_leaf[x]];
+        const double2 *a = reinterpret_cast<const double2 *>(
+            A + (kop ? Pn.offK : Pn.offV) + ((size_t)d * Pn.rows_pad + (x - Pn.row0)) * ncp + c);
+        const double2 p = a[0], q = a[1];
+        const double sc = pow2(rowexp[x]);
+        v = make_double4(p.x * sc, p.y * sc, q.x * sc, q.y * sc);
+    }
+    uint32_t w[kCrtModuli];
+    const double e[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-    for (int m = 0; m < kCrtModuli; ++m) res[(size_t)m * n + o] = __float2half_rn(r[m]);
+    for (int j = 0; j < 4; ++j) {
+        float r[kCrtModuli];
+        residues16(__double2ll_rn(e[j]), r);
+#pragma unroll
+        for (int m = 0; m < kCrtModuli; ++m) w[m] = (j ? w[m] : 0u) | (uint32_t)((int)r[m] + 128) << (8 * j);
+    }
+    const size_t per_m = (size_t)ntiles * nkb * A8_STAGE;
+    const size_t o = ((size_t)(x / BM) * nkb + c / BK) * A8_STAGE + d * A8_TILE + row * 64 + ch * 16 + (c & 15);
+#pragma unroll
+    for (int m = 0; m < kCrtModuli; ++m) *reinterpret_cast<uint32_t *>(res + m * per_m + o) = w[m];
 }
 
-// per-row exponents of global panel rows: rowexp_R[R] = e of the row's triangle
-__global__ void k_row_exps(const PanelGPU *__restrict__ panels, int npanel, int kop, int nd, int ncp, int b,
-                           const unsigned long long *__restrict__ rowmax, int *__restrict__ rowexp_tri,
-                           int *__restrict__ rowexp_R)
+// per-row exponents
+__global__ void k_row_exps(const unsigned long long *__restrict__ rowmax, int nt, int b, int *__restrict__ rowexp)
 {
-    const PanelGPU &Pn = panels[blockIdx.x];
-    const long long R0 = (kop ? Pn.offK : Pn.offV) / ncp;
-    for (int i = threadIdx.x; i < nd * Pn.rows_pad; i += blockDim.x) {
-        const int r = i % Pn.rows_pad;
-        const int e = r < Pn.nrows ? crt_scale_exp(rowmax[Pn.row0 + r], b) : 0;
-        rowexp_R[R0 + i] = e;
-        if (i < Pn.nrows) rowexp_tri[Pn.row0 + r] = e;
-    }
+    const int x = blockIdx.x * blockDim.x + threadIdx.x;
+    if (x < nt) rowexp[x] = crt_scale_exp(rowmax[x], b);
 }
 
 // input: per-rhs scale 2^s (|W'| <= 2^b), W' = rint(2^s x) permuted (V) or padded (K) into
@@ -727,10 +668,14 @@ int crt_upload_constants(cudaStream_t st)
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return -1;
     if (done[dev]) return 0;
     float invp[kCrtModuli], pf[kCrtModuli], pow11[kCrtModuli][5];
+    int red[kCrtModuli];
     float pj[kCrtModuli][kCrtModuli] = {{0.f}}, invPi[kCrtModuli];
     for (int i = 0; i < kCrtModuli; ++i) {
         pf[i] = (float)g_moduli[i];
         invp[i] = 1.0f / (float)g_moduli[i];
+        // largest even r with 256 r ((p - 1) / 2)^2 + 1.5 p < 2^24
+        const long long hp = (g_moduli[i] - 1) / 2;
+        red[i] = (int)(((1ll << 24) - 2 * g_moduli[i]) / (256 * hp * hp)) & ~1;
         long long q = 1;  // p_0 ... p_{j-1} mod p_i, for j = 0 .. i
         for (int j = 0; j < i; ++j) {
             pj[j][i] = (float)q;
@@ -745,6 +690,7 @@ int crt_upload_constants(cudaStream_t st)
     }
     if (cudaMemcpyToSymbolAsync(c_p, g_moduli, sizeof(g_moduli), 0, cudaMemcpyHostToDevice, st) != cudaSuccess ||
         cudaMemcpyToSymbolAsync(c_pf, pf, sizeof(pf), 0, cudaMemcpyHostToDevice, st) != cudaSuccess ||
+        cudaMemcpyToSymbolAsync(c_red, red, sizeof(red), 0, cudaMemcpyHostToDevice, st) != cudaSuccess ||
         cudaMemcpyToSymbolAsync(c_invp, invp, sizeof(invp), 0, cudaMemcpyHostToDevice, st) != cudaSuccess ||
         cudaMemcpyToSymbolAsync(c_pow11, pow11, sizeof(pow11), 0, cudaMemcpyHostToDevice, st) != cudaSuccess ||
         cudaMemcpyToSymbolAsync(c_pjmodpif, pj, sizeof(pj), 0, cudaMemcpyHostToDevice, st) != cudaSuccess ||
@@ -765,18 +711,22 @@ int crt_bits(long long k_total)
     return std::min(b, 53);
 }
 
-void launch_crt_row_exps(const double *A, const PanelGPU *panels, int npanel, int kop, int nd, int ncp, int b,
-                         unsigned long long *rowmax, int nt, int *rowexp_tri, int *rowexp_R, cudaStream_t st)
+void launch_crt_row_exps(const double *A, const PanelGPU *panels, int npanel, int kop, int nd, int b,
+                         unsigned long long *rowmax, int nt, int *rowexp, cudaStream_t st)
 {
     cudaMemsetAsync(rowmax, 0, sizeof(unsigned long long) * nt, st);
     k_row_absmax<<<dim3(64, npanel), 256, 0, st>>>(A, panels, npanel, kop, nd, rowmax);
-    k_row_exps<<<npanel, 256, 0, st>>>(panels, npanel, kop, nd, ncp, b, rowmax, rowexp_tri, rowexp_R);
+    k_row_exps<<<(nt + 255) / 256, 256, 0, st>>>(rowmax, nt, b, rowexp);
 }
 
-void launch_crt_split_panel(const double *A, const int *rowexp_R, size_t n, int ncp, void *res, cudaStream_t st)
+size_t crt_panel_bytes(int nt, int ncp) { return (size_t)kCrtModuli * ((nt + BM - 1) / BM) * (ncp / BK) * A8_STAGE; }
+
+void launch_crt_split_panel(const double *A, const PanelGPU *panels, const int *tri_leaf, const int *rowexp, int kop,
+                            int nt, int ncp, unsigned char *res, cudaStream_t st)
 {
-    if (n == 0) return;
-    k_crt_split_panel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(A, rowexp_R, n, ncp, (__half *)res);
+    const int ntiles = (nt + BM - 1) / BM;
+    const size_t n = (size_t)ntiles * BM * 4 * (ncp / 4);
+    k_crt_split_panel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(A, panels, tri_leaf, rowexp, kop, nt, ntiles, ncp, res);
 }
 
 void launch_crt_split_input(const double *x, const int *perm, int ncol, int ncol_pad, int nrhs, int Et, int b,
@@ -798,27 +748,29 @@ void launch_crt_combine(const unsigned char *res, int nrhs, int Et, int nt, cons
     k_crt_combine<<<(unsigned)((per_mod + 255) / 256), 256, 0, st>>>(res, per_mod, per_rhs, nt, rowexp, wmax, b, f);
 }
 
-size_t nf_crt_smem_bytes() { return (size_t)NSTAGE * STAGE_BYTES + 1024 + 256; }
-
-int launch_nf_apply_crt(const CUtensorMap &A, const CUtensorMap &W, const NfCrtParams &P, int nsm, cudaStream_t st,
-                        int form)
+int nf_crt_intervals(int nint, int form)
 {
-    if (form == 2) {  // two row tiles per CTA, one modulus per item
-        NfCrtParams Q = P;
-        Q.nitems = kCrtModuli * ((P.ntiles + 1) / 2) * P.nib * P.nrhs;
-        const size_t smem = (size_t)NSTAGE2 * STAGE2 + 1024 + 256;
-        cudaError_t e = cudaFuncSetAttribute(k_nf_apply_crt2, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return -1;
-        const int grid = Q.nitems < nsm ? Q.nitems : nsm;
-        k_nf_apply_crt2<<<grid, kCrt2Threads, smem, st>>>(A, W, Q);
-        return cudaGetLastError() == cudaSuccess ? 0 : -1;
-    }
-    const size_t smem = nf_crt_smem_bytes();
-    cudaError_t e = cudaFuncSetAttribute(k_nf_apply_crt, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return -1;
-    const int grid = P.nitems < nsm ? P.nitems : nsm;
-    k_nf_apply_crt<<<grid, 192, smem, st>>>(A, W, P);
+    // the MMA's columns are 2 NI: few intervals take the narrowest block that holds them
+    return nint <= 32 ? 32 : (nint <= 64 || form == 2 ? 64 : 128);
+}
+
+template <int NI>
+static int launch_crt_T(const CUtensorMap &W, NfCrtParams P, int nsm, cudaStream_t st)
+{
+    P.nitems = kCrtModuli * P.ntiles * ((P.nint + NI - 1) / NI) * P.nrhs;
+    auto kf = k_nf_apply_crt<NI>;
+    if (cudaFuncSetAttribute(kf, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CrtSmem<NI>::bytes) != cudaSuccess)
+        return -1;
+    kf<<<std::min(P.nitems, nsm), kCrtThreads, CrtSmem<NI>::bytes, st>>>(W, P);
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
+}
+
+int launch_nf_apply_crt(const CUtensorMap &W, const NfCrtParams &P, int nsm, cudaStream_t st, int form)
+{
+    const int ni = nf_crt_intervals(P.nint, form);
+    return ni == 32   ? launch_crt_T<32>(W, P, nsm, st)
+           : ni == 64 ? launch_crt_T<64>(W, P, nsm, st)
+                      : launch_crt_T<128>(W, P, nsm, st);
 }
 
 }  // namespace pfmm

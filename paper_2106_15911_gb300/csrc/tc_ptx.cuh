@@ -47,6 +47,34 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *b, uint32_t parity, uint64_t
     }
 }
 
+// bounded wait whose clock starts at the first failed try (reading %globaltimer before every wait
+// costs more than most waits): false after about 2 s (2^32 SM cycles).  POLL: test without sleeping,
+// for the waits that a pipeline's rate hangs on; else tries that may sleep
+template <bool POLL>
+__device__ __forceinline__ bool mbar_wait_bounded(uint64_t *b, uint32_t parity)
+{
+    uint32_t ok = 0;
+    long long t0 = 0;
+    while (true) {
+        if (POLL)
+            asm volatile(
+                "{\n\t.reg .pred p;\n\tmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+                : "=r"(ok)
+                : "r"(su32(b)), "r"(parity)
+                : "memory");
+        else
+            asm volatile(
+                "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+                : "=r"(ok)
+                : "r"(su32(b)), "r"(parity)
+                : "memory");
+        if (ok) return true;
+        const long long t = clock64();
+        if (t0 == 0) t0 = t;
+        if (t - t0 > (1ll << 32)) return false;
+    }
+}
+
 // shared-memory matrix descriptor: K-major, 128-byte swizzle, 8-row groups 1024 bytes apart
 __device__ __forceinline__ uint64_t sw128_desc(uint32_t saddr)
 {
@@ -66,7 +94,8 @@ __device__ __forceinline__ void mma_commit(uint64_t *b)
                  : "memory");
 }
 
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32])
+// the loaded registers may be read only after a tcgen05.wait::ld
+__device__ __forceinline__ void tmem_ld32_async(uint32_t taddr, uint32_t (&r)[32])
 {
     asm volatile(
         "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
@@ -76,6 +105,11 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32])
           "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
           "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
         : "r"(taddr));
+}
+
+__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32])
+{
+    tmem_ld32_async(taddr, r);
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 

@@ -1,0 +1,37 @@
+"""The FP64 tensor-core nearfield at the edges of its tiling (128 target triangles, 64 columns, blocks
+of 32, 64 or 128 leaf intervals, reductions every 4 to 8 column blocks): row and column counts that
+leave remainders, one to several column blocks, interval counts on both sides of a block."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2106_15911_gb300 import pfmm as P
+from paper_2106_15911_gb300.inputs import cube_mesh, cube_sphere_mesh, random_density
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+
+
+@pytest.mark.parametrize("form", [1, 2])
+@pytest.mark.parametrize("mesh,n_a,Et,nrhs", [
+    (cube_mesh, 1, 4, 1),           # 12 triangles: one row tile, one column block, 2 leaf intervals
+    (cube_mesh, 3, 64, 3),          # 108 rows, 32 intervals: a full block of 32
+    (cube_sphere_mesh, 5, 128, 2),  # 300 rows: two tiles and 44 rows, 5 column blocks, 64 intervals
+    (cube_mesh, 7, 256, 1),         # 588 rows, 10 column blocks, 128 intervals
+    (cube_mesh, 9, 128, 1),         # 972 rows, 16 column blocks (8 for K): reductions on the last block
+])
+def test_residue_nearfield_at_tile_edges(mesh, n_a, Et, nrhs, form):
+    V, T = mesh(n_a)
+    kw = dict(m_t=2, m_x=2, c_st=1.0, quad_regular=2, quad_singular=2)
+    op = P.Operator(V, T, 1.0, Et, nf_form=form, **kw)
+    ref = P.Operator(V, T, 1.0, Et, nf_engine=P.PFMM_NF_CUDA_CORES, **kw)
+    assert op.info()["nf_tensor_cores"] == 3 and ref.info()["nf_tensor_cores"] == 0
+    for call, n in (("V", T.shape[0]), ("K", V.shape[0])):
+        x = torch.tensor(random_density(Et, n, nrhs, seed=17), device=DEV)
+        a = getattr(op, call)(x, parts=P.PFMM_PART_NEAR).cpu().numpy()
+        P.pfmm_check(op.h)
+        b = getattr(ref, call)(x, parts=P.PFMM_PART_NEAR).cpu().numpy()
+        # operands rounded to 52 bits of each row's and right-hand side's largest, exact sums
+        assert np.max(np.abs(a - b)) <= 1e-13 * np.max(np.abs(b))
+    op.close()
+    ref.close()
