@@ -47,21 +47,22 @@ __device__ __forceinline__ void erf_pair(R u, R &ef, R &efc)
     }
 }
 
-// erf(u)/u (Maclaurin series below 0.05)
+// erf(u)/u (Maclaurin series below 0.05), iu = 1/u
 template <typename R>
-__device__ __forceinline__ R erf_over_u(R u, R ef)
+__device__ __forceinline__ R erf_over_u(R u, R ef, R iu)
 {
     if (u < R(0.05)) {
         R u2 = u * u;
         R s = R(1) + u2 * (R(-1.0 / 3.0) + u2 * (R(1.0 / 10.0) + u2 * (R(-1.0 / 42.0) + u2 * R(1.0 / 216.0))));
         return R(2.0 / kSqrtPi) * s;
     }
-    return ef / u;
+    return ef * iu;
 }
 
 // phi2(u) = (erf(u) - 2u e^{-u^2}/sqrt(pi)) / u^3; series (2/sqrt(pi)) sum_{n>=1} (-1)^{n+1} 2n u^{2n-2} / (n! (2n+1))
+// iu = 1/u
 template <typename R>
-__device__ __forceinline__ R phi2(R u, R ef, R ex)
+__device__ __forceinline__ R phi2(R u, R ef, R ex, R iu)
 {
     if (u < R(0.5)) {
         R u2 = u * u, acc = R(0);
@@ -74,35 +75,53 @@ __device__ __forceinline__ R phi2(R u, R ef, R ex)
         }
         return R(2.0 / kSqrtPi) * acc;
     }
-    return (ef - R(2.0 / kSqrtPi) * u * ex) / (u * u * u);
+    return (ef - R(2.0 / kSqrtPi) * u * ex) * (iu * iu * iu);
 }
 
-// Single-layer time integrals for d = 0 .. nd-1 at distance r (nd <= 8).  r must be > 0 when
-// d = 0 is requested; for d >= 1 r = 0 is allowed.
+// Constants of the step ends s = k h, k = 1 .. nd, and of the formulas above, from the host in FP64
 template <typename R>
-__device__ __forceinline__ void time_V_all(R r, R h, R alpha, int nd, R *out)
+struct TimeConst {
+    R cu[8], icu[8];       // u = r cu, 1/u = icu / r:  cu = 1 / (2 sqrt(alpha s))
+    R s[8], b1[8], b2[8];  // s, sqrt(s) / (8 pi alpha^1.5), sqrt(s) / (4 pi^1.5 alpha^1.5)
+    R b3[8];               // sqrt(s / (pi alpha))
+    R a1, a2, clin, k8;    // 1 / (8 pi alpha^2), 1 / (2 alpha), 1 / (4 pi alpha), 1 / (8 pi alpha)
+};
+
+// Time integrals for d = 0 .. ND-1 at distance r: V[d] of the single layer and K[d] of the double
+// layer (to be multiplied by (x - y).n_y; 0 at r = 0).  r must be > 0 when d = 0 of V is used.  Both
+// layers share erf, erfc and exp of a step end; the divisions are one reciprocal of r (a step end
+// costs some 130 FP64 operations for both instead of some 700).
+template <typename R, bool DOV, bool DOK, int ND>
+__device__ __forceinline__ void time_integrals(R r, const TimeConst<R> &c, R *V, R *K)
 {
-    R g2[9], g2t[9];
-    g2[0] = R(0);
-    g2t[0] = R(0);
-    const R a32 = alpha * d_sqrt(alpha);
-    const R c_lin = R(1) / (R(4 * kPi) * alpha);
-    for (int k = 1; k <= nd; ++k) {
-        R s = R(k) * h;
-        R ss = d_sqrt(s);
-        R u = r / (R(2) * d_sqrt(alpha) * ss);
+    const R ir = r > R(0) ? R(1) / r : R(0), r2 = r * r;
+    R g1 = R(0), g2 = R(0), t1 = R(0), t2 = R(0);  // G2, bounded form at k - 1 and k - 2
+    R d1 = R(0), d2 = R(0), e1 = R(0), e2 = R(0);  // the same of the double layer
+#pragma unroll
+    for (int k = 0; k < ND; ++k) {
+        const R u = r * c.cu[k], iu = ir * c.icu[k];
         R ef, efc;
         erf_pair(u, ef, efc);
-        R ex = d_exp(-u * u);
-        g2t[k] = r * efc / (R(8 * kPi) * alpha * alpha) - ss * erf_over_u(u, ef) / (R(8 * kPi) * a32) -
-                 ss * ex / (R(4 * kPi * kSqrtPi) * a32);
-        g2[k] = (r > R(0)) ? ((s + r * r / (R(2) * alpha)) * efc - r * ss / d_sqrt(R(kPi) * alpha) * ex) * c_lin / r
-                           : R(0);
-    }
-    out[0] = g2[1];
-    for (int d = 1; d < nd; ++d) {
-        R u = r / (R(2) * d_sqrt(alpha * R(d + 1) * h));
-        out[d] = (u < R(1)) ? (g2t[d + 1] - g2t[d] - g2t[d] + g2t[d - 1]) : (g2[d + 1] - g2[d] - g2[d] + g2[d - 1]);
+        const R ex = d_exp(-u * u);
+        const bool small = u < R(1);
+        if (DOV) {
+            const R t = r * efc * c.a1 - c.b1[k] * erf_over_u(u, ef, iu) - c.b2[k] * ex;
+            const R g = ((c.s[k] + r2 * c.a2) * efc - r * c.b3[k] * ex) * (c.clin * ir);
+            V[k] = k == 0 ? g : (small ? t - t1 - t1 + t2 : g - g1 - g1 + g2);
+            g2 = g1;
+            g1 = g;
+            t2 = t1;
+            t1 = t;
+        }
+        if (DOK) {
+            const R g = ((c.s[k] * ir * ir - c.a2) * efc + c.b3[k] * ex * ir) * (R(1.0 / (4 * kPi)) * ir);
+            const R t = -(R(0.5) * u * phi2(u, ef, ex, iu) + efc) * (c.k8 * ir);
+            K[k] = k == 0 ? g : (small ? t - e1 - e1 + e2 : g - d1 - d1 + d2);
+            d2 = d1;
+            d1 = g;
+            e2 = e1;
+            e1 = t;
+        }
     }
 }
 
@@ -117,7 +136,7 @@ __device__ __forceinline__ void g2_and_g2t(double r, double s, double alpha, dou
     double ef, efc;
     erf_pair(u, ef, efc);
     const double ex = exp(-u * u);
-    g2t = r * efc / (8.0 * kPi * alpha * alpha) - ss * erf_over_u(u, ef) / (8.0 * kPi * a32) -
+    g2t = r * efc / (8.0 * kPi * alpha * alpha) - ss * erf_over_u(u, ef, 1.0 / u) / (8.0 * kPi * a32) -
           ss * ex / (4.0 * kPi * kSqrtPi * a32);
     g2 = r > 0.0 ? ((s + r * r / (2.0 * alpha)) * efc - r * ss / sqrt(kPi * alpha) * ex) / (4.0 * kPi * alpha * r) : 0.0;
 }
@@ -140,33 +159,6 @@ __device__ __forceinline__ double time_V_steps(double r, double tk0, double tk1,
     for (int i = 0; i < 4; ++i) g2_and_g2t(r, s[i], alpha, g[i], gt[i]);
     const double u = r / (2.0 * sqrt(alpha * s[0]));
     return u < 1.0 ? (gt[0] - gt[1]) - (gt[2] - gt[3]) : (g[0] - g[1]) - (g[2] - g[3]);
-}
-
-// Double-layer time factors for d = 0 .. nd-1 (multiply by (x - y).n_y); 0 at r = 0.
-template <typename R>
-__device__ __forceinline__ void time_K_all(R r, R h, R alpha, int nd, R *out)
-{
-    if (!(r > R(0))) {
-        for (int d = 0; d < nd; ++d) out[d] = R(0);
-        return;
-    }
-    R dl[9], dlt[9];
-    dl[0] = R(0);
-    dlt[0] = R(0);
-    for (int k = 1; k <= nd; ++k) {
-        R s = R(k) * h;
-        R u = r / (R(2) * d_sqrt(alpha * s));
-        R ef, efc;
-        erf_pair(u, ef, efc);
-        R ex = d_exp(-u * u);
-        dl[k] = ((s / (r * r) - R(1) / (R(2) * alpha)) * efc + d_sqrt(s / (R(kPi) * alpha)) * ex / r) / (R(4 * kPi) * r);
-        dlt[k] = -(R(0.5) * u * phi2(u, ef, ex) + efc) / (R(8 * kPi) * alpha * r);
-    }
-    out[0] = dl[1];
-    for (int d = 1; d < nd; ++d) {
-        R u = r / (R(2) * d_sqrt(alpha * R(d + 1) * h));
-        out[d] = (u < R(1)) ? (dlt[d + 1] - dlt[d] - dlt[d] + dlt[d - 1]) : (dl[d + 1] - dl[d] - dl[d] + dl[d - 1]);
-    }
 }
 
 // Chebyshev polynomials T_0..T_m at x (three-term recurrence)

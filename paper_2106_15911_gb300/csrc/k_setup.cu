@@ -11,6 +11,7 @@
 // Nearfield (Eq. eval_sl_nf_block with the entries of Section 2): collapsed Gauss-Legendre
 // n_r x n_r per triangle for regular pairs; Sauter-Schwab (Sauter & Schwab, Boundary Element
 // Methods, Sec. 5.2) with n_s points per direction for triangles sharing a vertex at d = 0, 1.
+#include <algorithm>
 #include <cstdio>
 
 #include "device_math.cuh"
@@ -131,50 +132,55 @@ void launch_e1_table(int na, int mt, int mx, int G, double hx, double hxp, doubl
 }
 
 // ------------------------------------------------------------------------------------------
-// Regular nearfield quadrature.  Thread per (row, column) of one panel.
-template <typename R, typename S, bool KOP>
-__global__ void __launch_bounds__(256) k_nf_regular(NfQuadArgs a, int panel_rows0, int nrows, int rows_pad,
-                                                      int cols_pad, const int *__restrict__ cols, S *__restrict__ A,
-                                                      const int *__restrict__ kmap_p, int colsK_pad, int ncols)
+// Regular nearfield quadrature of both layers.  Thread per (row, column) of one panel; bound by the
+// FP64 (FP32) pipe and the special functions, which the two layers share (see time_integrals).
+// One launch for all panels (grid z): a small mesh's panels have too few rows to fill the GPU alone.
+template <typename R, int ND>
+__global__ void __launch_bounds__(256) k_nf_regular(NfQuadArgs a, const PanelGPU *__restrict__ panels,
+                                                      R *__restrict__ AVs, R *__restrict__ AKs)
 {
+    const PanelGPU &P = panels[blockIdx.z];
     int col = blockIdx.x * blockDim.x + threadIdx.x;
     int row = blockIdx.y * blockDim.y + threadIdx.y;
-    if (row >= nrows || col >= ncols) return;
-    int y = cols[col];
+    if (row >= P.nrows || col >= P.ncolV) return;
+    int y = a.colV[P.colV_at + col];
     if (y < 0) return;
-    int x = panel_rows0 + row;
-    R acc[3 * 8];
+    int x = P.row0 + row;
+    R accV[ND], accK[3 * ND];
 #pragma unroll
-    for (int i = 0; i < 3 * 8; ++i) acc[i] = R(0);
-    const int d0 = nf_regular_pair<R, KOP>(a, x, y, acc);
-    const int nd = a.nd;
-    if (!KOP) {
-        for (int d = d0; d < nd; ++d) A[((size_t)d * rows_pad + row) * cols_pad + col] = S(acc[d]);
-    } else {
-        for (int v = 0; v < 3; ++v) {
-            int kc = kmap_p[a.tri[3 * y + v]];
-            for (int d = d0; d < nd; ++d) atomicAdd(&A[((size_t)d * rows_pad + row) * colsK_pad + kc], S(acc[3 * d + v]));
-        }
+    for (int i = 0; i < ND; ++i) accV[i] = R(0);
+#pragma unroll
+    for (int i = 0; i < 3 * ND; ++i) accK[i] = R(0);
+    const int d0 = nf_regular_pair<R, true, true, ND>(a, x, y, accV, accK);
+    R *AV = AVs + P.offV, *AK = AKs + P.offK;
+#pragma unroll
+    for (int d = 0; d < ND; ++d)
+        if (d >= d0) AV[((size_t)d * P.rows_pad + row) * P.colsV_pad + col] = accV[d];
+    for (int v = 0; v < 3; ++v) {
+        const int kc = a.kmap[(size_t)P.index * a.nv + a.tri[3 * y + v]];
+#pragma unroll
+        for (int d = 0; d < ND; ++d)
+            if (d >= d0) atomicAdd(&AK[((size_t)d * P.rows_pad + row) * P.colsK_pad + kc], accK[3 * d + v]);
     }
 }
 
-template <typename R, typename S>
-void launch_nf_regular_T(const NfQuadArgs &a, const PanelGPU &P, S *AV, S *AK, cudaStream_t st)
+template <typename R>
+void launch_nf_regular_T(const NfQuadArgs &a, const PanelGPU *panels, dim3 grd, R *AV, R *AK, cudaStream_t st)
 {
-    dim3 blk(32, 8);
-    dim3 grd((P.ncolV + 31) / 32, (P.nrows + 7) / 8);
-    k_nf_regular<R, S, false><<<grd, blk, 0, st>>>(a, P.row0, P.nrows, P.rows_pad, P.colsV_pad, a.colV + P.colV_at,
-                                                     AV + P.offV, nullptr, 0, P.ncolV);
-    k_nf_regular<R, S, true><<<grd, blk, 0, st>>>(a, P.row0, P.nrows, P.rows_pad, P.colsV_pad, a.colV + P.colV_at,
-                                                    AK + P.offK, a.kmap + (size_t)P.index * a.nv, P.colsK_pad, P.ncolV);
+    auto kf = a.nd == 2 ? k_nf_regular<R, 2> : a.nd == 4 ? k_nf_regular<R, 4> : a.nd == 6 ? k_nf_regular<R, 6> : k_nf_regular<R, 8>;
+    kf<<<grd, dim3(32, 8), 0, st>>>(a, panels, AV, AK);
 }
 
-void launch_nf_regular(const NfQuadArgs &a, const PanelGPU &P, void *AV, void *AK, bool mixed, cudaStream_t st)
+void launch_nf_regular(const NfQuadArgs &a, const PanelGPU *panels, int npanel, int max_rows, int max_cols, void *AV,
+                       void *AK, bool mixed, cudaStream_t st)
 {
-    if (mixed)
-        launch_nf_regular_T<float, float>(a, P, (float *)AV, (float *)AK, st);
-    else
-        launch_nf_regular_T<double, double>(a, P, (double *)AV, (double *)AK, st);
+    for (int p0 = 0; p0 < npanel; p0 += 65535) {  // grid z limit
+        const dim3 grd((max_cols + 31) / 32, (max_rows + 7) / 8, std::min(npanel - p0, 65535));
+        if (mixed)
+            launch_nf_regular_T<float>(a, panels + p0, grd, (float *)AV, (float *)AK, st);
+        else
+            launch_nf_regular_T<double>(a, panels + p0, grd, (double *)AV, (double *)AK, st);
+    }
 }
 
 // ------------------------------------------------------------------------------------------
@@ -224,8 +230,7 @@ __global__ void __launch_bounds__(128) k_nf_singular(NfQuadArgs a, const int *__
             double r = sqrt(dx[0] * dx[0] + dx[1] * dx[1] + dx[2] * dx[2]);
             double wt = w4 * jac[u] * Jx * Jy;
             double vv[2], kk[2];
-            time_V_all<double>(r, a.h, a.alpha, 2, vv);
-            time_K_all<double>(r, a.h, a.alpha, 2, kk);
+            time_integrals<double, true, true, 2>(r, a.tc, vv, kk);
             accV[0] += wt * vv[0];
             accV[1] += wt * vv[1];
             double dn = dx[0] * ny[0] + dx[1] * ny[1] + dx[2] * ny[2];

@@ -5,6 +5,7 @@
 
 #include <cstdint>
 
+#include "device_math.cuh"
 #include "pfmm_internal.h"
 
 namespace pfmm {
@@ -40,12 +41,16 @@ struct NfQuadArgs {
     int nq_sing;
     const int *colV;       // all panels' V columns
     const int *kmap;       // [npanel][nv]
+    dev::TimeConst<double> tc;  // constants of the nd step ends
+    dev::TimeConst<float> tcf;
 };
 
 void launch_space_tables(const SetupArgs &a, cudaStream_t st);
 void launch_e1_table(int na, int mt, int mx, int G, double hx, double hxp, double ht, double alpha, double *E1,
                      double *pref, cudaStream_t st);
-void launch_nf_regular(const NfQuadArgs &a, const PanelGPU &P, void *AV, void *AK, bool mixed, cudaStream_t st);
+// panels: device array; max_rows, max_cols: largest nrows and ncolV of the panels
+void launch_nf_regular(const NfQuadArgs &a, const PanelGPU *panels, int npanel, int max_rows, int max_cols, void *AV,
+                       void *AK, bool mixed, cudaStream_t st);
 void launch_nf_singular(const NfQuadArgs &a, const int *sing, int nsing, const PanelGPU *panels, void *AV, void *AK,
                         bool mixed, cudaStream_t st, double *cV = nullptr, double *cK = nullptr);
 

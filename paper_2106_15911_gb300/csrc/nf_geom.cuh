@@ -88,26 +88,34 @@ __device__ __forceinline__ int ss_points(int cls, double xi, double e1, double e
     return 2;
 }
 
-// Regular quadrature of the pair (x, y) (internal triangles) for the step offsets d0 .. nd-1 of
-// Eq. eval_sl_nf_block: acc[d] (V) or acc[3 d + v] (K, v: y's vertices in mesh order) are
-// accumulated (the caller zeroes them).  Touching pairs start at d0 = 2: their d = 0, 1 entries
-// come from the Sauter-Schwab rule.  Returns d0.
-template <typename R, bool KOP>
-__device__ __forceinline__ int nf_regular_pair(const NfQuadArgs &a, int x, int y, R *acc)
+template <typename R>
+__device__ __forceinline__ const dev::TimeConst<R> &time_const(const NfQuadArgs &a);
+template <>
+__device__ __forceinline__ const dev::TimeConst<double> &time_const<double>(const NfQuadArgs &a) { return a.tc; }
+template <>
+__device__ __forceinline__ const dev::TimeConst<float> &time_const<float>(const NfQuadArgs &a) { return a.tcf; }
+
+// Regular quadrature of the pair (x, y) (internal triangles) for the step offsets d0 .. ND-1 of
+// Eq. eval_sl_nf_block: accV[d] and accK[3 d + v] (v: y's vertices in mesh order) are accumulated
+// (the caller zeroes them).  Touching pairs start at d0 = 2: their d = 0, 1 entries come from the
+// Sauter-Schwab rule.  Returns d0.
+template <typename R, bool DOV, bool DOK, int ND>
+__device__ __forceinline__ int nf_regular_pair(const NfQuadArgs &a, int x, int y, R *accV, R *accK)
 {
     double PX[3][3], PY[3][3], nx[3], ny[3];
     load_tri(a.verts, a.tri, x, PX);
     load_tri(a.verts, a.tri, y, PY);
     double Jx = tri_jac(PX, nx), Jy = tri_jac(PY, ny);
     tri_normal_orig(PY, ny);
-    const int nd = a.nd;
-    int d0 = shared_count(a.tri, x, y) > 0 ? 2 : 0;  // d = 0, 1 of touching pairs: singular rule
+    const int d0 = shared_count(a.tri, x, y) > 0 ? 2 : 0;  // d = 0, 1 of touching pairs: singular rule
     const int nq = a.nq_reg;
-    const R h = R(a.h), alpha = R(a.alpha);
+    const dev::TimeConst<R> &tc = time_const<R>(a);
+#pragma unroll 1
     for (int i = 0; i < nq; ++i) {
         double s1 = a.rule_reg[i], s2 = a.rule_reg[nq + i], wi = a.rule_reg[2 * nq + i];
         double xp[3];
         for (int c = 0; c < 3; ++c) xp[c] = PX[0][c] + s1 * (PX[1][c] - PX[0][c]) + s2 * (PX[2][c] - PX[1][c]);
+#pragma unroll 1
         for (int j = 0; j < nq; ++j) {
             double t1 = a.rule_reg[j], t2 = a.rule_reg[nq + j], wj = a.rule_reg[2 * nq + j];
             double yp[3], dx[3];
@@ -117,24 +125,39 @@ __device__ __forceinline__ int nf_regular_pair(const NfQuadArgs &a, int x, int y
             }
             double r = sqrt(dx[0] * dx[0] + dx[1] * dx[1] + dx[2] * dx[2]);
             R wt = R(wi * wj * Jx * Jy);
-            R vals[8];
-            if (!KOP) {
-                dev::time_V_all<R>(R(r), h, alpha, nd, vals);
-                for (int d = d0; d < nd; ++d) acc[d] += wt * vals[d];
-            } else {
-                dev::time_K_all<R>(R(r), h, alpha, nd, vals);
+            R v[ND], k[ND];
+            dev::time_integrals<R, DOV, DOK, ND>(R(r), tc, v, k);
+            if (DOV)
+#pragma unroll
+                for (int d = 0; d < ND; ++d)
+                    if (d >= d0) accV[d] += wt * v[d];
+            if (DOK) {
                 R dn = R(dx[0] * ny[0] + dx[1] * ny[1] + dx[2] * ny[2]);
                 R by[3] = {R(1.0 - t1), R(t1 - t2), R(t2)};
-                for (int d = d0; d < nd; ++d) {
-                    R v = wt * dn * vals[d];
-                    acc[3 * d + 0] += v * by[0];
-                    acc[3 * d + 1] += v * by[1];
-                    acc[3 * d + 2] += v * by[2];
+#pragma unroll
+                for (int d = 0; d < ND; ++d) {
+                    if (d < d0) continue;
+                    R q = wt * dn * k[d];
+                    accK[3 * d + 0] += q * by[0];
+                    accK[3 * d + 1] += q * by[1];
+                    accK[3 * d + 2] += q * by[2];
                 }
             }
         }
     }
     return d0;
+}
+
+// one layer, offsets up to a.nd (2, 4, 6 or 8)
+template <typename R, bool KOP>
+__device__ __forceinline__ int nf_regular_pair(const NfQuadArgs &a, int x, int y, R *acc)
+{
+    switch (a.nd) {
+    case 2: return nf_regular_pair<R, !KOP, KOP, 2>(a, x, y, acc, acc);
+    case 4: return nf_regular_pair<R, !KOP, KOP, 4>(a, x, y, acc, acc);
+    case 6: return nf_regular_pair<R, !KOP, KOP, 6>(a, x, y, acc, acc);
+    default: return nf_regular_pair<R, !KOP, KOP, 8>(a, x, y, acc, acc);
+    }
 }
 
 }  // namespace pfmm
