@@ -285,11 +285,11 @@ int pfmm::run_nf_crt(pfmm_handle *H, int op, const double *x, int nrhs, double *
     const int cols = op == 0 ? H->colsV_u : H->colsK_u, b = op == 0 ? H->crt_bV : H->crt_bK;
     launch_crt_split_input(x, op == 0 ? H->d_perm : nullptr, op == 0 ? H->nt : H->nv, cols, nrhs, H->Et, b, H->d_Wres,
                            H->d_wmax, st);
-    const int nint = H->Et / 2;
-    uint64_t dims[5] = {(uint64_t)cols, 2, (uint64_t)nint, (uint64_t)nrhs, (uint64_t)kCrtModuli};
-    uint64_t str[4] = {(uint64_t)cols * 2, (uint64_t)cols * 4, (uint64_t)cols * 4 * nint,
-                       (uint64_t)cols * 4 * nint * nrhs};
-    uint32_t box[5] = {64, 1, (uint32_t)nf_crt_intervals(nint, H->crt_form), 1, 1};
+    const int ls = H->ls, nint = H->Et / ls;
+    uint64_t dims[5] = {(uint64_t)cols, (uint64_t)ls, (uint64_t)nint, (uint64_t)nrhs, (uint64_t)kCrtModuli};
+    uint64_t str[4] = {(uint64_t)cols * 2, (uint64_t)cols * 2 * ls, (uint64_t)cols * 2 * ls * nint,
+                       (uint64_t)cols * 2 * ls * nint * nrhs};
+    uint32_t box[5] = {64, 1, (uint32_t)nf_crt_intervals(nint, ls, H->crt_form), 1, 1};
     CUtensorMap mW;
     if ((rc = encode_map(&mW, H->d_Wres, 5, dims, str, box))) return rc;
     NfCrtParams P{};
@@ -303,7 +303,7 @@ int pfmm::run_nf_crt(pfmm_handle *H, int op, const double *x, int nrhs, double *
     P.res = H->d_res8;
     P.err = H->d_err;
     if (H->cur_ev) cudaEventRecord(H->cur_ev->ev[9], st);
-    if (launch_nf_apply_crt(mW, P, H->nsm, st, H->crt_form))
+    if (launch_nf_apply_crt(mW, P, ls, H->nsm, st, H->crt_form))
         return fail(PFMM_ERR_CUDA, std::string("FP64 tensor-core nearfield launch: ") +
                                        cudaGetErrorString(cudaGetLastError()));
     if (H->cur_ev) {
@@ -449,7 +449,7 @@ static int build_crt(pfmm_handle *H, const Tree &t, bool fullV, bool fullK, cuda
     size_t free_b = 0, total_b = 0;
     CK(cudaMemGetInfo(&free_b, &total_b));
     const int colsV = t.panels[0].colsV_pad, colsK = t.panels[0].colsK_pad;
-    const size_t need = (fullV ? crt_panel_bytes(H->nt, colsV) : 0) + (fullK ? crt_panel_bytes(H->nt, colsK) : 0);
+    const size_t need = (fullV ? crt_panel_bytes(H->nt, colsV, H->nd) : 0) + (fullK ? crt_panel_bytes(H->nt, colsK, H->nd) : 0);
     if (need > free_b / 10 * 7) return PFMM_OK;
     const int nd = H->nd, npanel = (int)t.panels.size();
     unsigned long long *rowmax = nullptr;
@@ -458,13 +458,13 @@ static int build_crt(pfmm_handle *H, const Tree &t, bool fullV, bool fullK, cuda
     for (int op = 0; op < 2; ++op) {
         if (!(op == 0 ? fullV : fullK)) continue;
         const int cols = op == 0 ? colsV : colsK;
-        const int b = crt_bits(4ll * cols);
+        const int b = crt_bits((long long)nd * cols);
         int *rexp = nullptr;
         unsigned char *res = nullptr;
-        if ((rc = H->alloc(&rexp, (size_t)H->nt)) || (rc = H->alloc(&res, crt_panel_bytes(H->nt, cols)))) return rc;
+        if ((rc = H->alloc(&rexp, (size_t)H->nt)) || (rc = H->alloc(&res, crt_panel_bytes(H->nt, cols, nd)))) return rc;
         const double *A = (const double *)(op == 0 ? H->d_AV : H->d_AK);
         launch_crt_row_exps(A, H->d_panels, npanel, op, nd, b, rowmax, H->nt, rexp, st);
-        launch_crt_split_panel(A, H->d_panels, H->d_tri_leaf, rexp, op, H->nt, cols, res, st);
+        launch_crt_split_panel(A, H->d_panels, H->d_tri_leaf, rexp, op, H->nt, cols, nd, res, st);
         CK(cudaStreamSynchronize(st));
         CK(cudaGetLastError());
         if (op == 0) {
@@ -823,7 +823,7 @@ static int build_impl(const pfmm_mesh *mesh, const pfmm_params *prm, cudaStream_
         }
         CK(cudaGetLastError());
 
-        // tensor-core nearfield: mixed mode, two steps per leaf, every panel spans all columns
+        // tensor-core nearfield: every panel spans all columns; mixed mode: two steps per leaf
         int dev = 0;
         CK(cudaGetDevice(&dev));
         CK(cudaDeviceGetAttribute(&H->nsm, cudaDevAttrMultiProcessorCount, dev));
@@ -832,7 +832,7 @@ static int build_impl(const pfmm_mesh *mesh, const pfmm_params *prm, cudaStream_
         CK(cudaDeviceGetAttribute(&cc_minor, cudaDevAttrComputeCapabilityMinor, dev));
         // tensor cores for the stored panels when every panel spans all columns: the FP16 split
         // (mixed mode) or the exact residue arithmetic (FP64 mode)
-        bool eligible = !H->otf && H->ls == 2 && prm->nf_engine == PFMM_NF_AUTO && cc_major == 10 && encode_fn() &&
+        bool eligible = !H->otf && (H->ls == 2 || !H->mixed) && prm->nf_engine == PFMM_NF_AUTO && cc_major == 10 && encode_fn() &&
                         (H->mixed || !prm->fp64_native);
         bool fullV = eligible, fullK = eligible;
         for (const Panel &P : t.panels) {
@@ -1168,8 +1168,8 @@ int pfmm_get_info(const pfmm_handle *h, pfmm_info *info)
     info->nf_form_ms[0] = h->crt_form_ms[0];
     info->nf_form_ms[1] = h->crt_form_ms[1];
     if (h->crtV || h->crtK)
-        info->nearfield_bytes += (h->crtV ? pfmm::crt_panel_bytes(h->nt, h->colsV_u) : 0) +
-                                 (h->crtK ? pfmm::crt_panel_bytes(h->nt, h->colsK_u) : 0);
+        info->nearfield_bytes += (h->crtV ? pfmm::crt_panel_bytes(h->nt, h->colsV_u, h->nd) : 0) +
+                                 (h->crtK ? pfmm::crt_panel_bytes(h->nt, h->colsK_u, h->nd) : 0);
     info->nearfield_v_elements = t.sizeV;
     info->nf_dense_columns = t.dense_cols ? 1 : 0;
     // separable M2L work per level: pass 1 over cells (X1, Y2, Y3) and the budget chains of every

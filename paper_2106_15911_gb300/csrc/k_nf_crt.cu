@@ -24,20 +24,20 @@
 // The residues of A' are stored as bytes (r + 128), half the bytes of FP16, because the stored
 // blocks are the bulk of the traffic: 16 bytes per element.  All panels index the same columns, so
 // the rows are tiled regardless of panels: tile t holds the target triangles 128 t .. 128 t + 127, and
-// the four step offsets of one 64-column block of a tile are 32 KB in one piece, [modulus][tile]
-// [column block][d][row][64], brought in by one bulk copy.  Converter warps turn the bytes into FP16
+// the 2 LS step offsets (LS steps per leaf) of one 64-column block of a tile are one piece, [modulus]
+// [tile][column block][d][row][64], brought in by one bulk copy (32 KB at LS = 2).  Converter warps turn the bytes into FP16
 // in registers (byte permute onto 1024 + u, one subtraction, exact) and write them to tensor memory,
 // from where tcgen05.mma takes them as the A operand.
 //
-// Tiles: 128 rows x (NI leaf intervals x 2 phases) columns; W is a TMA tensor [modulus][rhs]
+// Tiles: 128 rows x (NI leaf intervals x LS phases) columns; W is a TMA tensor [modulus][rhs]
 // [interval][phase][column], so the time shift d is a coordinate offset and causality the zero fill.
-// For one column block the four step offsets need only four W tiles, (phase 0 or 1) x (interval
-// shift 0 or 1); stored in the order (0, 1), (1, 1), (0, 0), (1, 0), phase ph of offset d is tile
-// 2 + ph - d, so both phases of an offset are one contiguous operand of 2 NI rows, and each W tile is
-// brought in once for its two uses.  A work item is (modulus, row tile, interval block, rhs).  The
-// accumulator of phase 0 is reduced modulo p before column blocks r, 2 r, ..., that of phase 1
-// before r / 2, 3 r / 2, ... (r = 4 .. 8 by the modulus: 256 r products of two residues stay below
-// 2^24): the other phase's MMAs of that block are issued first and hide the reduction.
+// For one column block the 2 LS step offsets need only 2 LS W tiles, one per step of the interval
+// before and of the interval itself; in that order phase ph of offset d is tile LS + ph - d, so all
+// phases of an offset are one contiguous operand of up to LS NI rows, and each W tile is brought in
+// once for its LS uses.  A work item is (modulus, row tile, interval block, rhs).  The accumulators
+// are reduced modulo p every r column blocks (r by the modulus and LS: 128 LS r products of two
+// residues stay below 2^24).  At LS = 2 the phases are reduced in turn, half a period apart, and the
+// other phase's MMAs of that block are issued first and hide the reduction.
 // The roles meet once per column block (16 MMAs): a wait, the issue and the commit of a step cost the
 // issuing thread some 400 cycles, which one step per offset (448 cycles of MMAs) did not hide.
 // Warps: 0 TMA of W, 1 TMEM allocation and MMA issue, 2-9 converters (two groups of four, two offsets
@@ -65,17 +65,15 @@ using namespace tc;
 __constant__ int c_p[kCrtModuli];              // the moduli
 __constant__ float c_invp[kCrtModuli];         // 1 / p (FP32)
 __constant__ float c_pf[kCrtModuli];           // the moduli (FP32)
-__constant__ int c_red[kCrtModuli];            // column blocks between two reductions of an accumulator (even)
+__constant__ int c_red[5][kCrtModuli];         // [LS] column blocks between two reductions (LS = 2: even)
 __constant__ float c_pow11[kCrtModuli][5];     // 2^(11 k) mod p_i (FP32), k = 0 .. 4
 __constant__ float c_pjmodpif[kCrtModuli][kCrtModuli];  // (p_0 ... p_{j-1}) mod p_i, j < i (FP32)
 __constant__ float c_invPif[kCrtModuli];       // (p_0 ... p_{i-1})^-1 mod p_i (FP32)
 
 constexpr int BM = 128, BK = 64;
 constexpr int A8_TILE = BM * BK;         // 8 KB of residue bytes
-constexpr int A8_STAGE = 4 * A8_TILE;    // the four offsets of a column block
-constexpr int NST = 2;                   // column blocks in flight (bytes, FP16 tiles in tensor memory, W)
+constexpr int NST = 2;                   // column blocks in flight (bytes, W)
 constexpr int kCrtThreads = 608;
-constexpr int kTmemA = 256;              // first tensor memory column of the A tiles (32 columns each, four a stage)
 constexpr uint64_t kTimeoutNs = 2000000000ull;
 
 __device__ __forceinline__ void bulk_copy(void *dst, const void *src, uint32_t bytes, uint64_t *bar)
@@ -174,10 +172,16 @@ __device__ __forceinline__ void bytes_to_half(uint32_t w, uint32_t &lo, uint32_t
     hi = *reinterpret_cast<const uint32_t *>(&y);
 }
 
-template <int NI>
-struct CrtSmem {
-    static constexpr int W_TILE = NI * BK * 2, W_STAGE = 4 * W_TILE;
-    static constexpr size_t bytes = (size_t)NST * (W_STAGE + A8_STAGE) + 1024 + 256;
+template <int NI, int LS>
+struct CrtShape {
+    static constexpr int ND = 2 * LS;  // step offsets
+    static constexpr int W_TILE = NI * BK * 2, W_STAGE = ND * W_TILE, A8_STAGE = ND * A8_TILE;
+    // tensor memory: LS NI accumulator columns, then TA stages of ND FP16 tiles of 32 columns
+    static constexpr int TA = LS <= 3 ? 2 : 1, kTmemA = 512 - TA * ND * 32;
+    static_assert(LS * NI <= kTmemA && LS * NI <= 256, "tensor memory");
+    static constexpr int NG = LS == 2 ? 2 : 1, GC = LS * NI / NG;  // groups reduced together, their columns
+    // one CTA per SM (it takes all of the tensor memory)
+    static constexpr size_t used = (size_t)NST * (W_STAGE + A8_STAGE) + 1024 + 256, bytes = used > 118784 ? used : 118784;
 };
 
 // x mod p into [-(p-1)/2 - p, (p-1)/2 + p] for an integer-valued |x| < 2^24 (exact): the FP32
@@ -192,10 +196,11 @@ __device__ __forceinline__ float mod_small(float x, float p, float invp)
 
 }  // namespace
 
-template <int NI>
+template <int NI, int LS>
 __global__ void __launch_bounds__(kCrtThreads, 1) k_nf_apply_crt(const __grid_constant__ CUtensorMap mapW, NfCrtParams P)
 {
-    using S = CrtSmem<NI>;
+    using S = CrtShape<NI, LS>;
+    constexpr int ND = S::ND, A8_STAGE = S::A8_STAGE, TA = S::TA, kTmemA = S::kTmemA, NG = S::NG, GC = S::GC;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char *smem = (unsigned char *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     unsigned char *sA = smem + NST * S::W_STAGE;
@@ -248,7 +253,7 @@ __global__ void __launch_bounds__(kCrtThreads, 1) k_nf_apply_crt(const __grid_co
     };
 
     if (warp == 0) {
-        // ---------------- TMA of W: the four (phase, shift) tiles of a column block
+        // ---------------- TMA of W: the tiles of a column block
         if (lane == 0) {
             int g = 0;
             for (int it = blockIdx.x; it < P.nitems && !s_abort; it += gridDim.x) {
@@ -259,8 +264,8 @@ __global__ void __launch_bounds__(kCrtThreads, 1) k_nf_apply_crt(const __grid_co
                     unsigned char *d = smem + s * S::W_STAGE;
                     mbar_expect_tx(&wfull[s], S::W_STAGE);
 #pragma unroll
-                    for (int q = 0; q < 4; ++q)  // (0, 1), (1, 1), (0, 0), (1, 0)
-                        tma_5d(d + q * S::W_TILE, &mapW, kb * BK, q & 1, I.ib * NI - (q < 2 ? 1 : 0), I.rhs, I.m,
+                    for (int q = 0; q < ND; ++q)  // the steps of the interval before, then its own
+                        tma_5d(d + q * S::W_TILE, &mapW, kb * BK, q % LS, I.ib * NI - (q < LS ? 1 : 0), I.rhs, I.m,
                                &wfull[s]);
                 }
             }
@@ -288,19 +293,19 @@ __global__ void __launch_bounds__(kCrtThreads, 1) k_nf_apply_crt(const __grid_co
         // ---------------- MMA issuer
         const uint32_t issue = elect_lane(), tm = __shfl_sync(0xffffffffu, tmem, 0);
         const uint32_t wlo = __shfl_sync(0xffffffffu, (su32(smem) >> 4) & 0x3FFFu, 0) | 1u << 16;
-        constexpr uint32_t id2 = idesc_f16(BM, 2 * NI), id1 = idesc_f16(BM, NI), WT = S::W_TILE >> 4;
+        constexpr uint32_t WT = S::W_TILE >> 4;
         int g = 0;
-        uint32_t ev0 = 0, ev1 = 0;  // accumulator hand-overs of the phases
+        uint32_t ev0 = 0, ev1 = 0;  // accumulator hand-overs of the groups
         for (int it = blockIdx.x; it < P.nitems && !s_abort; it += gridDim.x) {
             const CItem I(P, nib, it);
-            const int rp = c_red[I.m];
+            const int rp = c_red[LS][I.m];
             // the previous item's outputs have been read
             bool ok = (ev0 == 0 || wait(&tempty[0], (ev0 - 1) & 1, 13)) && (ev1 == 0 || wait(&tempty[1], (ev1 - 1) & 1, 13));
-            int next0 = rp, next1 = rp / 2;  // column blocks before which a phase is reduced
+            int next0 = rp, next1 = rp / 2;  // column blocks before which a group is reduced
             for (int kb = 0; kb < P.nkb && ok; ++kb, ++g) {
                 const int s = g % NST;
-                const uint32_t w0 = wlo + s * (S::W_STAGE >> 4), at = tm + kTmemA + s * 128;
-                const bool r0 = kb == next0, r1 = kb == next1;
+                const uint32_t w0 = wlo + s * (S::W_STAGE >> 4), at = tm + kTmemA + g % TA * (ND * 32);
+                const bool r0 = kb == next0, r1 = NG == 2 && kb == next1;
                 if (r0) {
                     mma_commit_if(issue, &tfull[0]);
                     ++ev0;
@@ -312,30 +317,30 @@ __global__ void __launch_bounds__(kCrtThreads, 1) k_nf_apply_crt(const __grid_co
                     next1 += rp;
                 }
                 ok = wait(&wfull[s], (g / NST) & 1, 14) && wait(&aready[s], (g / NST) & 1, 15);
+                if (ok && NG == 1 && r0) ok = wait(&tempty[0], (ev0 - 1) & 1, 16);
                 if (!ok) break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                if (!r0 && !r1) {
-                    const uint32_t more = kb > 0 ? 1u : 0u;  // an item's first MMA starts both phases from zero
+                // offset d for the np phases from p0
+                auto offset = [&](int d, int p0, int np, uint32_t first) {
+                    const uint32_t id = idesc_f16(BM, np * NI);
 #pragma unroll
-                    for (int d = 0; d < 3; ++d)
+                    for (int kk = 0; kk < BK / 16; ++kk)
+                        mma_f16_ts(issue, tm + p0 * NI, at + d * 32 + kk * 8, w0 + (LS + p0 - d) * WT + kk * 2, id,
+                                   kk == 0 ? first : 1u);
+                };
+                if (NG == 1 || (!r0 && !r1)) {
+                    // the first MMA of an item, of offset 0, starts all phases from zero
 #pragma unroll
-                        for (int kk = 0; kk < BK / 16; ++kk)
-                            mma_f16_ts(issue, tm, at + d * 32 + kk * 8, w0 + (2 - d) * WT + kk * 2, id2,
-                                       d == 0 && kk == 0 ? more : 1u);
-#pragma unroll
-                    for (int kk = 0; kk < BK / 16; ++kk) mma_f16_ts(issue, tm + NI, at + 96 + kk * 8, w0 + kk * 2, id1, 1u);
+                    for (int d = 0; d < ND; ++d) {
+                        const int p0 = d > LS ? d - LS : 0;
+                        offset(d, p0, LS - p0, d == 0 ? (kb > 0 ? 1u : 0u) : 1u);
+                    }
                 } else {
                     // the other phase first, while the epilogue reduces this one
                     auto phase = [&](int ph) {
 #pragma unroll
-                        for (int d = 0; d < 3; ++d)
-#pragma unroll
-                            for (int kk = 0; kk < BK / 16; ++kk)
-                                mma_f16_ts(issue, tm + ph * NI, at + d * 32 + kk * 8, w0 + (2 + ph - d) * WT + kk * 2, id1, 1u);
-                        if (ph == 1)
-#pragma unroll
-                            for (int kk = 0; kk < BK / 16; ++kk)
-                                mma_f16_ts(issue, tm + NI, at + 96 + kk * 8, w0 + kk * 2, id1, 1u);
+                        for (int d = 0; d < ND; ++d)
+                            if (d <= LS + ph) offset(d, ph, 1, 1u);
                     };
                     if (r0) {
                         phase(1);
@@ -352,13 +357,15 @@ __global__ void __launch_bounds__(kCrtThreads, 1) k_nf_apply_crt(const __grid_co
                 mma_commit_if(issue, &done[s]);
             }
             mma_commit_if(issue, &tfull[0]);
-            mma_commit_if(issue, &tfull[1]);
             ++ev0;
-            ++ev1;
+            if (NG == 2) {
+                mma_commit_if(issue, &tfull[1]);
+                ++ev1;
+            }
         }
     } else if (warp < 10) {
-        // ---------------- converters: thread = row; the bytes of two offsets to FP16 pairs in TMEM
-        const int row = (warp & 3) * 32 + lane, d0 = (warp - 2) >> 2 << 1;
+        // ---------------- converters: thread = row; the bytes of LS offsets to FP16 pairs in TMEM
+        const int row = (warp & 3) * 32 + lane, d0 = ((warp - 2) >> 2) * LS;
         const uint32_t tq = tmem + ((uint32_t)((warp & 3) * 32) << 16) + kTmemA + d0 * 32;
         int g = 0;
         bool ok = true;
@@ -366,9 +373,9 @@ __global__ void __launch_bounds__(kCrtThreads, 1) k_nf_apply_crt(const __grid_co
             for (int kb = 0; kb < P.nkb; ++kb, ++g) {
                 const int s = g % NST;
                 if (!(ok = warp_wait(&a8full[s], (g / NST) & 1, 18))) break;
-                uint4 b[2][4];
+                uint4 b[LS][4];
 #pragma unroll
-                for (int d = 0; d < 2; ++d) {
+                for (int d = 0; d < LS; ++d) {
                     // 16-byte chunk c of row r is at c ^ ((r / 2) mod 4): a quarter warp reads all banks
                     const unsigned char *src = sA + s * A8_STAGE + (d0 + d) * A8_TILE + row * 64;
 #pragma unroll
@@ -388,72 +395,80 @@ __global__ void __launch_bounds__(kCrtThreads, 1) k_nf_apply_crt(const __grid_co
                 convert(b[0]);
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&a8empty[s]);
-                if (!(ok = warp_wait(&done[s], ((g / NST) & 1) ^ 1, 19))) break;
+                // the MMAs of column block g - TA, which read these tiles' place, have completed
+                const int gd = g - TA;
+                if (gd >= 0 && !(ok = warp_wait(&done[gd % NST], (gd / NST) & 1, 19))) break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                tmem_st32_async(tq + s * 128, v);
-                convert(b[1]);
-                tmem_st32_async(tq + s * 128 + 32, v);
+                const uint32_t ts = tq + g % TA * (ND * 32);
+                tmem_st32_async(ts, v);
+#pragma unroll
+                for (int d = 1; d < LS; ++d) {
+                    convert(b[d]);
+                    tmem_st32_async(ts + d * 32, v);
+                }
                 asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
                 asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&aready[s]);
             }
     } else {
-        // ---------------- epilogue: warps 10..17, TMEM lane quadrant = warp % 4, half of a phase's columns
-        constexpr int NC = NI >= 64 ? NI / 2 : NI;  // columns of a phase per warp
-        const int quad = warp & 3, half = (warp - 10) >> 2, c00 = half * NC;
-        const bool active = NI >= 64 || half == 0;
+        // ---------------- epilogue: warps 10..17, TMEM lane quadrant = warp % 4, every other 32 columns
+        constexpr int NCH = GC / 32, NC = (NCH + 1) / 2;  // 32-column chunks of a group, of a warp
+        const int quad = warp & 3, half = (warp - 10) >> 2;
         uint32_t ev[2] = {0, 0};
         bool ok = true;
         for (int it = blockIdx.x; it < P.nitems && ok; it += gridDim.x) {
             const CItem I(P, nib, it);
             const float p = c_pf[I.m], invp = c_invp[I.m];
-            const int rp = c_red[I.m];
-            bool odd = true;  // phase 1 is reduced first, then in turn
-            for (int kb = rp / 2; ok; kb += rp / 2, odd = !odd) {
+            const int rp = c_red[LS][I.m] / NG;
+            bool odd = NG == 2;  // of two groups the second is reduced first, then in turn
+            for (int kb = rp; ok; kb += rp, odd = NG == 2 && !odd) {
                 const bool last = kb >= P.nkb;
 #pragma unroll
-                for (int ph = 0; ph < 2; ++ph) {
-                    if (!ok || (!last && (ph == 1) != odd)) continue;
-                    if (!(ok = warp_wait(&tfull[ph], ev[ph]++ & 1, 20))) continue;
+                for (int gr = 0; gr < NG; ++gr) {
+                    if (!ok || (!last && (gr == 1) != odd)) continue;
+                    if (!(ok = warp_wait(&tfull[gr], ev[gr]++ & 1, 20))) continue;
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                    const uint32_t tb = tmem + ((uint32_t)(quad * 32) << 16) + ph * NI + c00;
-                    if (active && !last) {
-                        uint32_t v[NC / 32][32];
+                    const uint32_t tb = tmem + ((uint32_t)(quad * 32) << 16) + gr * GC;
+                    if (!last) {
+                        uint32_t v[NC][32];
 #pragma unroll
-                        for (int c = 0; c < NC / 32; ++c) tmem_ld32_async(tb + c * 32, v[c]);
+                        for (int c = 0; c < NC; ++c)
+                            if (2 * c + half < NCH) tmem_ld32_async(tb + (2 * c + half) * 32, v[c]);
                         asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-                        for (int c = 0; c < NC / 32; ++c) {
+                        for (int c = 0; c < NC; ++c) {
+                            if (2 * c + half >= NCH) continue;
 #pragma unroll
                             for (int j = 0; j < 32; ++j)
                                 v[c][j] = __float_as_uint(mod_small(__uint_as_float(v[c][j]), p, invp));
-                            tmem_st32_async(tb + c * 32, v[c]);
+                            tmem_st32_async(tb + (2 * c + half) * 32, v[c]);
                         }
                         asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-                    } else if (active) {
+                    } else {
                         const int row = I.tile * BM + quad * 32 + lane;
                         unsigned char *out = P.res + ((size_t)I.m * P.nrhs + I.rhs) * P.Et * (size_t)P.nt + row;
 #pragma unroll 1
-                        for (int c0 = 0; c0 < NC; c0 += 32) {
+                        for (int c = half; c < NCH; c += 2) {
                             uint32_t v[32];
-                            tmem_ld32(tb + c0, v);
+                            tmem_ld32(tb + c * 32, v);
+                            const int col = gr * GC + c * 32, ph = col / NI, iv0 = I.ib * NI + col % NI;
                             if (row < P.nt) {
 #pragma unroll
                                 for (int j = 0; j < 32; ++j) {
-                                    const int iv = I.ib * NI + c00 + c0 + j;
                                     float r = mod_small(__uint_as_float(v[j]), p, invp);
                                     r = r < 0.f ? r + p : r;
                                     r = r < 0.f ? r + p : r;
                                     r = r >= p ? r - p : r;
-                                    if (iv < P.nint) out[(unsigned)(2 * iv + ph) * (unsigned)P.nt] = (unsigned char)(int)r;
+                                    if (iv0 + j < P.nint)
+                                        out[(unsigned)(LS * (iv0 + j) + ph) * (unsigned)P.nt] = (unsigned char)(int)r;
                                 }
                             }
                         }
                     }
                     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
                     __syncwarp();
-                    if (lane == 0) mbar_arrive(&tempty[ph]);
+                    if (lane == 0) mbar_arrive(&tempty[gr]);
                 }
                 if (last) break;
             }
@@ -547,12 +562,12 @@ __device__ __forceinline__ void residues16(long long a, float (&r)[kCrtModuli])
 // past the last triangle are zero.  Thread per (row, d, four columns)
 __global__ void k_crt_split_panel(const double *__restrict__ A, const PanelGPU *__restrict__ panels,
                                   const int *__restrict__ tri_leaf, const int *__restrict__ rowexp, int kop, int nt,
-                                  int ntiles, int ncp, unsigned char *__restrict__ res)
+                                  int ntiles, int ncp, int nd, unsigned char *__restrict__ res)
 {
     const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int nq = ncp / 4, c = (int)(i % nq) * 4;
     const size_t rd = i / nq;
-    const int d = (int)(rd & 3), x = (int)(rd >> 2);
+    const int x = (int)(rd / nd), d = (int)(rd - (size_t)x * nd);
     if (x >= ntiles * BM) return;
     const int nkb = ncp / BK, row = x & (BM - 1), ch = ((c & 63) >> 4) ^ ((row >> 1) & 3);
     double4 v = make_double4(0.0, 0.0, 0.0, 0.0);
@@ -573,8 +588,8 @@ __global__ void k_crt_split_panel(const double *__restrict__ A, const PanelGPU *
 #pragma unroll
         for (int m = 0; m < kCrtModuli; ++m) w[m] = (j ? w[m] : 0u) | (uint32_t)((int)r[m] + 128) << (8 * j);
     }
-    const size_t per_m = (size_t)ntiles * nkb * A8_STAGE;
-    const size_t o = ((size_t)(x / BM) * nkb + c / BK) * A8_STAGE + d * A8_TILE + row * 64 + ch * 16 + (c & 15);
+    const size_t per_m = (size_t)ntiles * nkb * nd * A8_TILE;
+    const size_t o = (((size_t)(x / BM) * nkb + c / BK) * nd + d) * A8_TILE + row * 64 + ch * 16 + (c & 15);
 #pragma unroll
     for (int m = 0; m < kCrtModuli; ++m) *reinterpret_cast<uint32_t *>(res + m * per_m + o) = w[m];
 }
@@ -668,14 +683,15 @@ int crt_upload_constants(cudaStream_t st)
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return -1;
     if (done[dev]) return 0;
     float invp[kCrtModuli], pf[kCrtModuli], pow11[kCrtModuli][5];
-    int red[kCrtModuli];
+    int red[5][kCrtModuli] = {{0}};
     float pj[kCrtModuli][kCrtModuli] = {{0.f}}, invPi[kCrtModuli];
     for (int i = 0; i < kCrtModuli; ++i) {
         pf[i] = (float)g_moduli[i];
         invp[i] = 1.0f / (float)g_moduli[i];
-        // largest even r with 256 r ((p - 1) / 2)^2 + 1.5 p < 2^24
+        // largest r (LS = 2: even) with 128 LS r ((p - 1) / 2)^2 + 1.5 p < 2^24
         const long long hp = (g_moduli[i] - 1) / 2;
-        red[i] = (int)(((1ll << 24) - 2 * g_moduli[i]) / (256 * hp * hp)) & ~1;
+        for (int ls = 1; ls <= 4; ++ls) red[ls][i] = (int)(((1ll << 24) - 2 * g_moduli[i]) / (128 * ls * hp * hp));
+        red[2][i] &= ~1;
         long long q = 1;  // p_0 ... p_{j-1} mod p_i, for j = 0 .. i
         for (int j = 0; j < i; ++j) {
             pj[j][i] = (float)q;
@@ -719,14 +735,18 @@ void launch_crt_row_exps(const double *A, const PanelGPU *panels, int npanel, in
     k_row_exps<<<(nt + 255) / 256, 256, 0, st>>>(rowmax, nt, b, rowexp);
 }
 
-size_t crt_panel_bytes(int nt, int ncp) { return (size_t)kCrtModuli * ((nt + BM - 1) / BM) * (ncp / BK) * A8_STAGE; }
+size_t crt_panel_bytes(int nt, int ncp, int nd)
+{
+    return (size_t)kCrtModuli * ((nt + BM - 1) / BM) * (ncp / BK) * nd * A8_TILE;
+}
 
 void launch_crt_split_panel(const double *A, const PanelGPU *panels, const int *tri_leaf, const int *rowexp, int kop,
-                            int nt, int ncp, unsigned char *res, cudaStream_t st)
+                            int nt, int ncp, int nd, unsigned char *res, cudaStream_t st)
 {
     const int ntiles = (nt + BM - 1) / BM;
-    const size_t n = (size_t)ntiles * BM * 4 * (ncp / 4);
-    k_crt_split_panel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(A, panels, tri_leaf, rowexp, kop, nt, ntiles, ncp, res);
+    const size_t n = (size_t)ntiles * BM * nd * (ncp / 4);
+    k_crt_split_panel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(A, panels, tri_leaf, rowexp, kop, nt, ntiles, ncp, nd,
+                                                                  res);
 }
 
 void launch_crt_split_input(const double *x, const int *perm, int ncol, int ncol_pad, int nrhs, int Et, int b,
@@ -748,29 +768,41 @@ void launch_crt_combine(const unsigned char *res, int nrhs, int Et, int nt, cons
     k_crt_combine<<<(unsigned)((per_mod + 255) / 256), 256, 0, st>>>(res, per_mod, per_rhs, nt, rowexp, wmax, b, f);
 }
 
-int nf_crt_intervals(int nint, int form)
+int nf_crt_intervals(int nint, int ls, int form)
 {
-    // the MMA's columns are 2 NI: few intervals take the narrowest block that holds them
+    // the MMA's columns are LS NI: few intervals take the narrowest block that holds them; three and
+    // four steps per leaf leave room for 32 intervals beside the A tiles in tensor memory
+    if (ls > 2) return 32;
     return nint <= 32 ? 32 : (nint <= 64 || form == 2 ? 64 : 128);
 }
 
-template <int NI>
+template <int NI, int LS>
 static int launch_crt_T(const CUtensorMap &W, NfCrtParams P, int nsm, cudaStream_t st)
 {
     P.nitems = kCrtModuli * P.ntiles * ((P.nint + NI - 1) / NI) * P.nrhs;
-    auto kf = k_nf_apply_crt<NI>;
-    if (cudaFuncSetAttribute(kf, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CrtSmem<NI>::bytes) != cudaSuccess)
-        return -1;
-    kf<<<std::min(P.nitems, nsm), kCrtThreads, CrtSmem<NI>::bytes, st>>>(W, P);
+    auto kf = k_nf_apply_crt<NI, LS>;
+    const size_t smem = CrtShape<NI, LS>::bytes;
+    if (cudaFuncSetAttribute(kf, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return -1;
+    kf<<<std::min(P.nitems, nsm), kCrtThreads, smem, st>>>(W, P);
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
-int launch_nf_apply_crt(const CUtensorMap &W, const NfCrtParams &P, int nsm, cudaStream_t st, int form)
+int launch_nf_apply_crt(const CUtensorMap &W, const NfCrtParams &P, int ls, int nsm, cudaStream_t st, int form)
 {
-    const int ni = nf_crt_intervals(P.nint, form);
-    return ni == 32   ? launch_crt_T<32>(W, P, nsm, st)
-           : ni == 64 ? launch_crt_T<64>(W, P, nsm, st)
-                      : launch_crt_T<128>(W, P, nsm, st);
+    const int ni = nf_crt_intervals(P.nint, ls, form);
+    switch (ls) {
+    case 1:
+        return ni == 32   ? launch_crt_T<32, 1>(W, P, nsm, st)
+               : ni == 64 ? launch_crt_T<64, 1>(W, P, nsm, st)
+                          : launch_crt_T<128, 1>(W, P, nsm, st);
+    case 2:
+        return ni == 32   ? launch_crt_T<32, 2>(W, P, nsm, st)
+               : ni == 64 ? launch_crt_T<64, 2>(W, P, nsm, st)
+                          : launch_crt_T<128, 2>(W, P, nsm, st);
+    case 3: return launch_crt_T<32, 3>(W, P, nsm, st);
+    case 4: return launch_crt_T<32, 4>(W, P, nsm, st);
+    default: return -1;
+    }
 }
 
 }  // namespace pfmm

@@ -30,10 +30,10 @@ int crt_bits(long long k_total);
 // in [2^(b-1), 2^b) after scaling)
 void launch_crt_row_exps(const double *A, const PanelGPU *panels, int npanel, int kop, int nd, int b,
                          unsigned long long *rowmax, int nt, int *rowexp, cudaStream_t st);
-// residues of the scaled, rounded panels of 4 step offsets (all of ncp columns) for NfCrtParams.A
-size_t crt_panel_bytes(int nt, int ncp);
+// residues of the scaled, rounded panels of nd step offsets (all of ncp columns) for NfCrtParams.A
+size_t crt_panel_bytes(int nt, int ncp, int nd);
 void launch_crt_split_panel(const double *A, const PanelGPU *panels, const int *tri_leaf, const int *rowexp, int kop,
-                            int nt, int ncp, unsigned char *res, cudaStream_t st);
+                            int nt, int ncp, int nd, unsigned char *res, cudaStream_t st);
 // per-rhs max |x| into wmax, residues [kCrtModuli][nrhs][Et][ncol_pad] of the scaled, rounded,
 // permuted (V) or padded (K) input
 void launch_crt_split_input(const double *x, const int *perm, int ncol, int ncol_pad, int nrhs, int Et, int b,
@@ -42,9 +42,9 @@ void launch_crt_split_input(const double *x, const int *perm, int ncol, int ncol
 void launch_crt_combine(const unsigned char *res, int nrhs, int Et, int nt, const int *rowexp,
                         const unsigned long long *wmax, int b, double *f, cudaStream_t st);
 // leaf intervals per work item: rows of the W tensor map's box
-int nf_crt_intervals(int nint, int form);
+int nf_crt_intervals(int nint, int ls, int form);
 // form 1: work items of up to 128 leaf intervals; form 2: of up to 64 (twice the items, each of half
 // the MMAs on the same blocks)
-int launch_nf_apply_crt(const CUtensorMap &W, const NfCrtParams &P, int nsm, cudaStream_t st, int form);
+int launch_nf_apply_crt(const CUtensorMap &W, const NfCrtParams &P, int ls, int nsm, cudaStream_t st, int form);
 
 }  // namespace pfmm
