@@ -671,30 +671,20 @@ static int build_impl(const pfmm_mesh *mesh, const pfmm_params *prm, cudaStream_
             if ((rc = H->alloc(&E1, ne)) || (rc = H->alloc(&pref, 2 * (size_t)na * na))) return rc;
             launch_e1_table(na, prm->m_t, mx, L.G, L.hx, L.hxp, L.ht, H->alpha, E1, pref, st);
             CK(cudaGetLastError());
-            if (L.G == 4 && H->fprec != 0) {  // before E1 is converted in place
-                if ((rc = H->alloc(&D.EF, m2l_fold_table_floats(na, mx, H->fprec)))) return rc;
-                launch_m2l_fold_table(E1, na, mx, D.ntr, H->fprec, D.EF, st);
-                for (int s = 0; s < 2; ++s) {
-                    const int eng = s ? kM2LFusedSliced : kM2LFused;
-                    if (H->fold[s].units || m2l_engine_for(H->fprec, 4, H->nk, H->ne, mx, s ? 4 : 2) != eng) continue;
-                    const M2LFoldPlan P = m2l_fold_plan(H->fprec, mx, kinv, s == 1);
-                    M2LFoldDev &F = H->fold[s];
+            if ((L.G == 4 && H->fprec != 0) || (L.G == 8 && H->fprec == 1)) {  // before E1 is converted in place
+                if ((rc = H->alloc(&D.EF, m2l_fold_table_floats(na, mx, L.G, H->fprec)))) return rc;
+                launch_m2l_fold_table(E1, na, mx, L.G, D.ntr, H->fprec, D.EF, st);
+                for (int s = (L.G == 4 ? 0 : 2); s < (L.G == 4 ? 2 : 3); ++s) {
+                    // T2 whole, sliced, 8^3: where that engine can run the level
+                    const int eng = s == 0 ? kM2LFused : s == 1 ? kM2LFusedSliced : kM2LSlab, force = s == 0 ? 2 : s == 1 ? 4 : 0;
+                    if (H->fold[s].units || m2l_engine_for(H->fprec, L.G, H->nk, H->ne, mx, force) != eng) continue;
+                    const M2LFoldPlan P = s == 2 ? m2l_slab_plan(mx, kinv) : m2l_fold_plan(H->fprec, mx, kinv, s == 1);
                     int *units = nullptr, *urow = nullptr;
                     if ((rc = upload(H, &units, P.units, st)) || (rc = upload(H, &urow, P.urow, st))) return rc;
                     CK(cudaStreamSynchronize(st));  // P's arrays go out of scope
-                    F.urows = P.urows;
-                    F.nslice = P.nslice;
-                    F.nunits = (int)P.units.size() / 2;
-                    F.first3 = P.first3;
-                    F.q3 = P.q3;
-                    for (int i = 0; i < 2; ++i) F.ntask[i] = P.ntask[i];
-                    for (int i = 0; i < kM2LMaxSlices; ++i) {
-                        F.first2[i] = P.first2[i];
-                        F.ntask2[i] = P.ntask2[i];
-                    }
-                    F.smem = P.smem;
-                    F.units = units;
-                    F.urow = urow;
+                    H->fold[s] = P.d;
+                    H->fold[s].units = units;
+                    H->fold[s].urow = urow;
                 }
             }
             if ((rc = device_to_R(H, &D.E1, E1, ne, st)) || (rc = device_to_R(H, &D.pref, pref, 2 * (size_t)na * na, st)))

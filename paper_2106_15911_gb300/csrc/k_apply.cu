@@ -1313,6 +1313,11 @@ int launch_m2l(int prec, const DevLevel &L, int l, const void *mu, void *lam, in
             return;
         }
         if (engine == kM2LSlab) {
+            if constexpr (std::is_same<R, float>::value) {
+                rc = launch_m2l_slab_folded(L, g.fold[2], (const R *)mb, (R *)lb, nrhs, g, (R *)T1, ws_elems, st);
+                if (rc <= 0) return;
+                rc = 0;  // no room for the folded moments
+            }
             const size_t ssm = m2l_slab_smem(g.nk, g.ne, g.mx, es);
             M2LArgs A{L.G, L.ntr, na, g.nk, g.mx, g.ne, L.nint, L.nbox, L.cellbox, L.boxcell, L.pk, L.pJ, 0,
                       g.kidx, g.kinv, g.eoff};

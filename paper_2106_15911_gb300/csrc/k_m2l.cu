@@ -42,6 +42,8 @@ namespace pfmm {
 
 namespace {
 
+constexpr int kSlabThreads = 256;  // 8^3 kernel
+
 template <typename R>
 struct Form;  // planes: FP32 words per value; NF: fibres per lane; threads and CTAs per SM
 template <>
@@ -239,9 +241,9 @@ k_m2l_folded(M2LFoldArgs A, const R *__restrict__ mu, R *__restrict__ lam)
     constexpr int PL = F::planes, NF = F::NF, LPU = 16 / NF, UPW = 32 / LPU, W = F::threads / 32, RW = 64 * PL;
     extern __shared__ __align__(16) float sm[];
     const int nk = A.nk, na = A.na, m1 = A.mx + 1;
-    float *T1 = sm, *U = T1 + A.ne * RW, *Es = U + A.urows * RW;
+    float *T1 = sm, *U = T1 + A.ne * RW, *Es = U + A.p.urows * RW;
     int2 *un = reinterpret_cast<int2 *>(Es + m1 * m1 * 8 * PL);
-    int *cbo = reinterpret_cast<int *>(un + A.nunits);  // [z][x][y] element offset of the cell's box, -1: empty
+    int *cbo = reinterpret_cast<int *>(un + A.p.nunits);  // [z][x][y] element offset of the cell's box, -1: empty
     int *urow = cbo + 64;                               // [nk] row of U of a moment
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, sub = lane / LPU, cl = lane % LPU;
     // grid x: (interval, node, chunk); even intervals have half the terms of odd ones
@@ -250,8 +252,8 @@ k_m2l_folded(M2LFoldArgs A, const R *__restrict__ mu, R *__restrict__ lam)
     const int nterm = k < 2 ? 0 : (k & 1 ? 2 * na : na);
     const int t_lo = chunk * A.tpc, t_hi = min(nterm, t_lo + A.tpc);
     if (A.part && t_lo >= t_hi) return;
-    for (int i = threadIdx.x; i < A.nunits; i += F::threads) un[i] = A.units[i];
-    for (int i = threadIdx.x; i < nk; i += F::threads) urow[i] = A.urow[i];
+    for (int i = threadIdx.x; i < A.p.nunits; i += F::threads) un[i] = reinterpret_cast<const int2 *>(A.p.units)[i];
+    for (int i = threadIdx.x; i < nk; i += F::threads) urow[i] = A.p.urow[i];
     for (int i = threadIdx.x; i < 64; i += F::threads) {
         const int box = A.cellbox[i];
         cbo[(i & 3) * 16 + (i >> 2)] = box < 0 ? -1 : box * na * nk;
@@ -312,7 +314,7 @@ k_m2l_folded(M2LFoldArgs A, const R *__restrict__ mu, R *__restrict__ lam)
         }
         __syncthreads();
         // pass 1: unit (k2, k3, nu1); the sum over k1 is cumulative, every partial sum is a row of T1
-        for (int ts = warp; ts < A.ntask[0]; ts += W) {
+        for (int ts = warp; ts < A.p.ntask1[0]; ts += W) {
             const UnitBits u(un[ts * UPW + sub]);
             int q[NF][4];
 #pragma unroll
@@ -329,11 +331,11 @@ k_m2l_folded(M2LFoldArgs A, const R *__restrict__ mu, R *__restrict__ lam)
             });
         }
         __syncthreads();
-        for (int sl = 0; sl < A.nslice; ++sl) {
+        for (int sl = 0; sl < A.p.nslice; ++sl) {
             if (sl > 0) __syncthreads();  // pass 3 of the previous slice is done with U
             // pass 2: unit = row of T2
-            for (int ts = warp; ts < A.ntask2[sl]; ts += W) {
-                const UnitBits u(un[A.first2[sl] + ts * UPW + sub]);
+            for (int ts = warp; ts < A.p.ntask2[sl]; ts += W) {
+                const UnitBits u(un[A.p.first2[sl] + ts * UPW + sub]);
                 R acc[NF][4];
                 chain_of(u.len, acc, T1 + u.row * RW + ((cl ^ (u.key << 1)) << 2), u.step * RW, RW, LPU * 4,
                             Es + u.nu * m1 * 8 * PL, [](int) {});
@@ -353,8 +355,8 @@ k_m2l_folded(M2LFoldArgs A, const R *__restrict__ mu, R *__restrict__ lam)
 #pragma unroll
             for (int q = 0; q < Q3; ++q) {
                 const int ts = warp + q * W;
-                if (ts >= A.ntask[1]) break;
-                const UnitBits u(un[A.first3 + ts * UPW + sub]);
+                if (ts >= A.p.ntask3) break;
+                const UnitBits u(un[A.p.first3 + ts * UPW + sub]);
                 if (u.slice != sl) continue;
                 R acc[NF][4];
                 chain_of(u.len, acc, U + u.row * RW + ((cl ^ (u.key << 1)) << 2), RW, 0, LPU * 4,
@@ -371,8 +373,8 @@ k_m2l_folded(M2LFoldArgs A, const R *__restrict__ mu, R *__restrict__ lam)
 #pragma unroll
     for (int q = 0; q < Q3; ++q) {
         const int ts = warp + q * W;
-        if (ts >= A.ntask[1]) break;
-        const UnitBits u(un[A.first3 + ts * UPW + sub]);
+        if (ts >= A.p.ntask3) break;
+        const UnitBits u(un[A.p.first3 + ts * UPW + sub]);
         if (!u.valid) continue;
         const bool odd = u.nu & 1;
 #pragma unroll
@@ -429,36 +431,38 @@ __global__ void k_m2l_sum_chunks(const R *__restrict__ part, int na, int tpc, si
 }
 
 // folded coefficients of a level from its FP64 table E1 [D][a][b][o][k][nu] (offsets beyond the
-// interaction radius are zero): EF [D][a][b][nu][k][8], in FP32 or as 8 high and 8 low parts
-__global__ void k_m2l_fold_table(const double *__restrict__ E1, int na, int m1, int ntr, int planes, float *__restrict__ EF)
+// interaction radius are zero): EF [D][a][b][nu][k][2 (G/2)^2] (sector, i, j), in FP32 or as high and low
+// parts
+__global__ void k_m2l_fold_table(const double *__restrict__ E1, int na, int m1, int G, int ntr, int planes,
+                                 float *__restrict__ EF)
 {
-    const int gid = blockIdx.x * blockDim.x + threadIdx.x, esz = m1 * m1;
+    const int gid = blockIdx.x * blockDim.x + threadIdx.x, esz = m1 * m1, H = G / 2, n = 2 * H * H;
     if (gid >= 2 * na * na * esz) return;
     const int k = gid % m1, nu = (gid / m1) % m1;
-    const double *E = E1 + (size_t)(gid / esz) * 7 * esz + k * m1 + nu;
-    float *o = EF + (size_t)gid * 8 * planes;
+    const double *E = E1 + ((size_t)(gid / esz) * (2 * G - 1) + G - 1) * esz + k * m1 + nu;
+    float *o = EF + (size_t)gid * n * planes;
     for (int s = 0; s < 2; ++s)
-        for (int i = 0; i < 2; ++i)
-            for (int j = 0; j < 2; ++j) {
-                const int o1 = i - j, o2 = i - 3 + j;
-                const double t1 = (o1 < 0 ? -o1 : o1) <= ntr ? E[(o1 + 3) * esz] : 0.0;
-                const double t2 = (o2 < 0 ? -o2 : o2) <= ntr ? E[(o2 + 3) * esz] : 0.0;
+        for (int i = 0; i < H; ++i)
+            for (int j = 0; j < H; ++j) {
+                const int o1 = i - j, o2 = i - (G - 1 - j);
+                const double t1 = (o1 < 0 ? -o1 : o1) <= ntr ? E[o1 * esz] : 0.0;
+                const double t2 = (o2 < 0 ? -o2 : o2) <= ntr ? E[o2 * esz] : 0.0;
                 const double m = 0.5 * (s == 0 ? t1 + t2 : t1 - t2);
-                const int at = s * 4 + i * 2 + j;
+                const int at = (s * H + i) * H + j;
                 o[at] = (float)m;
-                if (planes == 2) o[at + 8] = (float)(m - (double)(float)m);
+                if (planes == 2) o[at + n] = (float)(m - (double)(float)m);
             }
 }
 
-void launch_m2l_fold_table(const double *E1, int na, int mx, int ntr, int prec, float *EF, cudaStream_t st)
+void launch_m2l_fold_table(const double *E1, int na, int mx, int G, int ntr, int prec, float *EF, cudaStream_t st)
 {
     const int n = 2 * na * na * (mx + 1) * (mx + 1);
-    k_m2l_fold_table<<<(n + 127) / 128, 128, 0, st>>>(E1, na, mx + 1, ntr, prec == 1 ? 1 : 2, EF);
+    k_m2l_fold_table<<<(n + 127) / 128, 128, 0, st>>>(E1, na, mx + 1, G, ntr, prec == 1 ? 1 : 2, EF);
 }
 
-size_t m2l_fold_table_floats(int na, int mx, int prec)
+size_t m2l_fold_table_floats(int na, int mx, int G, int prec)
 {
-    return (size_t)2 * na * na * (mx + 1) * (mx + 1) * 8 * (prec == 1 ? 1 : 2);
+    return (size_t)na * na * (mx + 1) * (mx + 1) * G * G * (prec == 1 ? 1 : 2);
 }
 
 namespace {
@@ -530,54 +534,54 @@ int deal(const std::vector<Unit> &u, int upw, int warps, std::vector<int> &out)
 
 }  // namespace
 
-M2LFoldPlan m2l_fold_plan(int prec, int mx, const std::vector<int> &kinv, bool sliced)
+// slab: 8^3 levels (T1 by slices as well, keys of one bit that alternate with the budget)
+static M2LFoldPlan make_plan(int upw, int warps, int mx, const std::vector<int> &kinv, bool sliced, bool slab)
 {
-    const int m1 = mx + 1, nf = prec == 1 ? Form<float>::NF : Form<df64>::NF, upw = 2 * nf;
-    const int warps = (prec == 1 ? Form<float>::threads : Form<df64>::threads) / 32;
+    const int m1 = mx + 1, nk = (mx + 1) * (mx + 2) * (mx + 3) / 6;
     auto iv = [&](int a, int b, int c) { return kinv[((size_t)a * m1 + b) * m1 + c]; };
     auto tri = [](int n) { return n * (n + 1) / 2; };
     M2LFoldPlan P;
-    P.nk = (mx + 1) * (mx + 2) * (mx + 3) / 6;
-    P.ne = P.nk * (mx + 4) / 4;
-    // rows of U: (k2, k3), then k1; of T1: (nu1, k3), then k2, then C = nu1 + k3 + k2 .. m_x
-    P.urow.assign(P.nk, 0);
-    std::vector<int> ub((size_t)m1 * m1, 0), tb((size_t)m1 * m1, 0);
-    int r = 0, rt = 0;
-    for (int i = 0; i <= mx; ++i)
-        for (int j = 0; i + j <= mx; ++j) {
-            ub[i * m1 + j] = r;
-            for (int k1 = 0; k1 + i + j <= mx; ++k1) P.urow[iv(k1, i, j)] = r++;
-            tb[i * m1 + j] = rt;
-            rt += tri(mx - i - j + 1);
-        }
-    // slices of nu1: consecutive values whose rows of T2 fit the rows of the moments
+    M2LFoldDev &D = P.d;
+    // slices of nu1: consecutive values whose rows of T2 (as many as of T1) fit the rows of the moments
     std::vector<int> slice(m1, 0);
     auto rows2 = [&](int nu1) {
         int n = 0;
         for (int nu2 = 0; nu1 + nu2 <= mx; ++nu2) n += tri(mx - nu1 - nu2 + 1);
         return n;
     };
-    P.nslice = 1;
-    P.urows = P.nk;
+    D.nslice = 1;
+    D.urows = nk;
     for (int v = 0, fill = 0; v <= mx; ++v) {
-        if (sliced && fill && fill + rows2(v) > P.nk) {
-            P.nslice++;
+        if (sliced && fill && fill + rows2(v) > nk) {
+            D.nslice++;
             fill = 0;
         }
         fill += rows2(v);
-        slice[v] = P.nslice - 1;
-        P.urows = std::max(P.urows, fill);
+        slice[v] = D.nslice - 1;
+        D.urows = std::max(D.urows, fill);
     }
-    std::vector<Unit> u1, u3;
-    std::vector<std::vector<Unit>> u2(P.nslice);
+    // rows of U: (k2, k3), then k1; of T1: (nu1, k3), then k2, then C = nu1 + k3 + k2 .. m_x
+    P.urow.assign(nk, 0);
+    std::vector<int> ub((size_t)m1 * m1, 0), tb((size_t)m1 * m1, 0), f1(D.nslice, 0);
+    int r = 0;
+    for (int i = 0; i <= mx; ++i)
+        for (int j = 0; i + j <= mx; ++j) {
+            ub[i * m1 + j] = r;
+            for (int k1 = 0; k1 + i + j <= mx; ++k1) P.urow[iv(k1, i, j)] = r++;
+            int &rt = f1[slab ? slice[i] : 0];
+            tb[i * m1 + j] = rt;
+            rt += tri(mx - i - j + 1);
+        }
+    std::vector<Unit> u3;
+    std::vector<std::vector<Unit>> u1(slab ? D.nslice : 1), u2(D.nslice);
     for (int k2 = 0; k2 <= mx; ++k2)
         for (int k3 = 0; k2 + k3 <= mx; ++k3)
             for (int nu1 = 0; nu1 + k2 + k3 <= mx; ++nu1) {
                 const int n = mx - nu1 - k3;  // T1 rows of k2 start after n + 1, n, ... rows of smaller k2
-                u1.push_back({ub[k2 * m1 + k3], nu1, 0, k3 & 3, 0, 0, n - k2 + 1,
-                              tb[nu1 * m1 + k3] + k2 * (n + 1) - tri(k2 - 1), true});
+                u1[slab ? slice[nu1] : 0].push_back({ub[k2 * m1 + k3], nu1, 0, k3 & 3, 0, 0, n - k2 + 1,
+                                                     tb[nu1 * m1 + k3] + k2 * (n + 1) - tri(k2 - 1), true});
             }
-    std::vector<int> t2b((size_t)m1 * m1, 0), fill(P.nslice, 0);
+    std::vector<int> t2b((size_t)m1 * m1, 0), fill(D.nslice, 0);
     for (int nu1 = 0; nu1 <= mx; ++nu1)
         for (int nu2 = 0; nu1 + nu2 <= mx; ++nu2) {
             t2b[nu1 * m1 + nu2] = fill[slice[nu1]];
@@ -588,24 +592,43 @@ M2LFoldPlan m2l_fold_plan(int prec, int mx, const std::vector<int> &kinv, bool s
             for (int k3 = 0; nu1 + nu2 + k3 <= mx; ++k3)
                 for (int B = nu1 + nu2 + k3; B <= mx; ++B) {
                     const int C = B - nu2, s = nu1 + k3;  // k2 = 0 .. C - s; from k2 to k2 + 1: n - k2 rows
-                    u2[slice[nu1]].push_back({tb[nu1 * m1 + k3] + C - s, nu2, k3 & 3, nu1 & 3, mx - s, 0, C - s + 1,
-                                              t2b[nu1 * m1 + nu2] + tri(B - nu1 - nu2) + k3, true});
+                    u2[slice[nu1]].push_back({tb[nu1 * m1 + k3] + C - s, nu2, k3 & 3, slab ? B & 1 : nu1 & 3, mx - s, 0,
+                                              C - s + 1, t2b[nu1 * m1 + nu2] + tri(B - nu1 - nu2) + k3, true});
                 }
             for (int nu3 = 0; nu1 + nu2 + nu3 <= mx; ++nu3)
-                u3.push_back({t2b[nu1 * m1 + nu2] + tri(mx - nu3 - nu1 - nu2), nu3, nu1 & 3, 0, 0, slice[nu1],
-                              mx - nu1 - nu2 - nu3 + 1, iv(nu1, nu2, nu3), true});
+                u3.push_back({t2b[nu1 * m1 + nu2] + tri(mx - nu3 - nu1 - nu2), nu3, slab ? (mx - nu3) & 1 : nu1 & 3, 0, 0,
+                              slice[nu1], mx - nu1 - nu2 - nu3 + 1, iv(nu1, nu2, nu3), true});
         }
-    P.ntask[0] = deal(u1, upw, warps, P.units);
-    for (int s = 0; s < P.nslice; ++s) {
-        P.first2[s] = (int)P.units.size() / 2;
-        P.ntask2[s] = deal(u2[s], upw, warps, P.units);
+    for (int s = 0; s < (slab ? D.nslice : 1); ++s) {
+        D.first1[s] = (int)P.units.size() / 2;
+        D.ntask1[s] = deal(u1[s], upw, warps, P.units);
     }
-    P.first3 = (int)P.units.size() / 2;
-    P.ntask[1] = deal(u3, upw, warps, P.units);
-    P.q3 = (P.ntask[1] + warps - 1) / warps;
-    const int planes = prec == 1 ? 1 : 2;
-    P.smem = sizeof(float) * planes * ((size_t)(P.ne + P.urows) * 64 + (size_t)m1 * m1 * 8) + sizeof(int) * P.units.size() +
-             sizeof(int) * (64 + P.nk);
+    for (int s = 0; s < D.nslice; ++s) {
+        D.first2[s] = (int)P.units.size() / 2;
+        D.ntask2[s] = deal(u2[s], upw, warps, P.units);
+    }
+    D.first3 = (int)P.units.size() / 2;
+    D.ntask3 = deal(u3, upw, warps, P.units);
+    D.q3 = (D.ntask3 + warps - 1) / warps;
+    D.nunits = (int)P.units.size() / 2;
+    return P;
+}
+
+M2LFoldPlan m2l_fold_plan(int prec, int mx, const std::vector<int> &kinv, bool sliced)
+{
+    const int m1 = mx + 1, nf = prec == 1 ? Form<float>::NF : Form<df64>::NF, planes = prec == 1 ? 1 : 2;
+    const int warps = (prec == 1 ? Form<float>::threads : Form<df64>::threads) / 32;
+    M2LFoldPlan P = make_plan(2 * nf, warps, mx, kinv, sliced, false);
+    const size_t nk = P.urow.size(), ne = nk * (mx + 4) / 4;
+    P.d.smem = sizeof(float) * planes * ((ne + P.d.urows) * 64 + (size_t)m1 * m1 * 8) + sizeof(int) * P.units.size() +
+               sizeof(int) * (64 + nk);
+    return P;
+}
+
+M2LFoldPlan m2l_slab_plan(int mx, const std::vector<int> &kinv)
+{
+    M2LFoldPlan P = make_plan(2, kSlabThreads / 32, mx, kinv, true, true);
+    P.d.smem = sizeof(float) * ((size_t)2 * P.d.urows * 256 + (size_t)(mx + 1) * (mx + 1) * 32) + sizeof(int) * P.units.size();
     return P;
 }
 
@@ -629,17 +652,7 @@ int launch_m2l_folded(int prec, const DevLevel &L, const M2LFoldDev &P, const vo
     A.ne = g.ne;
     A.nint = L.nint;
     A.nbox = L.nbox;
-    A.urows = P.urows;
-    A.nslice = P.nslice;
-    A.nunits = P.nunits;
-    A.first3 = P.first3;
-    for (int i = 0; i < 2; ++i) A.ntask[i] = P.ntask[i];
-    for (int i = 0; i < kM2LMaxSlices; ++i) {
-        A.first2[i] = P.first2[i];
-        A.ntask2[i] = P.ntask2[i];
-    }
-    A.units = (const int2 *)P.units;
-    A.urow = P.urow;
+    A.p = P;
     A.cellbox = L.cellbox;
     A.EF = L.EF;
     A.pref = L.pref;
@@ -664,6 +677,344 @@ int launch_m2l_folded(int prec, const DevLevel &L, const M2LFoldDev &P, const vo
         else
             k_m2l_sum_chunks<df64><<<blocks, 256, 0, st>>>((const df64 *)ws, g.na, A.tpc, nlev, per_k, L.nint, (df64 *)lam);
     }
+    return 0;
+}
+
+// ------------------------------------------------------------------------------------------
+// 8^3 levels (FP32).  A direction folds into two sectors of four; the coefficients of (k, nu) are two
+// 4 x 4 blocks.  T1 and T2 of a whole level's cells do not fit shared memory, so a CTA takes the target
+// x-sector s1 (four X1 of a folded direction) and forms T1 and T2 a slice of nu1 at a time; rows have
+// 256 cells (4 X1 x 64).  The folded moments of the source intervals are laid out once in global memory
+// (every term is read by 5 b x 2 s1 CTAs of up to two intervals) and pass 1 reads them from L2.  The
+// two CTAs of (k, b) are a cluster: at the end they exchange their sector's locals through
+// distributed shared memory and each writes one half of the x range.  FP32 FMA and issue bound: a step
+// of a lane is 64 FMAs on 8 or 12 vector loads (the unfolded kernel had one FMA per load).
+
+// moments of (rhs, J, a) folded in x, y, z: F[((rhs, J, a)][row of U][X1][y >> 2][z][y & 3], positions of
+// the folded directions; 12 multi-indices per CTA
+constexpr int kFoldK = 12;
+__global__ void __launch_bounds__(256) k_m2l_fold_moments(const float *__restrict__ mu, const int *__restrict__ cellbox,
+                                                          const int *__restrict__ urow, int na, int nk, int nint, int nbox,
+                                                          int J0, int nJ, int r0, float *__restrict__ F)
+{
+    __shared__ float S[kFoldK][8][8][9];  // [k][x][y][z]
+    const int J = J0 + blockIdx.x / na, a = blockIdx.x % na, k0 = blockIdx.y * kFoldK, kn = min(kFoldK, nk - k0);
+    const float *mJ = mu + (((size_t)(r0 + blockIdx.z) * nint + J) * nbox * na + a) * nk + k0;
+    for (int i = threadIdx.x; i < 512 * kFoldK; i += 256) {
+        const int c = i / kFoldK, k = i % kFoldK, box = cellbox[c];
+        S[k][c >> 6][(c >> 3) & 7][c & 7] = box >= 0 && k < kn ? mJ[(size_t)box * na * nk + k] : 0.f;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int dir = 0; dir < 3; ++dir) {
+        for (int i = threadIdx.x; i < 64 * kFoldK; i += 256) {
+            const int k = i >> 6, u = (i >> 3) & 7, w = i & 7;
+            float v[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) v[j] = dir == 0 ? S[k][j][u][w] : dir == 1 ? S[k][u][j][w] : S[k][u][w][j];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const float p = v[j] + v[7 - j], m = v[j] - v[7 - j];
+                if (dir == 0) {
+                    S[k][j][u][w] = p;
+                    S[k][4 + j][u][w] = m;
+                } else if (dir == 1) {
+                    S[k][u][j][w] = p;
+                    S[k][u][4 + j][w] = m;
+                } else {
+                    S[k][u][w][j] = p;
+                    S[k][u][w][4 + j] = m;
+                }
+            }
+        }
+        __syncthreads();
+    }
+    float *o = F + (((size_t)blockIdx.z * nJ + (J - J0)) * na + a) * nk * 512;
+    for (int i = threadIdx.x; i < 512 * kn; i += 256) {
+        const int k = i >> 9, c = i & 511, x = c >> 6, y = ((c >> 5) & 1) * 4 + (c & 3), z = (c >> 2) & 7;
+        o[(size_t)urow[k0 + k] * 512 + c] = S[k][x][y][z];
+    }
+}
+
+// one (k, nu) step of a fibre of eight: both sectors, 4 x 4 each
+__device__ __forceinline__ void fibre8(float (&acc)[8], const float (&in)[8], const float (&e)[4], int s, int i, int o)
+{
+    float &a = acc[((s ^ o) << 2) + i];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) a = fmaf(e[j], in[s * 4 + j], a);
+}
+
+// chain of LEN steps of passes 2 and 3: two fibres per lane at p and p + fstep, halves 32 words apart
+template <int LEN>
+__device__ __forceinline__ void chain8(float (&acc)[2][8], const float *p, int stride, int dec, int fstep, const float *e)
+{
+#pragma unroll
+    for (int f = 0; f < 2; ++f)
+#pragma unroll
+        for (int r = 0; r < 8; ++r) acc[f][r] = 0.f;
+#pragma unroll
+    for (int j = 0; j < LEN; ++j) {
+        float in[2][8];
+#pragma unroll
+        for (int f = 0; f < 2; ++f) {
+            float h0[4], h1[4];
+            load4(p + f * fstep, h0);
+            load4(p + f * fstep + 32, h1);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                in[f][q] = h0[q];
+                in[f][4 + q] = h1[q];
+            }
+        }
+#pragma unroll
+        for (int s = 0; s < 2; ++s)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                float ev[4];
+                load4(e + j * 32 + s * 16 + i * 4, ev);
+                fibre8(acc[0], in[0], ev, s, i, j & 1);
+                fibre8(acc[1], in[1], ev, s, i, j & 1);
+            }
+        p += stride;
+        stride -= dec;
+    }
+}
+__device__ __forceinline__ void chain8_of(int len, float (&acc)[2][8], const float *p, int stride, int dec, int fstep,
+                                          const float *e)
+{
+    switch (len) {
+    case 1: chain8<1>(acc, p, stride, dec, fstep, e); break;
+    case 2: chain8<2>(acc, p, stride, dec, fstep, e); break;
+    case 3: chain8<3>(acc, p, stride, dec, fstep, e); break;
+    case 4: chain8<4>(acc, p, stride, dec, fstep, e); break;
+    case 5: chain8<5>(acc, p, stride, dec, fstep, e); break;
+    case 6: chain8<6>(acc, p, stride, dec, fstep, e); break;
+    default: chain8<7>(acc, p, stride, dec, fstep, e); break;
+    }
+}
+
+template <int Q3>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSlabThreads, 1)
+k_m2l_slab_folded(M2LFoldArgs A, const float *__restrict__ F, float *__restrict__ lam, int J0, int nJ, int r0)
+{
+    constexpr int W = kSlabThreads / 32, RW = 256;
+    extern __shared__ __align__(16) float sm[];
+    const int nk = A.nk, na = A.na, m1 = A.mx + 1;
+    float *T1 = sm, *T2 = T1 + A.p.urows * RW, *Es = T2 + A.p.urows * RW;
+    int2 *un = reinterpret_cast<int2 *>(Es + m1 * m1 * 32);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, sub = lane >> 4, cl = lane & 15;
+    const int s1 = blockIdx.x & 1, kb = blockIdx.x >> 1, b = kb % na, k = A.k_lo + kb / na, rhs = r0 + blockIdx.y;
+    const int nterm = k < 2 ? 0 : (k & 1 ? 2 * na : na);
+    for (int i = threadIdx.x; i < A.p.nunits; i += kSlabThreads) un[i] = reinterpret_cast<const int2 *>(A.p.units)[i];
+
+    float lamr[Q3][2][8];
+#pragma unroll
+    for (int q = 0; q < Q3; ++q)
+#pragma unroll
+        for (int f = 0; f < 2; ++f)
+#pragma unroll
+            for (int r = 0; r < 8; ++r) lamr[q][f][r] = 0.f;
+
+    for (int t = 0; t < nterm; ++t) {
+        const int a = t % na, D = (k & 1) ? 3 - t / na : 2, J = k - D;
+        __syncthreads();  // units in place; the previous term's passes are done with Es
+        const float4 *Eg = reinterpret_cast<const float4 *>(A.EF) + (size_t)(((D - 2) * na + a) * na + b) * m1 * m1 * 8;
+        for (int i = threadIdx.x; i < m1 * m1 * 8; i += kSlabThreads) reinterpret_cast<float4 *>(Es)[i] = Eg[i];
+        const float coef = reinterpret_cast<const float *>(A.pref)[((D - 2) * na + a) * na + b];
+        const float *Fj = F + (((size_t)blockIdx.y * nJ + (J - J0)) * na + a) * nk * 512 + cl * 4;
+        for (int sl = 0; sl < A.p.nslice; ++sl) {
+            __syncthreads();  // Es in place; pass 2 of the previous slice is done with T1
+            // pass 1: unit (k2, k3, nu1); lane = four cells (y of one half, z); inputs of the sector that
+            // feeds s1, outputs the four X1 of s1
+            for (int ts = warp; ts < A.p.ntask1[sl]; ts += W) {
+                const UnitBits u(un[A.p.first1[sl] + ts * 2 + sub]);
+                float acc[4][4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) acc[i][c] = 0.f;
+                const int s0 = s1 ^ (u.nu & 1);
+                const float *src = Fj + (size_t)u.row * 512;
+                const float *e = Es + u.nu * m1 * 32;
+                float *o = T1 + u.out * RW + cl * 4;
+#pragma unroll 2
+                for (int j = 0; j < u.len; ++j) {
+                    const int s = s0 ^ (j & 1);
+                    float4 in[4];
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) in[q] = __ldg(reinterpret_cast<const float4 *>(src + j * 512 + s * 256 + q * 64));
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        float ev[4];
+                        load4(e + j * 32 + s * 16 + i * 4, ev);
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) {
+                            acc[i][0] = fmaf(ev[q], in[q].x, acc[i][0]);
+                            acc[i][1] = fmaf(ev[q], in[q].y, acc[i][1]);
+                            acc[i][2] = fmaf(ev[q], in[q].z, acc[i][2]);
+                            acc[i][3] = fmaf(ev[q], in[q].w, acc[i][3]);
+                        }
+                        if (u.valid) store4(o + j * RW + i * 64, acc[i]);
+                    }
+                }
+            }
+            __syncthreads();
+            // pass 2: unit = row of T2; lane: fibres (X1, z) with X1 = cl / 8 and cl / 8 + 2
+            for (int ts = warp; ts < A.p.ntask2[sl]; ts += W) {
+                const UnitBits u(un[A.p.first2[sl] + ts * 2 + sub]);
+                const int z = cl & 7, i0 = cl >> 3;
+                float acc[2][8];
+                chain8_of(u.len, acc, T1 + u.row * RW + i0 * 64 + z * 4, u.step * RW, RW, 128, Es + u.nu * m1 * 32);
+                if (u.valid) {
+                    // to [X1][z / 4][X2 ^ swizzle][z % 4]: the lanes' eight groups of four words on all banks
+                    float *o = T2 + u.out * RW + i0 * 64 + (z >> 2) * 32 + (z & 3);
+                    const int sw = (z >> 2) | i0 << 1 | u.okey << 2, fl = (u.nu & 1) << 2;
+#pragma unroll
+                    for (int r = 0; r < 8; ++r) {
+                        const int x2 = ((r ^ fl) ^ sw) << 2;
+                        o[x2] = acc[0][r];
+                        o[x2 + 128] = acc[1][r];
+                    }
+                }
+            }
+            __syncthreads();
+            // pass 3: unit = multi-index of the locals; lane: fibres (X1, X2)
+#pragma unroll
+            for (int q = 0; q < Q3; ++q) {
+                const int ts = warp + q * W;
+                if (ts >= A.p.ntask3) break;
+                const UnitBits u(un[A.p.first3 + ts * 2 + sub]);
+                if (u.slice != sl) continue;
+                const int X2 = cl & 7, i0 = cl >> 3;
+                float acc[2][8];
+                // the halves of a fibre (z / 4) lie at different swizzles
+                const float *p = T2 + u.row * RW + i0 * 64;
+                const int c0 = (X2 ^ (i0 << 1 | u.key << 2)) << 2, c1 = (X2 ^ (1 | i0 << 1 | u.key << 2)) << 2;
+                const float *e = Es + u.nu * m1 * 32;
+#pragma unroll
+                for (int f = 0; f < 2; ++f)
+#pragma unroll
+                    for (int r = 0; r < 8; ++r) acc[f][r] = 0.f;
+#pragma unroll 1
+                for (int j = 0; j < u.len; j += 2) {
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        if (h == 1 && j + 1 >= u.len) break;
+                        float in[2][8];
+#pragma unroll
+                        for (int f = 0; f < 2; ++f) {
+                            float h0[4], h1[4];
+                            load4(p + f * 128 + c0, h0);
+                            load4(p + f * 128 + 32 + c1, h1);
+#pragma unroll
+                            for (int v = 0; v < 4; ++v) {
+                                in[f][v] = h0[v];
+                                in[f][4 + v] = h1[v];
+                            }
+                        }
+#pragma unroll
+                        for (int s = 0; s < 2; ++s)
+#pragma unroll
+                            for (int i = 0; i < 4; ++i) {
+                                float ev[4];
+                                load4(e + s * 16 + i * 4, ev);
+                                fibre8(acc[0], in[0], ev, s, i, h);
+                                fibre8(acc[1], in[1], ev, s, i, h);
+                            }
+                        p += RW;
+                        e += 32;
+                    }
+                }
+#pragma unroll
+                for (int f = 0; f < 2; ++f)
+#pragma unroll
+                    for (int r = 0; r < 8; ++r) lamr[q][f][r] = fmaf(coef, acc[f][r], lamr[q][f][r]);
+            }
+        }
+    }
+    // unfold in z per lane into rows [multi-index][X1][X2][X3] over T1 and T2 (nk <= urows)
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < Q3; ++q) {
+        const int ts = warp + q * W;
+        if (ts >= A.p.ntask3) break;
+        const UnitBits u(un[A.p.first3 + ts * 2 + sub]);
+        if (!u.valid) continue;
+        const int X2 = cl & 7, i0 = cl >> 3;
+        const bool odd = u.nu & 1;
+#pragma unroll
+        for (int f = 0; f < 2; ++f) {
+            float *p = T1 + u.out * RW + (i0 + 2 * f) * 64 + X2 * 8;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const float P = odd ? lamr[q][f][4 + i] : lamr[q][f][i], M = odd ? lamr[q][f][i] : lamr[q][f][4 + i];
+                p[i] = P + M;
+                p[7 - i] = P - M;
+            }
+        }
+    }
+    __syncthreads();
+    // unfold in y
+    for (int i = threadIdx.x; i < nk * 32; i += kSlabThreads) {
+        float *p = T1 + (i >> 5) * RW + ((i >> 3) & 3) * 64 + (i & 7);
+        float v[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) v[j] = p[j * 8];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            p[j * 8] = v[j] + v[4 + j];
+            p[(7 - j) * 8] = v[j] - v[4 + j];
+        }
+    }
+    // unfold in x with the other CTA's sector: sector 0 writes X1 = i (sum), sector 1 X1 = 7 - i (difference)
+    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+    uint32_t mine = (uint32_t)__cvta_generic_to_shared(T1), other;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(other) : "r"(mine), "r"(s1 ^ 1));
+    float *out = lam + (((size_t)rhs * A.nint + k) * A.nbox * na + b) * nk;
+    for (int i = threadIdx.x; i < nk * 256; i += kSlabThreads) {
+        const int iv = i % nk, c = i / nk, i1 = c >> 6;
+        const int box = A.cellbox[(s1 ? 7 - i1 : i1) * 64 + (c & 63)];
+        if (box < 0) continue;
+        float o;
+        asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(o) : "r"(other + 4u * (iv * RW + c)) : "memory");
+        const float m = T1[iv * RW + c];
+        out[(size_t)box * na * nk + iv] = s1 ? o - m : m + o;
+    }
+    // the other CTA has read this one's rows
+    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+
+int launch_m2l_slab_folded(const DevLevel &L, const M2LFoldDev &P, const float *mu, float *lam, int nrhs,
+                           const ApplyGeo &g, float *ws, size_t ws_elems, cudaStream_t st)
+{
+    // folded moments: per_int floats an interval and right-hand side; a target interval needs two
+    // intervals (k - 3, k - 2), n targets n + 1
+    const size_t per_int = (size_t)512 * g.na * g.nk, cap = ws_elems / per_int;
+    if (!P.units || cap < 2) return 1;
+    M2LFoldArgs A{};
+    A.na = g.na;
+    A.nk = g.nk;
+    A.mx = g.mx;
+    A.nint = L.nint;
+    A.nbox = L.nbox;
+    A.p = P;
+    A.cellbox = L.cellbox;
+    A.EF = L.EF;
+    A.pref = L.pref;
+    auto kf = P.q3 <= 4 ? k_m2l_slab_folded<4> : k_m2l_slab_folded<7>;
+    if (P.q3 > 7 || cudaFuncSetAttribute(kf, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)P.smem) != cudaSuccess) return -1;
+    const int rc = (int)std::min<size_t>(nrhs, std::max<size_t>(1, cap / std::min(L.nint, 16)));  // rhs at a time
+    const int nt = (int)std::min<size_t>(cap / rc - 1, L.nint);                                    // targets at a time
+    for (int r0 = 0; r0 < nrhs; r0 += rc)
+        for (int k0 = 0; k0 < L.nint; k0 += nt) {
+            const int nr = std::min(rc, nrhs - r0), k1 = std::min(L.nint, k0 + nt);
+            const int J0 = std::max(0, k0 - 3), nJ = std::max(0, k1 - 2 - J0);
+            if (nJ > 0)
+                k_m2l_fold_moments<<<dim3(nJ * g.na, (g.nk + kFoldK - 1) / kFoldK, nr), 256, 0, st>>>(
+                    mu, L.cellbox, P.urow, g.na, g.nk, L.nint, L.nbox, J0, nJ, r0, ws);
+            A.k_lo = k0;
+            kf<<<dim3((unsigned)((k1 - k0) * g.na * 2), nr), kSlabThreads, P.smem, st>>>(A, ws, lam, J0, nJ, r0);
+        }
     return 0;
 }
 

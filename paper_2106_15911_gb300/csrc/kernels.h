@@ -73,11 +73,11 @@ struct OtfArgs {
 void launch_nf_otf(bool mixed, bool kop, const OtfArgs &a, int nsm, cudaStream_t st);
 
 // ---- apply ------------------------------------------------------------------------------
-// unit tables of the folded M2L of 4^3 levels on the device (k_m2l.cu); units null: not built
+// unit tables of the folded M2L (k_m2l.cu) on the device; units null: not built
 constexpr int kM2LMaxSlices = 8;
 struct M2LFoldDev {
-    int urows, nslice, nunits, first3, q3;
-    int ntask[2], first2[kM2LMaxSlices], ntask2[kM2LMaxSlices];
+    int urows, nslice, nunits, first3, ntask3, q3;  // rows of U, units, pass 3: first unit, tasks (in all, per warp)
+    int first1[kM2LMaxSlices], ntask1[kM2LMaxSlices], first2[kM2LMaxSlices], ntask2[kM2LMaxSlices];
     const int *units, *urow;
     size_t smem;
 };
@@ -97,7 +97,7 @@ struct ApplyGeo {
     const int *box_tiles;  // [nbox_p + 1] first tile of each leaf box (tiles are box-major)
     int nsm;               // streaming multiprocessors of the device (grid sizing)
     int m2l_force;         // M2L engine asked for by the batch autotuner (PFMM_M2L_* code, 0: none)
-    const M2LFoldDev *fold;// [2] unit tables of the folded M2L: T2 whole, T2 sliced
+    const M2LFoldDev *fold;// [3] unit tables of the folded M2L: 4^3 with T2 whole, sliced; 8^3
 };
 
 // prec of the FMM launchers: 0 FP64, 1 FP32 (mixed mode), 2 double-FP32 (FP64 mode); every

@@ -125,7 +125,8 @@ struct DevLevel {
     int *ch_ptr, *ch_idx;
     void *E1;        // [2][na][na][2G-1][m1][m1]  (R)
     void *pref;      // [2][na][na]                (R)
-    float *EF;       // 4^3 levels: folded coefficients [2][na][na][m1][m1][8] (FP32, or high and low parts)
+    float *EF;       // 4^3 and 8^3 levels: folded coefficients [2][na][na][m1][m1][8 or 32] (FP32, or high
+                     // and low parts)
     void *qx;        // [2 bits][m1][m1] q^(x) from this level's boxes into their parents (R)
     int64_t mom_off; // element offset of this level's moments in the moment buffer (per rhs)
     int ntr;         // interaction-area radius (Eq. 03:Iarea)
