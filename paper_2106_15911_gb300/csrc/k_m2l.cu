@@ -42,7 +42,7 @@ namespace pfmm {
 
 namespace {
 
-constexpr int kSlabThreads = 256;  // 8^3 kernel
+constexpr int kSlabThreads = 512;  // 8^3 kernel
 
 template <typename R>
 struct Form;  // planes: FP32 words per value; NF: fibres per lane; threads and CTAs per SM
@@ -837,12 +837,19 @@ k_m2l_slab_folded(M2LFoldArgs A, const float *__restrict__ F, float *__restrict_
                 const float *src = Fj + (size_t)u.row * 512;
                 const float *e = Es + u.nu * m1 * 32;
                 float *o = T1 + u.out * RW + cl * 4;
-#pragma unroll 2
+                float4 nx[4];  // the next step's inputs, one L2 latency ahead
+#pragma unroll
+                for (int q = 0; q < 4; ++q) nx[q] = __ldg(reinterpret_cast<const float4 *>(src + s0 * 256 + q * 64));
+#pragma unroll 1
                 for (int j = 0; j < u.len; ++j) {
                     const int s = s0 ^ (j & 1);
                     float4 in[4];
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) in[q] = __ldg(reinterpret_cast<const float4 *>(src + j * 512 + s * 256 + q * 64));
+                    for (int q = 0; q < 4; ++q) in[q] = nx[q];
+                    if (j + 1 < u.len)
+#pragma unroll
+                        for (int q = 0; q < 4; ++q)
+                            nx[q] = __ldg(reinterpret_cast<const float4 *>(src + (j + 1) * 512 + (s ^ 1) * 256 + q * 64));
 #pragma unroll
                     for (int i = 0; i < 4; ++i) {
                         float ev[4];
@@ -1001,8 +1008,8 @@ int launch_m2l_slab_folded(const DevLevel &L, const M2LFoldDev &P, const float *
     A.cellbox = L.cellbox;
     A.EF = L.EF;
     A.pref = L.pref;
-    auto kf = P.q3 <= 4 ? k_m2l_slab_folded<4> : k_m2l_slab_folded<7>;
-    if (P.q3 > 7 || cudaFuncSetAttribute(kf, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)P.smem) != cudaSuccess) return -1;
+    auto kf = P.q3 <= 2 ? k_m2l_slab_folded<2> : k_m2l_slab_folded<3>;
+    if (P.q3 > 3 || cudaFuncSetAttribute(kf, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)P.smem) != cudaSuccess) return -1;
     const int rc = (int)std::min<size_t>(nrhs, std::max<size_t>(1, cap / std::min(L.nint, 16)));  // rhs at a time
     const int nt = (int)std::min<size_t>(cap / rc - 1, L.nint);                                    // targets at a time
     for (int r0 = 0; r0 < nrhs; r0 += rc)
