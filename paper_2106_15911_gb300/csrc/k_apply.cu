@@ -466,164 +466,201 @@ void launch_s2m(int prec, bool kop, const void *x, int ncolg, const void *Stab, 
 }
 
 // ------------------------------------------------------------------------------------------
-// M2M from level l+1 to level l (Eq. temp_m2m, st_m2m): thread per parent moment.
+// Temporal M2M from level l+1 to level l (Eq. temp_m2m): thread per (parent interval, box, kap), which
+// reads the 2 (m_t + 1) child moments once for all parent time nodes (bytes of the moments once;
+// one thread per node read them m_t + 1 times)
 template <typename R>
 __global__ void k_m2m(const R *__restrict__ mu_c, R *__restrict__ mu_p, const int *__restrict__ ch_ptr,
-                      const int *__restrict__ ch_idx, const int *__restrict__ oct_c, const R *__restrict__ q1,
-                      const R *__restrict__ qt, const int *__restrict__ kidx, const int *__restrict__ kinv, int st, int na,
-                      int nk, int mx, int nint_p, int nbox_p, int nbox_c, int nrhs)
+                      const int *__restrict__ ch_idx, const R *__restrict__ qt, int na, int nk, int nint_p, int nbox_p,
+                      int nbox_c, int nrhs)
 {
-    size_t gid = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    size_t total = (size_t)nrhs * nint_p * nbox_p * na * nk;
-    if (gid >= total) return;
-    int iv = gid % nk;
-    size_t r_ = gid / nk;
-    int ap = r_ % na;
-    r_ /= na;
-    int bp = r_ % nbox_p;
-    r_ /= nbox_p;
-    int kp = r_ % nint_p;
-    int rhs = (int)(r_ / nint_p);
-    const int m1 = mx + 1;
-    int n0 = kidx[3 * iv], n1 = kidx[3 * iv + 1], n2 = kidx[3 * iv + 2];
-    R acc = R(0);
-    for (int e = ch_ptr[bp]; e < ch_ptr[bp + 1]; ++e) {
-        int bc = ch_idx[e], oc = oct_c[bc];
-        const R *qa = q1 + (oc & 1) * m1 * m1, *qb = q1 + ((oc >> 1) & 1) * m1 * m1, *qc = q1 + ((oc >> 2) & 1) * m1 * m1;
-        for (int c = 0; c < 2; ++c) {
-            int kc = 2 * kp + c;
-            const R *mc = mu_c + (((size_t)rhs * 2 * nint_p + kc) * nbox_c + bc) * na * nk;
-            for (int ac = 0; ac < na; ++ac) {
-                R qtv = qt[(c * na + ac) * na + ap];
-                const R *m = mc + ac * nk;
-                if (!st) {
-                    acc += qtv * m[iv];
-                } else {
-                    R s = R(0);
-                    for (int k0 = 0; k0 <= n0; ++k0)
-                        for (int k1 = 0; k1 <= n1; ++k1)
-                            for (int k2 = 0; k2 <= n2; ++k2)
-                                s += qa[k0 * m1 + n0] * qb[k1 * m1 + n1] * qc[k2 * m1 + n2] *
-                                     m[kinv[(k0 * m1 + k1) * m1 + k2]];
-                    acc += qtv * s;
-                }
-            }
+    const size_t gid = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (gid >= (size_t)nrhs * nint_p * nbox_p * nk) return;
+    const int ik = (int)(gid % nk);
+    const size_t rb = gid / nk, rk = rb / nbox_p;  // (rhs, kp)
+    const int bp = (int)(rb - rk * nbox_p), bc = ch_idx[ch_ptr[bp]];
+    R v[kMaxNa];
+#pragma unroll
+    for (int a = 0; a < kMaxNa; ++a) v[a] = R(0);
+    for (int c = 0; c < 2; ++c) {
+        const R *m = mu_c + ((2 * rk + c) * nbox_c + bc) * na * nk + ik;
+        for (int ac = 0; ac < na; ++ac) {
+            const R x = m[(size_t)ac * nk];
+            const R *q = qt + (c * na + ac) * na;
+#pragma unroll
+            for (int a = 0; a < kMaxNa; ++a)
+                if (a < na) mac(v[a], q[a], x);
         }
     }
-    mu_p[gid] = acc;
+    R *o = mu_p + rb * na * nk + ik;
+#pragma unroll
+    for (int a = 0; a < kMaxNa; ++a)
+        if (a < na) o[(size_t)a * nk] = v[a];
 }
 
-// Space-time M2M (Eq. st_m2m) with one CTA per parent (interval kp, box bp, rhs): the temporal
-// contraction of each child's moments is staged in shared memory,
-//   tmp_c[ap][kap] = sum_{c, ac} q^(t)_c[ac][ap] mu[2 kp + c][child][ac][kap],
-// then mu_p[ap][nu] = sum_children sum_{kap <= nu} q^(x)_{kap,nu}(child) tmp_c[ap][kap].
+// Space-time M2M (Eq. st_m2m), one CTA per (parent interval kp, box bp, chunk of parent time nodes,
+// rhs), one direction at a time:
+//   B3[child][ap][kap]   = sum_{c, ac} q^(t)_c[ac][ap] mu[2 kp + c][child][ac][kap]
+//   B2[z, y][ap][n0,k1,k2] = sum_x sum_{k0 <= n0} q^(x)_{k0 n0}(x half) B3[z, y, x][ap][k0,k1,k2]
+// and likewise in y and z, the last into mu_p[ap][n0,n1,n2].  kap <= nu keeps every intermediate in the
+// graded index set.  Latency bound (a parent is some 10^4 multiply-adds): the direct sum over
+// kap <= nu per child took 48 us for the 256 parents of the 12288 x 256 tree, one node per CTA.
 template <typename R>
 __global__ void __launch_bounds__(256) k_m2m_st(const R *__restrict__ mu_c, R *__restrict__ mu_p,
                                                   const int *__restrict__ ch_ptr, const int *__restrict__ ch_idx,
                                                   const int *__restrict__ oct_c, const R *__restrict__ q1,
                                                   const R *__restrict__ qt, const int *__restrict__ kidx,
                                                   const int *__restrict__ kinv, int na, int nk, int mx, int nint_p,
-                                                  int nbox_p, int nbox_c)
+                                                  int nbox_p, int nbox_c, int apc)
 {
-    extern __shared__ unsigned char smem_raw[];
+    extern __shared__ __align__(16) unsigned char smem_raw[];
     const int m1 = mx + 1;
-    R *tmp = reinterpret_cast<R *>(smem_raw);  // [8][nk]: children's contracted moments for node ap
-    R *part = tmp + 8 * nk;                    // [8][nk]: partial sums over children, per thread group
-    R *qs = part + 8 * nk;                     // [2][m1][m1]
-    int *kin = reinterpret_cast<int *>(qs + 2 * m1 * m1);
-    // one CTA per (kp, bp, ap): the outputs of one parent time node
-    const int ap = blockIdx.x % na, pb = blockIdx.x / na;
-    const int kp = pb / nbox_p, bp = pb % nbox_p, rhs = blockIdx.y;
-    const int c0 = ch_ptr[bp], nch = ch_ptr[bp + 1] - c0;
+    R *B3 = reinterpret_cast<R *>(smem_raw);  // [8][apc][nk]
+    R *B2 = B3 + 8 * apc * nk;                // [4][apc][nk]
+    R *qs = B2 + 4 * apc * nk;                // [2][m1][m1]
+    int *kin = reinterpret_cast<int *>(qs + 2 * m1 * m1), *kid = kin + m1 * m1 * m1;
+    __shared__ int child[8];                  // box of the child in octant oc, or -1
+    const int kp = blockIdx.x / nbox_p, bp = blockIdx.x % nbox_p, rhs = blockIdx.y;
+    const int a0 = blockIdx.z * apc, an = min(apc, na - a0);
+    if (threadIdx.x < 8) child[threadIdx.x] = -1;
+    __syncthreads();
+    if (threadIdx.x < ch_ptr[bp + 1] - ch_ptr[bp]) {
+        const int bc = ch_idx[ch_ptr[bp] + threadIdx.x];
+        child[oct_c[bc]] = bc;
+    }
     for (int i = threadIdx.x; i < 2 * m1 * m1; i += blockDim.x) qs[i] = q1[i];
     for (int i = threadIdx.x; i < m1 * m1 * m1; i += blockDim.x) kin[i] = kinv[i];
-    for (int i = threadIdx.x; i < nch * nk; i += blockDim.x) {
-        int e = i / nk, ik = i % nk, bc = ch_idx[c0 + e];
-        R v = R(0);
-        for (int c = 0; c < 2; ++c) {
-            const R *m = mu_c + (((size_t)rhs * 2 * nint_p + 2 * kp + c) * nbox_c + bc) * na * nk + ik;
-            for (int ac = 0; ac < na; ++ac) v += qt[(c * na + ac) * na + ap] * m[(size_t)ac * nk];
-        }
-        tmp[i] = v;
-    }
+    for (int i = threadIdx.x; i < nk; i += blockDim.x) kid[i] = kidx[3 * i] | kidx[3 * i + 1] << 8 | kidx[3 * i + 2] << 16;
     __syncthreads();
-    // output iv: `per` threads take every per-th child; their partial sums are added in a fixed
-    // order afterwards (deterministic)
-    const int per = max(1, min((int)blockDim.x / nk, 8));
-    for (int o = threadIdx.x; o < nk * per; o += blockDim.x) {
-        const int iv = o % nk, g = o / nk;
-        const int n0 = kidx[3 * iv], n1 = kidx[3 * iv + 1], n2 = kidx[3 * iv + 2];
-        R acc = R(0);
-        for (int e = g; e < nch; e += per) {
-            const int oc = oct_c[ch_idx[c0 + e]];
-            const R *qa = qs + (oc & 1) * m1 * m1, *qb = qs + ((oc >> 1) & 1) * m1 * m1, *qc = qs + ((oc >> 2) & 1) * m1 * m1;
-            const R *tp = tmp + e * nk;
-            for (int k0 = 0; k0 <= n0; ++k0)
-                for (int k1 = 0; k1 <= n1; ++k1) {
-                    const R q01 = qa[k0 * m1 + n0] * qb[k1 * m1 + n1];
-                    for (int k2 = 0; k2 <= n2; ++k2) acc += q01 * qc[k2 * m1 + n2] * tp[kin[(k0 * m1 + k1) * m1 + k2]];
+    for (int i = threadIdx.x; i < 8 * nk; i += blockDim.x) {
+        const int oc = i / nk, ik = i - oc * nk, bc = child[oc];
+        R v[kMaxNa];
+#pragma unroll
+        for (int a = 0; a < kMaxNa; ++a) v[a] = R(0);
+        if (bc >= 0)
+            for (int c = 0; c < 2; ++c) {
+                const R *m = mu_c + ((((size_t)rhs * nint_p + kp) * 2 + c) * nbox_c + bc) * na * nk + ik;
+                for (int ac = 0; ac < na; ++ac) {
+                    const R x = m[(size_t)ac * nk];
+                    const R *q = qt + (c * na + ac) * na + a0;
+#pragma unroll
+                    for (int a = 0; a < kMaxNa; ++a)
+                        if (a < an) mac(v[a], q[a], x);
                 }
-        }
-        part[g * nk + iv] = acc;
+            }
+#pragma unroll
+        for (int a = 0; a < kMaxNa; ++a)
+            if (a < an) B3[(oc * apc + a) * nk + ik] = v[a];
     }
     __syncthreads();
-    R *out = mu_p + (((size_t)rhs * nint_p + kp) * nbox_p + bp) * na * nk + (size_t)ap * nk;
-    for (int iv = threadIdx.x; iv < nk; iv += blockDim.x) {
-        R sum = R(0);
-        for (int g = 0; g < per; ++g) sum += part[g * nk + iv];
-        out[iv] = sum;
+    R *out = mu_p + (((size_t)rhs * nint_p + kp) * nbox_p + bp) * na * nk + (size_t)a0 * nk;
+    // direction dir sums over the octants' bit 0 of what is left; its degree moves from k to n
+    R *src = B3, *dst = B2;
+    for (int dir = 0; dir < 3; ++dir) {
+        const int ng = 4 >> dir, st = dir == 0 ? m1 * m1 : dir == 1 ? m1 : 1;  // stride of the degree in kin
+        for (int i = threadIdx.x; i < ng * an * nk; i += blockDim.x) {
+            const int t = i % nk, ga = i / nk, g = ga / an, a = ga - g * an;
+            const int id = kid[t], d0 = id & 255, d1 = (id >> 8) & 255, d2 = id >> 16;
+            const int n = dir == 0 ? d0 : dir == 1 ? d1 : d2, base = (d0 * m1 + d1) * m1 + d2 - n * st;
+            R s = R(0);
+            for (int bit = 0; bit < 2; ++bit) {
+                const R *x = src + ((2 * g + bit) * apc + a) * nk, *q = qs + bit * m1 * m1 + n;
+                for (int k = 0; k <= n; ++k) mac(s, q[k * m1], x[kin[base + k * st]]);
+            }
+            if (dir < 2) dst[(g * apc + a) * nk + t] = s;
+            else out[(size_t)a * nk + t] = s;
+        }
+        __syncthreads();
+        R *sw = src;
+        src = dst;
+        dst = sw;
     }
 }
 
-// Space-time L2L (transpose of Eq. st_m2m) with one CTA per (parent (kp, bp), child box, rhs):
-//   tmp[bp_][kap] = sum_{nu >= kap, |nu| <= m_x} q^(x)_{kap,nu}(child) lam_p[bp_][nu],
-//   lam_c[2 kp + c][child][bc][kap] += sum_{bp_} q^(t)_c[bc][bp_] tmp[bp_][kap].
+// Space-time L2L (transpose of Eq. st_m2m), one CTA per (parent (kp, bp), chunk of parent time nodes,
+// rhs), one direction at a time: z, y and x expand the parent's locals to its octants,
+//   C1[z][bp][n0,n1,k2] = sum_{n2 >= k2, n0+n1+n2 <= m_x} q^(x)_{k2 n2}(z half) lam_p[bp][n0,n1,n2],  ...,
+// then lam_c[2 kp + c][child][bc][kap] += sum_bp q^(t)_c[bc][bp] C3[child][bp][kap].  All parent nodes are
+// in one CTA unless their arrays do not fit (then the chunks add one after the other's launch).  Few
+// parents: one CTA per octant (grid z = 8), 1.7 times the sums over eight times the CTAs.
 template <typename R>
 __global__ void __launch_bounds__(256) k_l2l_st(const R *__restrict__ lam_p, R *__restrict__ lam_c,
                                                   const int *__restrict__ ch_ptr, const int *__restrict__ ch_idx,
                                                   const int *__restrict__ oct_c, const R *__restrict__ q1,
                                                   const R *__restrict__ qt, const int *__restrict__ kidx,
                                                   const int *__restrict__ kinv, int na, int nk, int mx, int nint_p,
-                                                  int nbox_p, int nbox_c)
+                                                  int nbox_p, int nbox_c, int apc, int a0)
 {
-    extern __shared__ unsigned char smem_raw[];
-    const int m1 = mx + 1;
-    R *lp = reinterpret_cast<R *>(smem_raw);  // [na][nk]
-    R *tmp = lp + na * nk;                    // [na][nk]
-    R *qs = tmp + na * nk;                    // [2][m1][m1]
-    int *kin = reinterpret_cast<int *>(qs + 2 * m1 * m1);
-    const int e = blockIdx.x % 8, pb = blockIdx.x / 8;
-    const int kp = pb / nbox_p, bp = pb % nbox_p, rhs = blockIdx.y;
-    const int c0 = ch_ptr[bp], nch = ch_ptr[bp + 1] - c0;
-    if (e >= nch) return;  // the parent has fewer children
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int m1 = mx + 1, an = min(apc, na - a0);
+    R *C3 = reinterpret_cast<R *>(smem_raw);  // [8][apc][nk]; the parent's locals at first
+    R *C2 = C3 + 8 * apc * nk;                // [4][apc][nk]
+    R *qs = C2 + 4 * apc * nk;                // [2][m1][m1]
+    int *kin = reinterpret_cast<int *>(qs + 2 * m1 * m1), *kid = kin + m1 * m1 * m1;
+    __shared__ int child[8];
+    const int kp = blockIdx.x / nbox_p, bp = blockIdx.x % nbox_p, rhs = blockIdx.y;
+    if (threadIdx.x < 8) child[threadIdx.x] = -1;
+    __syncthreads();
+    if (threadIdx.x < ch_ptr[bp + 1] - ch_ptr[bp]) {
+        const int bc = ch_idx[ch_ptr[bp] + threadIdx.x];
+        child[oct_c[bc]] = bc;
+    }
     for (int i = threadIdx.x; i < 2 * m1 * m1; i += blockDim.x) qs[i] = q1[i];
     for (int i = threadIdx.x; i < m1 * m1 * m1; i += blockDim.x) kin[i] = kinv[i];
-    const R *src = lam_p + (((size_t)rhs * nint_p + kp) * nbox_p + bp) * na * nk;
-    for (int i = threadIdx.x; i < na * nk; i += blockDim.x) lp[i] = src[i];
-    {
-        const int bc = ch_idx[c0 + e], oc = oct_c[bc];
-        const R *qa = qs + (oc & 1) * m1 * m1, *qb = qs + ((oc >> 1) & 1) * m1 * m1, *qc = qs + ((oc >> 2) & 1) * m1 * m1;
-        __syncthreads();
-        for (int o = threadIdx.x; o < na * nk; o += blockDim.x) {
-            const int bpI = o / nk, ik = o % nk;
-            const int k0 = kidx[3 * ik], k1 = kidx[3 * ik + 1], k2 = kidx[3 * ik + 2];
-            const R *l = lp + bpI * nk;
+    for (int i = threadIdx.x; i < nk; i += blockDim.x) kid[i] = kidx[3 * i] | kidx[3 * i + 1] << 8 | kidx[3 * i + 2] << 16;
+    const R *lp = lam_p + (((size_t)rhs * nint_p + kp) * nbox_p + bp) * na * nk + (size_t)a0 * nk;
+    const int one = gridDim.z > 1 ? (int)blockIdx.z : -1;  // the only octant of this CTA, or all
+    // z: parent (in C2) -> [2] in C3; y: -> [4] in C2; x: -> [8] in C3
+    for (int i = threadIdx.x; i < an * nk; i += blockDim.x) C2[i] = lp[i];
+    __syncthreads();
+    R *src = C2, *dst = C3;
+    for (int dir = 2; dir >= 0; --dir) {
+        const int ng = one < 0 ? 8 >> dir : 1, st = dir == 0 ? m1 * m1 : dir == 1 ? m1 : 1;
+        for (int i = threadIdx.x; i < ng * an * nk; i += blockDim.x) {
+            const int t = i % nk, ga = i / nk, gi = ga / an, a = ga - gi * an, g = one < 0 ? gi : one >> dir;
+            const int id = kid[t], d0 = id & 255, d1 = (id >> 8) & 255, d2 = id >> 16;
+            const int k = dir == 0 ? d0 : dir == 1 ? d1 : d2, base = (d0 * m1 + d1) * m1 + d2 - k * st;
+            const int nmax = mx - (d0 + d1 + d2 - k);
+            // octant bits from the top: z, y, x
+            const R *x = src + ((g >> 1) * (dir == 2 ? an : apc) + a) * nk, *q = qs + (g & 1) * m1 * m1 + k * m1;
             R s = R(0);
-            for (int n0 = k0; n0 <= mx; ++n0)
-                for (int n1 = k1; n0 + n1 <= mx; ++n1) {
-                    const R q01 = qa[k0 * m1 + n0] * qb[k1 * m1 + n1];
-                    for (int n2 = k2; n0 + n1 + n2 <= mx; ++n2) s += q01 * qc[k2 * m1 + n2] * l[kin[(n0 * m1 + n1) * m1 + n2]];
-                }
-            tmp[o] = s;
+            for (int n = k; n <= nmax; ++n) mac(s, q[n], x[kin[base + n * st]]);
+            dst[(g * apc + a) * nk + t] = s;
         }
         __syncthreads();
-        for (int o = threadIdx.x; o < 2 * na * nk; o += blockDim.x) {
-            const int c = o / (na * nk), bcI = (o / nk) % na, ik = o % nk;
-            R v = R(0);
-            for (int bpI = 0; bpI < na; ++bpI) v += qt[(c * na + bcI) * na + bpI] * tmp[bpI * nk + ik];
-            lam_c[((((size_t)rhs * 2 * nint_p + 2 * kp + c) * nbox_c + bc) * na + bcI) * nk + ik] += v;
+        R *sw = src;
+        src = dst;
+        dst = sw;
+    }
+    // src = C3 holds the octants' locals at the parent's time nodes
+    for (int i = threadIdx.x; i < (one < 0 ? 8 : 1) * nk; i += blockDim.x) {
+        const int oi = i / nk, ik = i - oi * nk, oc = one < 0 ? oi : one, bc = child[oc];
+        if (bc < 0) continue;
+        R v[kMaxNa];
+#pragma unroll
+        for (int a = 0; a < kMaxNa; ++a) v[a] = a < an ? src[(oc * apc + a) * nk + ik] : R(0);
+        for (int c = 0; c < 2; ++c) {
+            R *o = lam_c + ((((size_t)rhs * nint_p + kp) * 2 + c) * nbox_c + bc) * na * nk + ik;
+            for (int b = 0; b < na; ++b) {
+                const R *q = qt + (c * na + b) * na + a0;
+                R s = R(0);
+#pragma unroll
+                for (int a = 0; a < kMaxNa; ++a)
+                    if (a < an) mac(s, q[a], v[a]);
+                o[(size_t)b * nk] += s;
+            }
         }
     }
+}
+
+// parent time nodes per CTA of the space-time M2M / L2L (at most `most`): as many as 12 arrays of
+// n_kappa leave room for (100 KB), and the shared memory they take
+static int st_nodes(const ApplyGeo &g, size_t es, int most, size_t *smem)
+{
+    const int m1 = g.mx + 1;
+    const int apc = std::max(1, std::min(most, (int)((size_t)100 * 1024 / (12 * (size_t)g.nk * es))));
+    *smem = es * ((size_t)12 * apc * g.nk + 2 * m1 * m1) + 4 * ((size_t)m1 * m1 * m1 + g.nk);
+    return apc;
 }
 
 void launch_m2m(int prec, const DevLevel &par, const DevLevel &ch, int l, const void *qt, void *mu, int nrhs,
@@ -631,26 +668,27 @@ void launch_m2m(int prec, const DevLevel &par, const DevLevel &ch, int l, const 
 {
     (void)l;
     (void)mu_stride;
-    const size_t total = (size_t)nrhs * par.nint * par.nbox * g.na * g.nk;
-    const unsigned blocks = (unsigned)((total + 127) / 128);
     const size_t es = prec == 1 ? 4 : 8;
     char *base = (char *)mu;
-    const int m1 = g.mx + 1;
     dispatch_prec(prec, [&](auto tag) {
         using R = decltype(tag);
         const R *mc = (const R *)(base + ch.mom_off * es * nrhs);
         R *mp = (R *)(base + par.mom_off * es * nrhs);
         if (ch.st) {
-            const size_t smem = es * ((size_t)16 * g.nk + 2 * m1 * m1) + 4 * (size_t)m1 * m1 * m1;
-            const dim3 grd(par.nint * par.nbox * g.na, nrhs);
+            size_t smem = 0;
+            // few parents: one time node per CTA (each forms its own temporal sums of the children)
+            const bool few = (int64_t)par.nint * par.nbox * nrhs < (g.nsm > 0 ? g.nsm : 152);
+            const int apc = st_nodes(g, es, few ? 1 : g.na, &smem);
+            const dim3 grd(par.nint * par.nbox, nrhs, (g.na + apc - 1) / apc);
             cudaFuncSetAttribute(k_m2m_st<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             k_m2m_st<R><<<grd, 256, smem, st>>>(mc, mp, par.ch_ptr, par.ch_idx, ch.octant, (const R *)ch.qx,
                                                 (const R *)qt, g.kidx, g.kinv, g.na, g.nk, g.mx, par.nint, par.nbox,
-                                                ch.nbox);
+                                                ch.nbox, apc);
             return;
         }
-        k_m2m<R><<<blocks, 128, 0, st>>>(mc, mp, par.ch_ptr, par.ch_idx, ch.octant, (const R *)ch.qx, (const R *)qt,
-                                         g.kidx, g.kinv, ch.st, g.na, g.nk, g.mx, par.nint, par.nbox, ch.nbox, nrhs);
+        const size_t total = (size_t)nrhs * par.nint * par.nbox * g.nk;
+        k_m2m<R><<<(unsigned)((total + 127) / 128), 128, 0, st>>>(mc, mp, par.ch_ptr, par.ch_idx, (const R *)qt, g.na, g.nk,
+                                                                  par.nint, par.nbox, ch.nbox, nrhs);
     });
 }
 
@@ -1358,45 +1396,33 @@ int launch_m2l(int prec, const DevLevel &L, int l, const void *mu, void *lam, in
 }
 
 // ------------------------------------------------------------------------------------------
-// L2L from level l-1 to level l (transposes of Eq. temp_m2m, st_m2m): thread per child local.
+// Temporal L2L from level l-1 to level l (transpose of Eq. temp_m2m): thread per (parent interval, box,
+// kap), which reads the parent's locals once for both child intervals.
 template <typename R>
-__global__ void k_l2l(const R *__restrict__ lam_p, R *__restrict__ lam_c, const int *__restrict__ parent,
-                      const int *__restrict__ oct_c, const R *__restrict__ q1, const R *__restrict__ qt,
-                      const int *__restrict__ kidx, const int *__restrict__ kinv, int st, int na, int nk, int mx,
-                      int nint_c, int nbox_c, int nbox_p, int nrhs)
+__global__ void k_l2l(const R *__restrict__ lam_p, R *__restrict__ lam_c, const int *__restrict__ ch_ptr,
+                      const int *__restrict__ ch_idx, const R *__restrict__ qt, int na, int nk, int nbox_c, int nint_p,
+                      int nbox_p, int nrhs)
 {
-    size_t gid = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    size_t total = (size_t)nrhs * nint_c * nbox_c * na * nk;
-    if (gid >= total) return;
-    int ik = gid % nk;
-    size_t r_ = gid / nk;
-    int bcI = r_ % na;
-    r_ /= na;
-    int bc = r_ % nbox_c;
-    r_ /= nbox_c;
-    int kc = r_ % nint_c;
-    int rhs = (int)(r_ / nint_c);
-    const int m1 = mx + 1;
-    int kp = kc >> 1, c = kc & 1, bp = parent[bc], oc = oct_c[bc];
-    const R *qa = q1 + (oc & 1) * m1 * m1, *qb = q1 + ((oc >> 1) & 1) * m1 * m1, *qc = q1 + ((oc >> 2) & 1) * m1 * m1;
-    int k0 = kidx[3 * ik], k1 = kidx[3 * ik + 1], k2 = kidx[3 * ik + 2];
-    const R *lp = lam_p + (((size_t)rhs * (nint_c >> 1) + kp) * nbox_p + bp) * na * nk;
-    R acc = R(0);
-    for (int bpI = 0; bpI < na; ++bpI) {
-        R qtv = qt[(c * na + bcI) * na + bpI];
-        const R *l = lp + bpI * nk;
-        if (!st) {
-            acc += qtv * l[ik];
-        } else {
-            R s = R(0);
-            for (int n0 = k0; n0 <= mx; ++n0)
-                for (int n1 = k1; n0 + n1 <= mx; ++n1)
-                    for (int n2 = k2; n0 + n1 + n2 <= mx; ++n2)
-                        s += qa[k0 * m1 + n0] * qb[k1 * m1 + n1] * qc[k2 * m1 + n2] * l[kinv[(n0 * m1 + n1) * m1 + n2]];
-            acc += qtv * s;
+    const size_t gid = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (gid >= (size_t)nrhs * nint_p * nbox_p * nk) return;
+    const int ik = (int)(gid % nk);
+    const size_t rb = gid / nk, rk = rb / nbox_p;  // (rhs, kp)
+    const int bp = (int)(rb - rk * nbox_p), bc = ch_idx[ch_ptr[bp]];
+    const R *l = lam_p + rb * na * nk + ik;
+    R v[kMaxNa];
+#pragma unroll
+    for (int a = 0; a < kMaxNa; ++a) v[a] = a < na ? l[(size_t)a * nk] : R(0);
+    for (int c = 0; c < 2; ++c) {
+        R *o = lam_c + ((2 * rk + c) * nbox_c + bc) * na * nk + ik;
+        for (int b = 0; b < na; ++b) {
+            const R *q = qt + (c * na + b) * na;
+            R s = o[(size_t)b * nk];
+#pragma unroll
+            for (int a = 0; a < kMaxNa; ++a)
+                if (a < na) mac(s, q[a], v[a]);
+            o[(size_t)b * nk] = s;
         }
     }
-    lam_c[gid] += acc;
 }
 
 void launch_l2l(int prec, const DevLevel &par, const DevLevel &ch, int l, const void *qt, void *lam, int nrhs,
@@ -1404,25 +1430,27 @@ void launch_l2l(int prec, const DevLevel &par, const DevLevel &ch, int l, const 
 {
     (void)l;
     (void)mu_stride;
-    const size_t total = (size_t)nrhs * ch.nint * ch.nbox * g.na * g.nk;
-    const unsigned blocks = (unsigned)((total + 127) / 128);
     const size_t es = prec == 1 ? 4 : 8;
     char *base = (char *)lam;
-    const int m1 = g.mx + 1;
     dispatch_prec(prec, [&](auto tag) {
         using R = decltype(tag);
         const R *lp = (const R *)(base + par.mom_off * es * nrhs);
         R *lc = (R *)(base + ch.mom_off * es * nrhs);
         if (ch.st) {
-            const size_t smem = es * ((size_t)2 * g.na * g.nk + 2 * m1 * m1) + 4 * (size_t)m1 * m1 * m1;
-            const dim3 grd(par.nint * par.nbox * 8, nrhs);  // one CTA per (parent, child slot); empty slots exit
-            k_l2l_st<R><<<grd, 256, smem, st>>>(lp, lc, par.ch_ptr, par.ch_idx, ch.octant, (const R *)ch.qx,
-                                                (const R *)qt, g.kidx, g.kinv, g.na, g.nk, g.mx, par.nint, par.nbox,
-                                                ch.nbox);
+            size_t smem = 0;
+            const bool few = (int64_t)par.nint * par.nbox * nrhs < 2 * (g.nsm > 0 ? g.nsm : 152);
+            const int apc = st_nodes(g, es, g.na, &smem);
+            const dim3 grd(par.nint * par.nbox, nrhs, few ? 8 : 1);
+            cudaFuncSetAttribute(k_l2l_st<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            for (int a0 = 0; a0 < g.na; a0 += apc)
+                k_l2l_st<R><<<grd, 256, smem, st>>>(lp, lc, par.ch_ptr, par.ch_idx, ch.octant, (const R *)ch.qx,
+                                                    (const R *)qt, g.kidx, g.kinv, g.na, g.nk, g.mx, par.nint, par.nbox,
+                                                    ch.nbox, apc, a0);
             return;
         }
-        k_l2l<R><<<blocks, 128, 0, st>>>(lp, lc, ch.parent, ch.octant, (const R *)ch.qx, (const R *)qt, g.kidx,
-                                         g.kinv, ch.st, g.na, g.nk, g.mx, ch.nint, ch.nbox, par.nbox, nrhs);
+        const size_t total = (size_t)nrhs * par.nint * par.nbox * g.nk;
+        k_l2l<R><<<(unsigned)((total + 127) / 128), 128, 0, st>>>(lp, lc, par.ch_ptr, par.ch_idx, (const R *)qt, g.na, g.nk,
+                                                                  ch.nbox, par.nint, par.nbox, nrhs);
     });
 }
 
