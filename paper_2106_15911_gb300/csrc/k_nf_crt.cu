@@ -99,15 +99,6 @@ __host__ __device__ constexpr uint32_t idesc_f16(int M, int N)
     return (1u << 4) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
-// The issuing warp runs its loop as a whole, so that addresses and descriptors stay in uniform
-// registers, and one lane issues (16 MMAs from a single lane's branch took 94 cycles each).
-__device__ __forceinline__ uint32_t elect_lane()
-{
-    uint32_t e;
-    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(e));
-    return e;
-}
-
 // A from tensor memory, B from shared memory at descriptor low word blo (K-major, 128-byte swizzle)
 __device__ __forceinline__ void mma_f16_ts(uint32_t issue, uint32_t dt, uint32_t a, uint32_t blo, uint32_t idesc,
                                            uint32_t acc)
@@ -119,15 +110,6 @@ __device__ __forceinline__ void mma_f16_ts(uint32_t issue, uint32_t dt, uint32_t
         "r"(a), "r"(blo), "r"(idesc), "r"(acc), "r"(issue), "n"(hi)
         : "memory");
 }
-__device__ __forceinline__ void mma_commit_if(uint32_t issue, uint64_t *b)
-{
-    asm volatile(
-        "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %1, 0;\n\t@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 "
-        "[%0];\n\t}" ::"r"(su32(b)),
-        "r"(issue)
-        : "memory");
-}
-
 __device__ __forceinline__ void tmem_st32_async(uint32_t taddr, const uint32_t (&r)[32])
 {
     asm volatile(
@@ -138,12 +120,6 @@ __device__ __forceinline__ void tmem_st32_async(uint32_t taddr, const uint32_t (
         "r"(r[19]), "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]), "r"(r[24]), "r"(r[25]), "r"(r[26]), "r"(r[27]),
         "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31])
         : "memory");
-}
-
-__device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&r)[32])
-{
-    tmem_st32_async(taddr, r);
-    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
 }
 
 struct CItem {
@@ -570,17 +546,19 @@ __global__ void k_crt_split_panel(const double *__restrict__ A, const PanelGPU *
     const int x = (int)(rd / nd), d = (int)(rd - (size_t)x * nd);
     if (x >= ntiles * BM) return;
     const int nkb = ncp / BK, row = x & (BM - 1), ch = ((c & 63) >> 4) ^ ((row >> 1) & 3);
-    double4 v = make_double4(0.0, 0.0, 0.0, 0.0);
+    double e[4] = {0.0, 0.0, 0.0, 0.0};
     if (x < nt) {
         const PanelGPU &Pn = panels[tri_leaf[x]];
         const double2 *a = reinterpret_cast<const double2 *>(
             A + (kop ? Pn.offK : Pn.offV) + ((size_t)d * Pn.rows_pad + (x - Pn.row0)) * ncp + c);
         const double2 p = a[0], q = a[1];
         const double sc = pow2(rowexp[x]);
-        v = make_double4(p.x * sc, p.y * sc, q.x * sc, q.y * sc);
+        e[0] = p.x * sc;
+        e[1] = p.y * sc;
+        e[2] = q.x * sc;
+        e[3] = q.y * sc;
     }
     uint32_t w[kCrtModuli];
-    const double e[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
         float r[kCrtModuli];

@@ -81,12 +81,15 @@ __host__ __device__ constexpr uint32_t idesc_f16(int M, int N)
            | ((uint32_t)(M >> 4) << 24);  // M / 16
 }
 
-__device__ __forceinline__ void mma_f16(uint32_t dt, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc)
+// operands at descriptor low words alo, blo (K-major, 128-byte swizzle)
+__device__ __forceinline__ void mma_f16(uint32_t issue, uint32_t dt, uint32_t alo, uint32_t blo, uint32_t idesc,
+                                        uint32_t acc)
 {
+    constexpr uint32_t hi = (1024 >> 4) | 1u << 14 | 2u << 29;  // 8-row groups 1024 bytes apart, version, swizzle
     asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\ttcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::
-            "r"(dt),
-        "l"(a), "l"(b), "r"(idesc), "r"(acc)
+        "{\n\t.reg .pred p, q;\n\t.reg .b64 a, b;\n\tmov.b64 a, {%1, %6};\n\tmov.b64 b, {%2, %6};\n\tsetp.ne.b32 p, %4, "
+        "0;\n\tsetp.ne.b32 q, %5, 0;\n\t@q tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, p;\n\t}\n" ::"r"(dt),
+        "r"(alo), "r"(blo), "r"(idesc), "r"(acc), "r"(issue), "n"(hi)
         : "memory");
 }
 
@@ -200,12 +203,14 @@ __global__ void __launch_bounds__(192, 1) k_nf_apply_tc(const __grid_constant__ 
         }
     } else if (warp == 1) {
         // ---------------- MMA issuer
-        if (lane == 0) {
-            int g = 0, n = 0;  // n: sub-chunks issued (the TMEM accumulators alternate per sub-chunk)
-            const uint32_t id256 = idesc_f16(BM, 256), id128 = idesc_f16(BM, 128);
-            for (int it = blockIdx.x; it < nitems && !s_abort; it += gridDim.x) {
-              Item I = decode_item(P, it);
-              for (int sc0 = I.st0; sc0 < I.st1 && !s_abort; sc0 += kSub, ++n) {
+        const uint32_t issue = elect_lane(), tm = __shfl_sync(0xffffffffu, tmem, 0);
+        const uint32_t base = __shfl_sync(0xffffffffu, (su32(smem) >> 4) & 0x3FFFu, 0) | 1u << 16;
+        constexpr uint32_t id256 = idesc_f16(BM, 256), id128 = idesc_f16(BM, 128);
+        constexpr uint32_t AT = A_TILE >> 4, BH = B_HALF >> 4;
+        int g = 0, n = 0;  // n: sub-chunks issued (the TMEM accumulators alternate per sub-chunk)
+        for (int it = blockIdx.x; it < nitems && !s_abort; it += gridDim.x) {
+            const Item I = decode_item(P, it);
+            for (int sc0 = I.st0; sc0 < I.st1 && !s_abort; sc0 += kSub, ++n) {
                 const int sc1 = min(I.st1, sc0 + kSub);
                 const int acc = n & 1;
                 if (!mbar_wait(&tempty[acc], ((n >> 1) & 1) ^ 1, deadline)) {
@@ -214,8 +219,7 @@ __global__ void __launch_bounds__(192, 1) k_nf_apply_tc(const __grid_constant__ 
                     break;
                 }
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const uint32_t dcol = tmem + acc * 256;
-                uint32_t first = 1;
+                const uint32_t dcol = tm + acc * 256;
                 for (int st = sc0; st < sc1; ++st, ++g) {
                     const int s = g % NSTAGE;
                     if (!mbar_wait(&full[s], (g / NSTAGE) & 1, deadline)) {
@@ -224,33 +228,28 @@ __global__ void __launch_bounds__(192, 1) k_nf_apply_tc(const __grid_constant__ 
                         break;
                     }
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                    const int d = st / P.nkb;
-                    const uint32_t a_hi = su32(smem + s * STAGE_BYTES), a_lo = a_hi + A_TILE;
-                    const uint32_t b_hi = a_hi + 2 * A_TILE, b_lo = b_hi + 2 * B_HALF;
+                    const uint32_t more = st > sc0 ? 1u : 0u;  // a sub-chunk's first MMA starts from zero
+                    const uint32_t ah = base + s * (STAGE_BYTES >> 4), al = ah + AT, bh = ah + 2 * AT, bl = bh + 2 * BH;
+                    if (st < 3 * P.nkb) {
 #pragma unroll
-                    for (int kk = 0; kk < BK / 16; ++kk) {  // K = 16 fp16 (32 bytes) per MMA
-                        const uint32_t ko = kk * 32;
-                        if (d < 3) {
-                            mma_f16(dcol, sw128_desc(a_hi + ko), sw128_desc(b_hi + ko), id256, first ? 0u : 1u);
-                            first = 0;
-                            mma_f16(dcol, sw128_desc(a_hi + ko), sw128_desc(b_lo + ko), id256, 1u);
-                            mma_f16(dcol, sw128_desc(a_lo + ko), sw128_desc(b_hi + ko), id256, 1u);
-                        } else {
-                            // d = 3 reaches back only from the second step of an interval
-                            mma_f16(dcol + 128, sw128_desc(a_hi + ko), sw128_desc(b_hi + B_HALF + ko), id128,
-                                     first ? 0u : 1u);
-                            mma_f16(dcol + 128, sw128_desc(a_hi + ko), sw128_desc(b_lo + B_HALF + ko), id128, 1u);
-                            mma_f16(dcol + 128, sw128_desc(a_lo + ko), sw128_desc(b_hi + B_HALF + ko), id128, 1u);
-                            if (first) {
-                                // the phase-0 half starts with no d < 3 stage in this chunk: clear it
-                                first = 0;
-                            }
+                        for (int kk = 0; kk < BK / 16; ++kk) {  // K = 16 fp16 (32 bytes) per MMA
+                            mma_f16(issue, dcol, ah + kk * 2, bh + kk * 2, id256, kk == 0 ? more : 1u);
+                            mma_f16(issue, dcol, ah + kk * 2, bl + kk * 2, id256, 1u);
+                            mma_f16(issue, dcol, al + kk * 2, bh + kk * 2, id256, 1u);
+                        }
+                    } else {
+                        // d = 3 reaches back only from the second step of an interval; the phase-0 half of
+                        // a sub-chunk without d < 3 stages is not read
+#pragma unroll
+                        for (int kk = 0; kk < BK / 16; ++kk) {
+                            mma_f16(issue, dcol + 128, ah + kk * 2, bh + BH + kk * 2, id128, kk == 0 ? more : 1u);
+                            mma_f16(issue, dcol + 128, ah + kk * 2, bl + BH + kk * 2, id128, 1u);
+                            mma_f16(issue, dcol + 128, al + kk * 2, bh + BH + kk * 2, id128, 1u);
                         }
                     }
-                    mma_commit(&empty[s]);  // frees the stage once these MMAs have read it
+                    mma_commit_if(issue, &empty[s]);  // frees the stage once these MMAs have read it
                 }
-                mma_commit(&tfull[acc]);
-              }
+                mma_commit_if(issue, &tfull[acc]);
             }
         }
     } else {

@@ -94,6 +94,25 @@ __device__ __forceinline__ void mma_commit(uint64_t *b)
                  : "memory");
 }
 
+// An MMA-issuing warp runs its loop as a whole, so that addresses and descriptors stay in uniform
+// registers, and one lane issues (16 MMAs from a single lane's branch took 94 cycles each).
+__device__ __forceinline__ uint32_t elect_lane()
+{
+    uint32_t e;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(e));
+    return e;
+}
+
+// the commit of an issuing warp (one lane: issue = elect_lane())
+__device__ __forceinline__ void mma_commit_if(uint32_t issue, uint64_t *b)
+{
+    asm volatile(
+        "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %1, 0;\n\t@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 "
+        "[%0];\n\t}" ::"r"(su32(b)),
+        "r"(issue)
+        : "memory");
+}
+
 // the loaded registers may be read only after a tcgen05.wait::ld
 __device__ __forceinline__ void tmem_ld32_async(uint32_t taddr, uint32_t (&r)[32])
 {
