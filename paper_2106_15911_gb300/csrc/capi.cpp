@@ -1017,10 +1017,8 @@ static int apply_impl(pfmm_handle *H, int op, const double *x, double *f, int nr
     if (far)
         for (int l = p - 1; l >= 2; --l) launch_m2m(H->fprec, H->dl[l], H->dl[l + 1], l, H->d_qt, mu, nrhs, g, 0, st);
     mark(4);
-    if (far)
-        for (int l = 2; l <= p; ++l)
-            if (launch_m2l(H->fprec, H->dl[l], l, mu, lam, nrhs, g, H->d_T1, H->d_T2, H->ws_m2l, st))
-                return fail(PFMM_ERR_OOM, "M2L workspace too small for one interval");
+    if (far && launch_m2l_levels(H->fprec, H->dl.data(), p, mu, lam, nrhs, g, H->d_T1, H->d_T2, H->ws_m2l, st))
+        return fail(PFMM_ERR_OOM, "M2L workspace too small for one interval");
     mark(5);
     if (far)
         for (int l = 3; l <= p; ++l) launch_l2l(H->fprec, H->dl[l - 1], H->dl[l], l, H->d_qt, lam, nrhs, g, 0, st);

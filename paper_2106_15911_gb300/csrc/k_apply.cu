@@ -307,11 +307,11 @@ __global__ void __launch_bounds__(256) k_s2m(const XT *__restrict__ xin, int nco
 }
 
 // Balanced S2M in two stages (leaf boxes hold from a few to several hundred triangles):
-// stage 1, CTA per (64-row tile of a leaf box, kTSB steps, rhs): the spatial moments of the
-// tile's triangles, P[tile][t][i] = sum_{x in tile} x[t][x] Sx[x][i], same register blocking as
+// stage 1, CTA per (64-row tile of a leaf box, kTSB steps, chunk of 32 CK moments, rhs): the spatial
+// moments of the tile's triangles, P[tile][t][i] = sum_{x in tile} x[t][x] Sx[x][i], same register blocking as
 // k_s2m; stage 2, thread per moment: mu[k][X][a][i] = sum_s St[s][a] sum_{tiles of X} P[tile][k ls + s][i]
 // in tile order (deterministic).
-template <typename R, typename XT, bool KOP>
+template <typename R, typename XT, bool KOP, int CK>
 __global__ void __launch_bounds__(256) k_s2m_tile(const XT *__restrict__ xin, int ncolg, const int *__restrict__ tri,
                                                     const R *__restrict__ Stab, R *__restrict__ part,
                                                     const int *__restrict__ tiles, int ntiles,
@@ -320,8 +320,8 @@ __global__ void __launch_bounds__(256) k_s2m_tile(const XT *__restrict__ xin, in
     extern __shared__ __align__(16) unsigned char s2m_raw[];
     R *sm = reinterpret_cast<R *>(s2m_raw);
     constexpr int XCH = KOP ? 16 : 32, PER = KOP ? 3 : 1, KC = XCH * PER;
-    const int tile = blockIdx.x, rhs = blockIdx.z / nchk, i0 = (blockIdx.z % nchk) * kS2MChunk;
-    const int nkc = min(nk - i0, kS2MChunk);
+    const int tile = blockIdx.x, rhs = blockIdx.z / nchk, i0 = (blockIdx.z % nchk) * (32 * CK);
+    const int nkc = min(nk - i0, 32 * CK);
     const int X = tiles[2 * tile];
     const int x0 = leaf_start[X] + tiles[2 * tile + 1], x1 = min(x0 + 64, leaf_start[X + 1]);
     const int t0 = blockIdx.y * kTSB, nts = min(kTSB, Et - t0);
@@ -329,11 +329,11 @@ __global__ void __launch_bounds__(256) k_s2m_tile(const XT *__restrict__ xin, in
     R *Ss = sm + KC * kTSP;  // [KC][nkc]
     const XT *xr = xin + (size_t)rhs * Et * ncolg;
     const int kg = threadIdx.x & 31, tg = threadIdx.x >> 5, ck = (nkc + 31) / 32;
-    R acc[4][kS2MCK];
+    R acc[4][CK];
 #pragma unroll
     for (int r = 0; r < 4; ++r)
 #pragma unroll
-        for (int c = 0; c < kS2MCK; ++c) acc[r][c] = R(0);
+        for (int c = 0; c < CK; ++c) acc[r][c] = R(0);
     for (int xb = x0; xb < x1; xb += XCH) {
         const int nx = min(XCH, x1 - xb);
         __syncthreads();
@@ -355,7 +355,7 @@ __global__ void __launch_bounds__(256) k_s2m_tile(const XT *__restrict__ xin, in
             R w[4];
             lds4(Ws + j * kTSP + tg * 4, w);
 #pragma unroll
-            for (int c = 0; c < kS2MCK; ++c) {
+            for (int c = 0; c < CK; ++c) {
                 const int i = kg + 32 * c;
                 if (c < ck && i < nkc) {
                     const R sv = Ss[j * nkc + i];
@@ -371,7 +371,7 @@ __global__ void __launch_bounds__(256) k_s2m_tile(const XT *__restrict__ xin, in
         const int ts = tg * 4 + r;
         if (ts >= nts) continue;
 #pragma unroll
-        for (int c = 0; c < kS2MCK; ++c) {
+        for (int c = 0; c < CK; ++c) {
             const int i = kg + 32 * c;
             if (c < ck && i < nkc) pt[(size_t)ts * nk + i0 + i] = acc[r][c];
         }
@@ -439,13 +439,20 @@ void launch_s2m(int prec, bool kop, const void *x, int ncolg, const void *Stab, 
         using R = decltype(tag);
         // input in the arithmetic type, or FP64 converted on load for the double-FP32 passes
         using XT = typename std::conditional<std::is_same<R, df64>::value, double, R>::type;
-        const int nchk = (g.nk + kS2MChunk - 1) / kS2MChunk, nkc = std::min(g.nk, kS2MChunk);
+        int nchk = (g.nk + kS2MChunk - 1) / kS2MChunk, nkc = std::min(g.nk, kS2MChunk);
         if (ws && g.tiles && (size_t)nrhs * g.ntiles * g.Et * g.nk <= ws_elems) {
             const int KC = kop ? 48 : 32;
+            // too few CTAs to give every SM one: 32 moments per CTA instead of 192
+            const bool few = (int64_t)g.ntiles * ((g.Et + kTSB - 1) / kTSB) * nrhs * nchk < (g.nsm > 0 ? g.nsm : 152);
+            if (few) {
+                nchk = (g.nk + 31) / 32;
+                nkc = std::min(g.nk, 32);
+            }
             const size_t smem = ((size_t)KC * kTSP + (size_t)KC * nkc) * es;
             const dim3 grd(g.ntiles, (g.Et + kTSB - 1) / kTSB, nrhs * nchk);
             const dim3 g2((unsigned)(nrhs * nint), (unsigned)((g.nbox_leaf * g.nk + 255) / 256));
-            auto kt = kop ? k_s2m_tile<R, XT, true> : k_s2m_tile<R, XT, false>;
+            auto kt = few ? (kop ? k_s2m_tile<R, XT, true, 1> : k_s2m_tile<R, XT, false, 1>)
+                          : (kop ? k_s2m_tile<R, XT, true, kS2MCK> : k_s2m_tile<R, XT, false, kS2MCK>);
             cudaFuncSetAttribute(kt, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             kt<<<grd, 256, smem, st>>>((const XT *)x, ncolg, g.tri, (const R *)Stab, (R *)ws, g.tiles, g.ntiles,
                                        g.leaf_start, g.nk, g.Et, nchk);
@@ -834,22 +841,36 @@ __global__ void k_m2l_s3(M2LArgs A, const R *__restrict__ E1, const R *__restric
     lam[((((size_t)rhs * A.nint + k) * A.nbox + box) * na + b) * A.nk + iv] = val;
 }
 
-// Fused M2L for grids of at most 4^3 cells: one CTA per (target interval k, time node b, rhs)
+// Fused M2L for the coarse levels (grids of at most 2^3 cells).  A tree of coarse levels only takes all of
+// them in one launch: they are independent and small, so one after the other each was a launch and a
+// term sum of mostly idle SMs (M2L of 192 x 16 in FP64 37 -> 22 us, 768 x 64 107 -> 81 us).  Below 4^3
+// levels that is lost in their time (2 % of the 1.54 ms of 12288 x 256 with one right-hand side, nothing
+// with several), and there every coarse level keeps its own launch.
+// One CTA per (level, target interval k, time node b, rhs)
 // keeps the source moments of all cells, the intermediates T1, T2 of all cells and the target
-// locals in shared memory.  The grid is padded to FG^3 cells (FG = 4, or 2 for levels with G <= 2,
-// whose CTAs then need an eighth of the shared memory and work).  A unit of passes 1 and 2 is a
+// locals in shared memory, with the grid padded to 2^3 cells.  A unit of passes 1 and 2 is a
 // multi-index triple, one budget chain (pass 1: the whole prefix chain; pass 2: one budget value)
-// and two grid coordinates, with the FG cells of the third in registers; an item of pass 3 is a
-// target multi-index and two target coordinates, whose FG locals stay in registers over all
-// terms.  Each step does FG^2 FMAs from FG loads of moments or intermediates and 7 coefficient
-// loads.  Units and items are short chains dealt round-robin over the CTA, so the passes end
+// and two grid coordinates, with the cells of the third in registers; an item of pass 3 is a
+// target multi-index and two target coordinates, whose locals stay in registers over all
+// terms.  Units and items are short chains dealt round-robin over the CTA, so the passes end
 // together.  Coefficients beyond the
 // interaction radius are zeroed once per (J, a), which applies Eq. 03:Iarea without branches.
-// Same arithmetic as the three-pass kernels (cells with G < 4 are padded with empty cells).
+// Same arithmetic as the three-pass kernels (empty cells where G = 1).
 // Split mode (levels with too few intervals to fill the GPU): one CTA per (k, b, source term)
 // with source term = (J, a) of the interaction list; each term's locals go to its own slice of a
 // workspace and k_m2l_sum_terms adds the slices in a fixed order (deterministic).
 constexpr int FGMax = 4;  // largest grid extent of the fused kernels
+constexpr int kMaxCoarse = 16;  // coarse levels of one launch
+
+struct M2LCoarse {
+    int n, nrhs;
+    int first[kMaxCoarse + 1];   // first CTA (grid x) of a level
+    int sfirst[kMaxCoarse + 1];  // first CTA of a level in k_m2l_sum_terms
+    int split[kMaxCoarse];
+    M2LArgs a[kMaxCoarse];
+    const void *E1[kMaxCoarse], *pref[kMaxCoarse];
+    size_t mom[kMaxCoarse], part[kMaxCoarse];  // element offsets of the level's moments and slices
+};
 
 // C(n, 4), 0 for n < 4: the budget rows of all triples with |t| <= n - 4 (slice offsets of T2)
 __host__ __device__ inline int binom4(int n) { return n < 4 ? 0 : n * (n - 1) * (n - 2) * (n - 3) / 24; }
@@ -860,12 +881,19 @@ constexpr int kM2LThreads = 384;
 // lose much of the last one; one-term CTAs are uniform and many
 constexpr int kM2LSplitCtasPerSm = 8;
 
-template <typename R, int FG, bool SL>
-__global__ void __launch_bounds__(kM2LThreads, FG == 2 ? 2 : (sizeof(R) == 4 && !SL ? 2 : 1)) k_m2l_fused(M2LArgs A, const R *__restrict__ mu,
-                                                                const R *__restrict__ E1, const R *__restrict__ pref,
-                                                                R *__restrict__ lam, int nrhs, int split,
-                                                                R *__restrict__ part)
+template <typename R, bool SL>
+__global__ void __launch_bounds__(kM2LThreads, 2) k_m2l_fused(const __grid_constant__ M2LCoarse M,
+                                                               const R *__restrict__ mu_all, R *__restrict__ lam_all,
+                                                               R *__restrict__ part_all)
 {
+    constexpr int FG = 2;
+    int lv = 0;
+    while (lv + 1 < M.n && (int)blockIdx.x >= M.first[lv + 1]) ++lv;
+    const M2LArgs &A = M.a[lv];
+    const int bx = blockIdx.x - M.first[lv], nrhs = M.nrhs, split = M.split[lv];
+    const R *mu = mu_all + M.mom[lv], *E1 = reinterpret_cast<const R *>(M.E1[lv]),
+            *pref = reinterpret_cast<const R *>(M.pref[lv]);
+    R *lam = lam_all + M.mom[lv], *part = part_all + M.part[lv];
     extern __shared__ unsigned char smem_raw[];
     constexpr int C3 = FG * FG * FG, CS = C3 + 1;  // cell rows are padded by one (bank spread)
     const int G = A.G, nk = A.nk, ne = A.ne, mx = A.mx, m1 = mx + 1, na = A.na, esz = m1 * m1;
@@ -882,8 +910,10 @@ __global__ void __launch_bounds__(kM2LThreads, FG == 2 ? 2 : (sizeof(R) == 4 && 
     int *cbx = eof + nk;                       // [C3] padded cell -> box or -1
     int *eofs = cbx + C3;                      // SL: offset of a triple's budget range within its nu1 slice
     int *rs = eofs + nk;                       // [ne] pass-2 rows: triple | budget index << 16, per slice
+    // units cover the G^3 cells; what they read beyond (with zero coefficients) stays finite
+    for (int i = threadIdx.x; i < (ne + nu_rows) * CS; i += blockDim.x) T1s[i] = R(0);
     const int nterm = split ? 2 * na : 1;  // source terms per CTA group: (J index, a)
-    const int kb = blockIdx.x / nterm, term = blockIdx.x % nterm;
+    const int kb = bx / nterm, term = bx % nterm;
     const int k = kb / na, b = kb % na, rhs = blockIdx.y;
     for (int i = threadIdx.x; i < nk; i += blockDim.x) {
         kid[i] = A.kidx[3 * i] | (A.kidx[3 * i + 1] << 8) | (A.kidx[3 * i + 2] << 16);
@@ -914,7 +944,7 @@ __global__ void __launch_bounds__(kM2LThreads, FG == 2 ? 2 : (sizeof(R) == 4 && 
     }
     // target locals of this thread's pass-3 items (nu, X1, X2), cells X3, kept in registers
     constexpr int Q3 = 2 * FG;  // items per thread: nk * FG <= 2 * blockDim.x
-    const int nit3 = nk * FG * FG;
+    const int nit3 = nk * G * G;
     R lamr[Q3][FG];
 #pragma unroll
     for (int q = 0; q < Q3; ++q)
@@ -925,7 +955,7 @@ __global__ void __launch_bounds__(kM2LThreads, FG == 2 ? 2 : (sizeof(R) == 4 && 
         if (k % 2 == 0) { js[0] = k - 2; nj = 1; }
         else { js[0] = k - 3; js[1] = k - 2; nj = 2; }
     }
-    const int no = 2 * G - 1, nitems = nk * FG;
+    const int no = 2 * G - 1, lg = G >> 1, G2 = G * G;  // G = 1 or 2: u mod G = u & lg, u / G = u >> lg
     const int j_lo = split ? term / na : 0, j_hi = split ? j_lo + 1 : nj;
     const int a_lo = split ? term % na : 0, a_hi = split ? a_lo + 1 : na;
     if (split && j_lo >= nj) return;  // this (k) has fewer source intervals
@@ -949,8 +979,8 @@ __global__ void __launch_bounds__(kM2LThreads, FG == 2 ? 2 : (sizeof(R) == 4 && 
             // pass 1 (direction x): unit = (triple (nu1, k2, k3), Y2, Y3); registers: cells X1.  The
             // budget loop over B is a prefix sum (T1 holds the cumulative budget), so a unit is a
             // sequential chain of 1 .. m_x + 1 steps; units are spread over all threads
-            for (int u = threadIdx.x; u < nitems * FG; u += blockDim.x) {
-                const int z = u % FG, Y2 = (u / FG) % FG, t = u / (FG * FG), tk = kid[t];
+            for (int u = threadIdx.x; u < nk * G2; u += blockDim.x) {
+                const int z = u & lg, Y2 = (u >> lg) & lg, t = u >> 2 * lg, tk = kid[t];
                 const int nu1 = tk & 255, k2 = (tk >> 8) & 255, k3 = tk >> 16, s0 = nu1 + k2 + k3;
                 R acc[FG];
 #pragma unroll
@@ -965,7 +995,7 @@ __global__ void __launch_bounds__(kM2LThreads, FG == 2 ? 2 : (sizeof(R) == 4 && 
                     for (int Y1 = 0; Y1 < FG; ++Y1) {
                         const R mv = mrow[Y1 * FG * FG];
 #pragma unroll
-                        for (int X1 = 0; X1 < FG; ++X1) acc[X1] += e[X1 - Y1 + 3] * mv;
+                        for (int X1 = 0; X1 < FG; ++X1) mac(acc[X1], e[X1 - Y1 + 3], mv);
                     }
                     R *out = T1s + (eof[t] + k1) * CS + Y2 * FG + z;
 #pragma unroll
@@ -980,8 +1010,8 @@ __global__ void __launch_bounds__(kM2LThreads, FG == 2 ? 2 : (sizeof(R) == 4 && 
             // steps) and spreads a slice's rows over all threads
             const int r0 = SL ? ne - binom4(mx - sl + 4) : 0;
             const int r1 = SL ? ne - binom4(mx - sl + 3) : ne;
-            for (int u = r0 * FG * FG + threadIdx.x; u < r1 * FG * FG; u += blockDim.x) {
-                const int z = u % FG, X1 = (u / FG) % FG, rw = rs[u / (FG * FG)];
+            for (int u = r0 * G2 + threadIdx.x; u < r1 * G2; u += blockDim.x) {
+                const int z = u & lg, X1 = (u >> lg) & lg, rw = rs[u >> 2 * lg];
                 const int t = rw & 0xffff, j = rw >> 16, tk = kid[t];
                 const int nu1 = tk & 255, nu2 = (tk >> 8) & 255, k3 = tk >> 16;
                 R acc[FG];
@@ -997,10 +1027,10 @@ __global__ void __launch_bounds__(kM2LThreads, FG == 2 ? 2 : (sizeof(R) == 4 && 
                     for (int Y2 = 0; Y2 < FG; ++Y2) {
                         const R tv = trow[Y2 * FG];
 #pragma unroll
-                        for (int X2 = 0; X2 < FG; ++X2) acc[X2] += e[X2 - Y2 + 3] * tv;
+                        for (int X2 = 0; X2 < FG; ++X2) mac(acc[X2], e[X2 - Y2 + 3], tv);
                     }
                 }
-                R *out = U + (u / (FG * FG) - r0) * CS + X1 * FG * FG + z;
+                R *out = U + ((u >> 2 * lg) - r0) * CS + X1 * FG * FG + z;
 #pragma unroll
                 for (int X2 = 0; X2 < FG; ++X2) out[X2 * FG] = acc[X2];
             }
@@ -1010,7 +1040,7 @@ __global__ void __launch_bounds__(kM2LThreads, FG == 2 ? 2 : (sizeof(R) == 4 && 
             for (int q = 0; q < Q3; ++q) {
                 const int it = threadIdx.x + q * blockDim.x;
                 if (it >= nit3) break;
-                const int iv = it / (FG * FG), X1 = (it / FG) % FG, X2 = it % FG, tk = kid[iv];
+                const int iv = it >> 2 * lg, X1 = (it >> lg) & lg, X2 = it & lg, tk = kid[iv];
                 const int nu1 = tk & 255, nu2 = (tk >> 8) & 255, nu3 = tk >> 16, smax = mx - nu1 - nu2 - nu3;
                 if (SL && nu1 != sl) continue;
                 R acc[FG];
@@ -1029,10 +1059,10 @@ __global__ void __launch_bounds__(kM2LThreads, FG == 2 ? 2 : (sizeof(R) == 4 && 
 #pragma unroll
                     for (int X3 = 0; X3 < FG; ++X3)
 #pragma unroll
-                        for (int Y3 = 0; Y3 < FG; ++Y3) acc[X3] += e[X3 - Y3 + 3] * tv[Y3];
+                        for (int Y3 = 0; Y3 < FG; ++Y3) mac(acc[X3], e[X3 - Y3 + 3], tv[Y3]);
                 }
 #pragma unroll
-                for (int X3 = 0; X3 < FG; ++X3) lamr[q][X3] += coef * acc[X3];
+                for (int X3 = 0; X3 < FG; ++X3) mac(lamr[q][X3], coef, acc[X3]);
             }
             }  // slices
         }
@@ -1045,8 +1075,7 @@ __global__ void __launch_bounds__(kM2LThreads, FG == 2 ? 2 : (sizeof(R) == 4 && 
     for (int q = 0; q < Q3; ++q) {
         const int it = threadIdx.x + q * blockDim.x;
         if (it >= nit3) break;
-        const int iv = it / (FG * FG), X1 = (it / FG) % FG, X2 = it % FG;
-        if (X1 >= G || X2 >= G) continue;
+        const int iv = it >> 2 * lg, X1 = (it >> lg) & lg, X2 = it & lg;
 #pragma unroll
         for (int X3 = 0; X3 < FG; ++X3) {
             if (X3 >= G) continue;
@@ -1056,19 +1085,23 @@ __global__ void __launch_bounds__(kM2LThreads, FG == 2 ? 2 : (sizeof(R) == 4 && 
     }
 }
 
-// lam = sum of the term slices in term order; interval k has nj(k) * na terms (nj = 0 for k < 2,
-// 1 for even k, 2 for odd k): the slices of the other terms are never written and are not read
+// lam = sum of the term slices in term order, of the split levels; interval k has nj(k) * na terms (nj = 0
+// for k < 2, 1 for even k, 2 for odd k): the slices of the other terms are never written and are not read
 template <typename R>
-__global__ void k_m2l_sum_terms(const R *__restrict__ part, int na, size_t n, size_t per_k, int nint,
-                                R *__restrict__ lam)
+__global__ void k_m2l_sum_terms(const __grid_constant__ M2LCoarse M, const R *__restrict__ part_all, R *__restrict__ lam_all)
 {
-    const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    int lv = 0;
+    while (lv + 1 < M.n && (int)blockIdx.x >= M.sfirst[lv + 1]) ++lv;
+    const M2LArgs &A = M.a[lv];
+    const size_t per_k = (size_t)A.nbox * A.na * A.nk, n = (size_t)M.nrhs * A.nint * per_k;
+    const size_t i = (size_t)(blockIdx.x - M.sfirst[lv]) * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    const int k = (int)((i / per_k) % nint);
-    const int nterm = k < 2 ? 0 : (k % 2 == 0 ? na : 2 * na);
+    const R *part = part_all + M.part[lv];
+    const int k = (int)((i / per_k) % A.nint);
+    const int nterm = k < 2 ? 0 : (k % 2 == 0 ? A.na : 2 * A.na);
     R s = R(0);
     for (int t = 0; t < nterm; ++t) s += part[(size_t)t * n + i];
-    lam[i] = s;
+    lam_all[M.mom[lv] + i] = s;
 }
 
 // M2L for grids of 5^3 .. 8^3 cells (FP32), one CTA per (target interval k, time node b, target
@@ -1311,45 +1344,81 @@ int m2l_engine_for(int prec, int G, int nk, int ne, int mx, int force)
     }
 }
 
-// Runs the three passes over chunks of target intervals so that the intermediates fit the
-// workspace (ws_elems elements of R for each of T1 and T2).
-int launch_m2l(int prec, const DevLevel &L, int l, const void *mu, void *lam, int nrhs, const ApplyGeo &g,
-               void *T1, void *T2, size_t ws_elems, cudaStream_t st)
+// coarse levels (fused kernel on at most 2^3 cells), per_launch of them in one launch and one term sum
+template <typename R>
+static void launch_m2l_coarse(int prec, const DevLevel *dl, const std::vector<int> &levels, bool sl, const R *mu, R *lam,
+                              int nrhs, const ApplyGeo &g, R *ws, size_t ws_elems, int per_launch, cudaStream_t st)
 {
-    (void)l;
+    const int na = g.na, nterm = 2 * na;
+    const int64_t split_ctas = (int64_t)kM2LSplitCtasPerSm * (g.nsm > 0 ? g.nsm : 152);
+    const size_t fsm = m2l_fused_smem(2, g.nk, g.ne, g.mx, prec == 1 ? 4 : 8, sl);
+    for (size_t at = 0; at < levels.size(); at += per_launch) {
+        M2LCoarse M{};
+        M.nrhs = nrhs;
+        size_t used = 0;
+        for (size_t i = at; i < levels.size() && M.n < per_launch; ++i) {
+            const DevLevel &L = dl[levels[i]];
+            const int n = M.n++;
+            M.a[n] = M2LArgs{L.G, L.ntr, na, g.nk, g.mx, g.ne, L.nint, L.nbox, L.cellbox, L.boxcell, L.pk, L.pJ, 0,
+                             g.kidx, g.kinv, g.eoff};
+            M.E1[n] = L.E1;
+            M.pref[n] = L.pref;
+            M.mom[n] = (size_t)L.mom_off * nrhs;
+            // few (interval, node) CTAs: one CTA per source term as well, when the terms' partial
+            // locals fit what is left of the workspace
+            const size_t nlev = (size_t)nrhs * L.nint * L.nbox * na * g.nk;
+            M.split[n] = (int64_t)L.nint * na * nrhs < split_ctas && used + nterm * nlev <= ws_elems ? 1 : 0;
+            M.part[n] = used;
+            used += M.split[n] ? nterm * nlev : 0;
+            M.first[n + 1] = M.first[n] + L.nint * na * (M.split[n] ? nterm : 1);
+            M.sfirst[n + 1] = M.sfirst[n] + (M.split[n] ? (int)((nlev + 255) / 256) : 0);
+        }
+        auto kf = sl ? k_m2l_fused<R, true> : k_m2l_fused<R, false>;
+        cudaFuncSetAttribute(kf, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fsm);
+        kf<<<dim3(M.first[M.n], nrhs), kM2LThreads, fsm, st>>>(M, mu, lam, ws);
+        if (M.sfirst[M.n] > 0) k_m2l_sum_terms<R><<<M.sfirst[M.n], 256, 0, st>>>(M, ws, lam);
+    }
+}
+
+static int launch_m2l(int prec, const DevLevel &L, const void *mu, void *lam, int nrhs, const ApplyGeo &g, void *T1, void *T2,
+                      size_t ws_elems, cudaStream_t st);
+
+int launch_m2l_levels(int prec, const DevLevel *dl, int p, const void *mu, void *lam, int nrhs, const ApplyGeo &g, void *T1,
+                      void *T2, size_t ws_elems, cudaStream_t st)
+{
+    std::vector<int> coarse[2];  // T2 whole, sliced
+    for (int l = 2; l <= p; ++l) {
+        const int e = m2l_engine_for(prec, dl[l].G, g.nk, g.ne, g.mx, g.m2l_force);
+        if ((e == kM2LFused || e == kM2LFusedSliced) && dl[l].G <= 2) coarse[e == kM2LFusedSliced].push_back(l);
+        else if (launch_m2l(prec, dl[l], mu, lam, nrhs, g, T1, T2, ws_elems, st)) return -1;
+    }
+    const int per = p >= 2 && dl[p].G <= 2 ? kMaxCoarse : 1;
+    for (int sl = 0; sl < 2; ++sl) {
+        if (coarse[sl].empty()) continue;
+        if (prec == 1)
+            launch_m2l_coarse<float>(prec, dl, coarse[sl], sl, (const float *)mu, (float *)lam, nrhs, g, (float *)T1, ws_elems, per,
+                                     st);
+        else if (prec == 2)
+            launch_m2l_coarse<df64>(prec, dl, coarse[sl], sl, (const df64 *)mu, (df64 *)lam, nrhs, g, (df64 *)T1, ws_elems, per, st);
+    }
+    return 0;
+}
+
+// One level that is not coarse.  The three-pass engine runs over chunks of target intervals so that the
+// intermediates fit the workspace (ws_elems elements of R for each of T1 and T2).
+static int launch_m2l(int prec, const DevLevel &L, const void *mu, void *lam, int nrhs, const ApplyGeo &g, void *T1, void *T2,
+                      size_t ws_elems, cudaStream_t st)
+{
     const size_t es = prec == 1 ? 4 : 8;
     const int G3 = L.G * L.G * L.G, na = g.na;
     const int engine = m2l_engine_for(prec, L.G, g.nk, g.ne, g.mx, g.m2l_force);
     const char *mb = (const char *)mu + L.mom_off * es * nrhs;
     char *lb = (char *)lam + L.mom_off * es * nrhs;
+    if (engine == kM2LFused || engine == kM2LFusedSliced)
+        return launch_m2l_folded(prec, L, g.fold[engine == kM2LFusedSliced ? 1 : 0], mb, lb, nrhs, g, T1, ws_elems, st);
     int rc = 0;
     dispatch_prec(prec, [&](auto tag) {
         using R = decltype(tag);
-        if (engine == kM2LFused || engine == kM2LFusedSliced) {
-            const bool sl = engine == kM2LFusedSliced;
-            if (m2l_fused_fg(L.G) == FGMax) {
-                rc = launch_m2l_folded(prec, L, g.fold[sl ? 1 : 0], mb, lb, nrhs, g, T1, ws_elems, st);
-                return;
-            }
-            const size_t fsm = m2l_fused_smem(L.G, g.nk, g.ne, g.mx, es, sl);
-            M2LArgs A{L.G, L.ntr, na, g.nk, g.mx, g.ne, L.nint, L.nbox, L.cellbox, L.boxcell, L.pk, L.pJ, 0,
-                      g.kidx, g.kinv, g.eoff};
-            // few (interval, node) CTAs: one CTA per source term as well, when the terms' partial
-            // locals fit the workspace
-            const size_t per_k = (size_t)L.nbox * na * g.nk, nlev = (size_t)nrhs * L.nint * per_k;
-            const int nterm = 2 * na;
-            const int64_t split_ctas = (int64_t)kM2LSplitCtasPerSm * (g.nsm > 0 ? g.nsm : 152);
-            const int split = ((int64_t)L.nint * na * nrhs < split_ctas && (size_t)nterm * nlev <= ws_elems) ? 1 : 0;
-            const dim3 grd(L.nint * na * (split ? nterm : 1), nrhs);
-            auto kf = sl ? k_m2l_fused<R, 2, true> : k_m2l_fused<R, 2, false>;
-            cudaFuncSetAttribute(kf, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fsm);
-            kf<<<grd, kM2LThreads, fsm, st>>>(A, (const R *)mb, (const R *)L.E1, (const R *)L.pref, (R *)lb, nrhs,
-                                              split, (R *)T1);
-            if (split)
-                k_m2l_sum_terms<R><<<(unsigned)((nlev + 255) / 256), 256, 0, st>>>((const R *)T1, na, nlev, per_k,
-                                                                                  L.nint, (R *)lb);
-            return;
-        }
         if (engine == kM2LSlab) {
             if constexpr (std::is_same<R, float>::value) {
                 rc = launch_m2l_slab_folded(L, g.fold[2], (const R *)mb, (R *)lb, nrhs, g, (R *)T1, ws_elems, st);

@@ -1,5 +1,5 @@
 // k_m2l.cu -- M2L of the levels with 4^3 cells (Eq. m2l with Eq. exp_coeffs_3d, one direction at a
-// time; the passes and their budget rows are described at launch_m2l), with every direction folded
+// time; the passes and their budget rows are described at M2LArgs in k_apply.cu), with every direction folded
 // into its even and odd part.
 //
 // The one-directional coefficients satisfy E_{k,nu}(-o) = (-1)^{k+nu} E_{k,nu}(o), so on the four

@@ -131,9 +131,11 @@ void launch_s2m(int prec, bool kop, const void *x, int ncolg, const void *Stab /
                 void *mu_leaf, int nrhs, const ApplyGeo &g, cudaStream_t st, void *ws = nullptr, size_t ws_elems = 0);
 void launch_m2m(int prec, const DevLevel &par, const DevLevel &ch, int l, const void *qt, void *mu, int nrhs,
                 const ApplyGeo &g, int64_t mu_stride, cudaStream_t st);
-int launch_m2l(int prec, const DevLevel &L, int l, const void *mu, void *lam, int nrhs, const ApplyGeo &g,
-               void *T1, void *T2, size_t ws_elems, cudaStream_t st);
-// M2L kernel of a level with a G^3 grid (launch_m2l's choice): only kM2LThreePass uses T1 / T2
+// M2L of the levels 2 .. p (dl[l]); T1, T2: scratch of ws_elems elements each; -1: one interval of a
+// three-pass level does not fit it
+int launch_m2l_levels(int prec, const DevLevel *dl, int p, const void *mu, void *lam, int nrhs, const ApplyGeo &g, void *T1,
+                      void *T2, size_t ws_elems, cudaStream_t st);
+// M2L kernel of a level with a G^3 grid (launch_m2l_levels' choice): only kM2LThreePass uses T1 / T2
 enum { kM2LThreePass = 0, kM2LFused = 1, kM2LSlab = 2, kM2LFusedSliced = 3 };
 int m2l_engine(int prec, int G, int nk, int ne, int mx);
 // the engine of a level when an autotuner asks for `force` (a PFMM_M2L_* code; 0: none): the forced

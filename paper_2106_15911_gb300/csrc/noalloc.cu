@@ -132,7 +132,7 @@ extern "C" int pfmm_apply_V_noalloc(pfmm_handle *H, const double *w, double *f, 
         g.box_tiles = H->d_box_tiles;
     }
     // every buffer below is fully written before it is read, except the locals of the first two
-    // intervals of each level, which launch_m2l clears; nothing depends on the previous call
+    // intervals of each level, which launch_m2l_levels clears; nothing depends on the previous call
     launch_permute_in(w, xint, H->mixed, nrhs, g, st);
     if (tc) {  // the same nearfield engine as pfmm_apply_V
         if ((rc = run_nf_tc(H, 0, w, nrhs, whi, wlo, wmax, fint, part, st))) return rc;
@@ -149,9 +149,8 @@ extern "C" int pfmm_apply_V_noalloc(pfmm_handle *H, const double *w, double *f, 
         launch_s2m(H->fprec, false, xint, H->nt, H->d_Sx, H->d_St, mu + H->dl[p].mom_off * H->es * nrhs, nrhs, g, st, T1,
                    ws_elems);
         for (int l = p - 1; l >= 2; --l) launch_m2m(H->fprec, H->dl[l], H->dl[l + 1], l, H->d_qt, mu, nrhs, g, 0, st);
-        for (int l = 2; l <= p; ++l)
-            if (launch_m2l(H->fprec, H->dl[l], l, mu, lam, nrhs, g, T1, T2, ws_elems, st))
-                return set_error(PFMM_ERR_OOM, "static scratch too small for one M2L interval");
+        if (launch_m2l_levels(H->fprec, H->dl.data(), p, mu, lam, nrhs, g, T1, T2, ws_elems, st))
+            return set_error(PFMM_ERR_OOM, "static scratch too small for one M2L interval");
         for (int l = 3; l <= p; ++l) launch_l2l(H->fprec, H->dl[l - 1], H->dl[l], l, H->d_qt, lam, nrhs, g, 0, st);
         launch_l2t(H->fprec, lam + H->dl[p].mom_off * H->es * nrhs, H->d_Sx, H->d_St, fint, nrhs, g, 0, st, T1, ws_elems);
     }
