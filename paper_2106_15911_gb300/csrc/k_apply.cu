@@ -1415,7 +1415,8 @@ static int launch_m2l(int prec, const DevLevel &L, const void *mu, void *lam, in
     const char *mb = (const char *)mu + L.mom_off * es * nrhs;
     char *lb = (char *)lam + L.mom_off * es * nrhs;
     if (engine == kM2LFused || engine == kM2LFusedSliced)
-        return launch_m2l_folded(prec, L, g.fold[engine == kM2LFusedSliced ? 1 : 0], mb, lb, nrhs, g, T1, ws_elems, st);
+        return launch_m2l_folded(prec, engine == kM2LFusedSliced, L, g.fold[engine == kM2LFusedSliced ? 1 : 0], mb, lb, nrhs, g, T1,
+                                 ws_elems, st);
     int rc = 0;
     dispatch_prec(prec, [&](auto tag) {
         using R = decltype(tag);

@@ -21,8 +21,7 @@
 //   T2 row (nu1, nu2, B'; k3):  [X2][X1][Y3]       pass 3 sums over k3, Y3
 // The rows of one sum are consecutive (passes 1 and 3) or at steps that shrink by one row (pass 2),
 // so all passes are the same short chain: a unit (its rows and its nu) is given to 16 / NF lanes,
-// each with NF fibres in registers, and a warp takes a task of 2 NF units of one length, whose
-// chain is unrolled for that length.  Where the lengths allow it the units of a task share nu
+// each with NF fibres in registers, and a warp takes a task of 2 NF units of one length.  Where the lengths allow it the units of a task share nu
 // (their coefficient loads are one broadcast) and differ in the row key (k3 of T1, nu1 of T2, modulo
 // 4): the chunks of a row are stored at chunk ^ 2 key, so the units' stores go to different banks.
 // Tasks are dealt to the warps longest first, back and forth.  The parity of k + nu alternates with
@@ -45,14 +44,16 @@ namespace {
 constexpr int kSlabThreads = 512;  // 8^3 kernel
 
 template <typename R>
-struct Form;  // planes: FP32 words per value; NF: fibres per lane; threads and CTAs per SM
+// planes: FP32 words per value; NF: fibres per lane; threads and CTAs per SM (sliced: threads of the
+// sliced form, whose shared memory leaves room for one CTA per SM)
+struct Form;
 template <>
 struct Form<float> {
-    static constexpr int planes = 1, NF = 2, threads = 256, ctas = 2;
+    static constexpr int planes = 1, NF = 2, threads = 256, ctas = 2, sliced = 512;
 };
 template <>
 struct Form<df64> {
-    static constexpr int planes = 2, NF = 1, threads = 384, ctas = 1;
+    static constexpr int planes = 2, NF = 1, threads = 384, ctas = 1, sliced = 384;
 };
 
 __device__ __forceinline__ void load4(const float *p, float (&v)[4])
@@ -135,69 +136,33 @@ __device__ __forceinline__ void fibre_step(R (&acc)[4], const R (&in)[4], const 
     step(acc[3 - o], e[7], in[3]);
 }
 
-// the chain of a unit: LEN steps from row address p (rows `stride` words apart, then `stride - dec`
-// and so on; fibre f is f chunks of LPU further on) with the coefficients at e; after(j) sees the
-// partial sums of every step
-template <typename R, int LEN, typename After>
-__device__ __forceinline__ void chain(R (&acc)[Form<R>::NF][4], const float *p, int stride, int dec, int fstep,
-                                      const float *e, After after)
+// the chain of a unit: len steps from row address p (rows `stride` words apart, then `stride - dec` and
+// so on; the second fibre fstep words further on) with the coefficients at e; after(j) sees the partial
+// sums of every step.  Two steps at a time: unrolled for every length the passes outgrow the
+// instruction cache (M2L of 12288 x 256: double-FP32 1.79 instead of 0.93 ms, FP32 with 4 rhs 1.11
+// instead of 1.07 ms)
+template <typename R, typename After>
+__device__ __forceinline__ void chain_of(int len, R (&acc)[Form<R>::NF][4], const float *p, int stride, int dec, int fstep,
+                                         const float *e, After after)
 {
     constexpr int PL = Form<R>::planes, NF = Form<R>::NF;
 #pragma unroll
     for (int f = 0; f < NF; ++f)
 #pragma unroll
         for (int r = 0; r < 4; ++r) acc[f][r] = R(0);
-#pragma unroll
-    for (int j = 0; j < LEN; ++j) {
-        R ev[8], in[NF][4];
-        load8(e + j * 8 * PL, ev);
-        load4(p, in[0]);
-        if (NF == 2) load4(p + fstep, in[NF - 1]);
-#pragma unroll
-        for (int f = 0; f < NF; ++f) fibre_step(acc[f], in[f], ev, j & 1);
-        after(j);
-        p += stride;
-        stride -= dec;
-    }
-}
-
-// run the chain for the task's length (at most m_x + 1 = 9): in FP32 unrolled for that length; in
-// double-FP32 two steps at a time (a step is some 120 instructions: unrolled for every length the
-// three passes no longer fit the instruction cache, and the 12288 x 256 product's M2L took 1.79 ms
-// instead of 0.97)
-template <typename After>
-__device__ __forceinline__ void chain_of(int len, float (&acc)[Form<float>::NF][4], const float *p, int stride, int dec,
-                                         int fstep, const float *e, After after)
-{
-    switch (len) {
-    case 1: chain<float, 1>(acc, p, stride, dec, fstep, e, after); break;
-    case 2: chain<float, 2>(acc, p, stride, dec, fstep, e, after); break;
-    case 3: chain<float, 3>(acc, p, stride, dec, fstep, e, after); break;
-    case 4: chain<float, 4>(acc, p, stride, dec, fstep, e, after); break;
-    case 5: chain<float, 5>(acc, p, stride, dec, fstep, e, after); break;
-    case 6: chain<float, 6>(acc, p, stride, dec, fstep, e, after); break;
-    case 7: chain<float, 7>(acc, p, stride, dec, fstep, e, after); break;
-    case 8: chain<float, 8>(acc, p, stride, dec, fstep, e, after); break;
-    default: chain<float, 9>(acc, p, stride, dec, fstep, e, after); break;
-    }
-}
-template <typename After>
-__device__ __forceinline__ void chain_of(int len, df64 (&acc)[Form<df64>::NF][4], const float *p, int stride, int dec,
-                                         int fstep, const float *e, After after)
-{
-#pragma unroll
-    for (int r = 0; r < 4; ++r) acc[0][r] = df64(0);
 #pragma unroll 1
     for (int j = 0; j < len; j += 2) {
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             if (h == 1 && j + 1 >= len) break;
-            df64 ev[8], in[4];
+            R ev[8], in[NF][4];
             load8(e, ev);
-            load4(p, in);
-            fibre_step(acc[0], in, ev, h == 1);
+            load4(p, in[0]);
+            if (NF == 2) load4(p + fstep, in[NF - 1]);
+#pragma unroll
+            for (int f = 0; f < NF; ++f) fibre_step(acc[f], in[f], ev, h == 1);
             after(j + h);
-            e += 16;
+            e += 8 * PL;
             p += stride;
             stride -= dec;
         }
@@ -233,12 +198,12 @@ struct UnitBits {
 
 }  // namespace
 
-template <typename R, int Q3>
-__global__ void __launch_bounds__(Form<R>::threads, Form<R>::ctas)
+template <typename R, int Q3, int NT>
+__global__ void __launch_bounds__(NT, NT == Form<R>::threads ? Form<R>::ctas : 1)
 k_m2l_folded(M2LFoldArgs A, const R *__restrict__ mu, R *__restrict__ lam)
 {
     using F = Form<R>;
-    constexpr int PL = F::planes, NF = F::NF, LPU = 16 / NF, UPW = 32 / LPU, W = F::threads / 32, RW = 64 * PL;
+    constexpr int PL = F::planes, NF = F::NF, LPU = 16 / NF, UPW = 32 / LPU, W = NT / 32, RW = 64 * PL;
     extern __shared__ __align__(16) float sm[];
     const int nk = A.nk, na = A.na, m1 = A.mx + 1;
     float *T1 = sm, *U = T1 + A.ne * RW, *Es = U + A.p.urows * RW;
@@ -252,9 +217,9 @@ k_m2l_folded(M2LFoldArgs A, const R *__restrict__ mu, R *__restrict__ lam)
     const int nterm = k < 2 ? 0 : (k & 1 ? 2 * na : na);
     const int t_lo = chunk * A.tpc, t_hi = min(nterm, t_lo + A.tpc);
     if (A.part && t_lo >= t_hi) return;
-    for (int i = threadIdx.x; i < A.p.nunits; i += F::threads) un[i] = reinterpret_cast<const int2 *>(A.p.units)[i];
-    for (int i = threadIdx.x; i < nk; i += F::threads) urow[i] = A.p.urow[i];
-    for (int i = threadIdx.x; i < 64; i += F::threads) {
+    for (int i = threadIdx.x; i < A.p.nunits; i += NT) un[i] = reinterpret_cast<const int2 *>(A.p.units)[i];
+    for (int i = threadIdx.x; i < nk; i += NT) urow[i] = A.p.urow[i];
+    for (int i = threadIdx.x; i < 64; i += NT) {
         const int box = A.cellbox[i];
         cbo[(i & 3) * 16 + (i >> 2)] = box < 0 ? -1 : box * na * nk;
     }
@@ -272,12 +237,12 @@ k_m2l_folded(M2LFoldArgs A, const R *__restrict__ mu, R *__restrict__ lam)
         const int a = t % na, D = (k & 1) ? 3 - t / na : 2, J = k - D;
         __syncthreads();  // tables in place; the previous term's pass 3 is done with U and Es
         const float4 *Eg = reinterpret_cast<const float4 *>(A.EF) + (size_t)(((D - 2) * na + a) * na + b) * m1 * m1 * 2 * PL;
-        for (int i = threadIdx.x; i < m1 * m1 * 2 * PL; i += F::threads) reinterpret_cast<float4 *>(Es)[i] = Eg[i];
+        for (int i = threadIdx.x; i < m1 * m1 * 2 * PL; i += NT) reinterpret_cast<float4 *>(Es)[i] = Eg[i];
         const R coef = reinterpret_cast<const R *>(A.pref)[((D - 2) * na + a) * na + b];
         // moments of (J, a): lane = (multi-index, Y3) takes the 16 cells (Y1, Y2), folds them in x and
         // y and, with the lane of the mirrored Y3, in z
         const R *mJ = mu + (((size_t)rhs * A.nint + J) * A.nbox * na + a) * nk;
-        for (int i = threadIdx.x; i < ((nk + 7) & ~7) * 4; i += F::threads) {
+        for (int i = threadIdx.x; i < ((nk + 7) & ~7) * 4; i += NT) {
             const int z = i & 3, ik = i >> 2;
             const bool ok = ik < nk;
             const R *mi = mJ + (ok ? ik : 0);
@@ -392,7 +357,7 @@ k_m2l_folded(M2LFoldArgs A, const R *__restrict__ mu, R *__restrict__ lam)
     __syncthreads();
     R *out = (A.part ? reinterpret_cast<R *>(A.part) + (size_t)chunk * A.nlev : lam) +
              (((size_t)rhs * A.nint + k) * A.nbox * na + b) * nk;
-    for (int i = threadIdx.x; i < nk * 4; i += F::threads) {
+    for (int i = threadIdx.x; i < nk * 4; i += NT) {
         const int z = i & 3, iv = i >> 2;
         const float *p = U + iv * RW + z * 16;
         R v[4][4];  // [y][x]
@@ -617,7 +582,8 @@ static M2LFoldPlan make_plan(int upw, int warps, int mx, const std::vector<int> 
 M2LFoldPlan m2l_fold_plan(int prec, int mx, const std::vector<int> &kinv, bool sliced)
 {
     const int m1 = mx + 1, nf = prec == 1 ? Form<float>::NF : Form<df64>::NF, planes = prec == 1 ? 1 : 2;
-    const int warps = (prec == 1 ? Form<float>::threads : Form<df64>::threads) / 32;
+    const int warps = (prec == 1 ? (sliced ? Form<float>::sliced : Form<float>::threads)
+                                 : (sliced ? Form<df64>::sliced : Form<df64>::threads)) / 32;
     M2LFoldPlan P = make_plan(2 * nf, warps, mx, kinv, sliced, false);
     const size_t nk = P.urow.size(), ne = nk * (mx + 4) / 4;
     P.d.smem = sizeof(float) * planes * ((ne + P.d.urows) * 64 + (size_t)m1 * m1 * 8) + sizeof(int) * P.units.size() +
@@ -633,16 +599,19 @@ M2LFoldPlan m2l_slab_plan(int mx, const std::vector<int> &kinv)
 }
 
 template <typename R>
-static int launch_T(const M2LFoldArgs &A, int q3, size_t smem, dim3 grd, const void *mu, void *lam, cudaStream_t st)
+static int launch_T(const M2LFoldArgs &A, bool sliced, dim3 grd, const void *mu, void *lam, cudaStream_t st)
 {
-    auto kf = q3 <= 4 ? k_m2l_folded<R, 4> : k_m2l_folded<R, 7>;
-    if (q3 > 7) return -1;
-    if (cudaFuncSetAttribute(kf, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return -1;
-    kf<<<grd, Form<R>::threads, smem, st>>>(A, (const R *)mu, (R *)lam);
+    constexpr int NT = Form<R>::threads, NS = Form<R>::sliced;
+    auto kf = sliced && NS != NT ? (A.p.q3 <= 4 ? k_m2l_folded<R, 4, NS> : nullptr)
+              : A.p.q3 <= 4     ? k_m2l_folded<R, 4, NT>
+              : A.p.q3 <= 6     ? k_m2l_folded<R, 6, NT>
+                                : nullptr;
+    if (!kf || cudaFuncSetAttribute(kf, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)A.p.smem) != cudaSuccess) return -1;
+    kf<<<grd, sliced ? NS : NT, A.p.smem, st>>>(A, (const R *)mu, (R *)lam);
     return 0;
 }
 
-int launch_m2l_folded(int prec, const DevLevel &L, const M2LFoldDev &P, const void *mu, void *lam, int nrhs,
+int launch_m2l_folded(int prec, bool sliced, const DevLevel &L, const M2LFoldDev &P, const void *mu, void *lam, int nrhs,
                       const ApplyGeo &g, void *ws, size_t ws_elems, cudaStream_t st)
 {
     M2LFoldArgs A{};
@@ -668,7 +637,7 @@ int launch_m2l_folded(int prec, const DevLevel &L, const M2LFoldDev &P, const vo
     A.part = split ? ws : nullptr;
     A.nlev = nlev;
     const dim3 grd((unsigned)((L.nint - A.k_lo) * g.na * A.nchunk), nrhs);
-    const int rc = prec == 1 ? launch_T<float>(A, P.q3, P.smem, grd, mu, lam, st) : launch_T<df64>(A, P.q3, P.smem, grd, mu, lam, st);
+    const int rc = prec == 1 ? launch_T<float>(A, sliced, grd, mu, lam, st) : launch_T<df64>(A, sliced, grd, mu, lam, st);
     if (rc) return rc;
     if (split) {
         const unsigned blocks = (unsigned)((nlev + 255) / 256);
@@ -744,52 +713,45 @@ __device__ __forceinline__ void fibre8(float (&acc)[8], const float (&in)[8], co
     for (int j = 0; j < 4; ++j) a = fmaf(e[j], in[s * 4 + j], a);
 }
 
-// chain of LEN steps of passes 2 and 3: two fibres per lane at p and p + fstep, halves 32 words apart
-template <int LEN>
-__device__ __forceinline__ void chain8(float (&acc)[2][8], const float *p, int stride, int dec, int fstep, const float *e)
+// chain of passes 2 and 3: two fibres per lane (fstep words apart), the halves of a fibre at p + c0 and
+// p + c1
+__device__ __forceinline__ void chain8(int len, float (&acc)[2][8], const float *p, int c0, int c1, int stride, int dec,
+                                       int fstep, const float *e)
 {
 #pragma unroll
     for (int f = 0; f < 2; ++f)
 #pragma unroll
         for (int r = 0; r < 8; ++r) acc[f][r] = 0.f;
+#pragma unroll 1
+    for (int j = 0; j < len; j += 2) {
 #pragma unroll
-    for (int j = 0; j < LEN; ++j) {
-        float in[2][8];
+        for (int h = 0; h < 2; ++h) {
+            if (h == 1 && j + 1 >= len) break;
+            float in[2][8];
 #pragma unroll
-        for (int f = 0; f < 2; ++f) {
-            float h0[4], h1[4];
-            load4(p + f * fstep, h0);
-            load4(p + f * fstep + 32, h1);
+            for (int f = 0; f < 2; ++f) {
+                float h0[4], h1[4];
+                load4(p + f * fstep + c0, h0);
+                load4(p + f * fstep + c1, h1);
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                in[f][q] = h0[q];
-                in[f][4 + q] = h1[q];
+                for (int q = 0; q < 4; ++q) {
+                    in[f][q] = h0[q];
+                    in[f][4 + q] = h1[q];
+                }
             }
+#pragma unroll
+            for (int s = 0; s < 2; ++s)
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    float ev[4];
+                    load4(e + s * 16 + i * 4, ev);
+                    fibre8(acc[0], in[0], ev, s, i, h);
+                    fibre8(acc[1], in[1], ev, s, i, h);
+                }
+            p += stride;
+            stride -= dec;
+            e += 32;
         }
-#pragma unroll
-        for (int s = 0; s < 2; ++s)
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                float ev[4];
-                load4(e + j * 32 + s * 16 + i * 4, ev);
-                fibre8(acc[0], in[0], ev, s, i, j & 1);
-                fibre8(acc[1], in[1], ev, s, i, j & 1);
-            }
-        p += stride;
-        stride -= dec;
-    }
-}
-__device__ __forceinline__ void chain8_of(int len, float (&acc)[2][8], const float *p, int stride, int dec, int fstep,
-                                          const float *e)
-{
-    switch (len) {
-    case 1: chain8<1>(acc, p, stride, dec, fstep, e); break;
-    case 2: chain8<2>(acc, p, stride, dec, fstep, e); break;
-    case 3: chain8<3>(acc, p, stride, dec, fstep, e); break;
-    case 4: chain8<4>(acc, p, stride, dec, fstep, e); break;
-    case 5: chain8<5>(acc, p, stride, dec, fstep, e); break;
-    case 6: chain8<6>(acc, p, stride, dec, fstep, e); break;
-    default: chain8<7>(acc, p, stride, dec, fstep, e); break;
     }
 }
 
@@ -871,7 +833,7 @@ k_m2l_slab_folded(M2LFoldArgs A, const float *__restrict__ F, float *__restrict_
                 const UnitBits u(un[A.p.first2[sl] + ts * 2 + sub]);
                 const int z = cl & 7, i0 = cl >> 3;
                 float acc[2][8];
-                chain8_of(u.len, acc, T1 + u.row * RW + i0 * 64 + z * 4, u.step * RW, RW, 128, Es + u.nu * m1 * 32);
+                chain8(u.len, acc, T1 + u.row * RW + i0 * 64 + z * 4, 0, 32, u.step * RW, RW, 128, Es + u.nu * m1 * 32);
                 if (u.valid) {
                     // to [X1][z / 4][X2 ^ swizzle][z % 4]: the lanes' eight groups of four words on all banks
                     float *o = T2 + u.out * RW + i0 * 64 + (z >> 2) * 32 + (z & 3);
@@ -895,43 +857,8 @@ k_m2l_slab_folded(M2LFoldArgs A, const float *__restrict__ F, float *__restrict_
                 const int X2 = cl & 7, i0 = cl >> 3;
                 float acc[2][8];
                 // the halves of a fibre (z / 4) lie at different swizzles
-                const float *p = T2 + u.row * RW + i0 * 64;
-                const int c0 = (X2 ^ (i0 << 1 | u.key << 2)) << 2, c1 = (X2 ^ (1 | i0 << 1 | u.key << 2)) << 2;
-                const float *e = Es + u.nu * m1 * 32;
-#pragma unroll
-                for (int f = 0; f < 2; ++f)
-#pragma unroll
-                    for (int r = 0; r < 8; ++r) acc[f][r] = 0.f;
-#pragma unroll 1
-                for (int j = 0; j < u.len; j += 2) {
-#pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        if (h == 1 && j + 1 >= u.len) break;
-                        float in[2][8];
-#pragma unroll
-                        for (int f = 0; f < 2; ++f) {
-                            float h0[4], h1[4];
-                            load4(p + f * 128 + c0, h0);
-                            load4(p + f * 128 + 32 + c1, h1);
-#pragma unroll
-                            for (int v = 0; v < 4; ++v) {
-                                in[f][v] = h0[v];
-                                in[f][4 + v] = h1[v];
-                            }
-                        }
-#pragma unroll
-                        for (int s = 0; s < 2; ++s)
-#pragma unroll
-                            for (int i = 0; i < 4; ++i) {
-                                float ev[4];
-                                load4(e + s * 16 + i * 4, ev);
-                                fibre8(acc[0], in[0], ev, s, i, h);
-                                fibre8(acc[1], in[1], ev, s, i, h);
-                            }
-                        p += RW;
-                        e += 32;
-                    }
-                }
+                chain8(u.len, acc, T2 + u.row * RW + i0 * 64, (X2 ^ (i0 << 1 | u.key << 2)) << 2,
+                       32 + ((X2 ^ (1 | i0 << 1 | u.key << 2)) << 2), RW, 0, 128, Es + u.nu * m1 * 32);
 #pragma unroll
                 for (int f = 0; f < 2; ++f)
 #pragma unroll

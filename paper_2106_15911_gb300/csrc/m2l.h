@@ -39,7 +39,7 @@ struct M2LFoldArgs {
 // folded coefficients of a level with G = 4 or 8 cells per direction
 size_t m2l_fold_table_floats(int na, int mx, int G, int prec);
 void launch_m2l_fold_table(const double *E1, int na, int mx, int G, int ntr, int prec, float *EF, cudaStream_t st);
-int launch_m2l_folded(int prec, const DevLevel &L, const M2LFoldDev &P, const void *mu, void *lam, int nrhs,
+int launch_m2l_folded(int prec, bool sliced, const DevLevel &L, const M2LFoldDev &P, const void *mu, void *lam, int nrhs,
                       const ApplyGeo &g, void *ws, size_t ws_elems, cudaStream_t st);
 // 8^3 level, FP32; ws: scratch of ws_elems floats for the folded moments of some source intervals.
 // Returns 1 (nothing launched) when ws does not hold those of one target interval
