@@ -78,9 +78,9 @@ EncodeTiledFn encode_fn()
     return fn;
 }
 
-// FP16 tensor map, 128-byte swizzle, zero fill out of bounds; dims innermost first
+// FP16 tensor map, 128-byte swizzle unless given, zero fill out of bounds; dims innermost first
 int encode_map(CUtensorMap *m, const void *base, int rank, const uint64_t *dims, const uint64_t *strides_bytes,
-               const uint32_t *box)
+               const uint32_t *box, CUtensorMapSwizzle swizzle = CU_TENSOR_MAP_SWIZZLE_128B)
 {
     EncodeTiledFn fn = encode_fn();
     if (!fn) return fail(PFMM_ERR_CUDA, "cuTensorMapEncodeTiled is not available");
@@ -93,7 +93,7 @@ int encode_map(CUtensorMap *m, const void *base, int rank, const uint64_t *dims,
         if (i > 0) s[i - 1] = strides_bytes[i - 1];
     }
     CUresult r = fn(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, rank, const_cast<void *>(base), d, s, b, e,
-                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                    CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                     CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) return fail(PFMM_ERR_CUDA, "cuTensorMapEncodeTiled failed (" + std::to_string((int)r) + ")");
     return PFMM_OK;
@@ -175,9 +175,13 @@ int ensure_workspace(pfmm_handle *H, int nrhs)
     H->d_nfpart = nullptr;
     if (H->tcV || H->tcK) {
         H->w_elems = (size_t)nrhs * H->Et * std::max(H->colsV_u, H->colsK_u);
-        const int planes = std::max(H->tcV ? pfmm::nf_tc_planes(H, 0, nrhs) : 1, H->tcK ? pfmm::nf_tc_planes(H, 1, nrhs) : 1);
+        // fewer right-hand sides may take more planes each
+        size_t planes = 1;
+        for (int r = 1; r <= nrhs; ++r)
+            for (int op = 0; op < 2; ++op)
+                if (op == 0 ? H->tcV : H->tcK) planes = std::max(planes, (size_t)r * pfmm::nf_tc_planes(H, op, r));
         if ((rc = H->alloc(&H->d_Whi, H->w_elems)) || (rc = H->alloc(&H->d_Wlo, H->w_elems)) ||
-            (rc = H->alloc(&H->d_wmax, (size_t)nrhs)) || (rc = H->alloc(&H->d_nfpart, (size_t)planes * n_in)))
+            (rc = H->alloc(&H->d_wmax, (size_t)nrhs)) || (rc = H->alloc(&H->d_nfpart, planes * H->Et * H->nt)))
             return rc;
     }
     H->release(H->d_Wres);
@@ -226,12 +230,11 @@ int pfmm::ensure_ws(pfmm_handle *H, int nrhs) { return ensure_workspace(H, nrhs)
 // wmax), encodes their TMA views and launches.
 int pfmm::nf_tc_planes(const pfmm_handle *H, int op, int nrhs)
 {
-    const int cols = op == 0 ? H->colsV_u : H->colsK_u, nint = H->Et / 2;
-    return nf_tc_ksplit(nrhs * H->ntiles128 * ((nint + 127) / 128), cols / 64, H->nsm);
+    return nf_tc_ksplit(H->nt, H->Et / 2, H->Et, nrhs, op == 0 ? H->colsV_u : H->colsK_u, H->nsm);
 }
 
 int pfmm::run_nf_tc(pfmm_handle *H, int op, const double *x, int nrhs, void *whi, void *wlo,
-                    unsigned long long *wmax, double *fint, double *part, cudaStream_t st)
+                    unsigned long long *wmax, double *fint, double *part, int planes, cudaStream_t st)
 {
     int rc;
     const int cols = op == 0 ? H->colsV_u : H->colsK_u;
@@ -240,23 +243,19 @@ int pfmm::run_nf_tc(pfmm_handle *H, int op, const double *x, int nrhs, void *whi
     const int nint = H->Et / 2;
     uint64_t dims[4] = {(uint64_t)cols, 2, (uint64_t)nint, (uint64_t)nrhs};
     uint64_t str[3] = {(uint64_t)cols * 2, (uint64_t)cols * 4, (uint64_t)cols * 4 * nint};
-    uint32_t box[4] = {64, 1, 128, 1};
+    uint32_t box[4] = {32, 1, (uint32_t)nf_tc_intervals(nint), 1};
     CUtensorMap mWhi, mWlo;
-    if ((rc = encode_map(&mWhi, whi, 4, dims, str, box)) || (rc = encode_map(&mWlo, wlo, 4, dims, str, box))) return rc;
+    if ((rc = encode_map(&mWhi, whi, 4, dims, str, box, CU_TENSOR_MAP_SWIZZLE_64B)) ||
+        (rc = encode_map(&mWlo, wlo, 4, dims, str, box, CU_TENSOR_MAP_SWIZZLE_64B)))
+        return rc;
     NfTcParams P{};
-    P.panels = H->d_panels;
-    P.tiles = H->d_tiles128;
-    P.ntiles = H->ntiles128;
-    P.nib = (nint + 127) / 128;
-    P.nkb = cols / 64;
-    const int tiles = nrhs * P.ntiles * P.nib;
-    // split K into a few chunks for SM balance (each chunk accumulates 32-stage sub-chunks into its
-    // own FP64 partial plane; the planes are summed in order afterwards)
-    const int ks = nf_tc_ksplit(tiles, P.nkb, H->nsm);
+    P.A = (const unsigned char *)(op == 0 ? H->d_AVsplit : H->d_AKsplit);
+    P.ntiles = (H->nt + 127) / 128;
+    P.nkb = cols / 32;
+    // K chunks for SM balance (each accumulates its sub-chunks into its own FP64 partial plane; the
+    // planes are summed in order afterwards)
+    const int ks = std::min(nf_tc_planes(H, op, nrhs), planes);
     P.ksplit = ks;
-    P.nitems = tiles * ks;
-    P.cols_pad = cols;
-    P.kop = op;
     P.nint = nint;
     P.Et = H->Et;
     P.nt = H->nt;
@@ -266,8 +265,7 @@ int pfmm::run_nf_tc(pfmm_handle *H, int op, const double *x, int nrhs, void *whi
     P.nrhs = nrhs;
     P.err = H->d_err;
     if (H->cur_ev) cudaEventRecord(H->cur_ev->ev[9], st);
-    if (launch_nf_apply_tc(op == 0 ? H->mapAVhi : H->mapAKhi, op == 0 ? H->mapAVlo : H->mapAKlo, mWhi, mWlo, P, H->nsm,
-                           st))
+    if (launch_nf_apply_tc(mWhi, mWlo, P, H->nsm, st))
         return fail(PFMM_ERR_CUDA, std::string("tensor-core nearfield launch: ") + cudaGetErrorString(cudaGetLastError()));
     if (H->cur_ev) {
         cudaEventRecord(H->cur_ev->ev[10], st);
@@ -837,55 +835,34 @@ static int build_impl(const pfmm_mesh *mesh, const pfmm_params *prm, cudaStream_
         CK(cudaMalloc((void **)&H->d_err, sizeof(int)));
         H->allocs.push_back(H->d_err);
         CK(cudaMemsetAsync(H->d_err, 0, sizeof(int), st));
-        if (fullV || fullK) {
-            std::vector<int> t128;
-            for (size_t i = 0; i < t.panels.size(); ++i)
-                for (int r0 = 0; r0 < t.panels[i].nrows; r0 += 128) {
-                    t128.push_back((int)i);
-                    t128.push_back(r0);
-                }
-            H->ntiles128 = (int)t128.size() / 2;
-            if ((rc = upload(H, &H->d_tiles128, t128, st))) return rc;
-        }
         if (!H->mixed && (fullV || fullK)) {
             if ((rc = build_crt(H, t, fullV, fullK, st))) return rc;
             fullV = fullK = false;
         }
         if (fullV) {
             H->colsV_u = t.panels[0].colsV_pad;
-            size_t n = (size_t)t.sizeV;
-            if ((rc = H->alloc(&H->d_AVhi, n)) || (rc = H->alloc(&H->d_AVlo, n))) return rc;
-            H->a_expV = panel_scale_exp((const float *)H->d_AV, n, (unsigned *)H->d_err, st);
+            H->a_expV = panel_scale_exp((const float *)H->d_AV, (size_t)t.sizeV, (unsigned *)H->d_err, st);
             if (H->a_expV == INT32_MIN) return fail(PFMM_ERR_CUDA, "panel scale");
             CK(cudaMemsetAsync(H->d_err, 0, sizeof(int), st));
-            launch_split_panel((const float *)H->d_AV, H->d_AVhi, H->d_AVlo, n, H->colsV_u, H->a_expV, st);
+            if ((rc = H->alloc(&H->d_AVsplit, split_panel_halves(nt, H->colsV_u)))) return rc;
+            launch_split_panel((const float *)H->d_AV, H->d_panels, H->d_tri_leaf, 0, nt, H->colsV_u, H->a_expV,
+                               H->d_AVsplit, st);
             CK(cudaStreamSynchronize(st));
             H->release(H->d_AV);  // hi + lo represent it; the CUDA-core path reads their sum
             H->d_AV = nullptr;
-            // [block][64 rows][64 columns] view of the 64 x 64 blocks (n is a multiple of 4096)
-            uint64_t dims[3] = {64, 64, (uint64_t)(n / 4096)}, str[2] = {128, 8192};
-            uint32_t box[3] = {64, 64, 1};
-            if ((rc = encode_map(&H->mapAVhi, H->d_AVhi, 3, dims, str, box)) ||
-                (rc = encode_map(&H->mapAVlo, H->d_AVlo, 3, dims, str, box)))
-                return rc;
             H->tcV = true;
         }
         if (fullK) {
             H->colsK_u = t.panels[0].colsK_pad;
-            size_t n = (size_t)t.sizeK;
-            if ((rc = H->alloc(&H->d_AKhi, n)) || (rc = H->alloc(&H->d_AKlo, n))) return rc;
-            H->a_expK = panel_scale_exp((const float *)H->d_AK, n, (unsigned *)H->d_err, st);
+            H->a_expK = panel_scale_exp((const float *)H->d_AK, (size_t)t.sizeK, (unsigned *)H->d_err, st);
             if (H->a_expK == INT32_MIN) return fail(PFMM_ERR_CUDA, "panel scale");
             CK(cudaMemsetAsync(H->d_err, 0, sizeof(int), st));
-            launch_split_panel((const float *)H->d_AK, H->d_AKhi, H->d_AKlo, n, H->colsK_u, H->a_expK, st);
+            if ((rc = H->alloc(&H->d_AKsplit, split_panel_halves(nt, H->colsK_u)))) return rc;
+            launch_split_panel((const float *)H->d_AK, H->d_panels, H->d_tri_leaf, 1, nt, H->colsK_u, H->a_expK,
+                               H->d_AKsplit, st);
             CK(cudaStreamSynchronize(st));
-            H->release(H->d_AK);
+            H->release(H->d_AK);  // hi + lo represent it; the CUDA-core path reads their sum
             H->d_AK = nullptr;
-            uint64_t dims[3] = {64, 64, (uint64_t)(n / 4096)}, str[2] = {128, 8192};
-            uint32_t box[3] = {64, 64, 1};
-            if ((rc = encode_map(&H->mapAKhi, H->d_AKhi, 3, dims, str, box)) ||
-                (rc = encode_map(&H->mapAKlo, H->d_AKlo, 3, dims, str, box)))
-                return rc;
             H->tcK = true;
         }
         CK(cudaGetLastError());
@@ -991,7 +968,8 @@ static int apply_impl(pfmm_handle *H, int op, const double *x, double *f, int nr
     const bool tc = (parts & PFMM_PART_NEAR) && (op == 0 ? H->tcV : H->tcK) && !H->nf_cuda_cores;
     const bool crt = (parts & PFMM_PART_NEAR) && (op == 0 ? H->crtV : H->crtK) && !H->nf_cuda_cores;
     if (tc) {
-        if ((rc = pfmm::run_nf_tc(H, op, x, nrhs, H->d_Whi, H->d_Wlo, H->d_wmax, H->d_fint, H->d_nfpart, st)))
+        if ((rc = pfmm::run_nf_tc(H, op, x, nrhs, H->d_Whi, H->d_Wlo, H->d_wmax, H->d_fint, H->d_nfpart,
+                                  pfmm::nf_tc_planes(H, op, nrhs), st)))
             return rc;
     } else if (crt) {
         if ((rc = pfmm::run_nf_crt(H, op, x, nrhs, H->d_fint, st))) return rc;
@@ -1149,7 +1127,8 @@ int pfmm_get_info(const pfmm_handle *h, pfmm_info *info)
     info->n_m2l_pairs = t.n_m2l_pairs;
     // stored blocks: the arithmetic-type panels, or their two FP32 parts once split for tcgen05
     info->nearfield_bytes = h->otf ? h->otf_bytes
-                                   : t.sizeV * (h->tcV ? 4 : (int64_t)h->es) + t.sizeK * (h->tcK ? 4 : (int64_t)h->es);
+                                   : (h->tcV ? 2 * (int64_t)pfmm::split_panel_halves(h->nt, h->colsV_u) : t.sizeV * (int64_t)h->es) +
+                                         (h->tcK ? 2 * (int64_t)pfmm::split_panel_halves(h->nt, h->colsK_u) : t.sizeK * (int64_t)h->es);
     info->device_bytes = h->dev_bytes;
     info->nf_tensor_cores = (h->tcV || h->crtV ? 1 : 0) | (h->tcK || h->crtK ? 2 : 0);
     info->nf_form = h->crtV || h->crtK ? h->crt_form : 0;

@@ -22,9 +22,9 @@ struct pfmm_handle;
 namespace pfmm {
 // tensor-core nearfield of op (0: V, 1: K) into fint; whi/wlo: [nrhs][E_t][cols] FP32 workspaces
 // whi, wlo: FP16 input parts ([nrhs][E_t][cols] each); wmax: nrhs words of scratch
-// part: FP64 partial planes, nf_tc_planes(H, op, nrhs) x nrhs x E_t x E_x doubles
+// part: FP64 partial planes, `planes` (at most nf_tc_planes(H, op, nrhs)) x nrhs x E_t x E_x doubles
 int run_nf_tc(pfmm_handle *H, int op, const double *x, int nrhs, void *whi, void *wlo, unsigned long long *wmax,
-              double *fint, double *part, cudaStream_t st);
+              double *fint, double *part, int planes, cudaStream_t st);
 // K-chunk partial planes of the tensor-core nearfield of op for nrhs right-hand sides
 int nf_tc_planes(const pfmm_handle *H, int op, int nrhs);
 // FP64 mode: exact residue-arithmetic nearfield of op on the tensor cores into fint (overwritten)
@@ -93,12 +93,10 @@ struct pfmm_handle {
     bool nf_cuda_cores = false;     // engine override chosen by the batch autotuner
     pfmm::M2LFoldDev fold[3]{};     // unit tables of the folded M2L: 4^3 with T2 whole, sliced; 8^3
     int m2l_force = 0;              // M2L engine chosen by the batch autotuner (PFMM_M2L_* code, 0: per-level default)
-    uint16_t *d_AVhi = nullptr, *d_AVlo = nullptr, *d_AKhi = nullptr, *d_AKlo = nullptr;  // FP16 parts
+    uint16_t *d_AVsplit = nullptr, *d_AKsplit = nullptr;  // FP16 parts (nf_split_index)
     int a_expV = 0, a_expK = 0;     // scale exponents of the panels' FP16 split
-    CUtensorMap mapAVhi{}, mapAVlo{}, mapAKhi{}, mapAKlo{};
     int colsV_u = 0, colsK_u = 0;  // common padded column count of the panels
-    int *d_tiles128 = nullptr;
-    int ntiles128 = 0, nsm = 0;
+    int nsm = 0;
     int *d_err = nullptr;           // bounded-wait error word of the device kernels
     // FP64 mode, exact residue-arithmetic nearfield on the tensor cores (k_nf_crt.cu)
     bool crtV = false, crtK = false;
@@ -129,8 +127,7 @@ struct pfmm_handle {
     pfmm::NfHalfSplit split_desc(int op) const
     {
         pfmm::NfHalfSplit s;
-        s.hi = op == 0 ? d_AVhi : d_AKhi;
-        s.lo = op == 0 ? d_AVlo : d_AKlo;
+        s.parts = op == 0 ? d_AVsplit : d_AKsplit;
         s.inv_scale = std::ldexp(1.0f, -(op == 0 ? a_expV : a_expK));
         return s;
     }

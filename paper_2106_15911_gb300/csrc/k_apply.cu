@@ -113,9 +113,9 @@ __global__ void __launch_bounds__(256) k_nf_apply(const S *__restrict__ A, const
     const S *xr = x + (size_t)rhs * Et * ncolg;
     const int *cols = colidx + (kop ? P.colK_at : P.colV_at);
     const int ncp = kop ? P.colsK_pad : P.colsV_pad;
-    const bool half = hs.hi != nullptr;  // FP32 only
+    const bool half = hs.parts != nullptr;  // FP32 only
     const size_t off = kop ? P.offK : P.offV;
-    const __half *Hh = reinterpret_cast<const __half *>(hs.hi), *Hl = reinterpret_cast<const __half *>(hs.lo);
+    const __half *Hp = reinterpret_cast<const __half *>(hs.parts);
     S acc[4][4];
     double accd[4][4];
 #pragma unroll
@@ -129,15 +129,18 @@ __global__ void __launch_bounds__(256) k_nf_apply(const S *__restrict__ A, const
     int ktiles = 0;
     for (int d = 0; d < nd; ++d) {
         const size_t dbase = off + ((size_t)d * P.rows_pad + r0) * ncp;
-        const size_t rbase = off / ncp + (size_t)d * P.rows_pad + r0;  // global row (FP16 parts)
         for (int k0 = 0; k0 < ncp; k0 += BK) {
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
                 int e = tid + 256 * q;
                 int i = e >> 4, j = e & 15;
                 if (half) {
-                    const size_t ia = nf_tiled_index(rbase + i, k0 + j, ncp >> 6);
-                    As[j][i] = S((__half2float(Hh[ia]) + __half2float(Hl[ia])) * hs.inv_scale);
+                    S v = S(0);
+                    if (r0 + i < P.nrows) {
+                        const __half *h = Hp + nf_split_index(P.row0 + r0 + i, d, k0 + j, ncp >> 5);
+                        v = S((__half2float(h[0]) + __half2float(h[kSplitPart])) * hs.inv_scale);
+                    }
+                    As[j][i] = v;
                 } else {
                     As[j][i] = A[dbase + (size_t)i * ncp + k0 + j];
                 }

@@ -34,9 +34,8 @@ __host__ __device__ inline int f64_scale_exp(unsigned long long bits)
 }
 
 struct NfTcParams {
-    const PanelGPU *panels;
-    const int *tiles;   // [ntiles][2] (panel, first row) with 128-row tiles
-    int ntiles, nib, ksplit, nkb, nitems, cols_pad, kop;
+    const unsigned char *A;  // FP16 parts of the blocks (nf_split_index)
+    int ntiles, ksplit, nkb, nitems;  // 128-row tiles, K chunks, 32-column blocks; nitems is set by the launch
     int nint, Et, nt;
     int a_exp;              // scale exponent of the panels' FP16 split
     const unsigned long long *wmax;  // [nrhs] FP64 bits of max |W| per rhs (scale of the input split)
@@ -48,21 +47,20 @@ struct NfTcParams {
 // per-rhs max |x| of x [nrhs][per_rhs] FP64 into wmax (FP64 bits, accumulated with atomicMax: zero it first)
 void launch_absmax_input(const double *x, size_t per_rhs, int nrhs, unsigned grid_x, unsigned long long *wmax,
                          cudaStream_t st);
-size_t nf_tc_smem_bytes();
-// K chunks (partial planes) of the tensor-core nearfield for `tiles` output tiles of nkb column
-// blocks: 1 .. 8 (at most the tile's 32-stage sub-chunks), chosen so the work items fill the
-// rounds of the persistent grid of nsm CTAs best
-int nf_tc_ksplit(int tiles, int nkb, int nsm);
+// leaf intervals per work item: rows of the W tensor maps' box
+int nf_tc_intervals(int nint);
+// K chunks (partial planes) of the tensor-core nearfield: 1 .. 16
+int nf_tc_ksplit(int nt, int nint, int Et, int nrhs, int cols, int nsm);
 // f[i] = sum_kc part[kc][i] (n elements per plane, plane order)
 void launch_nf_tc_reduce(const double *part, int ks, size_t n, double *f, cudaStream_t st);
-int launch_nf_apply_tc(const CUtensorMap &Ahi, const CUtensorMap &Alo, const CUtensorMap &Whi, const CUtensorMap &Wlo,
-                       const NfTcParams &P, int nsm, cudaStream_t st);
+int launch_nf_apply_tc(const CUtensorMap &Whi, const CUtensorMap &Wlo, const NfTcParams &P, int nsm, cudaStream_t st);
 // scale exponent of n stored FP32 panel values (synchronises st; scratch: one device word);
 // INT32_MIN on a CUDA error
 int panel_scale_exp(const float *A, size_t n, unsigned *scratch, cudaStream_t st);
-// hi/lo FP16 parts ([n] each, 64 x 64 blocks of nf_tiled_index) of 2^a_exp A (row-major, ncp
-// columns, a multiple of 64)
-void launch_split_panel(const float *A, void *hi, void *lo, size_t n, int ncp, int a_exp, cudaStream_t st);
+// FP16 parts (nf_split_index) of 2^a_exp A, panels of 4 step offsets and ncp columns (a multiple of 64)
+size_t split_panel_halves(int nt, int ncp);
+void launch_split_panel(const float *A, const PanelGPU *panels, const int *tri_leaf, int kop, int nt, int ncp, int a_exp,
+                        void *out, cudaStream_t st);
 // per-rhs max |x| into wmax[nrhs], then the hi/lo FP16 parts [nrhs][Et][ncol_pad] of the scaled,
 // permuted (V) or padded (K) input
 void launch_split_input(const double *x, const int *perm, int ncol, int ncol_pad, int nrhs, int Et, void *hi,

@@ -73,8 +73,7 @@ extern "C" int pfmm_apply_V_noalloc(pfmm_handle *H, const double *w, double *f, 
     const bool tc = H->tcV && !H->nf_cuda_cores;
     const size_t b_w = tc ? up256((size_t)nrhs * H->Et * H->colsV_u * sizeof(uint16_t)) : 0;
     const size_t b_m = tc ? up256((size_t)nrhs * sizeof(unsigned long long)) : 0;
-    const size_t b_p = tc ? up256((size_t)nf_tc_planes(H, 0, nrhs) * n_in * sizeof(double)) : 0;
-    const size_t fixed = b_x + b_f + 2 * b_mu + 2 * b_w + b_m + b_p;
+    int planes = tc ? nf_tc_planes(H, 0, nrhs) : 0;  // fewer where the array is short of room
     // elements of T1 (and of T2) for the largest single-interval chunk of the levels whose M2L
     // takes the three separable passes (the fused and slab kernels keep their intermediates in
     // shared memory; the fused kernel's split mode and the two-stage S2M / L2T use T1 only when
@@ -86,6 +85,12 @@ extern "C" int pfmm_apply_V_noalloc(pfmm_handle *H, const double *w, double *f, 
         int maxpairs = 0;
         for (int k = 0; k < L.nint; ++k) maxpairs = std::max(maxpairs, L.kptr_host[k + 1] - L.kptr_host[k]);
         need_T = std::max(need_T, (size_t)nrhs * maxpairs * H->na * H->na * L.G * L.G * L.G * H->ne);
+    }
+    size_t b_p = 0, fixed = 0;
+    for (;; --planes) {
+        b_p = up256((size_t)planes * n_in * sizeof(double));
+        fixed = b_x + b_f + 2 * b_mu + 2 * b_w + b_m + b_p;
+        if (planes <= 1 || fixed + 2 * up256(need_T * H->es) <= kScratchBytes) break;
     }
     if (fixed + 2 * up256(need_T * H->es) > kScratchBytes)
         return set_error(PFMM_ERR_OOM, "pfmm_apply_V_noalloc needs " + std::to_string(fixed + 2 * up256(need_T * H->es)) +
@@ -135,7 +140,7 @@ extern "C" int pfmm_apply_V_noalloc(pfmm_handle *H, const double *w, double *f, 
     // intervals of each level, which launch_m2l_levels clears; nothing depends on the previous call
     launch_permute_in(w, xint, H->mixed, nrhs, g, st);
     if (tc) {  // the same nearfield engine as pfmm_apply_V
-        if ((rc = run_nf_tc(H, 0, w, nrhs, whi, wlo, wmax, fint, part, st))) return rc;
+        if ((rc = run_nf_tc(H, 0, w, nrhs, whi, wlo, wmax, fint, part, planes, st))) return rc;
     } else if (H->otf) {
         cudaMemsetAsync(fint, 0, n_in * sizeof(double), st);
         if ((rc = run_nf_otf(H, 0, xint, H->nt, H->Et, H->ls, nrhs, 1 << 30, fint, st))) return rc;
