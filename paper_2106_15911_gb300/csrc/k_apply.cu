@@ -91,7 +91,8 @@ void launch_to_df64(double *x, size_t n, cudaStream_t st)
 // of uniform steps: for target step t = k*ls + s of leaf interval k the temporal nearfield
 // N(I_k) = {I_{k-1}, I_k} contributes the step offsets d = 0 .. ls + s, so
 //   f[t][rows of X] = sum_{d=0}^{ls+s} A_d[X] x[t - d][cols of X].
-// One CTA computes a 64 x 64 tile (64 rows of a panel x 64 steps of one phase s) over all d
+// k_nf_apply, for a bounded number of offsets (the same-step block) or more than four steps per leaf:
+// one CTA computes a 64 x 64 tile (64 rows of a panel x 64 steps of one phase s) over all d
 // and all columns, so every output element is written exactly once.
 template <typename S>
 __global__ void __launch_bounds__(256) k_nf_apply(const S *__restrict__ A, const int *__restrict__ colidx,
@@ -191,10 +192,214 @@ __global__ void __launch_bounds__(256) k_nf_apply(const S *__restrict__ A, const
     }
 }
 
+// The same product, all step offsets, 8 rows of a panel per CTA.  64 x 64 tiles left 90 % padding on panels
+// of few rows (leaf boxes of an 8^3 grid on 1728 triangles hold 4 to 8), read as much from shared memory as
+// they multiplied, and staged the inputs once per offset.  Here a thread owns two leaf intervals (one at
+// LS > 2) with all their LS steps, so a column's 2 LS inputs of the interval and the one before it serve
+// every offset, and the 8 rows of A_d are broadcast reads: per column 4 LS (3 LS + 1) FMAs per interval
+// against 2 LS inputs and 16 LS broadcast coefficients.  Two stages of columns, copied behind the FMAs
+// (copies through registers took 2.7 ms at the first size below).  FP32 sums over
+// 128 products, added with their rounding errors kept (two FP32: the FP64 unit would be busy for half of the
+// FMAs' time, and sums over 512 products, all offsets in one, came out 20 % further from FP64 than the tiles').
+// Bound by the FMAs.  Nearfield, 64 x 64 tiles -> here: 1728 triangles x 1024 steps mixed 8.36 -> 1.12 ms,
+// FP64 134 -> 23.2; 768 x 256, 4 right-hand sides, mixed 0.99 -> 0.38; 192 x 16 FP64 0.79 -> 0.73; 3072 x 128
+// FP64 13.1 -> 11.8; 12288 x 64 mixed 9.0 -> 6.2; three steps per leaf FP64 3.9 -> 2.7; one step mixed, K,
+// 0.127 -> 0.113.
+constexpr int kNfRows = 8;
+__host__ __device__ constexpr int nf_rows_bk(size_t size) { return size == 4 ? 16 : 8; }
+__host__ __device__ constexpr int nf_rows_intervals(int ls) { return ls <= 2 ? 2 : 1; }  // per thread
+
+// one element to shared memory behind the computation, zero where !ok
+template <typename S>
+__device__ __forceinline__ void cp_async(S *dst, const S *src, bool ok)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src),
+                 "n"((int)sizeof(S)), "r"(ok ? (int)sizeof(S) : 0)
+                 : "memory");
+}
+
+template <typename S, int LS>
+__global__ void __launch_bounds__(128, 3) k_nf_rows(const S *__restrict__ A, const int *__restrict__ colidx,
+                                                 const int *__restrict__ tiles, const PanelGPU *__restrict__ panels,
+                                                 const S *__restrict__ x, int ncolg, int Et, int nint,
+                                                 double *__restrict__ f, int nt, int kop, int R, NfHalfSplit hs)
+{
+    constexpr int BM = kNfRows, BK = nf_rows_bk(sizeof(S)), ND = 2 * LS, NV = nf_rows_intervals(LS);
+    constexpr bool kFloat = sizeof(S) == 4;
+    constexpr int AS = ND * BM + 16 / (int)sizeof(S);  // 16-byte rows; two-way conflicts of the stores at most
+    extern __shared__ __align__(16) unsigned char smem_nf[];
+    S *sm = reinterpret_cast<S *>(smem_nf);
+    const int stage = BK * (AS + R);
+    const int tid = threadIdx.x, nthr = blockDim.x;
+    const int tile = blockIdx.x / (kRowTile / BM);
+    const PanelGPU P = panels[tiles[2 * tile]];
+    const int r0 = tiles[2 * tile + 1] + blockIdx.x % (kRowTile / BM) * BM;
+    if (r0 >= P.nrows) return;
+    const int i0 = blockIdx.y * nthr * NV, rhs = blockIdx.z;
+    const S *xr = x + (size_t)rhs * Et * ncolg;
+    const int *cols = colidx + (kop ? P.colK_at : P.colV_at);
+    const int ncp = kop ? P.colsK_pad : P.colsV_pad;
+    const bool half = hs.parts != nullptr;  // FP32 only
+    const size_t off = kop ? P.offK : P.offV;
+    const __half *Hp = reinterpret_cast<const __half *>(hs.parts);
+    const int j_st = tid % BK, nstep = LS * min(nthr * NV + 1, nint - i0 + 1), t0 = (i0 - 1) * LS;
+    const bool active = i0 + (tid & ~31) < nint;
+    S acc[NV][LS][BM];
+    float sh[NV][LS][BM], sl[NV][LS][BM];  // FP32 only: sum and its rounding errors
+#pragma unroll
+    for (int v = 0; v < NV; ++v)
+#pragma unroll
+        for (int s = 0; s < LS; ++s)
+#pragma unroll
+            for (int r = 0; r < BM; ++r) {
+                acc[v][s][r] = S(0);
+                sh[v][s][r] = sl[v][s][r] = 0.f;
+            }
+    auto load = [&](int k0, S *As) {
+        S *Ws = As + BK * AS;
+        const int col = cols[k0 + j_st];
+        for (int e = tid / BK; e < ND * BM; e += nthr / BK) {
+            const int r = e % BM, d = e / BM;
+            if (half) {
+                S v = S(0);
+                if (r0 + r < P.nrows) {
+                    const __half *h = Hp + nf_split_index(P.row0 + r0 + r, d, k0 + j_st, ncp >> 5);
+                    v = S((__half2float(h[0]) + __half2float(h[kSplitPart])) * hs.inv_scale);
+                }
+                As[j_st * AS + e] = v;
+            } else {
+                cp_async(As + j_st * AS + e, A + off + ((size_t)d * P.rows_pad + r0 + r) * ncp + k0 + j_st, true);
+            }
+        }
+        const S *src = xr + max(col, 0);
+        for (int c = tid / BK; c < nstep; c += nthr / BK) {
+            const int t = t0 + c;
+            cp_async(Ws + j_st * R + c, src + (size_t)max(t, 0) * ncolg, col >= 0 && t >= 0);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    int ktiles = 0;
+    if (ncp > 0) load(0, sm);
+    for (int k0 = 0, b = 0; k0 < ncp; k0 += BK, b ^= 1) {
+        const S *As = sm + b * stage, *Ws = As + BK * AS;
+        if (k0 + BK < ncp) {
+            load(k0 + BK, sm + (b ^ 1) * stage);
+            asm volatile("cp.async.wait_group 1;" ::: "memory");
+        } else {
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
+        }
+        __syncthreads();
+        if (active) {
+#pragma unroll 2
+            for (int j = 0; j < BK; ++j) {
+                S w[NV][ND];
+#pragma unroll
+                for (int v = 0; v < NV; ++v) {
+                    const S *src = Ws + j * R + (tid + v * nthr) * LS;
+                    if (LS % 2 == 0) {
+                        using S2 = typename std::conditional<kFloat, float2, double2>::type;
+#pragma unroll
+                        for (int q = 0; q < ND / 2; ++q) {
+                            const S2 p = reinterpret_cast<const S2 *>(src)[q];
+                            w[v][2 * q] = p.x;
+                            w[v][2 * q + 1] = p.y;
+                        }
+                    } else {
+#pragma unroll
+                        for (int q = 0; q < ND; ++q) w[v][q] = src[q];
+                    }
+                }
+#pragma unroll
+                for (int d = 0; d < ND; ++d) {
+                    S a[BM];
+                    constexpr int NB = 16 / (int)sizeof(S);
+#pragma unroll
+                    for (int q = 0; q < BM / NB; ++q)
+                        *reinterpret_cast<uint4 *>(&a[q * NB]) = reinterpret_cast<const uint4 *>(As + j * AS + d * BM)[q];
+#pragma unroll
+                    for (int s = 0; s < LS; ++s) {
+                        if (d > LS + s) continue;
+#pragma unroll
+                        for (int v = 0; v < NV; ++v)
+#pragma unroll
+                            for (int r = 0; r < BM; ++r) acc[v][s][r] += a[r] * w[v][LS + s - d];
+                    }
+                }
+            }
+        }
+        __syncthreads();
+        if (kFloat && ++ktiles == 128 / (BK * ND)) {
+            ktiles = 0;
+#pragma unroll
+            for (int v = 0; v < NV; ++v)
+#pragma unroll
+                for (int s = 0; s < LS; ++s)
+#pragma unroll
+                    for (int r = 0; r < BM; ++r) {
+                        float e;
+                        df_two_sum(sh[v][s][r], (float)acc[v][s][r], sh[v][s][r], e);
+                        sl[v][s][r] += fabsf(sh[v][s][r]) <= 3.402823466e38f ? e : 0.f;  // an infinite sum stays one
+                        acc[v][s][r] = S(0);
+                    }
+        }
+    }
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+        const int iv = i0 + tid + v * nthr;
+        if (iv >= nint) continue;
+#pragma unroll
+        for (int s = 0; s < LS; ++s)
+#pragma unroll
+            for (int r = 0; r < BM; ++r)
+                if (r0 + r < P.nrows)
+                    f[((size_t)rhs * Et + iv * LS + s) * nt + P.row0 + r0 + r] = (double)sh[v][s][r] + ((double)sl[v][s][r] + (double)acc[v][s][r]);
+    }
+}
+
+template <typename S, int LS>
+static void launch_nf_rows(const S *A, bool kop, const int *colidx, const int *tiles, int ntiles, const PanelGPU *panels,
+                           const S *x, int ncolg, int nrhs, const ApplyGeo &g, double *f, const NfHalfSplit *hs,
+                           cudaStream_t st)
+{
+    constexpr int NV = nf_rows_intervals(LS);
+    const int nint = g.Et / LS, nthr = std::min(128, ((nint + NV - 1) / NV + 31) / 32 * 32);
+    // row stride 32 / BK mod 32: the staging stores (BK columns x 32 / BK steps a warp) meet every bank once
+    constexpr int BK = nf_rows_bk(sizeof(S));
+    const int R = (LS * (nthr * NV + 1) - 32 / BK + 31) / 32 * 32 + 32 / BK;
+    const size_t smem = 2 * sizeof(S) * BK * ((size_t)2 * LS * kNfRows + 16 / sizeof(S) + R);
+    cudaFuncSetAttribute(k_nf_rows<S, LS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const dim3 grd(ntiles * (kRowTile / kNfRows), (nint + nthr * NV - 1) / (nthr * NV), nrhs);
+    k_nf_rows<S, LS><<<grd, nthr, smem, st>>>(A, colidx, tiles, panels, x, ncolg, g.Et, nint, f, g.nt, kop ? 1 : 0, R,
+                                             hs ? *hs : NfHalfSplit{});
+}
+
+template <typename S>
+static bool launch_nf_rows_ls(const S *A, bool kop, const int *colidx, const int *tiles, int ntiles,
+                              const PanelGPU *panels, const S *x, int ncolg, int nrhs, const ApplyGeo &g, double *f,
+                              const NfHalfSplit *hs, cudaStream_t st)
+{
+    switch (g.ls) {
+    case 1: launch_nf_rows<S, 1>(A, kop, colidx, tiles, ntiles, panels, x, ncolg, nrhs, g, f, hs, st); return true;
+    case 2: launch_nf_rows<S, 2>(A, kop, colidx, tiles, ntiles, panels, x, ncolg, nrhs, g, f, hs, st); return true;
+    case 3: launch_nf_rows<S, 3>(A, kop, colidx, tiles, ntiles, panels, x, ncolg, nrhs, g, f, hs, st); return true;
+    case 4: launch_nf_rows<S, 4>(A, kop, colidx, tiles, ntiles, panels, x, ncolg, nrhs, g, f, hs, st); return true;
+    default: return false;
+    }
+}
+
 void launch_nf_apply(bool mixed, bool kop, const void *A, const int *colidx, const int *tiles, int ntiles,
                      const PanelGPU *panels, const void *x, int ncolg, int nrhs, const ApplyGeo &g, double *f_int,
                      cudaStream_t st, int ndmax, const NfHalfSplit *hs)
 {
+    // all offsets of up to four steps per leaf: k_nf_rows, at 4 to 90 rows a panel and 8 to 512 intervals
+    // never behind the 64 x 64 tiles (k_nf_rows has the figures)
+    if (ndmax >= 2 * g.ls) {
+        if (mixed ? launch_nf_rows_ls<float>((const float *)A, kop, colidx, tiles, ntiles, panels, (const float *)x, ncolg,
+                                             nrhs, g, f_int, hs, st)
+                  : launch_nf_rows_ls<double>((const double *)A, kop, colidx, tiles, ntiles, panels, (const double *)x,
+                                              ncolg, nrhs, g, f_int, nullptr, st))
+            return;
+    }
     int nint = g.Et / g.ls;
     dim3 grd(ntiles, g.ls * ((nint + 63) / 64), nrhs);
     if (mixed)
