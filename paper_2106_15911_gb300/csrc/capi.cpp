@@ -360,7 +360,7 @@ int pfmm::apply_same_step(pfmm_handle *H, const double *x, double *f, int ns, vo
     } else {
         NfHalfSplit hs;
         launch_nf_apply(H->mixed, false, H->nf_blocks(0), H->d_colV, H->d_tiles, H->ntiles, H->d_panels, xint, H->nt, 1, g,
-                        fint, st, 1, H->nf_split(0, &hs));
+                        fint, st, true, H->nf_split(0, &hs));
     }
     launch_permute_out(fint, f, 1, g, st);
     cudaError_t e = cudaGetLastError();
@@ -979,7 +979,7 @@ static int apply_impl(pfmm_handle *H, int op, const double *x, double *f, int nr
     } else if (parts & PFMM_PART_NEAR) {
         NfHalfSplit hs;
         launch_nf_apply(H->mixed, op == 1, H->nf_blocks(op), op == 0 ? H->d_colV : H->d_colK, H->d_tiles, H->ntiles,
-                        H->d_panels, xin, ncolg, nrhs, g, H->d_fint, st, 1 << 30, H->nf_split(op, &hs));
+                        H->d_panels, xin, ncolg, nrhs, g, H->d_fint, st, false, H->nf_split(op, &hs));
     } else {
         CK(cudaMemsetAsync(H->d_fint, 0, sizeof(double) * nrhs * (size_t)H->Et * H->nt, st));
     }

@@ -91,15 +91,13 @@ void launch_to_df64(double *x, size_t n, cudaStream_t st)
 // of uniform steps: for target step t = k*ls + s of leaf interval k the temporal nearfield
 // N(I_k) = {I_{k-1}, I_k} contributes the step offsets d = 0 .. ls + s, so
 //   f[t][rows of X] = sum_{d=0}^{ls+s} A_d[X] x[t - d][cols of X].
-// k_nf_apply, for a bounded number of offsets (the same-step block) or more than four steps per leaf:
-// one CTA computes a 64 x 64 tile (64 rows of a panel x 64 steps of one phase s) over all d
+// k_nf_apply, for more than four steps per leaf: one CTA computes a 64 x 64 tile (64 rows of a panel x 64 steps of one phase s) over all d
 // and all columns, so every output element is written exactly once.
 template <typename S>
 __global__ void __launch_bounds__(256) k_nf_apply(const S *__restrict__ A, const int *__restrict__ colidx,
                                                     const int *__restrict__ tiles, const PanelGPU *__restrict__ panels,
                                                     const S *__restrict__ x, int ncolg, int Et, int ls, int nint,
-                                                    double *__restrict__ f, int nt, int kop, int ndmax,
-                                                    NfHalfSplit hs)
+                                                    double *__restrict__ f, int nt, int kop)
 {
     constexpr int BM = 64, BN = 64, BK = 16;
     constexpr bool kFloat = sizeof(S) == 4;
@@ -114,9 +112,7 @@ __global__ void __launch_bounds__(256) k_nf_apply(const S *__restrict__ A, const
     const S *xr = x + (size_t)rhs * Et * ncolg;
     const int *cols = colidx + (kop ? P.colK_at : P.colV_at);
     const int ncp = kop ? P.colsK_pad : P.colsV_pad;
-    const bool half = hs.parts != nullptr;  // FP32 only
     const size_t off = kop ? P.offK : P.offV;
-    const __half *Hp = reinterpret_cast<const __half *>(hs.parts);
     S acc[4][4];
     double accd[4][4];
 #pragma unroll
@@ -126,7 +122,7 @@ __global__ void __launch_bounds__(256) k_nf_apply(const S *__restrict__ A, const
             acc[i][j] = S(0);
             accd[i][j] = 0.0;
         }
-    const int nd = min(ls + s + 1, ndmax);
+    const int nd = ls + s + 1;
     int ktiles = 0;
     for (int d = 0; d < nd; ++d) {
         const size_t dbase = off + ((size_t)d * P.rows_pad + r0) * ncp;
@@ -135,16 +131,7 @@ __global__ void __launch_bounds__(256) k_nf_apply(const S *__restrict__ A, const
             for (int q = 0; q < 4; ++q) {
                 int e = tid + 256 * q;
                 int i = e >> 4, j = e & 15;
-                if (half) {
-                    S v = S(0);
-                    if (r0 + i < P.nrows) {
-                        const __half *h = Hp + nf_split_index(P.row0 + r0 + i, d, k0 + j, ncp >> 5);
-                        v = S((__half2float(h[0]) + __half2float(h[kSplitPart])) * hs.inv_scale);
-                    }
-                    As[j][i] = v;
-                } else {
-                    As[j][i] = A[dbase + (size_t)i * ncp + k0 + j];
-                }
+                As[j][i] = A[dbase + (size_t)i * ncp + k0 + j];
                 int c = e >> 4;
                 int t = ((ib * BN + c) * ls + s);
                 int col = cols[k0 + j];
@@ -387,27 +374,149 @@ static bool launch_nf_rows_ls(const S *A, bool kop, const int *colidx, const int
     }
 }
 
+// f_b = A_0 x_b for ns independent slices (each its own step, offset 0 only).  CTA: 8 rows of a panel x 32
+// slices (lane = slice), the columns dealt to its four warps in groups of 16, each warp with its own two
+// stages and its sum of eight rows; the four sums are added in order.  Bound by the reads of x from L2 (every
+// 8 rows read all of it).  On 3072 triangles and 32 slices, FP16 parts:
+// 441 us in 64 x 64 tiles (56 CTAs, one loop over all columns each) -> 79 us.
+template <typename S>
+__global__ void __launch_bounds__(128) k_nf_same_step(const S *__restrict__ A, const int *__restrict__ colidx,
+                                                      const int *__restrict__ tiles, const PanelGPU *__restrict__ panels,
+                                                      const S *__restrict__ x, int ncolg, int ns, double *__restrict__ f,
+                                                      int nt, int kop, NfHalfSplit hs)
+{
+    constexpr int BM = kNfRows, BK = 16, R = 34, NB = 16 / (int)sizeof(S), AS = BM + NB;
+    constexpr bool kFloat = sizeof(S) == 4;
+    extern __shared__ __align__(16) unsigned char smem_ss[];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, tile = blockIdx.x / (kRowTile / BM);
+    S *sm = reinterpret_cast<S *>(smem_ss) + warp * 2 * BK * (R + AS);
+    const PanelGPU P = panels[tiles[2 * tile]];
+    const int r0 = tiles[2 * tile + 1] + blockIdx.x % (kRowTile / BM) * BM, b0 = blockIdx.y * 32;
+    if (r0 >= P.nrows) return;
+    const int *cols = colidx + (kop ? P.colK_at : P.colV_at);
+    const int ncp = kop ? P.colsK_pad : P.colsV_pad, nb = min(32, ns - b0);
+    const bool half = hs.parts != nullptr;  // FP32 only
+    const S *Ap = A + (kop ? P.offK : P.offV) + (size_t)r0 * ncp;
+    const int jc = lane & 15;
+    // FP16 parts: lane = (row, 8 of the 16 columns, part)
+    const int hr = lane >> 2, hc = (lane >> 1) & 1, hp = lane & 1;
+    auto load = [&](int k0, S *Ws, uint4 &h) {
+        if (half) {
+            h = make_uint4(0, 0, 0, 0);
+            if (r0 + hr < P.nrows)
+                h = *reinterpret_cast<const uint4 *>(hs.parts + nf_split_index(P.row0 + r0 + hr, 0, k0 + 8 * hc, ncp >> 5) +
+                                                     hp * kSplitPart);
+        } else {
+#pragma unroll
+            for (int q = 0; q < BM / 2; ++q)
+                cp_async(Ws + BK * R + jc * AS + (lane >> 4) + 2 * q, Ap + (size_t)((lane >> 4) + 2 * q) * ncp + k0 + jc, true);
+        }
+        const int col = cols[k0 + jc];
+        const S *src = x + (size_t)b0 * ncolg + max(col, 0);
+        for (int c = lane >> 4; c < nb; c += 2) cp_async(Ws + jc * R + c, src + (size_t)c * ncolg, col >= 0);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    S acc[BM];
+    float sh[BM], sl[BM];  // FP32 only: sum and its rounding errors
+#pragma unroll
+    for (int r = 0; r < BM; ++r) {
+        acc[r] = S(0);
+        sh[r] = sl[r] = 0.f;
+    }
+    uint4 h, hn;
+    int n = 0;
+    if (warp * BK < ncp) load(warp * BK, sm, h);
+    for (int k0 = warp * BK, b = 0; k0 < ncp; k0 += 4 * BK, b ^= 1) {
+        S *Ws = sm + b * BK * (R + AS), *As = Ws + BK * R;
+        if (k0 + 4 * BK < ncp) {
+            load(k0 + 4 * BK, sm + (b ^ 1) * BK * (R + AS), hn);
+            asm volatile("cp.async.wait_group 1;" ::: "memory");
+        } else {
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
+        }
+        if (half) {
+            const __half *v = reinterpret_cast<const __half *>(&h);
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                const float mine = __half2float(v[q]), sum = mine + __shfl_xor_sync(0xffffffffu, mine, 1);
+                if ((q >> 2) == hp) As[(8 * hc + q) * AS + hr] = S(sum * hs.inv_scale);
+            }
+            h = hn;
+        }
+        __syncwarp();
+#pragma unroll
+        for (int j = 0; j < BK; ++j) {
+            S a[BM];
+#pragma unroll
+            for (int q = 0; q < BM / NB; ++q)
+                *reinterpret_cast<uint4 *>(&a[q * NB]) = reinterpret_cast<const uint4 *>(As + j * AS)[q];
+            const S w = Ws[j * R + lane];
+#pragma unroll
+            for (int r = 0; r < BM; ++r) acc[r] += a[r] * w;
+        }
+        __syncwarp();
+        if (kFloat && ++n == 128 / BK) {
+            n = 0;
+#pragma unroll
+            for (int r = 0; r < BM; ++r) {
+                float e;
+                df_two_sum(sh[r], (float)acc[r], sh[r], e);
+                sl[r] += fabsf(sh[r]) <= 3.402823466e38f ? e : 0.f;  // an infinite sum stays one
+                acc[r] = S(0);
+            }
+        }
+    }
+    double *red = reinterpret_cast<double *>(smem_ss);  // [warp][row][lane]
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < BM; ++r) red[(warp * BM + r) * 32 + lane] = (double)sh[r] + ((double)sl[r] + (double)acc[r]);
+    __syncthreads();
+    for (int e = threadIdx.x; e < BM * nb; e += 128) {  // rows innermost: f is [slice][triangle]
+        const int r = e % BM, c = e / BM;
+        double v = red[r * 32 + c];
+        for (int w = 1; w < 4; ++w) v += red[(w * BM + r) * 32 + c];
+        if (r0 + r < P.nrows) f[(size_t)(b0 + c) * nt + P.row0 + r0 + r] = v;
+    }
+}
+
+template <typename S>
+static void launch_same_step(const S *A, bool kop, const int *colidx, const int *tiles, int ntiles, const PanelGPU *panels,
+                             const S *x, int ncolg, const ApplyGeo &g, double *f, const NfHalfSplit *hs, cudaStream_t st)
+{
+    constexpr size_t smem = std::max(sizeof(S) * 4 * 2 * 16 * (34 + kNfRows + 16 / sizeof(S)), sizeof(double) * 4 * kNfRows * 32);
+    cudaFuncSetAttribute(k_nf_same_step<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    k_nf_same_step<S><<<dim3(ntiles * (kRowTile / kNfRows), (g.Et + 31) / 32), 128, smem, st>>>(
+        A, colidx, tiles, panels, x, ncolg, g.Et, f, g.nt, kop ? 1 : 0, hs ? *hs : NfHalfSplit{});
+}
+
 void launch_nf_apply(bool mixed, bool kop, const void *A, const int *colidx, const int *tiles, int ntiles,
                      const PanelGPU *panels, const void *x, int ncolg, int nrhs, const ApplyGeo &g, double *f_int,
-                     cudaStream_t st, int ndmax, const NfHalfSplit *hs)
+                     cudaStream_t st, bool same_step, const NfHalfSplit *hs)
 {
-    // all offsets of up to four steps per leaf: k_nf_rows, at 4 to 90 rows a panel and 8 to 512 intervals
-    // never behind the 64 x 64 tiles (k_nf_rows has the figures)
-    if (ndmax >= 2 * g.ls) {
-        if (mixed ? launch_nf_rows_ls<float>((const float *)A, kop, colidx, tiles, ntiles, panels, (const float *)x, ncolg,
-                                             nrhs, g, f_int, hs, st)
-                  : launch_nf_rows_ls<double>((const double *)A, kop, colidx, tiles, ntiles, panels, (const double *)x,
-                                              ncolg, nrhs, g, f_int, nullptr, st))
-            return;
+    if (same_step) {
+        if (mixed)
+            launch_same_step<float>((const float *)A, kop, colidx, tiles, ntiles, panels, (const float *)x, ncolg, g, f_int,
+                                    hs, st);
+        else
+            launch_same_step<double>((const double *)A, kop, colidx, tiles, ntiles, panels, (const double *)x, ncolg, g,
+                                     f_int, nullptr, st);
+        return;
     }
+    // up to four steps per leaf: k_nf_rows, at 4 to 90 rows a panel and 8 to 512 intervals never behind the
+    // 64 x 64 tiles (k_nf_rows has the figures).  The FP16 parts exist at two steps per leaf only
+    if (mixed ? launch_nf_rows_ls<float>((const float *)A, kop, colidx, tiles, ntiles, panels, (const float *)x, ncolg, nrhs,
+                                         g, f_int, hs, st)
+              : launch_nf_rows_ls<double>((const double *)A, kop, colidx, tiles, ntiles, panels, (const double *)x, ncolg,
+                                          nrhs, g, f_int, nullptr, st))
+        return;
     int nint = g.Et / g.ls;
     dim3 grd(ntiles, g.ls * ((nint + 63) / 64), nrhs);
     if (mixed)
         k_nf_apply<float><<<grd, 256, 0, st>>>((const float *)A, colidx, tiles, panels, (const float *)x, ncolg, g.Et,
-                                               g.ls, nint, f_int, g.nt, kop ? 1 : 0, ndmax, hs ? *hs : NfHalfSplit{});
+                                               g.ls, nint, f_int, g.nt, kop ? 1 : 0);
     else
         k_nf_apply<double><<<grd, 256, 0, st>>>((const double *)A, colidx, tiles, panels, (const double *)x, ncolg,
-                                                g.Et, g.ls, nint, f_int, g.nt, kop ? 1 : 0, ndmax, NfHalfSplit{});
+                                                g.Et, g.ls, nint, f_int, g.nt, kop ? 1 : 0);
 }
 
 // ------------------------------------------------------------------------------------------

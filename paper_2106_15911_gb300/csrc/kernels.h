@@ -125,8 +125,9 @@ __host__ __device__ inline size_t nf_split_index(int x, int d, int c, int nkb)
 }
 void launch_nf_apply(bool mixed, bool kop, const void *A, const int *colidx, const int *tiles, int ntiles,
                      const PanelGPU *panels, const void *x, int ncolg, int nrhs, const ApplyGeo &g, double *f_int,
-                     cudaStream_t st, int ndmax = 1 << 30,  // ndmax: only offsets d < ndmax
-                     const NfHalfSplit *hs = nullptr);      // FP32 only: blocks from the FP16 parts, A unused
+                     cudaStream_t st,
+                     bool same_step = false,            // offset 0 only, each of the g.Et steps a slice of its own
+                     const NfHalfSplit *hs = nullptr);  // FP32 only: blocks from the FP16 parts, A unused
 // ws: scratch of ws_elems elements of the arithmetic type for the per-tile partial moments (the
 // M2L workspace, idle at this point); too small: one CTA per whole leaf box instead
 void launch_s2m(int prec, bool kop, const void *x, int ncolg, const void *Stab /*Sx or SK*/, const void *St,

@@ -147,7 +147,7 @@ extern "C" int pfmm_apply_V_noalloc(pfmm_handle *H, const double *w, double *f, 
     } else {
         NfHalfSplit hs;
         launch_nf_apply(H->mixed, false, H->nf_blocks(0), H->d_colV, H->d_tiles, H->ntiles, H->d_panels, xint, H->nt, nrhs,
-                        g, fint, st, 1 << 30, H->nf_split(0, &hs));
+                        g, fint, st, false, H->nf_split(0, &hs));
     }
     const int p = H->p;
     if (p >= 2) {

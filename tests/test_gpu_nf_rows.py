@@ -37,3 +37,26 @@ def test_nearfield_rows_match_oracle(precision, mesh, n_a, ls, nint, nrhs, c_st)
             ref = O.pfmm_apply(Pr, k, w[r], targets=rows, parts=P.PFMM_PART_NEAR)[:, rows]
             assert np.max(np.abs(out[r][:, rows] - ref)) <= tol * np.max(np.abs(ref))
     op.close()
+
+
+@pytest.mark.parametrize("ns", [1, 32, 33])  # one slice of a CTA's 32, all, and a second CTA
+@pytest.mark.parametrize("kw", [dict(precision=P.PFMM_MIXED, c_st=1.0),   # FP16 parts
+                                dict(precision=P.PFMM_MIXED, c_st=0.15, n_tr=1),  # FP32 panels of their own columns
+                                dict(precision=P.PFMM_FP64, c_st=0.15, n_tr=1)])
+def test_same_step_block_of_slices(kw, ns):
+    V, T = cube_mesh(4)
+    Et = 32
+    kw = dict(kw, m_t=2, m_x=2)
+    op = P.Operator(V, T, 1.0, Et, **kw)
+    otf = P.Operator(V, T, 1.0, Et, nearfield=P.PFMM_NEARFIELD_ONTHEFLY, **dict(kw, precision=P.PFMM_FP64))
+    net = P.Mpnn(V, T, 1.0, Et, width=16, layers=1, seed=1)
+    net.output_scale = 1.0
+    R = torch.tensor(random_density(Et, len(T), 2, seed=32), device=DEV)
+    sl = (np.arange(ns) * 7 % (2 * Et)).astype(np.int32)
+    l1, g1 = net.loss_grad(R, None, sl, handle=op.h)
+    l2, g2 = net.loss_grad(R, None, sl, handle=otf.h)
+    # the panels' FP32 rounding and FP32 sums enter the residual and its gradient
+    assert l1 == pytest.approx(l2, rel=1e-5)
+    assert np.max(np.abs(g1 - g2)) <= 1e-5 * np.max(np.abs(g2))
+    for h in (net, op, otf):
+        h.close()
