@@ -342,17 +342,29 @@ __global__ void __launch_bounds__(NTH) k_layer_bwd(const float *__restrict__ G1,
 }
 
 // layer backward, graph part: G0[i] += sum_{j in N(i)} U[j] (the adjacency is symmetric, so this
-// is the transpose of the neighbour mean)
+// is the transpose of the neighbour mean).  Four columns a thread, the neighbours' reads in flight
+// together (98304 rows of 64: 48 us with one column and one read at a time -> 17 us)
 __global__ void k_scatter_nbr(const float *__restrict__ U, float *__restrict__ G0, const int *__restrict__ adj_ptr,
                               const int *__restrict__ adj, int nt, int64_t rows, int W)
 {
     const int64_t gid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (gid >= rows * W) return;
-    const int64_t row = gid / W, base = row - row % nt;
-    const int k = (int)(gid % W), i = (int)(row % nt);
-    float s = 0.f;
-    for (int q = adj_ptr[i]; q < adj_ptr[i + 1]; ++q) s += U[(base + adj[q]) * W + k];
-    G0[gid] += s;
+    const int W4 = W / 4;
+    if (gid >= rows * W4) return;
+    const int64_t row = gid / W4;
+    const int i = (int)(row % nt), k = (int)(gid % W4) * 4, q1 = adj_ptr[i + 1];
+    const float *Un = U + (row - i) * W + k;
+    float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 4
+    for (int q = adj_ptr[i]; q < q1; ++q) {
+        const float4 u = *reinterpret_cast<const float4 *>(Un + (int64_t)adj[q] * W);
+        s.x += u.x;
+        s.y += u.y;
+        s.z += u.z;
+        s.w += u.w;
+    }
+    float4 *g = reinterpret_cast<float4 *>(G0 + row * W + k);
+    const float4 v = *g;
+    *g = make_float4(v.x + s.x, v.y + s.y, v.z + s.z, v.w + s.w);
 }
 
 // encoder backward: d loss / d (W_g^T f + b_g) = G0 (v / s) SiLU'(PRE)
@@ -365,7 +377,11 @@ __global__ void k_enc_bwd(const float *__restrict__ G, const float *__restrict__
 
 // weight gradients of one dense map:  Gw[k][o] += sum_rows IN[row][k] DP[row][o] for k < kvalid,
 // gb[o] += sum_rows DP[row][o] (gb nullable); IN = the first KA columns of A (row stride lda), or
-// [A | mean_N(A)] when nbr_mean
+// [A | mean_N(A)] when nbr_mean (KA = lda = W: rows of float4).  A thread owns 8 x 4 outputs (three 16-byte
+// reads from shared memory per 32 FMAs; one output a read bound the kernel to the reads), the rows of a tile
+// are dealt to the thread groups that this leaves, whose sums are added before they go to memory (as many
+// additions there as groups lost accuracy).  98304 rows of 128 x 64: 275 -> 79 us, the neighbours' rows from
+// L2 most of it; encoder 5 x 64: 21 us.
 template <int W>
 __global__ void __launch_bounds__(NTH) k_wgrad(const float *__restrict__ A, int lda, int KA, int kvalid, int nbr_mean,
                                                const int *__restrict__ adj_ptr, const int *__restrict__ adj,
@@ -373,56 +389,101 @@ __global__ void __launch_bounds__(NTH) k_wgrad(const float *__restrict__ A, int 
                                                const float *__restrict__ DP, int64_t rows, float *__restrict__ Gw,
                                                float *__restrict__ gb)
 {
-    constexpr int NRG = NTH / W, EPT = (2 * W + NRG - 1) / NRG;
+    constexpr int TK = 8, TO = 4, W4 = W / 4;
     extern __shared__ __align__(16) float sm[];
-    const int K = nbr_mean ? 2 * KA : KA;
+    const int KT = nbr_mean ? 2 * W / TK : (KA + TK - 1) / TK, K = KT * TK;  // zero past the last column
     float *in = sm;            // [RW][K]
     float *dp = sm + RW * K;   // [RW][W]
-    const int o = threadIdx.x % W, kg = threadIdx.x / W;
-    float acc[EPT];
+    const int tpt = KT * W4, ngrp = NTH / tpt, grp = threadIdx.x / tpt;
+    const int k0 = threadIdx.x % tpt / W4 * TK, o0 = threadIdx.x % W4 * TO;
+    float acc[TK][TO], accb[TO];
 #pragma unroll
-    for (int q = 0; q < EPT; ++q) acc[q] = 0.f;
-    float accb = 0.f;
+    for (int c = 0; c < TO; ++c) {
+        accb[c] = 0.f;
+#pragma unroll
+        for (int k = 0; k < TK; ++k) acc[k][c] = 0.f;
+    }
+    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
     for (int64_t r0 = (int64_t)blockIdx.x * RW; r0 < rows; r0 += (int64_t)gridDim.x * RW) {
         __syncthreads();
-        for (int e = threadIdx.x; e < RW * K; e += NTH) {
-            const int r = e / K, k = e % K;
-            const int64_t row = r0 + r;
-            float v = 0.f;
-            if (row < rows) {
-                if (k < KA) {
-                    v = A[row * lda + k];
-                } else {
-                    const int kk = k - KA;
-                    const int64_t base = row - row % nt;
+        if (nbr_mean) {
+            for (int e = threadIdx.x; e < RW * W4; e += NTH) {
+                const int r = e / W4, k = e % W4;
+                const int64_t row = r0 + r;
+                float4 v = zero, m = zero;
+                if (row < rows) {
+                    v = reinterpret_cast<const float4 *>(A + row * W)[k];
                     const int i = (int)(row % nt);
-                    for (int q = adj_ptr[i]; q < adj_ptr[i + 1]; ++q) v += A[(base + adj[q]) * lda + kk];
-                    v *= deg_inv[i];
+                    const float *An = A + (row - i) * W + 4 * k;
+                    const int q1 = adj_ptr[i + 1];
+#pragma unroll 4
+                    for (int q = adj_ptr[i]; q < q1; ++q) {
+                        const float4 n = *reinterpret_cast<const float4 *>(An + (int64_t)adj[q] * W);
+                        m.x += n.x;
+                        m.y += n.y;
+                        m.z += n.z;
+                        m.w += n.w;
+                    }
+                    const float d = deg_inv[i];
+                    m = make_float4(m.x * d, m.y * d, m.z * d, m.w * d);
                 }
+                reinterpret_cast<float4 *>(in + r * K)[k] = v;
+                reinterpret_cast<float4 *>(in + r * K + W)[k] = m;
             }
-            in[e] = v;
+        } else {
+            for (int e = threadIdx.x; e < RW * K; e += NTH) {
+                const int64_t row = r0 + e / K;
+                const int k = e % K;
+                in[e] = row < rows && k < KA ? A[row * lda + k] : 0.f;
+            }
         }
-        for (int e = threadIdx.x; e < RW * W; e += NTH) {
-            const int64_t row = r0 + e / W;
-            dp[e] = row < rows ? DP[row * W + e % W] : 0.f;
+        for (int e = threadIdx.x; e < RW * W4; e += NTH)
+            reinterpret_cast<float4 *>(dp)[e] = r0 + e / W4 < rows ? reinterpret_cast<const float4 *>(DP + r0 * W)[e] : zero;
+        __syncthreads();
+        if (grp < ngrp)
+            for (int r = grp; r < RW; r += ngrp) {
+                const float4 d = *reinterpret_cast<const float4 *>(dp + r * W + o0);
+                float a[TK];
+                *reinterpret_cast<float4 *>(a) = *reinterpret_cast<const float4 *>(in + r * K + k0);
+                *reinterpret_cast<float4 *>(a + 4) = *reinterpret_cast<const float4 *>(in + r * K + k0 + 4);
+#pragma unroll
+                for (int k = 0; k < TK; ++k) {
+                    acc[k][0] += a[k] * d.x;
+                    acc[k][1] += a[k] * d.y;
+                    acc[k][2] += a[k] * d.z;
+                    acc[k][3] += a[k] * d.w;
+                }
+                accb[0] += d.x;
+                accb[1] += d.y;
+                accb[2] += d.z;
+                accb[3] += d.w;
+            }
+    }
+    if (ngrp > 1) {  // the groups' sums first: one addition per CTA and output in memory
+        for (int g = 0; g < ngrp; ++g) {
+            __syncthreads();
+            if (grp != g) continue;
+            float *w = sm + k0 * W + o0, *wb = sm + K * W + o0;
+#pragma unroll
+            for (int c = 0; c < TO; ++c) {
+#pragma unroll
+                for (int k = 0; k < TK; ++k) w[k * W + c] = g == 0 ? acc[k][c] : w[k * W + c] + acc[k][c];
+                if (k0 == 0) wb[c] = g == 0 ? accb[c] : wb[c] + accb[c];
+            }
         }
         __syncthreads();
-        for (int r = 0; r < RW; ++r) {
-            const float d = dp[r * W + o];
-#pragma unroll
-            for (int q = 0; q < EPT; ++q) {
-                const int k = kg + NRG * q;
-                if (k < K) acc[q] += in[r * K + k] * d;
-            }
-            accb += d;
-        }
+        for (int e = threadIdx.x; e < kvalid * W; e += NTH) atomicAdd(&Gw[e], sm[e]);
+        if (gb && threadIdx.x < W) atomicAdd(&gb[threadIdx.x], sm[K * W + threadIdx.x]);
+        return;
     }
 #pragma unroll
-    for (int q = 0; q < EPT; ++q) {
-        const int k = kg + NRG * q;
-        if (k < kvalid) atomicAdd(&Gw[k * W + o], acc[q]);
-    }
-    if (gb && kg == 0) atomicAdd(&gb[o], accb);
+    for (int k = 0; k < TK; ++k)
+        if (k0 + k < kvalid)
+#pragma unroll
+            for (int c = 0; c < TO; ++c) atomicAdd(&Gw[(k0 + k) * W + o0 + c], acc[k][c]);
+    if (gb && k0 == 0)
+#pragma unroll
+        for (int c = 0; c < TO; ++c) atomicAdd(&gb[o0 + c], accb[c]);
 }
 
 __global__ void k_adam(float *__restrict__ p, float *__restrict__ m, float *__restrict__ v, const float *__restrict__ g,
@@ -830,7 +891,7 @@ void launch_backward(pfmm_mpnn *N, int64_t rows, cudaStream_t st)
                                                             N->p16 + N->off_layer(l));
         k_wgrad<W><<<gw, NTH, smem_w, st>>>(Hl, W, W, 2 * W, 1, N->adj_ptr, N->adj, N->deg_inv, N->nt, Gup, rows,
                                             N->grad + N->off_layer(l), nullptr);
-        k_scatter_nbr<<<nblk(rows * W), 256, 0, st>>>(N->U, Gdn, N->adj_ptr, N->adj, N->nt, rows, W);
+        k_scatter_nbr<<<nblk(rows * (W / 4)), 256, 0, st>>>(N->U, Gdn, N->adj_ptr, N->adj, N->nt, rows, W);
         std::swap(Gup, Gdn);
     }
     k_enc_bwd<<<nblk(rows * W), 256, 0, st>>>(Gup, N->PRE, N->X, W, rows * W, N->DP);
