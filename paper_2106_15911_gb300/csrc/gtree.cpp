@@ -107,6 +107,7 @@ struct pfmm_gen {
     std::vector<int> leaves_all, leaves_far, m2l_targets;
     std::vector<std::vector<int>> parents_lv, all_lv;  // non-leaf boxes / all boxes of each level (global ids)
     int64_t n_m2l_pairs = 0, n_blocks = 0, nf_entries = 0;
+    int nf_groups = 0;  // most groups of 32 target elements of a leaf
     // device
     std::vector<void *> allocs;
     int64_t dev_bytes = 0;
@@ -517,6 +518,10 @@ int build_impl(pfmm_gen *h, const pfmm_mesh &m, const double *ts_host, cudaStrea
                 kidx.insert(kidx.end(), {a, b, c});
             }
     h->nk = (int)kidx.size() / 3;
+    for (int b : h->leaves_all) {
+        const GBox &B = h->boxes[b];
+        h->nf_groups = std::max(h->nf_groups, ((B.t1 - B.t0) * (B.a1 - B.a0) + 31) / 32);
+    }
     std::vector<double> verts(m.vertices, m.vertices + 3 * (size_t)m.n_vertices), tsv(ts_host, ts_host + E + 1);
     double *d_verts = nullptr, *d_ts = nullptr;
     if ((rc = h->upload(&h->d_box, h->boxes, st)) || (rc = h->upload(&h->d_perm, perm, st)) ||
@@ -757,7 +762,7 @@ int pfmm_gen_apply_V(pfmm_gen *h, const double *w, double *f, int32_t nrhs, int3
     launch_gen_permute_in(w, h->d_wint, h->d_perm, h->nt, rows, st);
     if (parts & PFMM_PART_NEAR)
         launch_gen_nf_apply(h->d_box, h->d_leaves_all, (int)h->leaves_all.size(), h->d_nptr, h->d_blocks, h->d_A,
-                            h->d_wint, h->d_fint, h->nt, h->Et, nrhs, st);
+                            h->d_wint, h->d_fint, h->nt, h->Et, nrhs, h->nf_groups, st);
     else if (cudaMemsetAsync(h->d_fint, 0, sizeof(double) * rows * (size_t)h->nt, st) != cudaSuccess)
         return fail(PFMM_ERR_CUDA, "cudaMemsetAsync failed");
     if ((parts & PFMM_PART_FAR) && h->nlev >= 3) {

@@ -71,7 +71,7 @@ void launch_gen_permute_in(const double *w, double *w_int, const int *perm, int 
 void launch_gen_permute_out(const double *f_int, double *f, const int *perm, int nt, int rows, cudaStream_t st);
 void launch_gen_nf_apply(const GBox *box, const int *leaves, int nleaves, const int *nptr, const GNear *blocks,
                          const double *A, const double *w_int, double *f_int, int nt, int Et, int nrhs,
-                         cudaStream_t st);
+                         int ngroups, cudaStream_t st);  // ngroups: most groups of 32 target elements of a leaf
 void launch_gen_s2m(const GenDev &g, const int *leaves, int n, const double *w_int, cudaStream_t st);
 // M2M of the parents of one level: the children (all boxes of the next level) write their
 // contributions into contrib ([nrhs][boxes][na][nk]), the parents add them in child order

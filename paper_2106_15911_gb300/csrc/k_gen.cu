@@ -202,8 +202,10 @@ void launch_gen_permute_out(const double *f_int, double *f, const int *perm, int
 
 // f_int[r][k][x] = sum over the blocks of the leaf of A[jj][y][kk][x] w_int[r][j][y] (entries with
 // j > k are stored as zeros).  The target elements e = kk ntx + x of the leaf go 32 at a time to the
-// lanes; the 8 warps of the CTA take every 8th source column (jj, y) of the leaf's blocks (the
-// column's 32 entries are one coalesced load) and their partial sums are added in warp order.
+// lanes of a CTA each (grid y); its 8 warps take every 8th source column (jj, y) of the leaf's blocks
+// (the column's 32 entries are one coalesced load) and their partial sums are added in warp order.
+// Bound by the latency of the entries' loads: 768 triangles x 32 graded steps, 453 MB: 1179 us with a CTA per leaf,
+// which went through its groups one after the other, -> 207 us (2.2 TB/s)
 constexpr int kGenNfWarps = 8;
 template <int R>
 __global__ void __launch_bounds__(32 * kGenNfWarps) k_gen_nf_apply(const GBox *__restrict__ box,
@@ -220,53 +222,51 @@ __global__ void __launch_bounds__(32 * kGenNfWarps) k_gen_nf_apply(const GBox *_
     const int ntx = T.t1 - T.t0, ne = ntx * (T.a1 - T.a0);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const size_t per_rhs = (size_t)Et * nt;
-    for (int e0 = 0; e0 < ne; e0 += 32) {
-        const int e = e0 + lane;
-        const bool valid = e < ne;
-        double acc[R];
+    const int e = blockIdx.y * 32 + lane;
+    if (blockIdx.y * 32 >= ne) return;
+    const bool valid = e < ne;
+    double acc[R];
 #pragma unroll
-        for (int r = 0; r < R; ++r) acc[r] = 0.0;
-        for (int q = nptr[b]; q < nptr[b + 1]; ++q) {
-            const GNear B = blocks[q];
-            const GBox S = box[B.src];
-            const int nys = S.t1 - S.t0, ncol = nys * (S.a1 - S.a0);
-            const double *Ab = A + B.off + (valid ? e : 0);
-            const double *w0 = w_int + (size_t)r0 * per_rhs + (size_t)S.a0 * nt + S.t0;
-            int jj = warp / nys, y = warp - jj * nys;  // column c = jj nys + y, advanced by kGenNfWarps
-#pragma unroll 4
-            for (int c = warp; c < ncol; c += kGenNfWarps) {
-                const double a = valid ? Ab[(size_t)c * ne] : 0.0;
-                const double *wj = w0 + (size_t)jj * nt + y;
+    for (int r = 0; r < R; ++r) acc[r] = 0.0;
+    for (int q = nptr[b]; q < nptr[b + 1]; ++q) {
+        const GNear B = blocks[q];
+        const GBox S = box[B.src];
+        const int nys = S.t1 - S.t0, ncol = nys * (S.a1 - S.a0);
+        const double *Ab = A + B.off + (valid ? e : 0);
+        const double *w0 = w_int + (size_t)r0 * per_rhs + (size_t)S.a0 * nt + S.t0;
+        int jj = warp / nys, y = warp - jj * nys;  // column c = jj nys + y, advanced by kGenNfWarps
+#pragma unroll 8
+        for (int c = warp; c < ncol; c += kGenNfWarps) {
+            const double a = valid ? Ab[(size_t)c * ne] : 0.0;
+            const double *wj = w0 + (size_t)jj * nt + y;
 #pragma unroll
-                for (int r = 0; r < R; ++r) acc[r] = fma(a, wj[(size_t)r * per_rhs], acc[r]);
-                y += kGenNfWarps;
-                while (y >= nys) {
-                    y -= nys;
-                    ++jj;
-                }
+            for (int r = 0; r < R; ++r) acc[r] = fma(a, wj[(size_t)r * per_rhs], acc[r]);
+            y += kGenNfWarps;
+            while (y >= nys) {
+                y -= nys;
+                ++jj;
             }
         }
+    }
 #pragma unroll
-        for (int r = 0; r < R; ++r) red[warp][r][lane] = acc[r];
-        __syncthreads();
-        if (warp == 0 && valid) {
-            const int kk = e / ntx, x = e - kk * ntx;
-            for (int r = 0; r < R; ++r) {
-                double s = 0.0;
-                for (int w = 0; w < kGenNfWarps; ++w) s += red[w][r][lane];
-                f_int[(size_t)(r0 + r) * per_rhs + (size_t)(T.a0 + kk) * nt + T.t0 + x] = s;
-            }
+    for (int r = 0; r < R; ++r) red[warp][r][lane] = acc[r];
+    __syncthreads();
+    if (warp == 0 && valid) {
+        const int kk = e / ntx, x = e - kk * ntx;
+        for (int r = 0; r < R; ++r) {
+            double s = 0.0;
+            for (int w = 0; w < kGenNfWarps; ++w) s += red[w][r][lane];
+            f_int[(size_t)(r0 + r) * per_rhs + (size_t)(T.a0 + kk) * nt + T.t0 + x] = s;
         }
-        __syncthreads();
     }
 }
 
 void launch_gen_nf_apply(const GBox *box, const int *leaves, int nleaves, const int *nptr, const GNear *blocks,
                          const double *A, const double *w_int, double *f_int, int nt, int Et, int nrhs,
-                         cudaStream_t st)
+                         int ngroups, cudaStream_t st)
 {
     if (nleaves <= 0) return;
-    const dim3 grid(nleaves), blk(32 * kGenNfWarps);
+    const dim3 grid(nleaves, ngroups), blk(32 * kGenNfWarps);
     for (int r0 = 0; r0 < nrhs;) {
         const int n = nrhs - r0;
         if (n >= 4) {
@@ -312,7 +312,9 @@ void launch_gen_s2m(const GenDev &g, const int *leaves, int n, const double *w_i
 // M2M in two launches per level, deterministic: each child Z_c writes its contribution
 //   contrib(Z_c)[ap][nu] = sum_ac q^(t)_{ac,ap} (sum_{kappa <= nu} q^(x)_{kappa,nu} mu(Z_c)[ac][kappa])
 // (Eq. st_m2m; Eq. temp_m2m when refined in time only: kappa = nu), one CTA per child with its moments
-// staged as dense cubes [ac][m1^3] and the 1D factors applied one direction at a time; then every
+// staged as dense cubes [ap][m1^3] at the parent's time nodes (the temporal factor first: the spatial sums
+// then run once per parent node, not once per pair of nodes; 53 -> 15 us a level on 768 triangles x 32 graded
+// steps) and the 1D factors applied one direction at a time; then every
 // parent adds its children's contributions in child order.
 constexpr int kGenPassThreads = 256;
 __global__ void __launch_bounds__(kGenPassThreads) k_gen_m2m_child(GenDev g, const int *__restrict__ children,
@@ -320,7 +322,7 @@ __global__ void __launch_bounds__(kGenPassThreads) k_gen_m2m_child(GenDev g, con
 {
     extern __shared__ double sm[];
     const int na = g.na, nk = g.nk, m1 = g.mx + 1, m3 = m1 * m1 * m1;
-    double *sc = sm;  // [na][m1^3]
+    double *sc = sm;  // [na][m1^3], at the parent's time nodes
     const int c = children[blockIdx.x];
     const GBox C = g.box[c];
     const int st = g.lvst[C.level];
@@ -332,35 +334,33 @@ __global__ void __launch_bounds__(kGenPassThreads) k_gen_m2m_child(GenDev g, con
         __syncthreads();
         for (int i = threadIdx.x; i < na * nk; i += blockDim.x) {
             const int a = i / nk, ik = i - a * nk;
-            sc[a * m3 + (g.kidx[3 * ik] * m1 + g.kidx[3 * ik + 1]) * m1 + g.kidx[3 * ik + 2]] =
-                g.mu[gidx(g, r, c, 0, 0) + i];
+            const double *mu = g.mu + gidx(g, r, c, 0, 0) + ik;
+            double v = 0.0;
+            for (int ac = 0; ac < na; ++ac) v += qtc[ac * na + a] * mu[(size_t)ac * nk];
+            sc[a * m3 + (g.kidx[3 * ik] * m1 + g.kidx[3 * ik + 1]) * m1 + g.kidx[3 * ik + 2]] = v;
         }
         __syncthreads();
         for (int t = threadIdx.x; t < na * nk; t += blockDim.x) {
             const int ap = t / nk, iv = t - ap * nk;
             const int n0 = g.kidx[3 * iv], n1 = g.kidx[3 * iv + 1], n2 = g.kidx[3 * iv + 2];
-            double sum = 0.0;
-            for (int ac = 0; ac < na; ++ac) {
-                const double *cube = sc + ac * m3;
-                double v;
-                if (!st) {
-                    v = cube[(n0 * m1 + n1) * m1 + n2];
-                } else {
-                    v = 0.0;
-                    for (int k0 = 0; k0 <= n0; ++k0) {
-                        double v1 = 0.0;
-                        for (int k1 = 0; k1 <= n1; ++k1) {
-                            const double *row = cube + (k0 * m1 + k1) * m1;
-                            double v2 = 0.0;
-                            for (int k2 = 0; k2 <= n2; ++k2) v2 += qc[k2 * m1 + n2] * row[k2];
-                            v1 += qb[k1 * m1 + n1] * v2;
-                        }
-                        v += qa[k0 * m1 + n0] * v1;
+            const double *cube = sc + ap * m3;
+            double v;
+            if (!st) {
+                v = cube[(n0 * m1 + n1) * m1 + n2];
+            } else {
+                v = 0.0;
+                for (int k0 = 0; k0 <= n0; ++k0) {
+                    double v1 = 0.0;
+                    for (int k1 = 0; k1 <= n1; ++k1) {
+                        const double *row = cube + (k0 * m1 + k1) * m1;
+                        double v2 = 0.0;
+                        for (int k2 = 0; k2 <= n2; ++k2) v2 += qc[k2 * m1 + n2] * row[k2];
+                        v1 += qb[k1 * m1 + n1] * v2;
                     }
+                    v += qa[k0 * m1 + n0] * v1;
                 }
-                sum += qtc[ac * na + ap] * v;
             }
-            contrib[gidx(g, r, c, 0, 0) + t] = sum;
+            contrib[gidx(g, r, c, 0, 0) + t] = v;
         }
     }
 }
@@ -533,7 +533,7 @@ __global__ void __launch_bounds__(kGenPassThreads) k_gen_l2l(GenDev g, const int
 {
     extern __shared__ double sm[];
     const int na = g.na, nk = g.nk, m1 = g.mx + 1, m3 = m1 * m1 * m1;
-    double *sp = sm;  // [na][m1^3]
+    double *sp = sm;  // [na][m1^3], at the child's time nodes
     const int bc = children[blockIdx.x];
     const GBox C = g.box[bc];
     const int st = g.lvst[C.level], bp = C.par;
@@ -545,35 +545,33 @@ __global__ void __launch_bounds__(kGenPassThreads) k_gen_l2l(GenDev g, const int
         __syncthreads();
         for (int i = threadIdx.x; i < na * nk; i += blockDim.x) {
             const int a = i / nk, ik = i - a * nk;
-            sp[a * m3 + (g.kidx[3 * ik] * m1 + g.kidx[3 * ik + 1]) * m1 + g.kidx[3 * ik + 2]] =
-                g.lam[gidx(g, r, bp, 0, 0) + i];
+            const double *lam = g.lam + gidx(g, r, bp, 0, 0) + ik;
+            double v = 0.0;
+            for (int bpI = 0; bpI < na; ++bpI) v += qtc[a * na + bpI] * lam[(size_t)bpI * nk];
+            sp[a * m3 + (g.kidx[3 * ik] * m1 + g.kidx[3 * ik + 1]) * m1 + g.kidx[3 * ik + 2]] = v;
         }
         __syncthreads();
         for (int t = threadIdx.x; t < na * nk; t += blockDim.x) {
             const int bcI = t / nk, ik = t - bcI * nk;
             const int k0 = g.kidx[3 * ik], k1 = g.kidx[3 * ik + 1], k2 = g.kidx[3 * ik + 2];
-            double acc = 0.0;
-            for (int bpI = 0; bpI < na; ++bpI) {
-                const double *cube = sp + bpI * m3;
-                double v;
-                if (!st) {
-                    v = cube[(k0 * m1 + k1) * m1 + k2];
-                } else {
-                    v = 0.0;
-                    for (int n0 = k0; n0 <= g.mx; ++n0) {
-                        double v1 = 0.0;
-                        for (int n1 = k1; n0 + n1 <= g.mx; ++n1) {
-                            const double *row = cube + (n0 * m1 + n1) * m1;
-                            double v2 = 0.0;
-                            for (int n2 = k2; n0 + n1 + n2 <= g.mx; ++n2) v2 += qc[k2 * m1 + n2] * row[n2];
-                            v1 += qb[k1 * m1 + n1] * v2;
-                        }
-                        v += qa[k0 * m1 + n0] * v1;
+            const double *cube = sp + bcI * m3;
+            double v;
+            if (!st) {
+                v = cube[(k0 * m1 + k1) * m1 + k2];
+            } else {
+                v = 0.0;
+                for (int n0 = k0; n0 <= g.mx; ++n0) {
+                    double v1 = 0.0;
+                    for (int n1 = k1; n0 + n1 <= g.mx; ++n1) {
+                        const double *row = cube + (n0 * m1 + n1) * m1;
+                        double v2 = 0.0;
+                        for (int n2 = k2; n0 + n1 + n2 <= g.mx; ++n2) v2 += qc[k2 * m1 + n2] * row[n2];
+                        v1 += qb[k1 * m1 + n1] * v2;
                     }
+                    v += qa[k0 * m1 + n0] * v1;
                 }
-                acc += qtc[bcI * na + bpI] * v;
             }
-            g.lam[gidx(g, r, bc, bcI, ik)] += acc;
+            g.lam[gidx(g, r, bc, bcI, ik)] += v;
         }
     }
 }
