@@ -31,13 +31,21 @@ ROOT = os.path.dirname(os.path.abspath(__file__))
 sys.path.insert(0, ROOT)
 
 METRIC = "pFMM matvec space-time DOF/s"
-# DRAM bytes (read + write) per stored nearfield element of one FP64 residue-arithmetic nearfield
-# launch (k_nf_apply_crt, form 1), from an ncu capture of the 3072-triangle x 256-step case
-# (1.7167e9 B read + 1.18e7 B written over 50,331,648 stored elements); traffic grows with the
-# stored elements, so a full launch's traffic is this times its element count
-NF_CRT_DRAM_BYTES_PER_ELEMENT = (1.716715e9 + 1.1788e7) / 50331648
-NF_CRT_TRAFFIC_SOURCE = ("ncu capture of 3072 tri x 256 steps (profiles/nf_crt_3072x256_fp64.md), scaled by the "
+# DRAM bytes (read + write) per residue-form element of one FP64 residue-arithmetic nearfield launch
+# (k_nf_apply_crt, form 1), from an ncu capture of the 3072-triangle x 256-step case (6.326e8 B read
+# + 1.26e7 B written over 3072 rows x 3072 columns x 4 offsets); traffic grows with the elements, so a
+# full launch's traffic is this times its element count
+NF_CRT_DRAM_BYTES_PER_ELEMENT = (6.326149e8 + 1.259e7) / 37748736
+NF_CRT_TRAFFIC_SOURCE = ("ncu capture of 3072 tri x 256 steps (profiles/nf_crt_bytes_3072x256_fp64.md), scaled by the "
                          "stored elements")
+
+
+def nf_residue_elements(nt, ls=2):
+    """Elements the residue form stores for V: rows in tiles of 128 triangles, columns in blocks of 64,
+    2 ls step offsets; 16 residue bytes each."""
+    return -(-nt // 128) * 128 * (-(-nt // 64) * 64) * 2 * ls
+
+
 N_A, ET, M_X, M_T, C_ST = 32, 256, 6, 4, 1.0
 
 
@@ -167,7 +175,7 @@ def phase_rooflines(phases, info, es, nt, Et, mx, mt, peaks, arith=None):
     nearfield: 2 sum_t |D(t)| nnz(A_d) flops on the stored elements.  arith: "fp32" (mixed mode),
     "df64" (FP64 mode: passes in double-FP32 on the FP32 pipe, peak = FP32 rate /
     DF64_FP32_OPS_PER_MAC; nearfield as residue products on the tensor cores where the handle
-    has them, 32 B per stored element) or "fp64" (native FP64 on the FP64 pipe); default from es.
+    has them, info's nf_residue_bytes or else 32 B per stored element) or "fp64" (native FP64 on the FP64 pipe); default from es.
     peaks: hbm_gbs, fp64_tflops, fp32_tflops, fp16_tflops."""
     from math import comb
 
@@ -207,8 +215,8 @@ def phase_rooflines(phases, info, es, nt, Et, mx, mt, peaks, arith=None):
     if tc and arith == "fp32":  # scaled FP16 hi / lo parts: 4 B per element, 3 FP16 products
         put("nearfield", nf_flops, nel * 4 + 16.0 * dof, phases.get("nearfield"), peaks["fp16_tflops"] / 3,
             "FP16 tensor peak / 3 (hi / lo products)")
-    elif tc and arith == "df64":  # residues modulo 16 primes: 32 B per element, 16 FP16 products
-        put("nearfield", nf_flops, nel * 32 + 48.0 * dof, phases.get("nearfield"), peaks["fp16_tflops"] / 16,
+    elif tc and arith == "df64":  # residues modulo 16 primes, 16 FP16 products
+        put("nearfield", nf_flops, info.get("nf_residue_bytes", nel * 32) + 48.0 * dof, phases.get("nearfield"), peaks["fp16_tflops"] / 16,
             "FP16 tensor peak / 16 (residue products)")
     else:
         put("nearfield", nf_flops, nel * es + 16.0 * dof, phases.get("nearfield"), peaks["fp64_tflops"] if es == 8
@@ -893,6 +901,8 @@ def main():
     # ---- rooflines: every phase from its algorithmic work; the dominant kernel is the nearfield
     peaks = _peaks(P, stream)
     es = 8 if head == P.PFMM_FP64 else 4
+    if head == P.PFMM_FP64:
+        info = dict(info, nf_residue_bytes=16.0 * nf_residue_elements(nt))
     rl = phase_rooflines(phases, info, es, nt, ET, M_X, M_T, peaks, arith="df64" if head == P.PFMM_FP64 else "fp32")
     nf = rl["nearfield"]
     tc = head == P.PFMM_MIXED and bool(info["nf_tensor_cores"] & 1)
@@ -904,16 +914,21 @@ def main():
                else "the nearfield phase (kernel events unavailable)")
     if crt:
         # FP64 nearfield as exact residue products on the tensor cores: 16 FP16 products per
-        # product of the method; per launch the kernel reads 16 FP16 residues (32 bytes) per stored
-        # element and per input value, and writes 16 one-byte output residues per output value
-        nel = info["nearfield_v_elements"]
-        byts = 32.0 * nel + 48.0 * dof
+        # product of the method; per launch the kernel reads 16 one-byte residues per stored element and 16
+        # FP16 residues per input value, and writes 16 one-byte output residues per output value
+        nel = nf_residue_elements(nt)
+        byts = 16.0 * nel + 48.0 * dof
         gbs = byts / (kms * 1e-3) / 1e9
-        executed = 16.0 * nf["flops"] / (kms * 1e-3) / 1e12
-        roofline = {"bound": "hbm", "kernel": "k_nf_apply_crt", "achieved": gbs, "peak": peaks["hbm_gbs"],
-                    "unit": "GB/s", "frac": gbs / peaks["hbm_gbs"],
+        executed = 16.0 * 2.0 * nt * nt * (ET // 2) * 7 / (kms * 1e-3) / 1e12
+        tensor = executed / peaks["fp16_tflops"] >= gbs / peaks["hbm_gbs"]
+        roofline = {"bound": "tensor" if tensor else "hbm", "kernel": "k_nf_apply_crt",
+                    "achieved": executed if tensor else gbs,
+                    "peak": peaks["fp16_tflops"] if tensor else peaks["hbm_gbs"],
+                    "unit": "TFLOP/s" if tensor else "GB/s",
+                    "frac": max(executed / peaks["fp16_tflops"], gbs / peaks["hbm_gbs"]),
+                    "hbm": {"achieved_gbs": gbs, "frac_of_copy_rate": gbs / peaks["hbm_gbs"]},
                     "traffic": NF_CRT_DRAM_BYTES_PER_ELEMENT * nel, "traffic_source": NF_CRT_TRAFFIC_SOURCE,
-                    "peak_source": "measured copy rate (of measured)", "bytes_per_launch": byts,
+                    "peak_source": "measured (of measured)", "bytes_per_launch": byts,
                     "ms_per_launch": kms, "timing": ktiming, "nearfield_phase_ms": nf["ms"],
                     "tensor": {"executed_fp16_tflops": executed, "frac_of_fp16_peak": executed / peaks["fp16_tflops"]},
                     "method_fp64_tflops": nf["flops"] / (kms * 1e-3) / 1e12, "fp64_pipe_tflops": peaks["fp64_tflops"]}
@@ -926,7 +941,7 @@ def main():
                     "ms_per_launch": kms, "timing": ktiming, "nearfield_phase_ms": nf["ms"],
                     "tensor": {"algorithmic_tflops": tfl, "frac_of_fp16_peak": tfl / peaks["fp16_tflops"]}}
     else:
-        roofline = {"bound": "alu", "kernel": "k_nf_apply<double>" if es == 8 else "k_nf_apply<float>",
+        roofline = {"bound": "alu", "kernel": "k_nf_rows<double>" if es == 8 else "k_nf_rows<float>",
                     "achieved": nf["tflops"], "peak": peaks["fp64_tflops"] if es == 8 else peaks["fp32_tflops"],
                     "unit": "TFLOP/s", "frac": nf["frac_fp"], "traffic": None,
                     "peak_source": "FMA rate measured in this run by pfmm_probe_fma_rate (independent FMA chains)",
@@ -946,6 +961,8 @@ def main():
         f64, fmx = (f, fo) if head == P.PFMM_FP64 else (fo, f)
         rel = float((fmx - f64).abs().max() / f64.abs().max())
         info2 = op2.info()
+        if other == P.PFMM_FP64:
+            info2 = dict(info2, nf_residue_bytes=16.0 * nf_residue_elements(nt))
         other_line = {"precision": "mixed" if other == P.PFMM_MIXED else "fp64",
                       "value": dof / (statistics.mean(ms2) * 1e-3), "ms_per_step": statistics.mean(ms2),
                       "phases_ms": ph2, "build_s": t_build2, "mixed_vs_fp64_rel_maxnorm": rel,

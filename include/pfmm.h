@@ -134,8 +134,9 @@ typedef struct pfmm_info {
 } pfmm_info;
 
 /* M2L kernels (pfmm_info.m2l_engine): the three separable passes through a global workspace
- * (FP64, grids beyond 8^3 or high degrees), the fused kernel (FP32, grids of at most 4^3 cells,
- * m_x <= 7), the slab kernel (FP32, grids of 5^3 .. 8^3 cells, m_x <= 6). */
+ * (grids beyond 8^3, high degrees, native FP64), the fused kernels (grids of at most 4^3 cells, FP32
+ * m_x <= 7 or double-FP32 m_x <= 6; the 4^3 grid in even and odd parts per direction), the slab
+ * kernels (FP32, grids of 5^3 .. 8^3 cells, m_x <= 6; the 8^3 grid in even and odd parts). */
 #define PFMM_M2L_THREE_PASS 1
 #define PFMM_M2L_FUSED 2
 #define PFMM_M2L_SLAB 3
