@@ -98,7 +98,13 @@ typedef struct pfmm_params {
     int32_t nf_engine;  /* PFMM_NF_AUTO: tensor cores where the panel layout allows (mixed mode: the
                            scaled two-part FP16 split with FP32 accumulation; FP64 mode: exact
                            integer products modulo 16 primes, combined by the Chinese remainder
-                           theorem), else CUDA cores; PFMM_NF_CUDA_CORES: always CUDA cores */
+                           theorem), else CUDA cores; PFMM_NF_CUDA_CORES: always CUDA cores.
+                           The integers of the FP64 mode are fixed point: block entries are rounded to
+                           52 to 53 bits of the largest of their row, inputs to as many (two fewer at
+                           the worst) of the largest of the two leaf intervals that a step's products
+                           read, over all triangles or nodes.  An output far below the product of
+                           those two keeps that absolute accuracy, where PFMM_NF_CUDA_CORES keeps FP64's
+                           relative one of every term */
     int32_t fp64_native;/* FP64 mode only.  0 (default): FP64-accurate arithmetic on the fast units --
                            the nearfield as exact residue products on the tensor cores (see
                            nf_engine) and the FMM passes in double-FP32 arithmetic (pairs of FP32

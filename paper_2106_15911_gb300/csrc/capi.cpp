@@ -189,10 +189,24 @@ int ensure_workspace(pfmm_handle *H, int nrhs)
     H->d_Wres = nullptr;
     H->d_res8 = nullptr;
     if (H->crtV || H->crtK) {
-        const size_t nw = (size_t)kCrtModuli * nrhs * H->Et * std::max(H->colsV_u, H->colsK_u);
-        if ((rc = H->alloc(&H->d_Wres, nw)) || (rc = H->alloc(&H->d_res8, (size_t)kCrtModuli * n_in)) ||
-            (!H->d_wmax && (rc = H->alloc(&H->d_wmax, (size_t)nrhs))))
-            return rc;
+        // residues of as many right-hand sides at a time as 4 GiB hold (the product loops over them), or
+        // as the device has room for
+        const size_t w1 = (size_t)kCrtModuli * 2 * H->Et * std::max(H->colsV_u, H->colsK_u);
+        const size_t most = std::max<size_t>(1, ((size_t)4 << 30) / (w1 * sizeof(uint16_t)));
+        for (int n = (int)std::min<size_t>(nrhs, most);; n = (n + 1) / 2) {
+            rc = H->alloc(&H->d_Wres, n * w1);
+            if (!rc) rc = H->alloc(&H->d_res8, (size_t)kCrtModuli * n * H->Et * H->nt);
+            if (!rc) {
+                H->crt_rhs = n;
+                break;
+            }
+            H->release(H->d_Wres);
+            H->d_Wres = nullptr;
+            if (rc != PFMM_ERR_OOM || n == 1) return rc;
+        }
+        if ((rc = H->alloc(&H->d_wmax, pfmm::crt_scratch_words(H->crt_rhs, H->Et, H->ls)))) return rc;
+        CK(cudaMemset(H->d_wmax, 0, sizeof(unsigned long long)));  // CTAs done
+        CK(cudaStreamSynchronize(cudaStreamLegacy));
     }
     H->ws_nrhs = nrhs;
     return PFMM_OK;
@@ -276,18 +290,30 @@ int pfmm::run_nf_tc(pfmm_handle *H, int op, const double *x, int nrhs, void *whi
 }
 
 // FP64 exact nearfield: residues of x, the residue products on the tensor cores, their FP64
-// combination into fint (every element written)
-int pfmm::run_nf_crt(pfmm_handle *H, int op, const double *x, int nrhs, double *fint, cudaStream_t st)
+// combination into fint (every element written); crt_rhs right-hand sides at most
+static int run_nf_crt_some(pfmm_handle *H, int op, const double *x, int nrhs, double *fint, bool first, bool last,
+                           cudaStream_t st)
 {
+    using namespace pfmm;
     int rc;
-    const int cols = op == 0 ? H->colsV_u : H->colsK_u, b = op == 0 ? H->crt_bV : H->crt_bK;
-    launch_crt_split_input(x, op == 0 ? H->d_perm : nullptr, op == 0 ? H->nt : H->nv, cols, nrhs, H->Et, b, H->d_Wres,
-                           H->d_wmax, st);
-    const int ls = H->ls, nint = H->Et / ls;
-    uint64_t dims[5] = {(uint64_t)cols, (uint64_t)ls, (uint64_t)nint, (uint64_t)nrhs, (uint64_t)kCrtModuli};
-    uint64_t str[4] = {(uint64_t)cols * 2, (uint64_t)cols * 2 * ls, (uint64_t)cols * 2 * ls * nint,
-                       (uint64_t)cols * 2 * ls * nint * nrhs};
-    uint32_t box[5] = {64, 1, (uint32_t)nf_crt_intervals(nint, ls, H->crt_form), 1, 1};
+    const int cols = op == 0 ? H->colsV_u : H->colsK_u, ls = H->ls, nint = H->Et / ls;
+    CrtInput in{};
+    in.x = x;
+    in.perm = op == 0 ? H->d_perm : nullptr;
+    in.ncol = op == 0 ? H->nt : H->nv;
+    in.ncol_pad = cols;
+    in.nrhs = nrhs;
+    in.Et = H->Et;
+    in.ls = ls;
+    in.nt = H->nt;
+    in.b = op == 0 ? H->crt_bV : H->crt_bK;
+    crt_scratch(in, H->d_wmax);
+    const int ni = nf_crt_intervals(nint, ls, H->crt_form);
+    launch_crt_split_input(in, ni, H->d_Wres, st);
+    const uint64_t row = (uint64_t)cols * 2;  // bytes
+    uint64_t dims[5] = {(uint64_t)cols, (uint64_t)2 * ls, (uint64_t)nint, (uint64_t)nrhs, (uint64_t)kCrtModuli};
+    uint64_t str[4] = {row, row * 2 * ls, row * 2 * H->Et, row * 2 * H->Et * nrhs};
+    uint32_t box[5] = {64, 1, (uint32_t)ni, 1, 1};
     CUtensorMap mW;
     if ((rc = encode_map(&mW, H->d_Wres, 5, dims, str, box))) return rc;
     NfCrtParams P{};
@@ -298,17 +324,29 @@ int pfmm::run_nf_crt(pfmm_handle *H, int op, const double *x, int nrhs, double *
     P.nint = nint;
     P.Et = H->Et;
     P.nt = H->nt;
+    P.shared = in.shared;
     P.res = H->d_res8;
     P.err = H->d_err;
-    if (H->cur_ev) cudaEventRecord(H->cur_ev->ev[9], st);
+    if (H->cur_ev && first) cudaEventRecord(H->cur_ev->ev[9], st);
     if (launch_nf_apply_crt(mW, P, ls, H->nsm, st, H->crt_form))
         return fail(PFMM_ERR_CUDA, std::string("FP64 tensor-core nearfield launch: ") +
                                        cudaGetErrorString(cudaGetLastError()));
-    if (H->cur_ev) {
+    if (H->cur_ev && last) {
         cudaEventRecord(H->cur_ev->ev[10], st);
         H->cur_ev->nf = true;
     }
-    launch_crt_combine(H->d_res8, nrhs, H->Et, H->nt, op == 0 ? H->d_rexpV : H->d_rexpK, H->d_wmax, b, fint, st);
+    launch_crt_combine(H->d_res8, in, op == 0 ? H->d_rexpV : H->d_rexpK, fint, st);
+    return PFMM_OK;
+}
+
+int pfmm::run_nf_crt(pfmm_handle *H, int op, const double *x, int nrhs, double *fint, cudaStream_t st)
+{
+    const size_t nin = (size_t)H->Et * (op == 0 ? H->nt : H->nv), nout = (size_t)H->Et * H->nt;
+    for (int r = 0; r < nrhs; r += H->crt_rhs) {
+        const int n = std::min(nrhs - r, H->crt_rhs);
+        const int rc = run_nf_crt_some(H, op, x + r * nin, n, fint + r * nout, r == 0, r + n == nrhs, st);
+        if (rc) return rc;
+    }
     return PFMM_OK;
 }
 

@@ -105,10 +105,11 @@ struct pfmm_handle {
     double crt_form_ms[2] = {0, 0};                   // build-time timing of the two forms
     unsigned char *d_AVres = nullptr, *d_AKres = nullptr;  // residue bytes [16][panel elements]
     int *d_rexpV = nullptr, *d_rexpK = nullptr;       // row scale exponents by triangle
-    uint16_t *d_Wres = nullptr;                       // input residues [16][nrhs][E_t][cols]
-    unsigned char *d_res8 = nullptr;                  // output residues [16][nrhs][E_t][E_x]
+    int crt_rhs = 0;                                  // right-hand sides that the next two hold
+    uint16_t *d_Wres = nullptr;                       // input residues [16][crt_rhs][leaf intervals][2 ls][cols]
+    unsigned char *d_res8 = nullptr;                  // output residues [16][crt_rhs][E_t][E_x]
     uint16_t *d_Whi = nullptr, *d_Wlo = nullptr;  // FP16 input parts
-    unsigned long long *d_wmax = nullptr;          // [ws_nrhs] max |input| per rhs (FP64 bits)
+    unsigned long long *d_wmax = nullptr;          // [ws_nrhs] max |input| per rhs (FP64 bits); FP64 mode: crt_scratch
     double *d_nfpart = nullptr;                    // partial planes of the tensor-core nearfield
     size_t w_elems = 0;
 

@@ -8,7 +8,9 @@
 // The block-Toeplitz nearfield product F[r][t] = sum_d sum_k A_d[r][k] W[t-d][k] is therefore
 // computed exactly in integers and rounded to FP64 once:
 //   * every row r of the stored FP64 blocks is scaled by 2^e_r (largest |A_d[r][k]| over d, k in
-//     [2^(b-1), 2^b)) and rounded to the integer A'; the input by 2^s per rhs to W' (|W'| <= 2^b),
+//     [2^(b-1), 2^b)) and rounded to the integer A'; the input by 2^s to W' (|W'| <= 2^b), with s
+//     from the largest input of the two leaf intervals that an output's products read (or of
+//     the whole right-hand side while that takes at most kCrtSlack bits from them),
 //     b chosen so that the exact integer product X = sum A' W' satisfies 2 |X| < M;
 //   * X is computed modulo 16 primes p_i < 256 (M = prod p_i ~ 2^123): the residues of A' and W'
 //     in [-(p-1)/2, (p-1)/2] are exact FP16 numbers, their products are below 2^14, and a tcgen05
@@ -19,7 +21,8 @@
 //     FP32 arithmetic), X is assembled exactly in 128-bit integers and X 2^-(e_r + s) is rounded
 //     to FP64 (relative error ~2^-52).
 // The only rounding before the final FP64 result is that of A and W to b-bit fixed point per row /
-// per rhs (b = 52..53): the product is as accurate as an FP64 dot product of the same terms.
+// per output interval (b = 52..53): the error is that of an FP64 dot product whose terms are all of
+// the size of the row's largest entry times the interval's largest input.
 //
 // The residues of A' are stored as bytes (r + 128), half the bytes of FP16, because the stored
 // blocks are the bulk of the traffic: 16 bytes per element.  All panels index the same columns, so
@@ -30,9 +33,12 @@
 // from where tcgen05.mma takes them as the A operand.
 //
 // Tiles: 128 rows x (NI leaf intervals x LS phases) columns; W is a TMA tensor [modulus][rhs]
-// [interval][phase][column], so the time shift d is a coordinate offset and causality the zero fill.
-// For one column block the 2 LS step offsets need only 2 LS W tiles, one per step of the interval
-// before and of the interval itself; in that order phase ph of offset d is tile LS + ph - d, so all
+// [interval][2 LS steps][column]: the steps of the interval before and then of the interval itself, both
+// scaled for this interval's outputs.  Where all intervals of a tile have the scale of the one before
+// (P.shared), the first LS steps are not stored but read as the interval before's own (a coordinate
+// offset; the zero fill before the first): writing and reading both took 1.6 % of a product.
+// For one column block the 2 LS step offsets need only these 2 LS W tiles; in this
+// order phase ph of offset d is tile LS + ph - d, so all
 // phases of an offset are one contiguous operand of up to LS NI rows, and each W tile is brought in
 // once for its LS uses.  A work item is (modulus, row tile, interval block, rhs).  The accumulators
 // are reduced modulo p every r column blocks (r by the modulus and LS: 128 LS r products of two
@@ -234,6 +240,7 @@ __global__ void __launch_bounds__(kCrtThreads, 1) k_nf_apply_crt(const __grid_co
             int g = 0;
             for (int it = blockIdx.x; it < P.nitems && !s_abort; it += gridDim.x) {
                 const CItem I(P, nib, it);
+                const bool shared = P.shared[I.rhs * nib + I.ib] != 0;
                 for (int kb = 0; kb < P.nkb; ++kb, ++g) {
                     const int s = g % NST;
                     if (!wait(&done[s], ((g / NST) & 1) ^ 1, 11) || s_abort) break;
@@ -241,8 +248,8 @@ __global__ void __launch_bounds__(kCrtThreads, 1) k_nf_apply_crt(const __grid_co
                     mbar_expect_tx(&wfull[s], S::W_STAGE);
 #pragma unroll
                     for (int q = 0; q < ND; ++q)  // the steps of the interval before, then its own
-                        tma_5d(d + q * S::W_TILE, &mapW, kb * BK, q % LS, I.ib * NI - (q < LS ? 1 : 0), I.rhs, I.m,
-                               &wfull[s]);
+                        tma_5d(d + q * S::W_TILE, &mapW, kb * BK, q < LS && shared ? LS + q : q,
+                               I.ib * NI - (q < LS && shared ? 1 : 0), I.rhs, I.m, &wfull[s]);
                 }
             }
             const uint64_t dl2 = gtimer() + kTimeoutNs / 20;
@@ -496,11 +503,11 @@ __host__ __device__ inline int crt_scale_exp(unsigned long long bits, int b)
     return b - 1 - E;
 }
 
-__device__ __forceinline__ double pow2(int e)
+// v 2^e, rounded once where the result is subnormal
+__device__ __forceinline__ double scale2(double v, int e)
 {
-    // 2^e for -1022 <= e <= 1023 from its bits; beyond: two steps
-    if (e >= -1022 && e <= 1023) return __longlong_as_double((long long)(1023 + e) << 52);
-    return ldexp(1.0, e);
+    if (e >= -1022 && e <= 1023) return v * __longlong_as_double((long long)(1023 + e) << 52);
+    return ldexp(v, e);
 }
 
 // balanced residue of an integer-valued x (|x| < 2^22) modulo p, in [-(p-1)/2, (p-1)/2]: the
@@ -552,11 +559,11 @@ __global__ void k_crt_split_panel(const double *__restrict__ A, const PanelGPU *
         const double2 *a = reinterpret_cast<const double2 *>(
             A + (kop ? Pn.offK : Pn.offV) + ((size_t)d * Pn.rows_pad + (x - Pn.row0)) * ncp + c);
         const double2 p = a[0], q = a[1];
-        const double sc = pow2(rowexp[x]);
-        e[0] = p.x * sc;
-        e[1] = p.y * sc;
-        e[2] = q.x * sc;
-        e[3] = q.y * sc;
+        const int sc = rowexp[x];
+        e[0] = scale2(p.x, sc);
+        e[1] = scale2(p.y, sc);
+        e[2] = scale2(q.x, sc);
+        e[3] = scale2(q.y, sc);
     }
     uint32_t w[kCrtModuli];
 #pragma unroll
@@ -579,34 +586,109 @@ __global__ void k_row_exps(const unsigned long long *__restrict__ rowmax, int nt
     if (x < nt) rowexp[x] = crt_scale_exp(rowmax[x], b);
 }
 
-// input: per-rhs scale 2^s (|W'| <= 2^b), W' = rint(2^s x) permuted (V) or padded (K) into
-// [rhs][t][ncol_pad], residues [modulus][rhs][t][ncol_pad]
-__global__ void k_crt_split_input(const double *__restrict__ x, const int *__restrict__ perm, int ncol, int ncol_pad,
-                                  size_t per_rhs, size_t total, const unsigned long long *__restrict__ wmax, int b,
-                                  __half *__restrict__ res)
+// scales of the input.  Every (rhs, leaf interval) goes to nsplit CTAs, each of which writes its largest |x|
+// as FP64 bits to part.  The last CTA to finish adds them up and sets, for the outputs of each interval
+// (whose products read it and the one before), win = the scale exponent of the rhs's largest |x|, or of the
+// two intervals' where that is more than kCrtSlack binary orders smaller.  shared of a tile of ni intervals:
+// the exponent never changes.  ticket is zero between launches.  With the split that follows 1 to 4 us more than
+// one scale per rhs took (12288 triangles x 256 steps: product 4.43 -> 4.45 ms)
+constexpr int kCrtSlack = 2;
+__global__ void __launch_bounds__(256) k_crt_scales(CrtInput in, int nsplit, int ni)
+{
+    __shared__ unsigned long long red[8];
+    __shared__ bool last;
+    const int nint = in.Et / in.ls, nw = in.nrhs * nint, w = blockIdx.x / nsplit;
+    const size_t per = (size_t)in.ls * in.ncol;
+    const unsigned long long *xr = reinterpret_cast<const unsigned long long *>(in.x) + w * per;
+    unsigned long long m = 0ull;
+    for (size_t i = (size_t)(blockIdx.x % nsplit) * blockDim.x + threadIdx.x; i < per; i += (size_t)nsplit * blockDim.x) {
+        const unsigned long long v = xr[i] & 0x7fffffffffffffffull;
+        m = v > m ? v : m;
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long v = __shfl_xor_sync(0xffffffffu, m, o);
+        m = v > m ? v : m;
+    }
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int q = 1; q < 8; ++q) m = red[q] > m ? red[q] : m;
+        in.part[blockIdx.x] = m;
+        __threadfence();
+        last = atomicAdd(in.ticket, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    const int nib = (nint + ni - 1) / ni;
+    for (int i = threadIdx.x; i < in.nrhs * nib; i += blockDim.x) in.shared[i] = 1;
+    for (int i = threadIdx.x; i < in.nrhs; i += blockDim.x) in.all[i] = 0ull;
+    if (threadIdx.x == 0) *in.ticket = 0u;
+    __syncthreads();
+    for (int i = threadIdx.x; i < nw; i += blockDim.x) {
+        unsigned long long v = 0ull;
+        for (int q = 0; q < nsplit; ++q) {
+            const unsigned long long u = __ldcg(in.part + (size_t)i * nsplit + q);
+            v = u > v ? u : v;
+        }
+        in.wmax[i] = v;
+        atomicMax(in.all + i / nint, v);
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < nw; i += blockDim.x) {
+        const int iv = i % nint;
+        unsigned long long v[3];  // this interval's, the one's before and the one's before that
+#pragma unroll
+        for (int q = 0; q < 3; ++q) v[q] = iv >= q ? in.wmax[i - q] : 0ull;
+        const int ea = crt_scale_exp(__ldcg(in.all + i / nint), in.b);
+        auto window = [&](unsigned long long x, unsigned long long y) {
+            const unsigned long long m = x > y ? x : y;
+            const int e = crt_scale_exp(m, in.b);
+            return m == 0ull || e - ea <= kCrtSlack ? ea : e;
+        };
+        const int e = window(v[0], v[1]);
+        in.win[i] = e;
+        if (iv > 0 && e != window(v[1], v[2])) in.shared[i / nint * nib + iv / ni] = 0;
+    }
+}
+
+// input: W' = rint(2^s x) permuted (V) or padded (K), with the scale of its own
+// interval's outputs as steps ls .. 2 ls - 1 and, where a tile of ni intervals is not shared, with that of
+// the next interval's as its steps 0 .. ls - 1; residues [modulus][rhs][interval][2 ls][ncol_pad]
+__global__ void k_crt_split_input(CrtInput in, size_t total, int ni, __half *__restrict__ res)
 {
     const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= total) return;
-    const size_t rt = i / ncol_pad;
-    const int c = (int)(i - rt * ncol_pad);
-    long long wi = 0;
-    if (c < ncol) {
-        const double v = x[rt * ncol + (perm ? perm[c] : c)];
-        wi = __double2ll_rn(v * pow2(crt_scale_exp(wmax[i / per_rhs], b)));
-    }
-    float r[kCrtModuli];
-    residues16(wi, r);
+    const int ls = in.ls, nint = in.Et / ls, nib = (nint + ni - 1) / ni;
+    const unsigned rt = i >> 32 ? (unsigned)(i / in.ncol_pad) : (unsigned)i / (unsigned)in.ncol_pad, rhs = rt / (unsigned)in.Et;
+    const int c = (int)(i - (size_t)rt * in.ncol_pad), t = (int)(rt - rhs * in.Et), iv = t / ls, s = t - iv * ls;
+    const size_t w = (size_t)rhs * nint + iv;
+    const double v = c < in.ncol ? in.x[(size_t)rt * in.ncol + (in.perm ? in.perm[c] : c)] : 0.0;
+    const bool more = iv + 1 < nint;  // the next interval's outputs read this step as well
+    const int e0 = in.win[w], e1 = more ? in.win[w + 1] : e0;
+    const bool next_shared = !more || in.shared[rhs * nib + (iv + 1) / ni], first_shared = iv > 0 || in.shared[rhs * nib];
+    // element of (interval iv, step ls + s); the next interval's step s is ls steps on
+    __half *o = res + (w * 2 * ls + ls + s) * in.ncol_pad + c;
+    const size_t per_m = 2 * total, next = (size_t)ls * in.ncol_pad;
+    if (!first_shared) {
 #pragma unroll
-    for (int m = 0; m < kCrtModuli; ++m) res[(size_t)m * total + i] = __float2half_rn(r[m]);
+        for (int m = 0; m < kCrtModuli; ++m) (o - next)[m * per_m] = __float2half_rn(0.f);
+    }
+#pragma unroll 1
+    for (int q = 0; q < (next_shared ? 1 : 2); ++q, o += next) {
+        float r[kCrtModuli];
+        residues16(__double2ll_rn(scale2(v, q ? e1 : e0)), r);
+#pragma unroll
+        for (int m = 0; m < kCrtModuli; ++m) o[m * per_m] = __float2half_rn(r[m]);
+    }
 }
 
-// f[rhs][t][row] = X 2^-(e_row + s_rhs), X from its residues by Garner's algorithm: the balanced
+// f[rhs][t][row] = X 2^-(e_row + s), X from its residues by Garner's algorithm: the balanced
 // mixed-radix digits v_j = (r_j - sum_{k<j} v_k P_k) P_j^-1 mod p_j (P_j = p_0 ... p_{j-1}) in exact
 // FP32 arithmetic (every intermediate is an integer below 2^20), then X = sum_j v_j P_j by Horner's
 // rule in 128-bit integers (|X| < M / 2 < 2^123, exact) and one conversion to FP64
-__global__ void k_crt_combine(const unsigned char *__restrict__ res, size_t per_mod, size_t per_rhs, int nt,
-                              const int *__restrict__ rowexp, const unsigned long long *__restrict__ wmax, int b,
-                              double *__restrict__ f)
+__global__ void k_crt_combine(const unsigned char *__restrict__ res, size_t per_mod, CrtInput in,
+                              const int *__restrict__ rowexp, double *__restrict__ f)
 {
     const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= per_mod) return;
@@ -630,9 +712,9 @@ __global__ void k_crt_combine(const unsigned char *__restrict__ res, size_t per_
     const unsigned long long hi = (unsigned long long)(U >> 64), lo = (unsigned long long)U;
     const double ax = hi ? fma((double)hi, 18446744073709551616.0, (double)lo) : (double)lo;
     const double x = neg ? -ax : ax;
-    const int row = (int)(i % nt);
-    const int e = rowexp[row] + crt_scale_exp(wmax[i / per_rhs], b);
-    f[i] = x * pow2(-e);
+    const unsigned rt = i >> 32 ? (unsigned)(i / in.nt) : (unsigned)i / (unsigned)in.nt, rhs = rt / (unsigned)in.Et;
+    const int row = (int)(i - (size_t)rt * in.nt), t = (int)(rt - rhs * in.Et), nint = in.Et / in.ls, iv = t / in.ls;
+    f[i] = scale2(x, -(rowexp[row] + in.win[(size_t)rhs * nint + iv]));
 }
 
 // ------------------------------------------------------------------------------------------
@@ -727,23 +809,39 @@ void launch_crt_split_panel(const double *A, const PanelGPU *panels, const int *
                                                                   res);
 }
 
-void launch_crt_split_input(const double *x, const int *perm, int ncol, int ncol_pad, int nrhs, int Et, int b,
-                            void *res, unsigned long long *wmax, cudaStream_t st)
+// CTAs of k_crt_scales per interval: about 2048 values each, or more where the intervals fill the GPU
+static int crt_nsplit(size_t nw, size_t per)
 {
-    cudaMemsetAsync(wmax, 0, sizeof(unsigned long long) * nrhs, st);
-    const size_t per_in = (size_t)Et * ncol;
-    const unsigned gx = (unsigned)std::max<size_t>(1, std::min<size_t>((per_in + 2047) / 2048, 1216));
-    launch_absmax_input(x, per_in, nrhs, gx, wmax, st);
-    const size_t per_rhs = (size_t)Et * ncol_pad, total = (size_t)nrhs * per_rhs;
-    k_crt_split_input<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(x, perm, ncol, ncol_pad, per_rhs, total, wmax,
-                                                                       b, (__half *)res);
+    return (int)std::max<size_t>(1, std::min<size_t>((per + 2047) / 2048, (1216 + nw - 1) / nw));
 }
 
-void launch_crt_combine(const unsigned char *res, int nrhs, int Et, int nt, const int *rowexp,
-                        const unsigned long long *wmax, int b, double *f, cudaStream_t st)
+// part: at most nw + 1216 CTAs
+size_t crt_scratch_words(int nrhs, int Et, int ls) { return (size_t)nrhs * (Et / ls) * 3 + 1216 + nrhs + 1; }
+
+void crt_scratch(CrtInput &in, unsigned long long *p)
 {
-    const size_t per_rhs = (size_t)Et * nt, per_mod = (size_t)nrhs * per_rhs;
-    k_crt_combine<<<(unsigned)((per_mod + 255) / 256), 256, 0, st>>>(res, per_mod, per_rhs, nt, rowexp, wmax, b, f);
+    const size_t nw = (size_t)in.nrhs * (in.Et / in.ls);
+    in.ticket = (unsigned *)p;
+    in.all = p + 1;
+    in.wmax = in.all + in.nrhs;
+    in.part = in.wmax + nw;
+    in.win = (int *)(in.part + nw + 1216);
+    in.shared = in.win + nw;  // at most one a (rhs, interval)
+}
+
+void launch_crt_split_input(const CrtInput &in, int ni, void *res, cudaStream_t st)
+{
+    const size_t nw = (size_t)in.nrhs * (in.Et / in.ls), per = (size_t)in.ls * in.ncol;
+    const int nsplit = crt_nsplit(nw, per);
+    k_crt_scales<<<(unsigned)(nw * nsplit), 256, 0, st>>>(in, nsplit, ni);
+    const size_t total = (size_t)in.nrhs * in.Et * in.ncol_pad;
+    k_crt_split_input<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(in, total, ni, (__half *)res);
+}
+
+void launch_crt_combine(const unsigned char *res, const CrtInput &in, const int *rowexp, double *f, cudaStream_t st)
+{
+    const size_t per_mod = (size_t)in.nrhs * in.Et * in.nt;
+    k_crt_combine<<<(unsigned)((per_mod + 255) / 256), 256, 0, st>>>(res, per_mod, in, rowexp, f);
 }
 
 int nf_crt_intervals(int nint, int ls, int form)

@@ -18,6 +18,7 @@ struct NfCrtParams {
     const unsigned char *A;  // residue bytes of the blocks [modulus][tile][column block][d][128][64]
     int ntiles, nkb, nitems; // 128-row tiles, 64-column blocks; nitems is set by the launch
     int nint, Et, nt, nrhs;
+    const int *shared;       // CrtInput.shared
     unsigned char *res;      // out: residues [modulus][rhs][Et][nt] in [0, p)
     int *err;                // set non-zero when a bounded wait gave up
 };
@@ -34,13 +35,26 @@ void launch_crt_row_exps(const double *A, const PanelGPU *panels, int npanel, in
 size_t crt_panel_bytes(int nt, int ncp, int nd);
 void launch_crt_split_panel(const double *A, const PanelGPU *panels, const int *tri_leaf, const int *rowexp, int kop,
                             int nt, int ncp, int nd, unsigned char *res, cudaStream_t st);
-// per-rhs max |x| into wmax, residues [kCrtModuli][nrhs][Et][ncol_pad] of the scaled, rounded,
-// permuted (V) or padded (K) input
-void launch_crt_split_input(const double *x, const int *perm, int ncol, int ncol_pad, int nrhs, int Et, int b,
-                            void *res, unsigned long long *wmax, cudaStream_t st);
+// one product's input
+struct CrtInput {
+    const double *x;          // [rhs][Et][ncol]
+    const int *perm;          // internal -> caller column (V), or null
+    int ncol, ncol_pad, nrhs, Et, ls, nt, b;
+    // scratch (k_crt_scales): CTAs done (0 between launches); largest |x| as FP64 bits of each rhs, of the
+    // (rhs, leaf interval)s and of their parts; scale exponents of the outputs; 1 where all intervals of a tile [rhs][tile] have the scale of the one before
+    unsigned *ticket;
+    unsigned long long *all, *wmax, *part;
+    int *win, *shared;
+};
+// scratch of a product: its words (the first zero before the first launch), and the pointers into it
+size_t crt_scratch_words(int nrhs, int Et, int ls);
+void crt_scratch(CrtInput &in, unsigned long long *p);
+// scales and residues [kCrtModuli][nrhs][leaf intervals][2 ls][ncol_pad] of the scaled, rounded,
+// permuted (V) or padded (K) input: every interval's own steps after those of the one before (these only in
+// tiles of ni intervals that are not shared)
+void launch_crt_split_input(const CrtInput &in, int ni, void *res, cudaStream_t st);
 // f[rhs][t][row] (overwritten) from the residues of the exact products
-void launch_crt_combine(const unsigned char *res, int nrhs, int Et, int nt, const int *rowexp,
-                        const unsigned long long *wmax, int b, double *f, cudaStream_t st);
+void launch_crt_combine(const unsigned char *res, const CrtInput &in, const int *rowexp, double *f, cudaStream_t st);
 // leaf intervals per work item: rows of the W tensor map's box
 int nf_crt_intervals(int nint, int ls, int form);
 // form 1: work items of up to 128 leaf intervals; form 2: of up to 64 (twice the items, each of half
