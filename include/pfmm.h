@@ -100,11 +100,12 @@ typedef struct pfmm_params {
                            integer products modulo 16 primes, combined by the Chinese remainder
                            theorem), else CUDA cores; PFMM_NF_CUDA_CORES: always CUDA cores.
                            The integers of the FP64 mode are fixed point: block entries are rounded to
-                           52 to 53 bits of the largest of their row, inputs to as many (two fewer at
+                           51 to 53 bits of the largest of their row, inputs to as many (two fewer at
                            the worst) of the largest of the two leaf intervals that a step's products
                            read, over all triangles or nodes.  An output far below the product of
                            those two keeps that absolute accuracy, where PFMM_NF_CUDA_CORES keeps FP64's
-                           relative one of every term */
+                           relative one of every term.  Inputs that are not finite reach the outputs
+                           whose products read them, as in FP64, and no others */
     int32_t fp64_native;/* FP64 mode only.  0 (default): FP64-accurate arithmetic on the fast units --
                            the nearfield as exact residue products on the tensor cores (see
                            nf_engine) and the FMM passes in double-FP32 arithmetic (pairs of FP32

@@ -307,7 +307,11 @@ static int run_nf_crt_some(pfmm_handle *H, int op, const double *x, int nrhs, do
     in.ls = ls;
     in.nt = H->nt;
     in.b = op == 0 ? H->crt_bV : H->crt_bK;
+    in.kop = op;
     crt_scratch(in, H->d_wmax);
+    in.A = (const double *)H->nf_blocks(op);
+    in.panels = H->d_panels;
+    in.tri_leaf = H->d_tri_leaf;
     const int ni = nf_crt_intervals(nint, ls, H->crt_form);
     launch_crt_split_input(in, ni, H->d_Wres, st);
     const uint64_t row = (uint64_t)cols * 2;  // bytes

@@ -9,7 +9,7 @@
 // computed exactly in integers and rounded to FP64 once:
 //   * every row r of the stored FP64 blocks is scaled by 2^e_r (largest |A_d[r][k]| over d, k in
 //     [2^(b-1), 2^b)) and rounded to the integer A'; the input by 2^s to W' (|W'| <= 2^b), with s
-//     from the largest input of the two leaf intervals that an output's products read (or of
+//     from the largest finite input of the two leaf intervals that an output's products read (or of
 //     the whole right-hand side while that takes at most kCrtSlack bits from them),
 //     b chosen so that the exact integer product X = sum A' W' satisfies 2 |X| < M;
 //   * X is computed modulo 16 primes p_i < 256 (M = prod p_i ~ 2^123): the residues of A' and W'
@@ -21,8 +21,9 @@
 //     FP32 arithmetic), X is assembled exactly in 128-bit integers and X 2^-(e_r + s) is rounded
 //     to FP64 (relative error ~2^-52).
 // The only rounding before the final FP64 result is that of A and W to b-bit fixed point per row /
-// per output interval (b = 52..53): the error is that of an FP64 dot product whose terms are all of
-// the size of the row's largest entry times the interval's largest input.
+// per output interval (b = 51..53): the error is that of an FP64 dot product whose terms are all of
+// the size of the row's largest entry times the interval's largest input.  An input that is not
+// finite has residues of zero, and its products are added in FP64 to the outputs that they reach.
 //
 // The residues of A' are stored as bytes (r + 128), half the bytes of FP16, because the stored
 // blocks are the bulk of the traffic: 16 bytes per element.  All panels index the same columns, so
@@ -586,34 +587,39 @@ __global__ void k_row_exps(const unsigned long long *__restrict__ rowmax, int nt
     if (x < nt) rowexp[x] = crt_scale_exp(rowmax[x], b);
 }
 
-// scales of the input.  Every (rhs, leaf interval) goes to nsplit CTAs, each of which writes its largest |x|
-// as FP64 bits to part.  The last CTA to finish adds them up and sets, for the outputs of each interval
-// (whose products read it and the one before), win = the scale exponent of the rhs's largest |x|, or of the
-// two intervals' where that is more than kCrtSlack binary orders smaller.  shared of a tile of ni intervals:
-// the exponent never changes.  ticket is zero between launches.  With the split that follows 1 to 4 us more than
-// one scale per rhs took (12288 triangles x 256 steps: product 4.43 -> 4.45 ms)
+// scales of the input.  Every (rhs, leaf interval) goes to nsplit CTAs, each of which writes its largest finite |x|
+// as FP64 bits (sign bit: there are other values) to part.  The last CTA to finish adds them up and sets, for the
+// outputs of each interval (whose products read it and the one before), win = the scale exponent of the rhs's
+// largest |x|, or of the two intervals' where that is more than kCrtSlack binary orders smaller; bit 0 of win
+// tells of values that are not finite.  shared of a tile of ni intervals: the exponent never changes.
+// ticket is zero between launches.  With the split that follows 1 to 4 us more than one scale per rhs took
+// (12288 triangles x 256 steps: product 4.43 -> 4.45 ms)
 constexpr int kCrtSlack = 2;
 __global__ void __launch_bounds__(256) k_crt_scales(CrtInput in, int nsplit, int ni)
 {
+    constexpr unsigned long long kNot = 1ull << 63;
     __shared__ unsigned long long red[8];
     __shared__ bool last;
     const int nint = in.Et / in.ls, nw = in.nrhs * nint, w = blockIdx.x / nsplit;
     const size_t per = (size_t)in.ls * in.ncol;
     const unsigned long long *xr = reinterpret_cast<const unsigned long long *>(in.x) + w * per;
     unsigned long long m = 0ull;
+    bool nf = false;
     for (size_t i = (size_t)(blockIdx.x % nsplit) * blockDim.x + threadIdx.x; i < per; i += (size_t)nsplit * blockDim.x) {
-        const unsigned long long v = xr[i] & 0x7fffffffffffffffull;
-        m = v > m ? v : m;
+        const unsigned long long v = xr[i] & ~kNot;
+        const bool finite = v < 0x7ff0000000000000ull;
+        nf |= !finite;
+        m = finite && v > m ? v : m;
     }
     for (int o = 16; o > 0; o >>= 1) {
         const unsigned long long v = __shfl_xor_sync(0xffffffffu, m, o);
         m = v > m ? v : m;
     }
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
-    __syncthreads();
+    nf = __syncthreads_or(nf) != 0;
     if (threadIdx.x == 0) {
         for (int q = 1; q < 8; ++q) m = red[q] > m ? red[q] : m;
-        in.part[blockIdx.x] = m;
+        in.part[blockIdx.x] = nf ? m | kNot : m;
         __threadfence();
         last = atomicAdd(in.ticket, 1u) == gridDim.x - 1;
     }
@@ -626,20 +632,25 @@ __global__ void __launch_bounds__(256) k_crt_scales(CrtInput in, int nsplit, int
     if (threadIdx.x == 0) *in.ticket = 0u;
     __syncthreads();
     for (int i = threadIdx.x; i < nw; i += blockDim.x) {
-        unsigned long long v = 0ull;
+        unsigned long long v = 0ull, bad = 0ull;
         for (int q = 0; q < nsplit; ++q) {
             const unsigned long long u = __ldcg(in.part + (size_t)i * nsplit + q);
-            v = u > v ? u : v;
+            v = (u & ~kNot) > v ? u & ~kNot : v;
+            bad |= u & kNot;
         }
-        in.wmax[i] = v;
+        in.wmax[i] = v | bad;
         atomicMax(in.all + i / nint, v);
     }
     __syncthreads();
     for (int i = threadIdx.x; i < nw; i += blockDim.x) {
         const int iv = i % nint;
-        unsigned long long v[3];  // this interval's, the one's before and the one's before that
+        unsigned long long v[3], bad = 0ull;  // this interval's, the one's before and the one's before that
 #pragma unroll
-        for (int q = 0; q < 3; ++q) v[q] = iv >= q ? in.wmax[i - q] : 0ull;
+        for (int q = 0; q < 3; ++q) {
+            v[q] = iv >= q ? in.wmax[i - q] : 0ull;
+            if (q < 2) bad |= v[q] & kNot;
+            v[q] &= ~kNot;
+        }
         const int ea = crt_scale_exp(__ldcg(in.all + i / nint), in.b);
         auto window = [&](unsigned long long x, unsigned long long y) {
             const unsigned long long m = x > y ? x : y;
@@ -647,12 +658,12 @@ __global__ void __launch_bounds__(256) k_crt_scales(CrtInput in, int nsplit, int
             return m == 0ull || e - ea <= kCrtSlack ? ea : e;
         };
         const int e = window(v[0], v[1]);
-        in.win[i] = e;
+        in.win[i] = e * 2 + (bad ? 1 : 0);
         if (iv > 0 && e != window(v[1], v[2])) in.shared[i / nint * nib + iv / ni] = 0;
     }
 }
 
-// input: W' = rint(2^s x) permuted (V) or padded (K), with the scale of its own
+// input: W' = rint(2^s x) permuted (V) or padded (K), 0 where x is not finite, with the scale of its own
 // interval's outputs as steps ls .. 2 ls - 1 and, where a tile of ni intervals is not shared, with that of
 // the next interval's as its steps 0 .. ls - 1; residues [modulus][rhs][interval][2 ls][ncol_pad]
 __global__ void k_crt_split_input(CrtInput in, size_t total, int ni, __half *__restrict__ res)
@@ -663,9 +674,10 @@ __global__ void k_crt_split_input(CrtInput in, size_t total, int ni, __half *__r
     const unsigned rt = i >> 32 ? (unsigned)(i / in.ncol_pad) : (unsigned)i / (unsigned)in.ncol_pad, rhs = rt / (unsigned)in.Et;
     const int c = (int)(i - (size_t)rt * in.ncol_pad), t = (int)(rt - rhs * in.Et), iv = t / ls, s = t - iv * ls;
     const size_t w = (size_t)rhs * nint + iv;
-    const double v = c < in.ncol ? in.x[(size_t)rt * in.ncol + (in.perm ? in.perm[c] : c)] : 0.0;
+    double v = c < in.ncol ? in.x[(size_t)rt * in.ncol + (in.perm ? in.perm[c] : c)] : 0.0;
+    if (!isfinite(v)) v = 0.0;
     const bool more = iv + 1 < nint;  // the next interval's outputs read this step as well
-    const int e0 = in.win[w], e1 = more ? in.win[w + 1] : e0;
+    const int e0 = in.win[w] >> 1, e1 = more ? in.win[w + 1] >> 1 : e0;
     const bool next_shared = !more || in.shared[rhs * nib + (iv + 1) / ni], first_shared = iv > 0 || in.shared[rhs * nib];
     // element of (interval iv, step ls + s); the next interval's step s is ls steps on
     __half *o = res + (w * 2 * ls + ls + s) * in.ncol_pad + c;
@@ -686,7 +698,8 @@ __global__ void k_crt_split_input(CrtInput in, size_t total, int ni, __half *__r
 // f[rhs][t][row] = X 2^-(e_row + s), X from its residues by Garner's algorithm: the balanced
 // mixed-radix digits v_j = (r_j - sum_{k<j} v_k P_k) P_j^-1 mod p_j (P_j = p_0 ... p_{j-1}) in exact
 // FP32 arithmetic (every intermediate is an integer below 2^20), then X = sum_j v_j P_j by Horner's
-// rule in 128-bit integers (|X| < M / 2 < 2^123, exact) and one conversion to FP64
+// rule in 128-bit integers (|X| < M / 2 < 2^123, exact) and one conversion to FP64.  The products of inputs
+// that are not finite follow in FP64 from the stored blocks
 __global__ void k_crt_combine(const unsigned char *__restrict__ res, size_t per_mod, CrtInput in,
                               const int *__restrict__ rowexp, double *__restrict__ f)
 {
@@ -714,7 +727,18 @@ __global__ void k_crt_combine(const unsigned char *__restrict__ res, size_t per_
     const double x = neg ? -ax : ax;
     const unsigned rt = i >> 32 ? (unsigned)(i / in.nt) : (unsigned)i / (unsigned)in.nt, rhs = rt / (unsigned)in.Et;
     const int row = (int)(i - (size_t)rt * in.nt), t = (int)(rt - rhs * in.Et), nint = in.Et / in.ls, iv = t / in.ls;
-    f[i] = scale2(x, -(rowexp[row] + in.win[(size_t)rhs * nint + iv]));
+    const int win = in.win[(size_t)rhs * nint + iv];
+    double y = scale2(x, -(rowexp[row] + (win >> 1)));
+    if (win & 1) {
+        const PanelGPU &Pn = in.panels[in.tri_leaf[row]];
+        const double *a = in.A + (in.kop ? Pn.offK : Pn.offV) + (size_t)(row - Pn.row0) * in.ncol_pad;
+        for (int d = 0; d <= t - (iv - 1) * in.ls && d <= t; ++d, a += (size_t)Pn.rows_pad * in.ncol_pad)
+            for (int c = 0; c < in.ncol; ++c) {
+                const double v = in.x[(size_t)(rt - d) * in.ncol + (in.perm ? in.perm[c] : c)];
+                if (!isfinite(v)) y += a[c] * v;
+            }
+    }
+    f[i] = y;
 }
 
 // ------------------------------------------------------------------------------------------

@@ -35,16 +35,20 @@ void launch_crt_row_exps(const double *A, const PanelGPU *panels, int npanel, in
 size_t crt_panel_bytes(int nt, int ncp, int nd);
 void launch_crt_split_panel(const double *A, const PanelGPU *panels, const int *tri_leaf, const int *rowexp, int kop,
                             int nt, int ncp, int nd, unsigned char *res, cudaStream_t st);
-// one product's input
+// one product's input, and the stored blocks for the entries that are not finite
 struct CrtInput {
     const double *x;          // [rhs][Et][ncol]
     const int *perm;          // internal -> caller column (V), or null
-    int ncol, ncol_pad, nrhs, Et, ls, nt, b;
-    // scratch (k_crt_scales): CTAs done (0 between launches); largest |x| as FP64 bits of each rhs, of the
-    // (rhs, leaf interval)s and of their parts; scale exponents of the outputs; 1 where all intervals of a tile [rhs][tile] have the scale of the one before
+    int ncol, ncol_pad, nrhs, Et, ls, nt, b, kop;
+    // scratch (k_crt_scales): CTAs done (0 between launches); largest finite |x| as FP64 bits of each rhs, of the
+    // (rhs, leaf interval)s and of their parts; scale exponents of the outputs (x 2, + 1 where values that are not
+    // finite reach them); 1 where all intervals of a tile [rhs][tile] have the scale of the one before
     unsigned *ticket;
     unsigned long long *all, *wmax, *part;
     int *win, *shared;
+    const double *A;          // FP64 panels
+    const PanelGPU *panels;
+    const int *tri_leaf;
 };
 // scratch of a product: its words (the first zero before the first launch), and the pointers into it
 size_t crt_scratch_words(int nrhs, int Et, int ls);

@@ -1,5 +1,6 @@
 """The FP64 tensor-core nearfield on inputs that its fixed point could lose, against the CUDA-core FP64
-engine: densities that grow or decay over the steps by far more than FP64's 53 bits, and magnitudes near both ends
+engine: entries that are not finite (they reach the outputs whose products read them, and no others),
+densities that grow or decay over the steps by far more than FP64's 53 bits, and magnitudes near both ends
 of FP64's range."""
 import numpy as np
 import pytest
@@ -25,6 +26,30 @@ def _pair(ls, nint):
 
 def _near(op, call, x):
     return getattr(op, call)(x, parts=P.PFMM_PART_NEAR).cpu().numpy()
+
+
+@pytest.mark.parametrize("ls", LS)
+def test_entries_that_are_not_finite(ls):
+    V, T, Et, op, ref = _pair(ls, 8)
+    for call, n in (("V", len(T)), ("K", len(V))):
+        for bad in ({(0, ls, 3): np.nan}, {(0, Et - 1, n - 1): np.inf, (1, 0, 0): -np.inf},
+                    {(1, 4 * ls, 5): np.inf, (1, 4 * ls, 6): -np.inf, (2, 0, 1): 1e300}):
+            w = random_density(Et, n, 3, seed=23)
+            for at, v in bad.items():
+                w[at] = v
+            x = torch.tensor(w, device=DEV)
+            a, b = _near(op, call, x), _near(ref, call, x)
+            assert not np.isfinite(b).all() and np.isfinite(b).any()
+            np.testing.assert_array_equal(np.isnan(a), np.isnan(b))
+            np.testing.assert_array_equal(a[np.isinf(b)], b[np.isinf(b)])
+            # 52 bits of the largest finite input that a step's outputs read
+            for r in range(3):
+                for t in range(Et):
+                    ok = np.isfinite(b[r, t])
+                    if ok.any():
+                        assert np.max(np.abs(a[r, t] - b[r, t])[ok]) <= 1e-13 * np.max(np.abs(b[r, t])[ok])
+    op.close()
+    ref.close()
 
 
 @pytest.mark.parametrize("ls", LS)
