@@ -188,7 +188,9 @@ __global__ void __launch_bounds__(256) k_nf_apply(const S *__restrict__ A, const
 // (copies through registers took 2.7 ms at the first size below).  FP32 sums over
 // 128 products, added with their rounding errors kept (two FP32: the FP64 unit would be busy for half of the
 // FMAs' time, and sums over 512 products, all offsets in one, came out 20 % further from FP64 than the tiles').
-// Bound by the FMAs.  Nearfield, 64 x 64 tiles -> here: 1728 triangles x 1024 steps mixed 8.36 -> 1.12 ms,
+// Outputs beyond the FP32 range are summed once more in FP64 (nf_direct); the call costs 3 to 5 % at two steps per
+// leaf, whose registers are short, and nothing at others.
+// Bound by the FMAs.  Nearfield, 64 x 64 tiles -> here: 1728 triangles x 1024 steps mixed 8.36 -> 1.18 ms,
 // FP64 134 -> 23.2; 768 x 256, 4 right-hand sides, mixed 0.99 -> 0.38; 192 x 16 FP64 0.79 -> 0.73; 3072 x 128
 // FP64 13.1 -> 11.8; 12288 x 64 mixed 9.0 -> 6.2; three steps per leaf FP64 3.9 -> 2.7; one step mixed, K,
 // 0.127 -> 0.113.
@@ -203,6 +205,35 @@ __device__ __forceinline__ void cp_async(S *dst, const S *src, bool ok)
     asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src),
                  "n"((int)sizeof(S)), "r"(ok ? (int)sizeof(S) : 0)
                  : "memory");
+}
+
+// those of the n outputs f of the mixed mode that are not finite once more, in FP64: rows row .. row + n - 1 of a panel
+// at step t, offsets 0 .. nd - 1 (the first steps have fewer)
+__device__ __noinline__ void nf_direct(const float *__restrict__ A, const uint16_t *__restrict__ parts, float inv_scale,
+                                       const PanelGPU *__restrict__ Pp, int kop, const int *__restrict__ colidx,
+                                       const float *__restrict__ x, int ncolg, int row, int n, int t, int nd, double *f)
+{
+    const PanelGPU P = *Pp;
+    const int *cols = colidx + (kop ? P.colK_at : P.colV_at);
+    const int ncp = kop ? P.colsK_pad : P.colsV_pad;
+    const __half *Hp = reinterpret_cast<const __half *>(parts);
+    for (int r = 0; r < n; ++r) {
+        if (isfinite(f[r])) continue;
+        double y = 0.0;
+        for (int d = 0; d < nd && d <= t; ++d)
+            for (int c = 0; c < ncp && y == y; ++c) {  // NaN stays
+                if (cols[c] < 0) continue;
+                float a;
+                if (Hp) {
+                    const __half *h = Hp + nf_split_index(P.row0 + row + r, d, c, ncp >> 5);
+                    a = (__half2float(h[0]) + __half2float(h[kSplitPart])) * inv_scale;
+                } else {
+                    a = A[(kop ? P.offK : P.offV) + ((size_t)d * P.rows_pad + row + r) * ncp + c];
+                }
+                y += (double)a * (double)x[(size_t)(t - d) * ncolg + cols[c]];
+            }
+        f[r] = y;
+    }
 }
 
 template <typename S, int LS>
@@ -335,11 +366,21 @@ __global__ void __launch_bounds__(128, 3) k_nf_rows(const S *__restrict__ A, con
         const int iv = i0 + tid + v * nthr;
         if (iv >= nint) continue;
 #pragma unroll
-        for (int s = 0; s < LS; ++s)
+        for (int s = 0; s < LS; ++s) {
+            double *o = f + ((size_t)rhs * Et + iv * LS + s) * nt + P.row0 + r0;
+            bool finite = true;
 #pragma unroll
             for (int r = 0; r < BM; ++r)
-                if (r0 + r < P.nrows)
-                    f[((size_t)rhs * Et + iv * LS + s) * nt + P.row0 + r0 + r] = (double)sh[v][s][r] + ((double)sl[v][s][r] + (double)acc[v][s][r]);
+                if (r0 + r < P.nrows) {
+                    const double y = (double)sh[v][s][r] + ((double)sl[v][s][r] + (double)acc[v][s][r]);
+                    o[r] = y;
+                    finite &= isfinite(y);
+                }
+            if constexpr (kFloat)
+                if (!finite)
+                    nf_direct(A, hs.parts, hs.inv_scale, panels + tiles[2 * tile], kop, colidx, xr, ncolg, r0,
+                              min(BM, P.nrows - r0), iv * LS + s, LS + s + 1, o);
+        }
     }
 }
 
@@ -475,7 +516,13 @@ __global__ void __launch_bounds__(128) k_nf_same_step(const S *__restrict__ A, c
         const int r = e % BM, c = e / BM;
         double v = red[r * 32 + c];
         for (int w = 1; w < 4; ++w) v += red[(w * BM + r) * 32 + c];
-        if (r0 + r < P.nrows) f[(size_t)(b0 + c) * nt + P.row0 + r0 + r] = v;
+        if (r0 + r >= P.nrows) continue;
+        double *o = f + (size_t)(b0 + c) * nt + P.row0 + r0 + r;
+        *o = v;
+        if constexpr (kFloat)
+            if (!isfinite(v))
+                nf_direct(A, hs.parts, hs.inv_scale, panels + tiles[2 * tile], kop, colidx, x + (size_t)(b0 + c) * ncolg, ncolg,
+                          r0 + r, 1, 0, 1, o);
     }
 }
 

@@ -39,6 +39,26 @@ def test_nearfield_rows_match_oracle(precision, mesh, n_a, ls, nint, nrhs, c_st)
     op.close()
 
 
+@pytest.mark.parametrize("ls,n_a", [(1, 8), (2, 8), (3, 6), (4, 6)])
+def test_sums_beyond_the_fp32_range(ls, n_a):
+    # products and the sums of 128 of them are FP32 numbers, the outputs are not: FP64 sums
+    V, T = cube_mesh(n_a)
+    V = 100.0 * V  # entries of order one
+    Et = 8 * ls
+    kw = dict(m_t=2, m_x=2, c_st=1.0, leaf_steps=ls, quad_regular=2, quad_singular=2)
+    op = P.Operator(V, T, 1e4, Et, precision=P.PFMM_MIXED, nf_engine=P.PFMM_NF_CUDA_CORES, **kw)
+    ref = P.Operator(V, T, 1e4, Et, nf_engine=P.PFMM_NF_CUDA_CORES, **kw)
+    x = torch.ones(1, Et, len(T), device=DEV, dtype=torch.float64)
+    one = ref.V(x, parts=P.PFMM_PART_NEAR)
+    x *= 5e38 / float(one.max())
+    assert float(x.max()) < 3e38
+    a, b = op.V(x, parts=P.PFMM_PART_NEAR), ref.V(x, parts=P.PFMM_PART_NEAR)
+    assert float(b.max()) > 4.9e38
+    assert float((a - b).abs().max()) <= 1e-5 * float(b.max())  # FP32 blocks and sums
+    op.close()
+    ref.close()
+
+
 @pytest.mark.parametrize("ns", [1, 32, 33])  # one slice of a CTA's 32, all, and a second CTA
 @pytest.mark.parametrize("kw", [dict(precision=P.PFMM_MIXED, c_st=1.0),   # FP16 parts
                                 dict(precision=P.PFMM_MIXED, c_st=0.15, n_tr=1),  # FP32 panels of their own columns
