@@ -812,31 +812,8 @@ static int build_impl(const pfmm_mesh *mesh, const pfmm_params *prm, cudaStream_
         a.nq_sing = prm->quad_singular;
         a.colV = H->d_colV;
         a.kmap = H->d_kmap;
-        for (int k = 0; k < H->nd; ++k) {
-            const double sk = (k + 1) * H->h, ss = std::sqrt(sk), al = H->alpha, a32 = al * std::sqrt(al), sp = std::sqrt(kPi);
-            a.tc.cu[k] = 1.0 / (2.0 * std::sqrt(al) * ss);
-            a.tc.icu[k] = 2.0 * std::sqrt(al) * ss;
-            a.tc.s[k] = sk;
-            a.tc.b1[k] = ss / (8.0 * kPi * a32);
-            a.tc.b2[k] = ss / (4.0 * kPi * sp * a32);
-            a.tc.b3[k] = ss / std::sqrt(kPi * al);
-        }
-        a.tc.a1 = 1.0 / (8.0 * kPi * H->alpha * H->alpha);
-        a.tc.a2 = 1.0 / (2.0 * H->alpha);
-        a.tc.clin = 1.0 / (4.0 * kPi * H->alpha);
-        a.tc.k8 = 1.0 / (8.0 * kPi * H->alpha);
-        for (int k = 0; k < H->nd; ++k) {
-            a.tcf.cu[k] = (float)a.tc.cu[k];
-            a.tcf.icu[k] = (float)a.tc.icu[k];
-            a.tcf.s[k] = (float)a.tc.s[k];
-            a.tcf.b1[k] = (float)a.tc.b1[k];
-            a.tcf.b2[k] = (float)a.tc.b2[k];
-            a.tcf.b3[k] = (float)a.tc.b3[k];
-        }
-        a.tcf.a1 = (float)a.tc.a1;
-        a.tcf.a2 = (float)a.tc.a2;
-        a.tcf.clin = (float)a.tc.clin;
-        a.tcf.k8 = (float)a.tc.k8;
+        a.tc.set(H->h, H->alpha, H->nd);
+        a.tcf.set(H->h, H->alpha, H->nd);
         if (H->otf) {
             H->quad = a;
             launch_nf_singular(a, d_sing, (int)t.sing.size(), H->d_panels, nullptr, nullptr, H->mixed, st, H->d_singV,

@@ -47,6 +47,38 @@ __device__ __forceinline__ void erf_pair(R u, R &ef, R &efc)
     }
 }
 
+// A constant of the formulas below: FP64, or in FP32 the rounded value and what that leaves.  One FP32
+// rounding of it would be the same for every entry, and the second differences in time amplify what
+// the step ends' constants differ by (768 triangles x 256 steps, alpha 0.5: the nearfield came out 7.5e-7 from FP64
+// instead of 3.4e-7)
+template <typename R>
+struct Num {
+    R hi;
+    __host__ __device__ constexpr void set(double v) { hi = v; }
+};
+template <>
+struct Num<float> {
+    float hi, lo;
+    __host__ __device__ constexpr void set(double v)
+    {
+        hi = (float)v;
+        lo = (float)(v - (double)hi);
+    }
+};
+__device__ __forceinline__ double mulc(double x, Num<double> c) { return x * c.hi; }
+__device__ __forceinline__ float mulc(float x, Num<float> c) { return fmaf(x, c.hi, x * c.lo); }
+__device__ __forceinline__ double addc(double x, Num<double> c) { return c.hi + x; }
+__device__ __forceinline__ float addc(float x, Num<float> c) { return c.hi + (x + c.lo); }
+__device__ __forceinline__ double subc(double x, Num<double> c) { return x - c.hi; }
+__device__ __forceinline__ float subc(float x, Num<float> c) { return (x - c.hi) - c.lo; }
+template <typename R>
+__device__ constexpr Num<R> num(double v)
+{
+    Num<R> c{};
+    c.set(v);
+    return c;
+}
+
 // erf(u)/u (Maclaurin series below 0.05), iu = 1/u
 template <typename R>
 __device__ __forceinline__ R erf_over_u(R u, R ef, R iu)
@@ -54,7 +86,7 @@ __device__ __forceinline__ R erf_over_u(R u, R ef, R iu)
     if (u < R(0.05)) {
         R u2 = u * u;
         R s = R(1) + u2 * (R(-1.0 / 3.0) + u2 * (R(1.0 / 10.0) + u2 * (R(-1.0 / 42.0) + u2 * R(1.0 / 216.0))));
-        return R(2.0 / kSqrtPi) * s;
+        return mulc(s, num<R>(2.0 / kSqrtPi));
     }
     return ef * iu;
 }
@@ -73,18 +105,35 @@ __device__ __forceinline__ R phi2(R u, R ef, R ex, R iu)
             double c = (2.0 * n) / (fact[n] * (2.0 * n + 1.0));
             acc = acc * u2 + R((n % 2) ? c : -c);
         }
-        return R(2.0 / kSqrtPi) * acc;
+        return mulc(acc, num<R>(2.0 / kSqrtPi));
     }
-    return (ef - R(2.0 / kSqrtPi) * u * ex) * (iu * iu * iu);
+    return (ef - mulc(u, num<R>(2.0 / kSqrtPi)) * ex) * (iu * iu * iu);
 }
 
 // Constants of the step ends s = k h, k = 1 .. nd, and of the formulas above, from the host in FP64
 template <typename R>
 struct TimeConst {
-    R cu[8], icu[8];       // u = r cu, 1/u = icu / r:  cu = 1 / (2 sqrt(alpha s))
-    R s[8], b1[8], b2[8];  // s, sqrt(s) / (8 pi alpha^1.5), sqrt(s) / (4 pi^1.5 alpha^1.5)
-    R b3[8];               // sqrt(s / (pi alpha))
-    R a1, a2, clin, k8;    // 1 / (8 pi alpha^2), 1 / (2 alpha), 1 / (4 pi alpha), 1 / (8 pi alpha)
+    Num<R> cu[8], icu[8];       // u = r cu, 1/u = icu / r:  cu = 1 / (2 sqrt(alpha s))
+    Num<R> s[8], b1[8], b2[8];  // s, sqrt(s) / (8 pi alpha^1.5), sqrt(s) / (4 pi^1.5 alpha^1.5)
+    Num<R> b3[8];               // sqrt(s / (pi alpha))
+    Num<R> a1, a2, clin, k8;    // 1 / (8 pi alpha^2), 1 / (2 alpha), 1 / (4 pi alpha), 1 / (8 pi alpha)
+    void set(double h, double alpha, int nd)
+    {
+        const double a32 = alpha * sqrt(alpha);
+        for (int k = 0; k < nd; ++k) {
+            const double sk = (k + 1) * h, ss = sqrt(sk);
+            cu[k].set(1.0 / (2.0 * sqrt(alpha) * ss));
+            icu[k].set(2.0 * sqrt(alpha) * ss);
+            s[k].set(sk);
+            b1[k].set(ss / (8.0 * kPi * a32));
+            b2[k].set(ss / (4.0 * kPi * sqrt(kPi) * a32));
+            b3[k].set(ss / sqrt(kPi * alpha));
+        }
+        a1.set(1.0 / (8.0 * kPi * alpha * alpha));
+        a2.set(1.0 / (2.0 * alpha));
+        clin.set(1.0 / (4.0 * kPi * alpha));
+        k8.set(1.0 / (8.0 * kPi * alpha));
+    }
 };
 
 // Time integrals for d = 0 .. ND-1 at distance r: V[d] of the single layer and K[d] of the double
@@ -99,14 +148,14 @@ __device__ __forceinline__ void time_integrals(R r, const TimeConst<R> &c, R *V,
     R d1 = R(0), d2 = R(0), e1 = R(0), e2 = R(0);  // the same of the double layer
 #pragma unroll
     for (int k = 0; k < ND; ++k) {
-        const R u = r * c.cu[k], iu = ir * c.icu[k];
+        const R u = mulc(r, c.cu[k]), iu = mulc(ir, c.icu[k]);
         R ef, efc;
         erf_pair(u, ef, efc);
         const R ex = d_exp(-u * u);
         const bool small = u < R(1);
         if (DOV) {
-            const R t = r * efc * c.a1 - c.b1[k] * erf_over_u(u, ef, iu) - c.b2[k] * ex;
-            const R g = ((c.s[k] + r2 * c.a2) * efc - r * c.b3[k] * ex) * (c.clin * ir);
+            const R t = mulc(r * efc, c.a1) - mulc(erf_over_u(u, ef, iu), c.b1[k]) - mulc(ex, c.b2[k]);
+            const R g = (addc(mulc(r2, c.a2), c.s[k]) * efc - mulc(r, c.b3[k]) * ex) * mulc(ir, c.clin);
             V[k] = k == 0 ? g : (small ? t - t1 - t1 + t2 : g - g1 - g1 + g2);
             g2 = g1;
             g1 = g;
@@ -114,8 +163,8 @@ __device__ __forceinline__ void time_integrals(R r, const TimeConst<R> &c, R *V,
             t1 = t;
         }
         if (DOK) {
-            const R g = ((c.s[k] * ir * ir - c.a2) * efc + c.b3[k] * ex * ir) * (R(1.0 / (4 * kPi)) * ir);
-            const R t = -(R(0.5) * u * phi2(u, ef, ex, iu) + efc) * (c.k8 * ir);
+            const R g = (subc(mulc(ir, c.s[k]) * ir, c.a2) * efc + mulc(ex, c.b3[k]) * ir) * mulc(ir, num<R>(1.0 / (4 * kPi)));
+            const R t = -(R(0.5) * u * phi2(u, ef, ex, iu) + efc) * mulc(ir, c.k8);
             K[k] = k == 0 ? g : (small ? t - e1 - e1 + e2 : g - d1 - d1 + d2);
             d2 = d1;
             d1 = g;
