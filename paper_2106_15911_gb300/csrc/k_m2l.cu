@@ -27,6 +27,10 @@
 // Tasks are dealt to the warps longest first, back and forth.  The parity of k + nu alternates with
 // k, so the accumulators are kept relative to the parity of nu and swapped by addressing when they
 // are written.  Double-FP32 rows hold 64 high then 64 low parts.
+//
+// Folding mixes all cells of a fibre, so where the interaction radius leaves some out, what is not finite would
+// reach them and their zeros would come out as rounding noise: there such moments are folded as zeros and
+// k_m2l_outside settles the cells afterwards.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -113,6 +117,8 @@ __device__ __forceinline__ void step(df64 &acc, df64 a, df64 b)
 }
 __device__ __forceinline__ float norm(float v) { return v; }
 __device__ __forceinline__ df64 norm(df64 v) { return df_fast_two_sum(v.hi, v.lo); }
+__device__ __forceinline__ float head(float v) { return v; }
+__device__ __forceinline__ float head(df64 v) { return v.hi; }
 __device__ __forceinline__ float diff(float a, float b) { return a - b; }
 __device__ __forceinline__ df64 diff(df64 a, df64 b) { return a + (-b); }
 __device__ __forceinline__ float shfl_x(float v, int m) { return __shfl_xor_sync(0xffffffffu, v, m); }
@@ -255,6 +261,13 @@ k_m2l_folded(M2LFoldArgs A, const R *__restrict__ mu, R *__restrict__ lam)
                 v[x][2] = o.z >= 0 ? mi[o.z] : R(0);
                 v[x][3] = o.w >= 0 ? mi[o.w] : R(0);
             }
+            if (A.truncated) {
+#pragma unroll
+                for (int x = 0; x < 4; ++x)
+#pragma unroll
+                    for (int y = 0; y < 4; ++y)
+                        if (!isfinite(head(v[x][y]))) v[x][y] = R(0);
+            }
 #pragma unroll
             for (int y = 0; y < 4; ++y) {
                 const R a0 = v[0][y], a1 = v[1][y], a2 = v[2][y], a3 = v[3][y];
@@ -393,6 +406,56 @@ __global__ void k_m2l_sum_chunks(const R *__restrict__ part, int na, int tpc, si
     R s = R(0);
     for (int t = 0; t < nc; ++t) s += part[(size_t)t * n + i];
     lam[i] = s;
+}
+
+// Locals of a level whose interaction radius leaves cells out: zero where no moment within the radius is other
+// than zero, NaN where one is not finite.  CTA: (target interval, rhs); reads the moments of its one or two source
+// intervals once.  Bound by the latency of these reads: many warps, eight loads each in flight
+constexpr int kOutsideThreads = 1024;
+template <typename R>
+__global__ void __launch_bounds__(kOutsideThreads) k_m2l_outside(const R *__restrict__ mu, R *__restrict__ lam,
+                                                     const int *__restrict__ boxcell, int G, int ntr, int na, int nk, int nint,
+                                                     int nbox)
+{
+    __shared__ int flag[2][512];  // bit 0: a moment that is not zero, bit 1: one that is not finite
+    const int k = blockIdx.x + 2, rhs = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n = na * nk, G3 = G * G * G;
+    for (int i = threadIdx.x; i < G3; i += kOutsideThreads) flag[0][i] = 0;
+    __syncthreads();
+    for (int w = warp; w < nbox * (1 + (k & 1)); w += kOutsideThreads / 32) {
+        const int b = w % nbox;
+        const R *m = mu + (((size_t)rhs * nint + k - 2 - w / nbox) * nbox + b) * n;
+        int f = 0;
+#pragma unroll 8
+        for (int i = lane; i < n; i += 32) {
+            const float v = head(m[i]);
+            f |= isfinite(v) ? (v != 0.f ? 1 : 0) : 3;
+        }
+        f = __reduce_or_sync(0xffffffffu, f);
+        if (lane == 0 && f) atomicOr(&flag[0][boxcell[b]], f);
+    }
+    __syncthreads();
+    for (int dir = 0, st = 1; dir < 3; ++dir, st *= G) {  // the cells within the radius, one direction at a time
+        for (int i = threadIdx.x; i < G3; i += kOutsideThreads) {
+            const int c = i / st % G;
+            int f = 0;
+            for (int o = max(-ntr, -c); o <= min(ntr, G - 1 - c); ++o) f |= flag[dir & 1][i + o * st];
+            flag[~dir & 1][i] = f;
+        }
+        __syncthreads();
+    }
+    for (int b = warp; b < nbox; b += kOutsideThreads / 32) {
+        const int f = flag[1][boxcell[b]];
+        if (f == 1) continue;
+        R *o = lam + (((size_t)rhs * nint + k) * nbox + b) * n;
+        for (int i = lane; i < n; i += 32) o[i] = f ? R(__int_as_float(0x7fffffff)) : R(0);
+    }
+}
+
+template <typename R>
+static void settle_outside(const DevLevel &L, const R *mu, R *lam, int nrhs, const ApplyGeo &g, cudaStream_t st)
+{
+    if (L.ntr < L.G - 1 && L.nint > 2)
+        k_m2l_outside<R><<<dim3(L.nint - 2, nrhs), kOutsideThreads, 0, st>>>(mu, lam, L.boxcell, L.G, L.ntr, g.na, g.nk, L.nint, L.nbox);
 }
 
 // folded coefficients of a level from its FP64 table E1 [D][a][b][o][k][nu] (offsets beyond the
@@ -621,6 +684,7 @@ int launch_m2l_folded(int prec, bool sliced, const DevLevel &L, const M2LFoldDev
     A.ne = g.ne;
     A.nint = L.nint;
     A.nbox = L.nbox;
+    A.truncated = L.ntr < L.G - 1;
     A.p = P;
     A.cellbox = L.cellbox;
     A.EF = L.EF;
@@ -646,6 +710,10 @@ int launch_m2l_folded(int prec, bool sliced, const DevLevel &L, const M2LFoldDev
         else
             k_m2l_sum_chunks<df64><<<blocks, 256, 0, st>>>((const df64 *)ws, g.na, A.tpc, nlev, per_k, L.nint, (df64 *)lam);
     }
+    if (prec == 1)
+        settle_outside(L, (const float *)mu, (float *)lam, nrhs, g, st);
+    else
+        settle_outside(L, (const df64 *)mu, (df64 *)lam, nrhs, g, st);
     return 0;
 }
 
@@ -664,14 +732,15 @@ int launch_m2l_folded(int prec, bool sliced, const DevLevel &L, const M2LFoldDev
 constexpr int kFoldK = 12;
 __global__ void __launch_bounds__(256) k_m2l_fold_moments(const float *__restrict__ mu, const int *__restrict__ cellbox,
                                                           const int *__restrict__ urow, int na, int nk, int nint, int nbox,
-                                                          int J0, int nJ, int r0, float *__restrict__ F)
+                                                          int J0, int nJ, int r0, int truncated, float *__restrict__ F)
 {
     __shared__ float S[kFoldK][8][8][9];  // [k][x][y][z]
     const int J = J0 + blockIdx.x / na, a = blockIdx.x % na, k0 = blockIdx.y * kFoldK, kn = min(kFoldK, nk - k0);
     const float *mJ = mu + (((size_t)(r0 + blockIdx.z) * nint + J) * nbox * na + a) * nk + k0;
     for (int i = threadIdx.x; i < 512 * kFoldK; i += 256) {
         const int c = i / kFoldK, k = i % kFoldK, box = cellbox[c];
-        S[k][c >> 6][(c >> 3) & 7][c & 7] = box >= 0 && k < kn ? mJ[(size_t)box * na * nk + k] : 0.f;
+        const float v = box >= 0 && k < kn ? mJ[(size_t)box * na * nk + k] : 0.f;
+        S[k][c >> 6][(c >> 3) & 7][c & 7] = truncated && !isfinite(v) ? 0.f : v;
     }
     __syncthreads();
 #pragma unroll
@@ -931,6 +1000,7 @@ int launch_m2l_slab_folded(const DevLevel &L, const M2LFoldDev &P, const float *
     A.mx = g.mx;
     A.nint = L.nint;
     A.nbox = L.nbox;
+    A.truncated = L.ntr < L.G - 1;
     A.p = P;
     A.cellbox = L.cellbox;
     A.EF = L.EF;
@@ -945,10 +1015,11 @@ int launch_m2l_slab_folded(const DevLevel &L, const M2LFoldDev &P, const float *
             const int J0 = std::max(0, k0 - 3), nJ = std::max(0, k1 - 2 - J0);
             if (nJ > 0)
                 k_m2l_fold_moments<<<dim3(nJ * g.na, (g.nk + kFoldK - 1) / kFoldK, nr), 256, 0, st>>>(
-                    mu, L.cellbox, P.urow, g.na, g.nk, L.nint, L.nbox, J0, nJ, r0, ws);
+                    mu, L.cellbox, P.urow, g.na, g.nk, L.nint, L.nbox, J0, nJ, r0, A.truncated, ws);
             A.k_lo = k0;
             kf<<<dim3((unsigned)((k1 - k0) * g.na * 2), nr), kSlabThreads, P.smem, st>>>(A, ws, lam, J0, nJ, r0);
         }
+    settle_outside(L, mu, lam, nrhs, g, st);
     return 0;
 }
 

@@ -28,6 +28,7 @@ M2LFoldPlan m2l_slab_plan(int mx, const std::vector<int> &kinv);
 
 struct M2LFoldArgs {
     int na, nk, mx, ne, nint, nbox, tpc, nchunk, k_lo;
+    int truncated;              // the interaction radius leaves cells out: moments that are not finite count as zeros
     M2LFoldDev p;
     const int *cellbox;         // [G^3]
     const float *EF;
