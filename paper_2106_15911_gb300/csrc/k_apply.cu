@@ -188,9 +188,8 @@ __global__ void __launch_bounds__(256) k_nf_apply(const S *__restrict__ A, const
 // (copies through registers took 2.7 ms at the first size below).  FP32 sums over
 // 128 products, added with their rounding errors kept (two FP32: the FP64 unit would be busy for half of the
 // FMAs' time, and sums over 512 products, all offsets in one, came out 20 % further from FP64 than the tiles').
-// Outputs beyond the FP32 range are summed once more in FP64 (nf_direct); the call costs 3 to 5 % at two steps per
-// leaf, whose registers are short, and nothing at others.
-// Bound by the FMAs.  Nearfield, 64 x 64 tiles -> here: 1728 triangles x 1024 steps mixed 8.36 -> 1.18 ms,
+// Outputs beyond the FP32 range are summed once more in FP64 (nf_direct).
+// Bound by the FMAs.  Nearfield, 64 x 64 tiles -> here: 1728 triangles x 1024 steps mixed 8.36 -> 1.20 ms,
 // FP64 134 -> 23.2; 768 x 256, 4 right-hand sides, mixed 0.99 -> 0.38; 192 x 16 FP64 0.79 -> 0.73; 3072 x 128
 // FP64 13.1 -> 11.8; 12288 x 64 mixed 9.0 -> 6.2; three steps per leaf FP64 3.9 -> 2.7; one step mixed, K,
 // 0.127 -> 0.113.
@@ -236,8 +235,13 @@ __device__ __noinline__ void nf_direct(const float *__restrict__ A, const uint16
     }
 }
 
+// CTAs per SM: 32 FP32 outputs a thread do not fit 168 registers beside their loop (with three CTAs 768 triangles x
+// 256 steps, n_tr 2, 4 right-hand sides took 265 instead of 209 us, 3072 x 64 with 2 998 instead of 918; 1728 x 1024
+// 1.19 and 1.20 ms)
+__host__ __device__ constexpr int nf_rows_ctas(size_t size, int ls) { return size == 4 && ls == 2 ? 2 : 3; }
+
 template <typename S, int LS>
-__global__ void __launch_bounds__(128, 3) k_nf_rows(const S *__restrict__ A, const int *__restrict__ colidx,
+__global__ void __launch_bounds__(128, nf_rows_ctas(sizeof(S), LS)) k_nf_rows(const S *__restrict__ A, const int *__restrict__ colidx,
                                                  const int *__restrict__ tiles, const PanelGPU *__restrict__ panels,
                                                  const S *__restrict__ x, int ncolg, int Et, int nint,
                                                  double *__restrict__ f, int nt, int kop, int R, NfHalfSplit hs)
