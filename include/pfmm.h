@@ -113,7 +113,8 @@ typedef struct pfmm_params {
                            the FP64 pipe (reference mode, about 50x slower on GB300) */
     int32_t nf_form;    /* FP64 tensor-core nearfield kernel form: 0 (default) the faster of the two,
                            timed at build; 1 work items of up to 128 leaf intervals; 2 of up to 64
-                           (twice the items, each reading the blocks again) */
+                           (twice the items, each reading the blocks again).  They differ only with more
+                           than 64 leaf intervals and one or two steps per leaf; else 0 is 1, untimed */
 } pfmm_params;
 
 typedef struct pfmm_handle pfmm_handle;

@@ -436,11 +436,14 @@ int pfmm_default_params(pfmm_params *p)
 
 // The faster of the two forms of the FP64 tensor-core nearfield (work items of up to 128 or of up to
 // 64 leaf intervals), timed with CUDA events on this handle's
-// V product of a zero input (the work does not depend on the values).
+// V product of a zero input (the work does not depend on the values).  Handles whose forms are the same kernel
+// keep form 1 untimed.
 static int tune_crt_form(pfmm_handle *H, cudaStream_t st)
 {
     int rc = ensure_workspace(H, 1);
     if (rc) return rc;
+    const int nint = H->Et / H->ls;
+    if (pfmm::nf_crt_intervals(nint, H->ls, 1) == pfmm::nf_crt_intervals(nint, H->ls, 2)) return PFMM_OK;
     double *x = nullptr;
     if ((rc = H->alloc(&x, (size_t)H->Et * H->nt))) return rc;
     CK(cudaMemsetAsync(x, 0, sizeof(double) * H->Et * H->nt, st));
