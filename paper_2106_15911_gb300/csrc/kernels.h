@@ -138,7 +138,9 @@ void launch_m2m(int prec, const DevLevel &par, const DevLevel &ch, int l, const 
 // three-pass level does not fit it
 int launch_m2l_levels(int prec, const DevLevel *dl, int p, const void *mu, void *lam, int nrhs, const ApplyGeo &g, void *T1,
                       void *T2, size_t ws_elems, cudaStream_t st);
-// M2L kernel of a level with a G^3 grid (launch_m2l_levels' choice): only kM2LThreePass uses T1 / T2
+// M2L kernel of a level with a G^3 grid (launch_m2l_levels' choice).  kM2LThreePass needs T1 and T2; the others
+// take T1 where it is large enough: the fused kernels for a launch by source terms, the slab kernel for its
+// folded moments (else it runs unfolded)
 enum { kM2LThreePass = 0, kM2LFused = 1, kM2LSlab = 2, kM2LFusedSliced = 3 };
 int m2l_engine(int prec, int G, int nk, int ne, int mx);
 // the engine of a level when an autotuner asks for `force` (a PFMM_M2L_* code; 0: none): the forced

@@ -74,23 +74,28 @@ extern "C" int pfmm_apply_V_noalloc(pfmm_handle *H, const double *w, double *f, 
     const size_t b_w = tc ? up256((size_t)nrhs * H->Et * H->colsV_u * sizeof(uint16_t)) : 0;
     const size_t b_m = tc ? up256((size_t)nrhs * sizeof(unsigned long long)) : 0;
     int planes = tc ? nf_tc_planes(H, 0, nrhs) : 0;  // fewer where the array is short of room
-    // elements of T1 (and of T2) for the largest single-interval chunk of the levels whose M2L
-    // takes the three separable passes (the fused and slab kernels keep their intermediates in
-    // shared memory; the fused kernel's split mode and the two-stage S2M / L2T use T1 only when
-    // it is large enough and fall back otherwise)
-    size_t need_T = 0;
+    // need_T: elements of T1 (and of T2) for the largest single-interval chunk of the levels whose M2L
+    // takes the three separable passes.  want_T: elements of T1 for the folded moments of 16 target
+    // intervals of an 8^3 level, which go before further planes: with fewer than one interval's the level
+    // takes the unfolded kernel, at five times the time.  The two-stage S2M / L2T and the M2L's launches
+    // by source term use T1 where it is large enough
+    size_t need_T = 0, want_T = 0;
     for (int l = 2; l <= H->p; ++l) {
         const DevLevel &L = H->dl[l];
-        if (m2l_engine_for(H->fprec, L.G, H->nk, H->ne, H->mx, H->m2l_force) != kM2LThreePass) continue;
+        const int engine = m2l_engine_for(H->fprec, L.G, H->nk, H->ne, H->mx, H->m2l_force);
+        if (engine == kM2LSlab && H->fold[2].units)
+            want_T = std::max(want_T, (size_t)(std::min(L.nint, 16) + 1) * 512 * H->na * H->nk);
+        if (engine != kM2LThreePass) continue;
         int maxpairs = 0;
         for (int k = 0; k < L.nint; ++k) maxpairs = std::max(maxpairs, L.kptr_host[k + 1] - L.kptr_host[k]);
         need_T = std::max(need_T, (size_t)nrhs * maxpairs * H->na * H->na * L.G * L.G * L.G * H->ne);
     }
+    const int nT = need_T ? 2 : 1;  // T2: three passes only
     size_t b_p = 0, fixed = 0;
     for (;; --planes) {
         b_p = up256((size_t)planes * n_in * sizeof(double));
         fixed = b_x + b_f + 2 * b_mu + 2 * b_w + b_m + b_p;
-        if (planes <= 1 || fixed + 2 * up256(need_T * H->es) <= kScratchBytes) break;
+        if (planes <= 1 || fixed + nT * up256(std::max(need_T, want_T) * H->es) <= kScratchBytes) break;
     }
     if (fixed + 2 * up256(need_T * H->es) > kScratchBytes)
         return set_error(PFMM_ERR_OOM, "pfmm_apply_V_noalloc needs " + std::to_string(fixed + 2 * up256(need_T * H->es)) +
@@ -106,8 +111,8 @@ extern "C" int pfmm_apply_V_noalloc(pfmm_handle *H, const double *w, double *f, 
     void *whi = lam + b_mu, *wlo = lam + b_mu + b_w;
     unsigned long long *wmax = (unsigned long long *)(lam + b_mu + 2 * b_w);
     double *part = (double *)(lam + b_mu + 2 * b_w + b_m);
-    const size_t t_bytes = (kScratchBytes - fixed) / 2 / 256 * 256;
-    void *T1 = base + fixed, *T2 = base + fixed + t_bytes;
+    const size_t t_bytes = (kScratchBytes - fixed) / nT / 256 * 256;
+    void *T1 = base + fixed, *T2 = base + fixed + (nT - 1) * t_bytes;
     const size_t ws_elems = t_bytes / H->es;
 
     ApplyGeo g{};

@@ -47,6 +47,33 @@ def test_noalloc_matches_apply_V_on_two_calls(precision, n_a, Et, kw):
     op.close()
 
 
+def test_noalloc_leaves_room_for_the_folded_moments_of_8_cubed_levels():
+    # tensor-core nearfield that would fill the array with nine partial planes
+    V, T = cube_mesh(12)
+    op = P.Operator(V, T, 1.0, 128, precision=P.PFMM_MIXED, m_t=4, m_x=4, c_st=0.1, n_tr=7, quad_regular=1, quad_singular=2)
+    info = op.info()
+    assert info["nf_tensor_cores"] & 1 and P.PFMM_M2L_SLAB in info["m2l_engine"]
+    w = torch.tensor(random_density(128, len(T), 1, seed=3), device=DEV)
+    ref, out = torch.empty_like(w), torch.empty_like(w)
+
+    def ms(f):
+        t = []
+        for _ in range(6):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            f()
+            b.record()
+            torch.cuda.synchronize()
+            t.append(a.elapsed_time(b))
+        return min(t)
+
+    t0, t1 = ms(lambda: P.pfmm_apply_V(op.h, w, ref, 1)), ms(lambda: P.pfmm_apply_V_noalloc(op.h, w, out, 1))
+    # one and nine chunks of the columns: FP32 sums of up to 2048 products, sqrt(2048) 2^-24 = 2.7e-6 each
+    assert float((out - ref).abs().max() / ref.abs().max()) <= 5.4e-6
+    assert t1 <= 2 * t0, (t1, t0)  # the unfolded kernel takes five times the far field's time
+    op.close()
+
+
 def test_noalloc_rejects_workspaces_beyond_the_static_array():
     V, T = cube_mesh(4)
     Et, nrhs = 16, 4096  # 4096 x 16 x 192 FP64 values: ~100 MB of workspace
