@@ -179,6 +179,12 @@ int pfmm_apply_M(pfmm_handle *h, const double *g, double *f, int32_t nrhs, void 
 int pfmm_apply_parts(pfmm_handle *h, int32_t op, const double *x, double *f, int32_t nrhs, int32_t parts,
                      void *stream);
 
+/* Measurement utility: the nearfield engine of a handle whose parameters let it use the tensor cores:
+ * PFMM_NF_CUDA_CORES runs the products on the CUDA cores from the blocks that the handle holds (the
+ * choice that the batch autotuner makes by time; in mixed precision the blocks are then the sums of
+ * their two FP16 parts), PFMM_NF_AUTO goes back.  Batches capture the choice at their next new call. */
+int pfmm_set_nf_engine(pfmm_handle *h, int32_t engine);
+
 /* Per-phase device times.  When enabled, every apply records CUDA events around its phases on
  * its stream; pfmm_phase_times synchronises the last apply's stream, writes the accumulated
  * milliseconds of the phases (0 permute in, 1 nearfield, 2 S2M, 3 M2M, 4 M2L, 5 L2L, 6 L2T,

@@ -1038,6 +1038,14 @@ int pfmm_apply_parts(pfmm_handle *h, int32_t op, const double *x, double *f, int
     return apply_impl(h, op, x, f, nrhs, parts, (cudaStream_t)stream);
 }
 
+int pfmm_set_nf_engine(pfmm_handle *h, int32_t engine)
+{
+    if (!h || (engine != PFMM_NF_AUTO && engine != PFMM_NF_CUDA_CORES))
+        return fail(PFMM_ERR_INVALID_ARG, "invalid pfmm_set_nf_engine arguments");
+    h->nf_cuda_cores = engine == PFMM_NF_CUDA_CORES;
+    return PFMM_OK;
+}
+
 int pfmm_count_apply_kernels(pfmm_handle *h, int32_t op, const double *x, double *f, int32_t nrhs, int32_t parts,
                              int64_t *kernels)
 {

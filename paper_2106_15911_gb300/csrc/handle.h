@@ -90,7 +90,7 @@ struct pfmm_handle {
 
     // tensor-core nearfield (mixed mode, untruncated panels of equal width, 2 steps per leaf)
     bool tcV = false, tcK = false;
-    bool nf_cuda_cores = false;     // engine override chosen by the batch autotuner
+    bool nf_cuda_cores = false;     // engine override: the batch autotuner's choice, or pfmm_set_nf_engine
     pfmm::M2LFoldDev fold[3]{};     // unit tables of the folded M2L: 4^3 with T2 whole, sliced; 8^3
     int m2l_force = 0;              // M2L engine chosen by the batch autotuner (PFMM_M2L_* code, 0: per-level default)
     uint16_t *d_AVsplit = nullptr, *d_AKsplit = nullptr;  // FP16 parts (nf_split_index)

@@ -87,6 +87,7 @@ SIGNATURES = {
     "pfmm_apply_V_noalloc": (ctypes.c_int, [_VP, _DP, _DP, _I, _VP]),
     "pfmm_set_profiling": (ctypes.c_int, [_VP, _I]),
     "pfmm_phase_times": (ctypes.c_int, [_VP, ctypes.POINTER(ctypes.c_double), ctypes.POINTER(ctypes.c_int32)]),
+    "pfmm_set_nf_engine": (ctypes.c_int, [_VP, _I]),
     "pfmm_nf_kernel_time": (ctypes.c_int, [_VP, ctypes.POINTER(ctypes.c_double), ctypes.POINTER(ctypes.c_int32)]),
     "pfmm_get_info": (ctypes.c_int, [_VP, ctypes.POINTER(pfmm_info)]),
     "pfmm_gen_create": (ctypes.c_int, [ctypes.POINTER(pfmm_mesh), ctypes.POINTER(ctypes.c_double),
@@ -278,6 +279,11 @@ def pfmm_count_apply_kernels(h, op: int, x, f, nrhs: int, parts: int = PFMM_PART
     n = ctypes.c_int64()
     _check(lib().pfmm_count_apply_kernels(h, int(op), _ptr(x), _ptr(f), int(nrhs), int(parts), ctypes.byref(n)))
     return n.value
+
+
+def pfmm_set_nf_engine(h, engine: int):
+    """Nearfield engine of a handle with tensor-core panels: PFMM_NF_CUDA_CORES or PFMM_NF_AUTO."""
+    _check(lib().pfmm_set_nf_engine(h, int(engine)))
 
 
 def pfmm_set_profiling(h, on: bool):

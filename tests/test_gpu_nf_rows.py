@@ -1,5 +1,5 @@
 """The CUDA-core nearfield (8 rows of a panel per CTA, 32 to 256 leaf intervals, columns two stages at a
-time) on panels of their own columns, against the oracle's nearfield: one to four steps per leaf, interval
+time), from the FP16 parts of a tensor-core handle against its tensor-core product and the FP32 panels, and on panels of their own columns, against the oracle's nearfield: one to four steps per leaf, interval
 counts of one, below and past a CTA's, panels of fewer than 8 rows and of several groups."""
 import numpy as np
 import pytest
@@ -37,6 +37,35 @@ def test_nearfield_rows_match_oracle(precision, mesh, n_a, ls, nint, nrhs, c_st)
             ref = O.pfmm_apply(Pr, k, w[r], targets=rows, parts=P.PFMM_PART_NEAR)[:, rows]
             assert np.max(np.abs(out[r][:, rows] - ref)) <= tol * np.max(np.abs(ref))
     op.close()
+
+
+@pytest.mark.parametrize("mesh,n_a,Et,nrhs", [
+    (cube_mesh, 1, 2, 1),          # 12 rows: 8 and 4; one interval
+    (cube_mesh, 2, 64, 2),         # 48 rows: six times 8
+    (cube_sphere_mesh, 4, 16, 3),  # 192 rows: a tile of 128 and a half
+    (cube_sphere_mesh, 5, 512, 1), # 300 rows: two tiles and 44 = 5 times 8 and 4; 256 intervals
+])
+def test_rows_from_the_fp16_parts(mesh, n_a, Et, nrhs):
+    # the blocks of a mixed handle on the tensor cores exist as FP16 parts only
+    V, T = mesh(n_a)
+    kw = dict(m_t=2, m_x=2, quad_regular=2, quad_singular=2, precision=P.PFMM_MIXED)
+    op, panels = P.Operator(V, T, 1.0, Et, **kw), P.Operator(V, T, 1.0, Et, nf_engine=P.PFMM_NF_CUDA_CORES, **kw)
+    assert op.info()["nf_tensor_cores"] == 3
+    for k, (call, n) in enumerate((("V", len(T)), ("K", len(V)))):
+        x = torch.tensor(random_density(Et, n, nrhs, seed=9), device=DEV)
+        P.pfmm_set_nf_engine(op.h, P.PFMM_NF_AUTO)
+        tc = getattr(op, call)(x, parts=P.PFMM_PART_NEAR)
+        P.pfmm_set_nf_engine(op.h, P.PFMM_NF_CUDA_CORES)
+        got = getattr(op, call)(x, parts=P.PFMM_PART_NEAR)
+        ref = getattr(panels, call)(x, parts=P.PFMM_PART_NEAR)
+        # the parts hold a block to 2^-22, a row's sums are the same FP32 ones; the tensor cores also round the input
+        # to two parts and sum in another order
+        assert float((got - ref).abs().max()) <= 1e-6 * float(ref.abs().max())
+        assert float((got - tc).abs().max()) <= 1e-5 * float(ref.abs().max())
+        # three kernels instead of six
+        assert P.pfmm_count_apply_kernels(op.h, k, x, torch.empty_like(ref), nrhs, P.PFMM_PART_NEAR) == 3
+    for h in (op, panels):
+        h.close()
 
 
 @pytest.mark.parametrize("ls,n_a", [(1, 8), (2, 8), (3, 6), (4, 6)])
