@@ -144,7 +144,8 @@ typedef struct pfmm_info {
 /* M2L kernels (pfmm_info.m2l_engine): the three separable passes through a global workspace
  * (grids beyond 8^3, high degrees, native FP64), the fused kernels (grids of at most 4^3 cells, FP32
  * m_x <= 7 or double-FP32 m_x <= 6; the 4^3 grid in even and odd parts per direction), the slab
- * kernels (FP32, grids of 5^3 .. 8^3 cells, m_x <= 6; the 8^3 grid in even and odd parts). */
+ * kernels (FP32, grids of 8^3 cells, m_x <= 6; in even and odd parts too).  Grids have 2^n cells per
+ * direction. */
 #define PFMM_M2L_THREE_PASS 1
 #define PFMM_M2L_FUSED 2
 #define PFMM_M2L_SLAB 3

@@ -91,95 +91,8 @@ void launch_to_df64(double *x, size_t n, cudaStream_t st)
 // of uniform steps: for target step t = k*ls + s of leaf interval k the temporal nearfield
 // N(I_k) = {I_{k-1}, I_k} contributes the step offsets d = 0 .. ls + s, so
 //   f[t][rows of X] = sum_{d=0}^{ls+s} A_d[X] x[t - d][cols of X].
-// k_nf_apply, for more than four steps per leaf: one CTA computes a 64 x 64 tile (64 rows of a panel x 64 steps of one phase s) over all d
-// and all columns, so every output element is written exactly once.
-template <typename S>
-__global__ void __launch_bounds__(256) k_nf_apply(const S *__restrict__ A, const int *__restrict__ colidx,
-                                                    const int *__restrict__ tiles, const PanelGPU *__restrict__ panels,
-                                                    const S *__restrict__ x, int ncolg, int Et, int ls, int nint,
-                                                    double *__restrict__ f, int nt, int kop)
-{
-    constexpr int BM = 64, BN = 64, BK = 16;
-    constexpr bool kFloat = sizeof(S) == 4;
-    __shared__ S As[BK][BM + 1];
-    __shared__ S Ws[BK][BN + 1];
-    const int tid = threadIdx.x;
-    const int rg = tid & 15, cg = tid >> 4;
-    const PanelGPU P = panels[tiles[2 * blockIdx.x]];
-    const int r0 = tiles[2 * blockIdx.x + 1];
-    const int s = blockIdx.y % ls, ib = blockIdx.y / ls;
-    const int rhs = blockIdx.z;
-    const S *xr = x + (size_t)rhs * Et * ncolg;
-    const int *cols = colidx + (kop ? P.colK_at : P.colV_at);
-    const int ncp = kop ? P.colsK_pad : P.colsV_pad;
-    const size_t off = kop ? P.offK : P.offV;
-    S acc[4][4];
-    double accd[4][4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            acc[i][j] = S(0);
-            accd[i][j] = 0.0;
-        }
-    const int nd = ls + s + 1;
-    int ktiles = 0;
-    for (int d = 0; d < nd; ++d) {
-        const size_t dbase = off + ((size_t)d * P.rows_pad + r0) * ncp;
-        for (int k0 = 0; k0 < ncp; k0 += BK) {
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                int e = tid + 256 * q;
-                int i = e >> 4, j = e & 15;
-                As[j][i] = A[dbase + (size_t)i * ncp + k0 + j];
-                int c = e >> 4;
-                int t = ((ib * BN + c) * ls + s);
-                int col = cols[k0 + j];
-                S v = S(0);
-                if (col >= 0 && ib * BN + c < nint && t - d >= 0) v = xr[(size_t)(t - d) * ncolg + col];
-                Ws[j][c] = v;
-            }
-            __syncthreads();
-#pragma unroll
-            for (int j = 0; j < BK; ++j) {
-                S a[4], b[4];
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    a[q] = As[j][rg + 16 * q];
-                    b[q] = Ws[j][cg + 16 * q];
-                }
-#pragma unroll
-                for (int qi = 0; qi < 4; ++qi)
-#pragma unroll
-                    for (int qj = 0; qj < 4; ++qj) acc[qi][qj] += a[qi] * b[qj];
-            }
-            __syncthreads();
-            if (kFloat && ++ktiles == 32) {  // FP32 partial sums over 512 columns, then FP64
-                ktiles = 0;
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        accd[i][j] += (double)acc[i][j];
-                        acc[i][j] = S(0);
-                    }
-            }
-        }
-    }
-#pragma unroll
-    for (int qj = 0; qj < 4; ++qj) {
-        int iv = ib * BN + cg + 16 * qj;
-        if (iv >= nint) continue;
-        int t = iv * ls + s;
-#pragma unroll
-        for (int qi = 0; qi < 4; ++qi) {
-            int row = r0 + rg + 16 * qi;
-            if (row < P.nrows) f[((size_t)rhs * Et + t) * nt + P.row0 + row] = accd[qi][qj] + (double)acc[qi][qj];
-        }
-    }
-}
-
-// The same product, all step offsets, 8 rows of a panel per CTA.  64 x 64 tiles left 90 % padding on panels
+//
+// k_nf_rows: all step offsets, 8 rows of a panel per CTA.  64 x 64 tiles left 90 % padding on panels
 // of few rows (leaf boxes of an 8^3 grid on 1728 triangles hold 4 to 8), read as much from shared memory as
 // they multiplied, and staged the inputs once per offset.  Here a thread owns two leaf intervals (one at
 // LS > 2) with all their LS steps, so a column's 2 LS inputs of the interval and the one before it serve
@@ -406,16 +319,16 @@ static void launch_nf_rows(const S *A, bool kop, const int *colidx, const int *t
 }
 
 template <typename S>
-static bool launch_nf_rows_ls(const S *A, bool kop, const int *colidx, const int *tiles, int ntiles,
+static void launch_nf_rows_ls(const S *A, bool kop, const int *colidx, const int *tiles, int ntiles,
                               const PanelGPU *panels, const S *x, int ncolg, int nrhs, const ApplyGeo &g, double *f,
                               const NfHalfSplit *hs, cudaStream_t st)
 {
     switch (g.ls) {
-    case 1: launch_nf_rows<S, 1>(A, kop, colidx, tiles, ntiles, panels, x, ncolg, nrhs, g, f, hs, st); return true;
-    case 2: launch_nf_rows<S, 2>(A, kop, colidx, tiles, ntiles, panels, x, ncolg, nrhs, g, f, hs, st); return true;
-    case 3: launch_nf_rows<S, 3>(A, kop, colidx, tiles, ntiles, panels, x, ncolg, nrhs, g, f, hs, st); return true;
-    case 4: launch_nf_rows<S, 4>(A, kop, colidx, tiles, ntiles, panels, x, ncolg, nrhs, g, f, hs, st); return true;
-    default: return false;
+    case 1: launch_nf_rows<S, 1>(A, kop, colidx, tiles, ntiles, panels, x, ncolg, nrhs, g, f, hs, st); break;
+    case 2: launch_nf_rows<S, 2>(A, kop, colidx, tiles, ntiles, panels, x, ncolg, nrhs, g, f, hs, st); break;
+    case 3: launch_nf_rows<S, 3>(A, kop, colidx, tiles, ntiles, panels, x, ncolg, nrhs, g, f, hs, st); break;
+    case 4: launch_nf_rows<S, 4>(A, kop, colidx, tiles, ntiles, panels, x, ncolg, nrhs, g, f, hs, st); break;
+    default: break;  // a handle has no more than four steps per leaf
     }
 }
 
@@ -553,21 +466,13 @@ void launch_nf_apply(bool mixed, bool kop, const void *A, const int *colidx, con
                                      f_int, nullptr, st);
         return;
     }
-    // up to four steps per leaf: k_nf_rows, at 4 to 90 rows a panel and 8 to 512 intervals never behind the
-    // 64 x 64 tiles (k_nf_rows has the figures).  The FP16 parts exist at two steps per leaf only
-    if (mixed ? launch_nf_rows_ls<float>((const float *)A, kop, colidx, tiles, ntiles, panels, (const float *)x, ncolg, nrhs,
-                                         g, f_int, hs, st)
-              : launch_nf_rows_ls<double>((const double *)A, kop, colidx, tiles, ntiles, panels, (const double *)x, ncolg,
-                                          nrhs, g, f_int, nullptr, st))
-        return;
-    int nint = g.Et / g.ls;
-    dim3 grd(ntiles, g.ls * ((nint + 63) / 64), nrhs);
+    // the FP16 parts exist at two steps per leaf only
     if (mixed)
-        k_nf_apply<float><<<grd, 256, 0, st>>>((const float *)A, colidx, tiles, panels, (const float *)x, ncolg, g.Et,
-                                               g.ls, nint, f_int, g.nt, kop ? 1 : 0);
+        launch_nf_rows_ls<float>((const float *)A, kop, colidx, tiles, ntiles, panels, (const float *)x, ncolg, nrhs, g, f_int, hs,
+                                 st);
     else
-        k_nf_apply<double><<<grd, 256, 0, st>>>((const double *)A, colidx, tiles, panels, (const double *)x, ncolg,
-                                                g.Et, g.ls, nint, f_int, g.nt, kop ? 1 : 0);
+        launch_nf_rows_ls<double>((const double *)A, kop, colidx, tiles, ntiles, panels, (const double *)x, ncolg, nrhs, g, f_int,
+                                  nullptr, st);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -1472,7 +1377,8 @@ __global__ void k_m2l_sum_terms(const __grid_constant__ M2LCoarse M, const R *__
     lam_all[M.mom[lv] + i] = s;
 }
 
-// M2L for grids of 5^3 .. 8^3 cells (FP32), one CTA per (target interval k, time node b, target
+// M2L for grids of 8^3 cells (FP32) where the scratch array does not hold the folded moments of one interval
+// (k_m2l_slab_folded takes a fifth of the time), one CTA per (target interval k, time node b, target
 // x-slab X1, rhs) over all source terms (J, a) of the interaction list.  The three directional
 // passes of k_m2l_fused restricted to one X1: pass 1 streams the source x-slabs Y1 within the
 // interaction radius through shared memory (the moments of one slab, cells (Y2, Y3)) and adds
@@ -1674,7 +1580,7 @@ size_t m2l_fused_smem(int G, int nk, int ne, int mx, size_t es, bool sliced)
 // Which M2L kernel a level takes (prec: 0 FP64, 1 FP32, 2 double-FP32): the fused kernel for FP32
 // grids of at most 4^3 cells whose intermediates fit its shared memory (m_x <= 7; double-FP32:
 // m_x <= 6 at one CTA per SM), the slab kernel
-// for FP32 grids of 5^3 .. 8^3 cells with m_x <= 6 (its per-thread arrays and shared memory are
+// for FP32 grids of 8^3 cells with m_x <= 6 (its per-thread arrays and shared memory are
 // sized for that), else the three separable passes through the global workspace (the 8-byte
 // formats, larger grids or degrees).  FP32 degrees whose full T2 does not fit the fused kernel
 // (m_x = 8) take its sliced form (T2 one nu1 value at a time).
@@ -1788,19 +1694,19 @@ static int launch_m2l(int prec, const DevLevel &L, const void *mu, void *lam, in
     int rc = 0;
     dispatch_prec(prec, [&](auto tag) {
         using R = decltype(tag);
-        if (engine == kM2LSlab) {
-            if constexpr (std::is_same<R, float>::value) {
+        if constexpr (std::is_same<R, float>::value) {
+            if (engine == kM2LSlab) {
                 rc = launch_m2l_slab_folded(L, g.fold[2], (const R *)mb, (R *)lb, nrhs, g, (R *)T1, ws_elems, st);
                 if (rc <= 0) return;
                 rc = 0;  // no room for the folded moments
+                const size_t ssm = m2l_slab_smem(g.nk, g.ne, g.mx, es);
+                M2LArgs A{L.G, L.ntr, na, g.nk, g.mx, g.ne, L.nint, L.nbox, L.cellbox, L.boxcell, L.pk, L.pJ, 0,
+                          g.kidx, g.kinv, g.eoff};
+                cudaFuncSetAttribute(k_m2l_slab<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ssm);
+                k_m2l_slab<R><<<dim3((unsigned)(L.nint * na * L.G), nrhs), kM2LSlabThreads, ssm, st>>>(
+                    A, (const R *)mb, (const R *)L.E1, (const R *)L.pref, (R *)lb);
+                return;
             }
-            const size_t ssm = m2l_slab_smem(g.nk, g.ne, g.mx, es);
-            M2LArgs A{L.G, L.ntr, na, g.nk, g.mx, g.ne, L.nint, L.nbox, L.cellbox, L.boxcell, L.pk, L.pJ, 0,
-                      g.kidx, g.kinv, g.eoff};
-            cudaFuncSetAttribute(k_m2l_slab<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ssm);
-            k_m2l_slab<R><<<dim3((unsigned)(L.nint * na * L.G), nrhs), kM2LSlabThreads, ssm, st>>>(
-                A, (const R *)mb, (const R *)L.E1, (const R *)L.pref, (R *)lb);
-            return;
         }
         const size_t per_pair = (size_t)nrhs * na * na * G3 * g.ne;
         // intervals 0 and 1 have no interaction list: their locals start at zero

@@ -222,7 +222,7 @@ __global__ void __launch_bounds__(kCrtThreads, 1) k_nf_apply_crt(const __grid_co
     const int nib = (P.nint + NI - 1) / NI;
     // each wait is bounded by about 2 s; the abort flag ends the other roles' loops
     auto wait = [&](uint64_t *bar, uint32_t parity, int code) {
-        if (mbar_wait_bounded<true>(bar, parity)) return true;
+        if (mbar_wait_bounded(bar, parity)) return true;
         atomicExch(P.err, code);
         s_abort = 1;
         return false;

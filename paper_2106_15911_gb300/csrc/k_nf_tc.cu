@@ -182,7 +182,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_nf_apply_tc(const __grid_cons
     const uint32_t tmem = *tmem_slot;
     const int nib = (P.nint + NI - 1) / NI;
     auto wait = [&](uint64_t *bar, uint32_t parity, int code) {
-        if (mbar_wait_bounded<true>(bar, parity)) return true;
+        if (mbar_wait_bounded(bar, parity)) return true;
         atomicExch(P.err, code);
         s_abort = 1;
         return false;
@@ -208,7 +208,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_nf_apply_tc(const __grid_cons
                 }
             }
             // before the CTA exits, the copies it issued must have landed (bounded wait)
-            for (int j = (g > NW ? g - NW : 0); j < g; ++j) mbar_wait_bounded<true>(&wfull[j % NW], (j / NW) & 1);
+            for (int j = (g > NW ? g - NW : 0); j < g; ++j) mbar_wait_bounded(&wfull[j % NW], (j / NW) & 1);
         }
     } else if (warp == 2) {
         // ---------------- bulk copies of A: hi and lo of one offset per slot
@@ -224,7 +224,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_nf_apply_tc(const __grid_cons
                     bulk_copy(sA + s * A_SLOT, src, A_SLOT, &afull[s]);
                 }
             }
-            for (int j = (g > NA ? g - NA : 0); j < g; ++j) mbar_wait_bounded<true>(&afull[j % NA], (j / NA) & 1);
+            for (int j = (g > NA ? g - NA : 0); j < g; ++j) mbar_wait_bounded(&afull[j % NA], (j / NA) & 1);
         }
     } else if (warp == 1) {
         // ---------------- MMA issuer

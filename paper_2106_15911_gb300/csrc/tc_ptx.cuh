@@ -48,26 +48,18 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *b, uint32_t parity, uint64_t
 }
 
 // bounded wait whose clock starts at the first failed try (reading %globaltimer before every wait
-// costs more than most waits): false after about 2 s (2^32 SM cycles).  POLL: test without sleeping,
-// for the waits that a pipeline's rate hangs on; else tries that may sleep
-template <bool POLL>
+// costs more than most waits): false after about 2 s (2^32 SM cycles).  It tests without sleeping, for the
+// waits that a pipeline's rate hangs on
 __device__ __forceinline__ bool mbar_wait_bounded(uint64_t *b, uint32_t parity)
 {
     uint32_t ok = 0;
     long long t0 = 0;
     while (true) {
-        if (POLL)
-            asm volatile(
-                "{\n\t.reg .pred p;\n\tmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-                : "=r"(ok)
-                : "r"(su32(b)), "r"(parity)
-                : "memory");
-        else
-            asm volatile(
-                "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-                : "=r"(ok)
-                : "r"(su32(b)), "r"(parity)
-                : "memory");
+        asm volatile(
+            "{\n\t.reg .pred p;\n\tmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+            : "=r"(ok)
+            : "r"(su32(b)), "r"(parity)
+            : "memory");
         if (ok) return true;
         const long long t = clock64();
         if (t0 == 0) t0 = t;

@@ -108,7 +108,7 @@ def test_mixed_precision_within_1e5_of_fp64_oracle():
     (cube_mesh, 12, 32, dict(m_t=4, m_x=6, c_st=0.1)),                # 8^3 at the leaf level; radius 7
 ])
 def test_mixed_m2l_on_8_cubed_grids_matches_fp64(mesh, n_a, Et, kw):
-    """Levels with 5^3 .. 8^3 cells run the slab M2L in mixed precision (one CTA per target
+    """Levels with 8^3 cells run the slab M2L in mixed precision (one CTA per target
     x-slab); the FP64 handle runs the three-pass kernels.  The far field (S2M .. L2T) of the two
     agrees to FP32 accuracy, for V and K and two right-hand sides."""
     V, T = mesh(n_a)
