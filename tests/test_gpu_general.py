@@ -26,6 +26,11 @@ def _random_steps(E, seed):
     return np.concatenate([[0.0], np.cumsum(h)]) / h.sum()
 
 
+def _oracle(V, T, ts, kw):
+    names = dict(quad_regular="n_r", quad_singular="n_s")
+    return O.make_general_problem(V, T, ts, **{names.get(k, k): v for k, v in kw.items()})
+
+
 def _rel(a, b):
     return np.max(np.abs(a - b)) / np.max(np.abs(b))
 
@@ -36,6 +41,7 @@ CASES = [
     (cube_mesh, 4, _graded(32, 1.5), 60, dict(m_t=4, m_x=4), 4, True),
     (cube_mesh, 4, _random_steps(24, 5), 40, dict(m_t=3, m_x=5), 4, True),
     (cube_mesh, 8, _graded(16, 2.0), 200, dict(m_t=4, m_x=6), 16, True),
+    (cube_mesh, 8, _graded(32, 1.5), 200, dict(m_t=4, m_x=6, quad_regular=1, quad_singular=2), 8, True),
     (cube_mesh, 4, np.linspace(0.0, 1.0, 33), 100, dict(m_t=4, m_x=4, c_st=0.25), 4, False),
     (cube_sphere_mesh, 4, _graded(24, 2.5), 48, dict(m_t=4, m_x=4, c_st=0.5), 4, True),
 ]
@@ -45,7 +51,7 @@ CASES = [
 def test_general_tree_matches_oracle(mesh, n_a, ts, n_max, kw, stride, early):
     V, T = mesh(n_a)
     op = P.GeneralOperator(V, T, ts, n_max, **kw)
-    Pr = O.make_general_problem(V, T, ts, **kw)
+    Pr = _oracle(V, T, ts, kw)
     ref = O.gen_tree_info(Pr, n_max, boxes=True)
     got = op.info()
     for k in ("nlev", "lx", "nbox", "nleaf", "nint", "ntr_far", "ntr_near"):
@@ -66,7 +72,7 @@ def test_general_apply_matches_oracle(mesh, n_a, ts, n_max, kw, stride, early):
     info = op.info()
     assert info["nlev"] >= 3
     assert (sum(1 for n in info["nleaf"] if n > 0) >= 2) == early  # leaves on several levels
-    Pr = O.make_general_problem(V, T, ts, **kw)
+    Pr = _oracle(V, T, ts, kw)
     w = random_density(E, T.shape[0], 2, seed=91)
     wt = torch.tensor(w, device=DEV)
     near = op.V(wt, parts=P.PFMM_PART_NEAR).cpu().numpy()
