@@ -80,7 +80,7 @@ void launch_space_tables(const SetupArgs &a, cudaStream_t st)
 // E1 tables of one level: thread per (D, a, b, o, k, l).  E_{k,l}(-r) = (-1)^{k+l} E_{k,l}(r) holds
 // exactly in the table (the value of the offset's mirror image with its sign, 0 for o = 0 and odd
 // k + l): the folded M2L relies on it, and the double layer's far field amplifies the asymmetry that
-// rounding leaves otherwise about a hundredfold (1.3e-13; both tables are 4e-13 from exact ones)
+// rounding leaves otherwise about a hundredfold (1.3e-13; either table leaves it 3.5e-13 from exact ones)
 __global__ void k_e1_table(int na, int mt, int mx, int G, double hx, double hxp, double ht, double alpha,
                            double *__restrict__ E1, double *__restrict__ pref)
 {
