@@ -592,7 +592,7 @@ __global__ void k_row_exps(const unsigned long long *__restrict__ rowmax, int nt
 // outputs of each interval (whose products read it and the one before), win = the scale exponent of the rhs's
 // largest |x|, or of the two intervals' where that is more than kCrtSlack binary orders smaller; bit 0 of win
 // tells of values that are not finite.  shared of a tile of ni intervals: the exponent never changes.
-// ticket is zero between launches.  With the split that follows 1 to 4 us more than one scale per rhs took
+// ticket is zero between products.  With the split that follows 1 to 4 us more than one scale per rhs took
 // (12288 triangles x 256 steps: product 4.43 -> 4.45 ms)
 constexpr int kCrtSlack = 2;
 __global__ void __launch_bounds__(256) k_crt_scales(CrtInput in, int nsplit, int ni)
@@ -705,6 +705,7 @@ __global__ void k_crt_combine(const unsigned char *__restrict__ res, size_t per_
 {
     const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= per_mod) return;
+    if (i == 0) *in.ticket = 0u;  // whatever overlapped: the next product's scales count from zero
     float acc[kCrtModuli], v[kCrtModuli];
 #pragma unroll
     for (int k = 0; k < kCrtModuli; ++k) acc[k] = 0.f;
@@ -733,7 +734,7 @@ __global__ void k_crt_combine(const unsigned char *__restrict__ res, size_t per_
         const PanelGPU &Pn = in.panels[in.tri_leaf[row]];
         const double *a = in.A + (in.kop ? Pn.offK : Pn.offV) + (size_t)(row - Pn.row0) * in.ncol_pad;
         for (int d = 0; d <= t - (iv - 1) * in.ls && d <= t; ++d, a += (size_t)Pn.rows_pad * in.ncol_pad)
-            for (int c = 0; c < in.ncol; ++c) {
+            for (int c = 0; c < in.ncol && y == y; ++c) {  // NaN stays
                 const double v = in.x[(size_t)(rt - d) * in.ncol + (in.perm ? in.perm[c] : c)];
                 if (!isfinite(v)) y += a[c] * v;
             }
